@@ -1566,26 +1566,42 @@ __global__ void __launch_bounds__(kThreads, 3) k_multi(const __grid_constant__ M
 // Selection of points by many query polygons at once (§5.2 "Spatial
 // Selection", one pass over the points for all queries).  The join runs once
 // and yields (point, query) pairs in point order; the pairs are then
-// partitioned by query, keeping point order: each super-tile of kSuperTile
-// pairs counts its pairs per query into a query-major table; an exclusive scan
+// partitioned by query, keeping point order: each super-tile (super_tile(cap)
+// pairs) counts its pairs per query into a query-major table; an exclusive scan
 // of the table in query-major order makes entry (q, s) the output position of
 // super-tile s's first pair of query q; the emit kernel writes the point ids.
-constexpr int kSuperTile = 32768;
-constexpr int kSelMaxQ = 1024;                      // queries per index (shared-memory counters)
-constexpr int kSelWarpRange = kSuperTile / kWarps;  // pairs per warp of a super-tile
+// Pairs per super-tile: 32768 while the output is large (the table then costs
+// 8 B per 32768 / P pairs), halved while that leaves the chip without two
+// tiles per SM, down to 1024: an output of 50k ids is 50 tiles instead of 2,
+// and both kernels are chains of dependent steps per tile (50k ids of 16
+// queries: count + emit 169 -> 9.6 us; 84M ids of 256 queries keep 32768).
+constexpr int kSuperTileMax = 32768, kSuperTileMin = 1024;
+constexpr int kSelMaxQ = 1024;            // queries per index (shared-memory counters)
+constexpr int kPartTile = 4096;           // pairs that k_part_emit orders in shared memory at a time
+constexpr int kPartRounds = kPartTile / kThreads; // rounds of 32 pairs per warp and tile
+static_assert(kSelMaxQ == 4 * kThreads, "k_part_emit: four queries per thread");
+
+uint32_t super_tile(uint64_t cap)
+{
+    uint32_t t = kSuperTileMax;
+    while (t > kSuperTileMin && (cap + t - 1) / t < 2 * 152)
+        t >>= 1;
+    return t;
+}
 
 __global__ void __launch_bounds__(kThreads) k_part_count(const uint2 *__restrict__ pairs,
                                                          const unsigned long long *total, uint64_t cap, uint32_t P,
-                                                         unsigned long long *table, uint32_t n_super)
+                                                         unsigned long long *table, uint32_t n_super, uint32_t tile)
 {
     extern __shared__ uint32_t s_cnt[]; // P counters
     for (uint32_t q = threadIdx.x; q < P; q += kThreads)
         s_cnt[q] = 0;
     __syncthreads();
     const unsigned long long n = min(*total, (unsigned long long)cap); // pairs past cap were not written
-    const uint64_t base = (uint64_t)blockIdx.x * kSuperTile;
-    for (uint32_t j = threadIdx.x; j < (uint32_t)kSuperTile; j += kThreads) {
-        const bool has = base + j < n;
+    const uint64_t base = (uint64_t)blockIdx.x * tile;
+    const uint32_t m = base < n ? (uint32_t)min((unsigned long long)tile, n - base) : 0u;
+    for (uint32_t j = threadIdx.x; j < ((m + 31) & ~31u); j += kThreads) { // whole warps take part
+        const bool has = j < m;
         const uint32_t q = has ? __ldcg(&pairs[base + j].y) : 0u;
         hist_add_warp(s_cnt, has, q);
     }
@@ -1594,53 +1610,121 @@ __global__ void __launch_bounds__(kThreads) k_part_count(const uint2 *__restrict
         table[(uint64_t)q * n_super + blockIdx.x] = s_cnt[q];
 }
 
-__global__ void __launch_bounds__(kThreads) k_part_emit(const uint2 *__restrict__ pairs,
+// Writes the ids of a super-tile's pairs at their queries' positions.  Pairs
+// arrive in point order and neighbours rarely share a query, so writing each
+// id straight to its list touches another sector per lane (84M ids: 2.04 ms,
+// a quarter of the L2's sector rate and nothing else busy).  Instead the block
+// orders kPartTile pairs by query in shared memory (stable: every warp ranks
+// its own contiguous range with one match per round, a block scan turns
+// the (query, warp) counts into places), then writes them in that order, so
+// that consecutive threads write consecutive ids of a list (runs of 16 at 256
+// queries).  Shared memory: kPartSmem(P).
+constexpr size_t part_smem(uint32_t P)
+{
+    return size_t(P) * (8 + 8 + 2 * kWarps) + size_t(kPartTile) * (4 + 2);
+}
+
+__global__ void __launch_bounds__(kThreads, 4) k_part_emit(const uint2 *__restrict__ pairs,
                                                         const unsigned long long *total, uint32_t P,
                                                         const unsigned long long *table, uint32_t n_super,
-                                                        uint32_t *ids, uint64_t cap)
+                                                        uint32_t *ids, uint64_t cap, uint32_t tile)
 {
-    extern __shared__ unsigned long long s_run[]; // kWarps x P running positions
-    uint32_t *s_wc = reinterpret_cast<uint32_t *>(s_run + (size_t)kWarps * P); // kWarps x P counts
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    unsigned long long *s_run = reinterpret_cast<unsigned long long *>(s_raw); // P: next output position
+    unsigned long long *s_off = s_run + P;                                    // P: position - place in the tile
+    uint32_t *s_id = reinterpret_cast<uint32_t *>(s_off + P);                 // kPartTile ids in query order
+    uint16_t *s_qy = reinterpret_cast<uint16_t *>(s_id + kPartTile);          // and their queries
+    uint16_t *s_wc = s_qy + kPartTile;                                        // kWarps x P counts, then places
+    __shared__ uint32_t s_wsum[kWarps];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (uint32_t i = threadIdx.x; i < kWarps * P; i += kThreads)
-        s_wc[i] = 0;
-    __syncthreads();
     const unsigned long long n = min(*total, (unsigned long long)cap); // pairs past cap were not written
-    const uint64_t base = (uint64_t)blockIdx.x * kSuperTile + (uint64_t)warp * kSelWarpRange;
-    // 1. every warp counts its range per query
-    for (uint32_t j = lane; j < (uint32_t)kSelWarpRange; j += 32) {
-        const bool has = base + j < n;
-        const uint32_t q = has ? __ldcg(&pairs[base + j].y) : 0u;
-        hist_add_warp(s_wc + warp * P, has, q);
-    }
-    __syncthreads();
-    // 2. start positions per (warp, query)
-    for (uint32_t q = threadIdx.x; q < P; q += kThreads) {
-        unsigned long long pos = table[(uint64_t)q * n_super + blockIdx.x];
-        for (int w = 0; w < kWarps; ++w) {
-            s_run[w * P + q] = pos;
-            pos += s_wc[w * P + q];
+    const uint64_t base = (uint64_t)blockIdx.x * tile;
+    if (base >= n)
+        return;
+    const uint32_t mt = (uint32_t)min((unsigned long long)tile, n - base);
+    for (uint32_t q = threadIdx.x; q < P; q += kThreads)
+        s_run[q] = table[(uint64_t)q * n_super + blockIdx.x];
+    for (uint32_t t0 = 0; t0 < mt; t0 += kPartTile) {
+        const uint32_t m = min(mt - t0, (uint32_t)kPartTile);
+        for (uint32_t i = threadIdx.x; i < kWarps * P / 2; i += kThreads)
+            reinterpret_cast<uint32_t *>(s_wc)[i] = 0u; // kWarps is even
+        __syncthreads();
+        // 1. every warp counts its range per query and ranks its pairs
+        const uint32_t span = (m + kThreads - 1) / kThreads * 32, w0 = warp * span, w1 = min(m, w0 + span);
+        uint2 pr[kPartRounds]; // (id, query), the query's word then with the rank in its upper half
+#pragma unroll
+        for (int r = 0; r < kPartRounds; ++r) {
+            const uint32_t j = w0 + r * 32 + lane;
+            pr[r] = j < w1 ? __ldcs(&pairs[base + t0 + j]) : make_uint2(0u, 0xffffffffu);
         }
-    }
-    __syncthreads();
-    // 3. every warp writes its range in pair (= point) order: lanes with the
-    //    same query take consecutive positions in lane order
-    for (uint32_t j0 = 0; j0 < (uint32_t)kSelWarpRange; j0 += 32) {
-        if (base + j0 >= n)
-            break;
-        const bool has = base + j0 + lane < n;
-        const uint2 pr = has ? __ldcg(&pairs[base + j0 + lane]) : make_uint2(0u, 0xffffffffu);
-        const uint32_t peers = __match_any_sync(kFull, pr.y);
-        const unsigned long long start = has ? s_run[warp * P + pr.y] : 0ull;
-        __syncwarp();
-        if (has) {
-            const unsigned long long o = start + __popc(peers & lanemask_lt());
+        uint16_t *wc = s_wc + warp * P;
+#pragma unroll
+        for (int r = 0; r < kPartRounds; ++r) {
+            if (r * 32 >= span)
+                break;
+            const bool has = w0 + r * 32 + lane < w1;
+            const uint32_t q = pr[r].y, peers = __match_any_sync(kFull, q);
+            const uint32_t before = has ? wc[q] : 0u;
+            __syncwarp();
+            if (has && lane == __ffs(peers) - 1)
+                wc[q] = (uint16_t)(before + __popc(peers));
+            __syncwarp();
+            pr[r].y = q | (before + __popc(peers & lanemask_lt())) << 16;
+        }
+        __syncthreads();
+        // 2. places: queries in order, within a query the warps in order
+        uint32_t c4[4], mine = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t q = threadIdx.x * 4 + k;
+            c4[k] = 0;
+            if (q < P)
+                for (int w = 0; w < kWarps; ++w)
+                    c4[k] += s_wc[w * P + q];
+            mine += c4[k];
+        }
+        uint32_t inc = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t v = __shfl_up_sync(kFull, inc, o);
+            if (lane >= o)
+                inc += v;
+        }
+        if (lane == 31)
+            s_wsum[warp] = inc;
+        __syncthreads();
+        uint32_t at = inc - mine;
+        for (int w = 0; w < warp; ++w)
+            at += s_wsum[w];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t q = threadIdx.x * 4 + k;
+            if (q < P) {
+                s_off[q] = s_run[q] - at; // modulo 2^64: a place of the query is at or above `at`
+                s_run[q] += c4[k];
+                for (int w = 0; w < kWarps; ++w) {
+                    const uint16_t c = s_wc[w * P + q];
+                    s_wc[w * P + q] = (uint16_t)at;
+                    at += c;
+                }
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < kPartRounds; ++r)
+            if (w0 + r * 32 + lane < w1) {
+                const uint32_t q = pr[r].y & 0xffffu, pl = wc[q] + (pr[r].y >> 16);
+                s_id[pl] = pr[r].x;
+                s_qy[pl] = (uint16_t)q;
+            }
+        __syncthreads();
+        // 3. out, in list order
+        for (uint32_t i = threadIdx.x; i < m; i += kThreads) {
+            const unsigned long long o = s_off[s_qy[i]] + i;
             if (o < cap)
-                ids[o] = pr.x;
-            if ((int)lane == __ffs(peers) - 1)
-                s_run[warp * P + pr.y] = start + __popc(peers);
+                ids[o] = s_id[i];
         }
-        __syncwarp();
+        __syncthreads(); // s_off and the places are rewritten by the next tile
     }
 }
 
@@ -2968,7 +3052,10 @@ size_t select_scratch_bytes(uint64_t n, uint32_t P, uint64_t cap)
 
 size_t partition_scratch_bytes(uint64_t cap, uint32_t P)
 {
-    const uint64_t n_super = (cap + kSuperTile - 1) / kSuperTile;
+    // super_tile leaves fewer than 608 tiles, or takes the largest or the
+    // smallest size; this bound, unlike the count itself, grows with cap
+    const uint64_t n_super = std::max((cap + kSuperTileMax - 1) / kSuperTileMax,
+                                      std::min<uint64_t>((cap + kSuperTileMin - 1) / kSuperTileMin, 608));
     const uint64_t tab = uint64_t(P) * (n_super ? n_super : 1);
     return size_t(tab * 8 + (scan_partials(tab) + 2) * 8 + 64);
 }
@@ -2978,7 +3065,8 @@ cudaError_t launch_partition(const uint2 *pairs, const unsigned long long *total
 {
     if (P > (uint32_t)kSelMaxQ)
         return cudaErrorInvalidValue;
-    const uint64_t n_super64 = (cap + kSuperTile - 1) / kSuperTile;
+    const uint32_t tile = super_tile(cap);
+    const uint64_t n_super64 = (cap + tile - 1) / tile;
     if (n_super64 >= (1ull << 31))
         return cudaErrorInvalidValue;
     if (P == 0)
@@ -2988,18 +3076,17 @@ cudaError_t launch_partition(const uint2 *pairs, const unsigned long long *total
     unsigned long long *part = table + uint64_t(P) * n_super;
     unsigned long long *tab_total = part + scan_partials(uint64_t(P) * n_super) + 1;
     // per (query, super-tile) counts of the pairs, scanned in query-major order
-    k_part_count<<<n_super, kThreads, sizeof(uint32_t) * P, s>>>(pairs, total, cap, P, table, n_super);
+    k_part_count<<<n_super, kThreads, sizeof(uint32_t) * P, s>>>(pairs, total, cap, P, table, n_super, tile);
     cudaError_t e = launch_scan(table, uint64_t(P) * n_super, tab_total, part, s);
     if (e != cudaSuccess)
         return e;
     k_sel_offsets<<<(P + 256) / 256, 256, 0, s>>>(table, n_super, P, total, offsets);
     // point ids, ascending per query
     static bool done[64] = {};
-    if ((e = smem_opt_in(k_part_emit, (sizeof(unsigned long long) + 4) * kWarps * kSelMaxQ, done)) != cudaSuccess)
+    if ((e = smem_opt_in(k_part_emit, part_smem(kSelMaxQ), done)) != cudaSuccess)
         return e;
     if (cap)
-        k_part_emit<<<n_super, kThreads, (sizeof(unsigned long long) + 4) * size_t(kWarps) * P, s>>>(
-            pairs, total, P, table, n_super, ids, cap);
+        k_part_emit<<<n_super, kThreads, part_smem(P), s>>>(pairs, total, P, table, n_super, ids, cap, tile);
     return cudaGetLastError();
 }
 
