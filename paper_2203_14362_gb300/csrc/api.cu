@@ -72,6 +72,8 @@ struct Aux {
     unsigned long long total;           // internal total when the caller passes none
 };
 
+constexpr size_t kPinnedBytes = 128;
+
 } // namespace
 
 struct spx_ctx {
@@ -82,6 +84,7 @@ struct spx_ctx {
     std::map<uint64_t, std::unique_ptr<PolysObj>> polys;
     std::map<uint64_t, std::unique_ptr<IndexObj>> indexes;
     Aux *aux = nullptr;
+    char *pinned = nullptr; // kPinnedBytes of host memory: a call's status and total come back here
     void *scratch = nullptr;
     size_t scratch_bytes = 0;
     // staging buffers of spx_join_host
@@ -173,18 +176,49 @@ spx_status ensure(spx_ctx *ctx, void **buf, size_t *have, size_t need, cudaStrea
     return SPX_OK;
 }
 
-// Read and clear the kernel error word (synchronises the stream).
-spx_status check_kernel_err(spx_ctx *ctx, cudaStream_t s)
+// The status of what ran on s (synchronises it): reads the kernel error word,
+// and clears it when set, and with `total` (a device word) the output's size
+// into *n.  Both come over as asynchronous copies into pinned words with one
+// wait for the stream: a wait and two synchronous copies to pageable memory
+// took 40 us of a 63 us join of 20k points, this takes 21 us.
+spx_status read_status(spx_ctx *ctx, cudaStream_t s, const unsigned long long *total, uint64_t *n)
 {
+    static_assert(sizeof(Aux) <= kPinnedBytes - 8, "the pinned words hold Aux and one total");
+    Aux *h = reinterpret_cast<Aux *>(ctx->pinned);
+    unsigned long long *ht = reinterpret_cast<unsigned long long *>(ctx->pinned + kPinnedBytes - 8);
+    SPX_CUDA(cudaMemcpyAsync(h, ctx->aux, sizeof(Aux), cudaMemcpyDeviceToHost, s), "read error word");
+    const bool own = total == &ctx->aux->total;
+    if (total && !own)
+        SPX_CUDA(cudaMemcpyAsync(ht, total, 8, cudaMemcpyDeviceToHost, s), "read total");
     SPX_CUDA(cudaStreamSynchronize(s), "stream synchronize");
-    unsigned w = 0;
-    SPX_CUDA(cudaMemcpy(&w, &ctx->aux->err, sizeof(w), cudaMemcpyDeviceToHost), "read error word");
-    if (w) {
+    if (h->err) {
+        const unsigned w = h->err;
         SPX_CUDA(cudaMemset(&ctx->aux->err, 0, sizeof(unsigned)), "clear error word");
         if (w & kErrTimeout)
             return fail(ctx, SPX_ETIMEOUT, "a bounded device wait gave up; results of that call are invalid");
         return fail(ctx, SPX_EKERNEL, "kernel reported an internal error");
     }
+    if (total)
+        *n = own ? h->total : *ht;
+    return SPX_OK;
+}
+spx_status check_kernel_err(spx_ctx *ctx, cudaStream_t s) { return read_status(ctx, s, nullptr, nullptr); }
+
+// The end of a call that reports its output's size (n_out not null): waits,
+// and SPX_ECAPACITY when the size exceeds cap.
+spx_status report_total(spx_ctx *ctx, cudaStream_t s, const unsigned long long *total, uint64_t cap, uint64_t *n_out,
+                        const char *what, const char *unit)
+{
+    if (!n_out)
+        return SPX_OK;
+    uint64_t t = 0;
+    const spx_status st = read_status(ctx, s, total, &t);
+    if (st != SPX_OK)
+        return st;
+    *n_out = t;
+    if (t > cap)
+        return fail(ctx, SPX_ECAPACITY, std::string(what) + ": " + std::to_string(t) + " " + unit +
+                                            " exceed capacity " + std::to_string(cap));
     return SPX_OK;
 }
 
@@ -277,17 +311,7 @@ spx_status disk_join_common(spx_ctx *ctx, PointsObj *pts, IndexObj *ix, uint32_t
         return cuda_fail(ctx, e, "join launch");
     if (timed && pts->n && (st = add_phase_times(ctx, false)) != SPX_OK)
         return st;
-    if (n_pairs) {
-        if ((st = check_kernel_err(ctx, s)) != SPX_OK)
-            return st;
-        unsigned long long t = 0;
-        SPX_CUDA(cudaMemcpy(&t, a.total, sizeof(t), cudaMemcpyDeviceToHost), "read total");
-        *n_pairs = t;
-        if (t > cap)
-            return fail(ctx, SPX_ECAPACITY, "join: " + std::to_string(t) + " pairs exceed capacity " +
-                                                std::to_string(cap));
-    }
-    return SPX_OK;
+    return report_total(ctx, s, a.total, cap, n_pairs, "join", "pairs");
 }
 
 BufferLaunch buffer_launch(spx_ctx *ctx, PointsObj *pts, IndexObj *ix)
@@ -323,17 +347,7 @@ spx_status buffer_join_common(spx_ctx *ctx, PointsObj *pts, IndexObj *ix, uint32
     cudaError_t e = launch_buffer_join(a, ctx->scratch, s);
     if (e != cudaSuccess)
         return cuda_fail(ctx, e, "join launch");
-    if (n_pairs) {
-        if ((st = check_kernel_err(ctx, s)) != SPX_OK)
-            return st;
-        unsigned long long t = 0;
-        SPX_CUDA(cudaMemcpy(&t, a.total, sizeof(t), cudaMemcpyDeviceToHost), "read total");
-        *n_pairs = t;
-        if (t > cap)
-            return fail(ctx, SPX_ECAPACITY, "join: " + std::to_string(t) + " pairs exceed capacity " +
-                                                std::to_string(cap));
-    }
-    return SPX_OK;
+    return report_total(ctx, s, a.total, cap, n_pairs, "join", "pairs");
 }
 
 spx_status join_common(spx_ctx *ctx, spx_points points, spx_index index, uint32_t *pairs_dev, uint64_t cap,
@@ -380,18 +394,7 @@ spx_status join_common(spx_ctx *ctx, spx_points points, spx_index index, uint32_
         return cuda_fail(ctx, e, "join launch");
     if (timed && pts->n && (st = add_phase_times(ctx, true)) != SPX_OK)
         return st;
-    if (n_pairs) {
-        st = check_kernel_err(ctx, s);
-        if (st != SPX_OK)
-            return st;
-        unsigned long long t = 0;
-        SPX_CUDA(cudaMemcpy(&t, a.total, sizeof(t), cudaMemcpyDeviceToHost), "read total");
-        *n_pairs = t;
-        if (t > cap)
-            return fail(ctx, SPX_ECAPACITY, "join: " + std::to_string(t) + " pairs exceed capacity " +
-                                                std::to_string(cap));
-    }
-    return SPX_OK;
+    return report_total(ctx, s, a.total, cap, n_pairs, "join", "pairs");
 }
 
 // Scratch of the allocation-free plain join (spx_join_plain_static): one
@@ -696,6 +699,8 @@ spx_status spx_create(int device, spx_ctx **out)
         return SPX_ENOMEM;
     if (cudaMemset(c->aux, 0, sizeof(Aux)) != cudaSuccess)
         return SPX_ECUDA;
+    if (cudaMallocHost(reinterpret_cast<void **>(&c->pinned), kPinnedBytes) != cudaSuccess)
+        return SPX_ENOMEM;
     if (cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking) != cudaSuccess)
         return SPX_ECUDA;
     *out = c.release();
@@ -716,6 +721,7 @@ void spx_destroy(spx_ctx *ctx)
         cudaFree(kv.second->cell_end);
     }
     cudaFree(ctx->aux);
+    cudaFreeHost(ctx->pinned);
     cudaFree(ctx->scratch);
     cudaFree(ctx->st_pts);
     cudaFree(ctx->st_pairs);
@@ -1440,17 +1446,7 @@ spx_status spx_select(spx_ctx *ctx, spx_points points, spx_index index, uint32_t
         cudaError_t e = launch_buffer_select(buffer_launch(ctx, pts, ix), ids_dev, cap, offs, ctx->scratch, s);
         if (e != cudaSuccess)
             return cuda_fail(ctx, e, "select launch");
-        if (n_ids) {
-            if ((st = check_kernel_err(ctx, s)) != SPX_OK)
-                return st;
-            unsigned long long t = 0;
-            SPX_CUDA(cudaMemcpy(&t, offs + PQ, sizeof(t), cudaMemcpyDeviceToHost), "select total");
-            *n_ids = t;
-            if (t > cap)
-                return fail(ctx, SPX_ECAPACITY, "select: " + std::to_string(t) + " ids exceed capacity " +
-                                                    std::to_string(cap));
-        }
-        return SPX_OK;
+        return report_total(ctx, s, offs + PQ, cap, n_ids, "select", "ids");
     }
     if (ix->kind == 1) {
         // distance selection: points within r of each centre, ascending per disk
@@ -1467,17 +1463,7 @@ spx_status spx_select(spx_ctx *ctx, spx_points points, spx_index index, uint32_t
         cudaError_t e = launch_disk_select(a, ids_dev, cap, offs, ctx->scratch, s);
         if (e != cudaSuccess)
             return cuda_fail(ctx, e, "select launch");
-        if (n_ids) {
-            if ((st = check_kernel_err(ctx, s)) != SPX_OK)
-                return st;
-            unsigned long long t = 0;
-            SPX_CUDA(cudaMemcpy(&t, offs + PQ, sizeof(t), cudaMemcpyDeviceToHost), "select total");
-            *n_ids = t;
-            if (t > cap)
-                return fail(ctx, SPX_ECAPACITY, "select: " + std::to_string(t) + " ids exceed capacity " +
-                                                    std::to_string(cap));
-        }
-        return SPX_OK;
+        return report_total(ctx, s, offs + PQ, cap, n_ids, "select", "ids");
     }
     spx_status st = ensure(ctx, &ctx->scratch, &ctx->scratch_bytes, select_scratch_bytes(pts->n, ix->view.P, cap), s,
                            "select");
@@ -1521,18 +1507,7 @@ spx_status spx_select(spx_ctx *ctx, spx_points points, spx_index index, uint32_t
     } else {
         SPX_CUDA(cudaGraphLaunch(it->second, s), "select graph launch");
     }
-    if (n_ids) {
-        st = check_kernel_err(ctx, s);
-        if (st != SPX_OK)
-            return st;
-        unsigned long long t = 0;
-        SPX_CUDA(cudaMemcpy(&t, offs + ix->view.P, sizeof(t), cudaMemcpyDeviceToHost), "select total");
-        *n_ids = t;
-        if (t > cap)
-            return fail(ctx, SPX_ECAPACITY, "select: " + std::to_string(t) + " ids exceed capacity " +
-                                                std::to_string(cap));
-    }
-    return SPX_OK;
+    return report_total(ctx, s, offs + ix->view.P, cap, n_ids, "select", "ids");
 }
 
 spx_status spx_aggregate(spx_ctx *ctx, spx_points points, spx_index index, uint64_t *counts_dev, void *stream)
