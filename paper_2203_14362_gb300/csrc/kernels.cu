@@ -617,70 +617,70 @@ __global__ void __launch_bounds__(kPlainThreads) k_plain_count(JoinLaunch a, uns
     }
 }
 
-__global__ void __launch_bounds__(1024) k_scan(unsigned long long *v, uint64_t n, unsigned long long *total)
-{
-    // exclusive scan of n values by one block: chunks of 1024 with a carried total
-    __shared__ unsigned long long s_w[32];
-    __shared__ unsigned long long s_carry;
-    if (threadIdx.x == 0)
-        s_carry = 0;
-    __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (uint64_t b = 0; b < n; b += 1024) {
-        const uint64_t i = b + threadIdx.x;
-        const unsigned long long x = i < n ? v[i] : 0ull;
-        unsigned long long inc = x;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long t = __shfl_up_sync(kFull, inc, o);
-            if (lane >= o)
-                inc += t;
-        }
-        if (lane == 31)
-            s_w[warp] = inc;
-        __syncthreads();
-        if (warp == 0) {
-            const unsigned long long w = s_w[lane];
-            unsigned long long wi = w;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned long long t = __shfl_up_sync(kFull, wi, o);
-                if (lane >= o)
-                    wi += t;
-            }
-            s_w[lane] = wi - w;
-        }
-        __syncthreads();
-        const unsigned long long carry = s_carry;
-        if (i < n)
-            v[i] = carry + s_w[warp] + inc - x;
-        __syncthreads();
-        if (threadIdx.x == 1023)
-            s_carry = carry + s_w[warp] + inc;
-        __syncthreads();
-    }
-    if (threadIdx.x == 0 && total)
-        *total = s_carry;
-}
-
-// Device-wide exclusive scan for long arrays: per-chunk sums, a one-block scan
-// of the sums, then every chunk rescanned from its base.
+// Exclusive scan by blocks of 1024 threads, kScanChunk values per step.  A warp
+// takes 256 consecutive values as eight rows of 32, so its loads and stores are
+// whole lines (eight consecutive values per thread touched 16 lines per access:
+// 67M values 399 -> 163 us in k_scan_apply, 11,719 values 14.4 -> 7.7 us in
+// k_scan, where one SM's L1 does it all).
 constexpr int kScanItems = 8;
 constexpr uint64_t kScanChunk = 1024 * kScanItems;
 
-__device__ __forceinline__ unsigned long long block_exclusive_scan_1024(unsigned long long x, unsigned long long &total,
-                                                                        unsigned long long *s_w)
+// Loads this thread's values of the step that starts at v[b]: row j of warp w
+// is v[b + 256 w + 32 j ..].
+__device__ __forceinline__ void scan_load(const unsigned long long *v, uint64_t b, uint64_t n,
+                                          unsigned long long (&x)[kScanItems])
+{
+    const uint64_t i0 = b + (threadIdx.x >> 5) * (32 * kScanItems) + (threadIdx.x & 31);
+#pragma unroll
+    for (int j = 0; j < kScanItems; ++j)
+        x[j] = i0 + 32 * j < n ? v[i0 + 32 * j] : 0ull;
+}
+
+// Turns the values of a step into their exclusive prefixes within the step
+// (x[j] becomes the prefix) and returns the step's sum.  s_w: 33 words.
+__device__ __forceinline__ unsigned long long scan_step(unsigned long long (&x)[kScanItems], unsigned long long *s_w)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    unsigned long long inc = x;
+    unsigned long long any = 0, wsum = 0;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long t = __shfl_up_sync(kFull, inc, o);
-        if (lane >= o)
-            inc += t;
+    for (int j = 0; j < kScanItems; ++j)
+        any |= x[j];
+    if (!__any_sync(kFull, (any >> 27) != 0)) { // a row's sum fits 32 bits
+#pragma unroll
+        for (int j = 0; j < kScanItems; ++j) {
+            const uint32_t v = (uint32_t)x[j];
+            uint32_t inc = v;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t t = __shfl_up_sync(kFull, inc, o);
+                if (lane >= o)
+                    inc += t;
+            }
+            x[j] = wsum + (inc - v);
+            wsum += __shfl_sync(kFull, inc, 31);
+        }
+    } else {
+#pragma unroll 1
+        for (int j = 0; j < kScanItems; ++j) {
+            unsigned long long v = 0, inc;
+#pragma unroll
+            for (int k = 0; k < kScanItems; ++k) // x stays in registers
+                v = k == j ? x[k] : v;
+            inc = v;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned long long t = __shfl_up_sync(kFull, inc, o);
+                if (lane >= o)
+                    inc += t;
+            }
+#pragma unroll
+            for (int k = 0; k < kScanItems; ++k)
+                x[k] = k == j ? wsum + (inc - v) : x[k];
+            wsum += __shfl_sync(kFull, inc, 31);
+        }
     }
-    if (lane == 31)
-        s_w[warp] = inc;
+    if (lane == 0)
+        s_w[warp] = wsum;
     __syncthreads();
     if (warp == 0) {
         const unsigned long long w = s_w[lane];
@@ -696,46 +696,70 @@ __device__ __forceinline__ unsigned long long block_exclusive_scan_1024(unsigned
             s_w[32] = wi;
     }
     __syncthreads();
-    total = s_w[32];
-    const unsigned long long ex = s_w[warp] + inc - x;
-    __syncthreads();
-    return ex;
+    const unsigned long long before = s_w[warp], total = s_w[32];
+#pragma unroll
+    for (int j = 0; j < kScanItems; ++j)
+        x[j] += before;
+    __syncthreads(); // s_w is rewritten by the next step
+    return total;
 }
 
+__device__ __forceinline__ void scan_store(unsigned long long *v, uint64_t b, uint64_t n, unsigned long long base,
+                                           const unsigned long long (&x)[kScanItems])
+{
+    const uint64_t i0 = b + (threadIdx.x >> 5) * (32 * kScanItems) + (threadIdx.x & 31);
+#pragma unroll
+    for (int j = 0; j < kScanItems; ++j)
+        if (i0 + 32 * j < n)
+            v[i0 + 32 * j] = base + x[j];
+}
+
+// One block, the steps one after the other with a carried total.
+__global__ void __launch_bounds__(1024) k_scan(unsigned long long *v, uint64_t n, unsigned long long *total)
+{
+    __shared__ unsigned long long s_w[33];
+    unsigned long long carry = 0, x[kScanItems];
+    for (uint64_t b = 0; b < n; b += kScanChunk) {
+        scan_load(v, b, n, x);
+        const unsigned long long t = scan_step(x, s_w);
+        scan_store(v, b, n, carry, x);
+        carry += t;
+    }
+    if (threadIdx.x == 0 && total)
+        *total = carry;
+}
+
+// Device-wide exclusive scan for long arrays: per-chunk sums, a one-block scan
+// of the sums, then every chunk rescanned from its base.
 __global__ void __launch_bounds__(1024) k_scan_partials(const unsigned long long *v, uint64_t n,
                                                         unsigned long long *part)
 {
-    __shared__ unsigned long long s_w[33];
-    const uint64_t b0 = (uint64_t)blockIdx.x * kScanChunk + (uint64_t)threadIdx.x * kScanItems;
-    unsigned long long sum = 0;
+    __shared__ unsigned long long s_w[32];
+    unsigned long long x[kScanItems], sum = 0;
+    scan_load(v, (uint64_t)blockIdx.x * kScanChunk, n, x);
 #pragma unroll
     for (int j = 0; j < kScanItems; ++j)
-        sum += (b0 + j < n) ? v[b0 + j] : 0ull;
-    unsigned long long total;
-    block_exclusive_scan_1024(sum, total, s_w);
-    if (threadIdx.x == 0)
-        part[blockIdx.x] = total;
+        sum += x[j];
+    sum = warp_sum64(sum);
+    if ((threadIdx.x & 31) == 0)
+        s_w[threadIdx.x >> 5] = sum;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        sum = warp_sum64(s_w[threadIdx.x]);
+        if (threadIdx.x == 0)
+            part[blockIdx.x] = sum;
+    }
 }
 
 __global__ void __launch_bounds__(1024) k_scan_apply(unsigned long long *v, uint64_t n,
                                                      const unsigned long long *part_off)
 {
     __shared__ unsigned long long s_w[33];
-    const uint64_t b0 = (uint64_t)blockIdx.x * kScanChunk + (uint64_t)threadIdx.x * kScanItems;
-    unsigned long long x[kScanItems], sum = 0;
-#pragma unroll
-    for (int j = 0; j < kScanItems; ++j) {
-        x[j] = (b0 + j < n) ? v[b0 + j] : 0ull;
-        sum += x[j];
-    }
-    unsigned long long total;
-    unsigned long long run = part_off[blockIdx.x] + block_exclusive_scan_1024(sum, total, s_w);
-#pragma unroll
-    for (int j = 0; j < kScanItems; ++j) {
-        if (b0 + j < n)
-            v[b0 + j] = run;
-        run += x[j];
-    }
+    const uint64_t b = (uint64_t)blockIdx.x * kScanChunk;
+    unsigned long long x[kScanItems];
+    scan_load(v, b, n, x);
+    scan_step(x, s_w);
+    scan_store(v, b, n, part_off[blockIdx.x], x);
 }
 
 __device__ __forceinline__ uint32_t warp_sum32(uint32_t v)
@@ -911,11 +935,16 @@ constexpr int kWalkQueue = 64; // < 32 rows carried over + one gather step of 32
 #define SPX_WALK_BATCH 4
 #endif
 constexpr int kWalkBatch = SPX_WALK_BATCH;
-#ifndef SPX_WALK_RANGE
-#define SPX_WALK_RANGE 512
-#endif
-constexpr int kWalkRange = SPX_WALK_RANGE; // bitmap words (of 32 rows) per warp of pass 1b
-static_assert(kWalkRange % (32 * SPX_WALK_BATCH) == 0, "a warp's range is whole steps");
+// A warp's range: short enough that a small table's words fill the chip twice
+// over (1M points: 61 warps of 512 words took 20.3 us, 977 of 32 take 7.5; 3M:
+// 22.7 -> 14.0), at most 512 (100M points: within 2 us from 256 to 1024).
+constexpr int kWalkRangeMax = 512, kWalkRangeMin = 32; // bitmap words (of 32 rows) per warp of pass 1b
+uint32_t walk_range(uint64_t nwords)
+{
+    const uint64_t warps = 2ull * kWalkMinBlocks * kWarps * uint64_t(device_sm_count());
+    const uint64_t r = (nwords / warps + 31) & ~uint64_t(31); // whole steps of a lane per word
+    return uint32_t(std::min<uint64_t>(std::max<uint64_t>(r, kWalkRangeMin), kWalkRangeMax));
+}
 
 // With the block summary (SUM), a CTA of 1024 threads (one per SM) first
 // copies the summary into shared memory; a point whose block is empty or
@@ -1112,7 +1141,8 @@ __global__ void __launch_bounds__(THREADS, SUM ? 1 : (TMA ? 6 : kResolveMinBlock
 }
 
 template <bool FP32, bool R16>
-__global__ void __launch_bounds__(kThreads, kWalkMinBlocks) k_walk(JoinLaunch a, uint32_t *pend, uint32_t nwords)
+__global__ void __launch_bounds__(kThreads, kWalkMinBlocks) k_walk(JoinLaunch a, uint32_t *pend, uint32_t nwords,
+                                                                   uint32_t range)
 {
     __shared__ uint32_t s_qa[kWarps * kWalkQueue];
     __shared__ uint32_t s_pa[kWarps * kWaveWords];
@@ -1169,8 +1199,8 @@ __global__ void __launch_bounds__(kThreads, kWalkMinBlocks) k_walk(JoinLaunch a,
         __syncwarp(); // the queue is rewritten after the round
     };
     constexpr int B = kWalkBatch; // bitmap words per lane per step, the next step's loaded ahead
-    const uint64_t w0 = ((uint64_t)blockIdx.x * kWarps + warp) * kWalkRange;
-    const uint64_t w1 = min((uint64_t)nwords, w0 + kWalkRange);
+    const uint64_t w0 = ((uint64_t)blockIdx.x * kWarps + warp) * range;
+    const uint64_t w1 = min((uint64_t)nwords, w0 + range);
     uint32_t qn = 0;
     uint32_t nxt[B];
 #pragma unroll
@@ -1220,6 +1250,129 @@ __global__ void __launch_bounds__(kThreads, kWalkMinBlocks) k_walk(JoinLaunch a,
     add_stats(a.stats, 0u, n_tests, n_esc, n_pairs);
 }
 
+// Pass 1 of a small table in one launch: a warp per 256-point chunk resolves its
+// points as pass 1a does and walks its own list points at once.  A table of up
+// to kSmallChunks chunks is bound by launches and by chains of dependent loads,
+// not by bandwidth, and the persistent CTAs of pass 1a would copy the 128 KB
+// summary for a few chunks each.  CTA of kThreads, no barrier between its warps
+// but for the counters (a CTA's points counted in shared memory when P is at
+// most kSmallHist).  Whole join with k_wemit<SELF>, against pass 1a + 1b + scan
+// + pass 3, 2000-cell map: 20k points 18.5 against 28.8 us, 500k 20.6 / 32.8,
+// 1M 32.8 / 39.0, 1.5M 39.0 / 39.1, 2M 53.7 / 43.1; the line is at 1M points.
+constexpr uint32_t kSmallChunks = 4096;
+constexpr uint32_t kSmallHist = 2048;
+
+template <bool FP32, bool R16>
+__global__ void __launch_bounds__(kThreads, 3) k_small(const __grid_constant__ JoinLaunch a, uint32_t *pend,
+                                                       uint32_t nchunks, int use_hist)
+{
+    __shared__ uint4 s_qa[kWarps * kWChunk]; // (x, y, first entry, row in the chunk)
+    __shared__ uint32_t s_pa[kWarps * kWaveWords];
+    __shared__ uint32_t s_ma[kWarps * kWItems]; // rows in several polygons
+    __shared__ uint32_t s_hist[kSmallHist];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint4 *s_q = s_qa + warp * kWChunk;
+    uint32_t *s_m = s_ma + warp * kWItems;
+    const IndexView &ix = a.ix;
+    const uint64_t keep = policy_evict_last();
+    const bool hist = use_hist && a.counts;
+    uint32_t n_tests = 0, n_esc = 0, total = 0, npts = 0;
+    if (hist) {
+        for (uint32_t i = threadIdx.x; i < ix.P; i += kThreads)
+            s_hist[i] = 0;
+        __syncthreads();
+    }
+    auto count1 = [&](bool has, uint32_t q) {
+        if (has && a.counts)
+            hist ? (void)atomicAdd(s_hist + q, 1u) : (void)atomicAdd(a.counts + q, 1ull);
+    };
+    const uint32_t ch = blockIdx.x * kWarps + warp;
+    if (ch < nchunks) {
+        const uint64_t base = (uint64_t)ch * kWChunk;
+        npts = (uint32_t)min((uint64_t)kWChunk, a.n - base);
+        uint32_t *res = a.res + base;
+        unsigned short *res16 = reinterpret_cast<unsigned short *>(a.res) + base;
+        int2 p[kWItems];
+        uint32_t w[kWItems];
+#pragma unroll
+        for (int j = 0; j < kWItems; ++j) {
+            const uint32_t loc = j * 32 + lane;
+            p[j] = loc < npts ? __ldcs(a.pts + base + loc) : make_int2(-1, -1);
+        }
+#pragma unroll
+        for (int j = 0; j < kWItems; ++j) {
+            w[j] = 0u;
+            if ((uint32_t)(p[j].x | p[j].y) < kBox)
+                w[j] = coarse_word(ix, (uint32_t)p[j].x, (uint32_t)p[j].y, keep);
+        }
+#pragma unroll
+        for (int j = 0; j < kWItems; ++j)
+            if ((w[j] >> 30) == kCellSub)
+                w[j] = fine_word(ix, w[j], (uint32_t)p[j].x, (uint32_t)p[j].y, keep);
+        if (lane < kWItems)
+            s_m[lane] = 0u;
+        uint32_t qn = 0;
+#pragma unroll
+        for (int j = 0; j < kWItems; ++j) {
+            const uint32_t kind = w[j] >> 30, loc = j * 32 + lane, pay = w[j] & kPayloadMask;
+            const bool one = kind == kCellInsideOne && in_bounds(pay < ix.P, ix), lst = kind == kCellList;
+            total += one ? 1u : 0u;
+            count1(one, pay);
+            if (loc < npts && !lst) {
+                if (R16)
+                    __stcg(res16 + loc, (unsigned short)(one ? pay : kRes16None));
+                else
+                    __stcg(res + loc, one ? pay : kResNone);
+            }
+            const uint32_t bl = __ballot_sync(kFull, lst);
+            if (lst)
+                s_q[qn + __popc(bl & lanemask_lt())] = make_uint4((uint32_t)p[j].x, (uint32_t)p[j].y, pay, loc);
+            qn += __popc(bl);
+        }
+        __syncwarp();
+        for (uint32_t k0 = 0; k0 < qn; k0 += 32) {
+            const bool has = k0 + lane < qn;
+            const uint4 it = s_q[has ? k0 + lane : k0]; // idle lanes walk nothing
+            uint32_t f = 0, c = 0;
+            uint64_t ids = 0; // R16 and a.aux: the first four polygons, 16 bits each
+            walk_list_wave<FP32>(ix, has, it.z, (int)it.x, (int)it.y, n_tests, n_esc, keep, s_pa + warp * kWaveWords,
+                                 [&](uint32_t q) {
+                                     if (R16 && c < 4)
+                                         ids |= (uint64_t)q << (16 * c);
+                                     f = c ? f : q;
+                                     ++c;
+                                     count1(true, q);
+                                 });
+            total += c;
+            if (has) {
+                if (R16) {
+                    __stcg(res16 + it.w, (unsigned short)(c == 0 ? kRes16None : c == 1 ? f : c));
+                    if (c >= 2) {
+                        atomicOr(s_m + (it.w >> 5), 1u << (it.w & 31));
+                        if (a.aux && c <= 4)
+                            __stcg(reinterpret_cast<unsigned long long *>(a.aux) + base + it.w, (unsigned long long)ids);
+                    }
+                } else {
+                    __stcg(res + it.w, res_encode(c, f));
+                }
+            }
+        }
+        __syncwarp();
+        if (lane < kWItems)
+            __stcg(pend + (uint64_t)ch * kWItems + lane, s_m[lane]);
+        const uint32_t t = warp_sum32(total);
+        if (lane == 0)
+            a.tile_tot[ch] = t;
+    }
+    if (hist) {
+        __syncthreads();
+        for (uint32_t i = threadIdx.x; i < ix.P; i += kThreads)
+            if (s_hist[i])
+                atomicAdd(a.counts + i, (unsigned long long)s_hist[i]);
+    }
+    add_stats(a.stats, lane == 0 ? npts : 0u, n_tests, n_esc, total);
+}
+
 // Pass 3 of the join with warp chunks: every warp writes the pairs of its
 // chunks from the stored per-point results at the chunk's scanned offset.
 // Lane order within a round of 32 points, rounds in order: point order.  A
@@ -1231,10 +1384,15 @@ __global__ void __launch_bounds__(kThreads, kWalkMinBlocks) k_walk(JoinLaunch a,
 constexpr size_t kEmitSmem = size_t(kWarps) * kWChunk * (sizeof(uint32_t) + sizeof(unsigned long long)) +
                              size_t(kWarps) * kWaveWords * sizeof(uint32_t);
 
-template <bool FP32, bool R16>
+//
+// With SELF (small tables, a warp per chunk) chunk_off holds the chunks' totals,
+// not their offsets: every CTA sums the totals before its first chunk itself
+// (at most 8 B x kSmallChunks from L2), which saves the scan's launch.
+template <bool FP32, bool R16, bool SELF>
 __global__ void __launch_bounds__(kThreads, 3) k_wemit(JoinLaunch a, const unsigned long long *chunk_off,
                                                        uint32_t nchunks, const uint32_t *pend)
 {
+    __shared__ unsigned long long s_before[SELF ? kWarps : 1];
     extern __shared__ __align__(16) unsigned char s_raw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     unsigned long long *s_o = reinterpret_cast<unsigned long long *>(s_raw) + warp * kWChunk;
@@ -1245,10 +1403,27 @@ __global__ void __launch_bounds__(kThreads, 3) k_wemit(JoinLaunch a, const unsig
                       warp * kWaveWords; // words of walk_list_wave
     const uint64_t keep = policy_evict_last();
     const uint32_t nw = gridDim.x * kWarps;
+    unsigned long long before = 0; // SELF: the pairs before this warp's chunk
+    if (SELF) {
+        const uint32_t c0 = blockIdx.x * kWarps;
+        for (uint32_t i = threadIdx.x; i < c0; i += kThreads)
+            before += chunk_off[i];
+        before = warp_sum64(before);
+        if (lane == 0)
+            s_before[warp] = before;
+        __syncthreads();
+        before = 0;
+        for (int w = 0; w < kWarps; ++w)
+            before += s_before[w];
+        for (int w = 0; w < warp && c0 + w < nchunks; ++w)
+            before += chunk_off[c0 + w];
+        if (c0 + warp == nchunks - 1 && lane == 0 && a.total)
+            *a.total = before + chunk_off[nchunks - 1];
+    }
     for (uint32_t ch = blockIdx.x * kWarps + warp; ch < nchunks; ch += nw) {
         const uint64_t base = (uint64_t)ch * kWChunk;
         const uint32_t npts = (uint32_t)min((uint64_t)kWChunk, a.n - base);
-        unsigned long long run = chunk_off[ch] + (a.pair_base ? *a.pair_base : 0ull);
+        unsigned long long run = SELF ? before : chunk_off[ch] + (a.pair_base ? *a.pair_base : 0ull);
         uint32_t res[kWItems], mw = 0;
 #pragma unroll
         for (int j = 0; j < kWItems; ++j) {
@@ -1572,9 +1747,10 @@ __global__ void __launch_bounds__(kThreads, 3) k_multi(const __grid_constant__ M
 // super-tile s's first pair of query q; the emit kernel writes the point ids.
 // Pairs per super-tile: 32768 while the output is large (the table then costs
 // 8 B per 32768 / P pairs), halved while that leaves the chip without two
-// tiles per SM, down to 1024: an output of 50k ids is 50 tiles instead of 2,
-// and both kernels are chains of dependent steps per tile (50k ids of 16
-// queries: count + emit 169 -> 9.6 us; 84M ids of 256 queries keep 32768).
+// tiles per SM, down to 1024: both kernels are chains of dependent steps per
+// tile, and a small output was one or two of them (3M points x 16 queries,
+// room for 207k ids: count + emit 170 -> 11.6 us; 84M ids of 256 queries keep
+// 32768).
 constexpr int kSuperTileMax = 32768, kSuperTileMin = 1024;
 constexpr int kSelMaxQ = 1024;            // queries per index (shared-memory counters)
 constexpr int kPartTile = 4096;           // pairs that k_part_emit orders in shared memory at a time
@@ -2087,13 +2263,14 @@ cudaError_t launch_pass1(const JoinLaunch &a, uint32_t *pend, cudaStream_t s, cu
         return e;
     if (mid)
         cudaEventRecord(mid, s);
-    // pass 1b: a warp per kWalkRange bitmap words, as many CTAs as that takes
+    // pass 1b: a warp per `range` bitmap words, as many CTAs as that takes
     const uint64_t nwords = nchunks * kWItems;
-    const uint64_t wblk = (nwords + uint64_t(kWarps) * kWalkRange - 1) / (uint64_t(kWarps) * kWalkRange);
+    const uint32_t range = walk_range(nwords);
+    const uint64_t wblk = (nwords + uint64_t(kWarps) * range - 1) / (uint64_t(kWarps) * range);
     if (a.narrow)
-        k_walk<FP32, true><<<unsigned(wblk), kThreads, 0, s>>>(a, pend, uint32_t(nwords));
+        k_walk<FP32, true><<<unsigned(wblk), kThreads, 0, s>>>(a, pend, uint32_t(nwords), range);
     else
-        k_walk<FP32, false><<<unsigned(wblk), kThreads, 0, s>>>(a, pend, uint32_t(nwords));
+        k_walk<FP32, false><<<unsigned(wblk), kThreads, 0, s>>>(a, pend, uint32_t(nwords), range);
     return cudaGetLastError();
 }
 
@@ -2907,8 +3084,29 @@ cudaError_t launch_join_emit(const JoinLaunch &a, cudaStream_t s, const uint32_t
         return cudaGetLastError();
     };
     if (a.narrow)
-        return a.fp32 ? emit(k_wemit<true, true>, done[2]) : emit(k_wemit<false, true>, done[3]);
-    return a.fp32 ? emit(k_wemit<true, false>, done[0]) : emit(k_wemit<false, false>, done[1]);
+        return a.fp32 ? emit(k_wemit<true, true, false>, done[2]) : emit(k_wemit<false, true, false>, done[3]);
+    return a.fp32 ? emit(k_wemit<true, false, false>, done[0]) : emit(k_wemit<false, false, false>, done[1]);
+}
+
+// The join of a small table (at most kSmallChunks chunks, with an output): two
+// launches, k_small and k_wemit<SELF>.  ev as for launch_join.
+template <bool FP32, bool R16>
+static cudaError_t launch_small(const JoinLaunch &a, uint32_t *pend, cudaStream_t s, cudaEvent_t *ev)
+{
+    static bool done[64] = {};
+    const uint32_t nchunks = uint32_t((a.n + kWChunk - 1) / kWChunk), nblk = (nchunks + kWarps - 1) / kWarps;
+    if (ev)
+        cudaEventRecord(ev[0], s);
+    k_small<FP32, R16><<<nblk, kThreads, 0, s>>>(a, pend, nchunks, a.ix.P <= kSmallHist ? 1 : 0);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess)
+        e = smem_opt_in(k_wemit<FP32, R16, true>, kEmitSmem, done);
+    if (e != cudaSuccess)
+        return e;
+    for (int k = 1; ev && k < 4; ++k)
+        cudaEventRecord(ev[k], s);
+    k_wemit<FP32, R16, true><<<nblk, kThreads, kEmitSmem, s>>>(a, a.tile_tot, nchunks, pend);
+    return cudaGetLastError();
 }
 
 __global__ void k_sum_u64(unsigned long long *dst, const unsigned long long *x, const unsigned long long *y)
@@ -2990,7 +3188,24 @@ cudaError_t launch_join_write(const JoinLaunch &a, void *scratch, cudaStream_t s
 
 cudaError_t launch_join(const JoinLaunch &a, void *scratch, cudaStream_t s, cudaEvent_t *ev)
 {
-    cudaError_t e = launch_join_count(a, scratch, s, ev);
+    cudaError_t e;
+    if (a.n && (a.n + kWChunk - 1) / kWChunk <= kSmallChunks && a.cap && !a.pair_base) {
+        if (reinterpret_cast<uintptr_t>(a.pts) & 15)
+            return cudaErrorMisalignedAddress;
+        JoinLaunch b = a;
+        uint32_t *pend = reinterpret_cast<uint32_t *>(join_layout(b, scratch));
+        if (a.counts && a.ix.P && !a.keep_counts)
+            if ((e = cudaMemsetAsync(a.counts, 0, sizeof(unsigned long long) * a.ix.P, s)) != cudaSuccess)
+                return e;
+        if (b.narrow)
+            e = a.fp32 ? launch_small<true, true>(b, pend, s, ev) : launch_small<false, true>(b, pend, s, ev);
+        else
+            e = a.fp32 ? launch_small<true, false>(b, pend, s, ev) : launch_small<false, false>(b, pend, s, ev);
+        if (ev)
+            cudaEventRecord(ev[4], s);
+        return e;
+    }
+    e = launch_join_count(a, scratch, s, ev);
     if (e != cudaSuccess || a.n == 0)
         return e;
     if ((e = launch_join_write(a, scratch, s)) != cudaSuccess)
