@@ -73,6 +73,7 @@ struct Aux {
 };
 
 constexpr size_t kPinnedBytes = 128;
+constexpr uint64_t kPoolKeep = uint64_t(64) << 20; // the row bitmap of 512M points
 
 } // namespace
 
@@ -84,6 +85,7 @@ struct spx_ctx {
     std::map<uint64_t, std::unique_ptr<PolysObj>> polys;
     std::map<uint64_t, std::unique_ptr<IndexObj>> indexes;
     Aux *aux = nullptr;
+    cudaMemPool_t pool = nullptr; // stream-ordered scratch of the row-order count, at most kPoolKeep kept between calls
     char *pinned = nullptr; // kPinnedBytes of host memory: a call's status and total come back here
     void *scratch = nullptr;
     size_t scratch_bytes = 0;
@@ -699,6 +701,14 @@ spx_status spx_create(int device, spx_ctx **out)
         return SPX_ENOMEM;
     if (cudaMemset(c->aux, 0, sizeof(Aux)) != cudaSuccess)
         return SPX_ECUDA;
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = device;
+    uint64_t keep = kPoolKeep;
+    if (cudaMemPoolCreate(&c->pool, &props) != cudaSuccess ||
+        cudaMemPoolSetAttribute(c->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess)
+        return SPX_ENOMEM;
     if (cudaMallocHost(reinterpret_cast<void **>(&c->pinned), kPinnedBytes) != cudaSuccess)
         return SPX_ENOMEM;
     if (cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking) != cudaSuccess)
@@ -722,6 +732,8 @@ void spx_destroy(spx_ctx *ctx)
     }
     cudaFree(ctx->aux);
     cudaFreeHost(ctx->pinned);
+    if (ctx->pool)
+        cudaMemPoolDestroy(ctx->pool);
     cudaFree(ctx->scratch);
     cudaFree(ctx->st_pts);
     cudaFree(ctx->st_pairs);
@@ -1003,8 +1015,11 @@ spx_status spx_autotune(spx_ctx *ctx, spx_points points, spx_polys polys, const 
 
     // device memory of the tuner: sample | reference counts | candidate counts | counter words
     const size_t b_sample = (m * 8 + 255) & ~size_t(255), b_counts = ((size_t(P) + 1) * 8 + 255) & ~size_t(255);
+    JoinLaunch sized{};
+    sized.n = m;
+    sized.clustered = pts->cluster_log2 ? 1 : 0; // the strided sample keeps the table's order
     void *mem = nullptr;
-    if (cudaMalloc(&mem, b_sample + 2 * b_counts + 256) != cudaSuccess)
+    if (cudaMalloc(&mem, b_sample + 2 * b_counts + aggregate_scratch_bytes(sized) + 256) != cudaSuccess)
         return fail(ctx, SPX_ENOMEM, "autotune: cudaMalloc of the sample failed");
     std::unique_ptr<void, decltype(&cudaFree)> mem_guard(mem, &cudaFree);
     int2 *sample = static_cast<int2 *>(mem);
@@ -1049,7 +1064,7 @@ spx_status spx_autotune(spx_ctx *ctx, spx_points points, spx_polys polys, const 
         a.err = &ctx->aux->err;
         a.stats = ctx->aux->stats;
         a.fp32 = ix->fp32;
-        a.clustered = pts->cluster_log2 ? 1 : 0; // the strided sample keeps the table's order
+        a.clustered = sized.clustered;
         float best_t = 0;
         cudaError_t e = cudaSuccess;
         for (int r = 0; r <= reps && e == cudaSuccess; ++r) { // launch 0 warms the index into L2
@@ -1550,10 +1565,25 @@ spx_status spx_aggregate(spx_ctx *ctx, spx_points points, spx_index index, uint6
     a.cell_end = pts->cell_end;
     a.cluster_log2 = pts->cluster_log2;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    spx_status st = ensure(ctx, &ctx->scratch, &ctx->scratch_bytes, aggregate_scratch_bytes(a), s, "aggregate");
-    if (st != SPX_OK)
-        return st;
-    cudaError_t e = launch_aggregate(a, ctx->scratch, s, ctx->timing ? ctx->ev : nullptr);
+    // a table in row order takes its scratch from the ctx's pool, in stream
+    // order: counts on several streams, or beside a join, share nothing.  When
+    // there is none to have, the one-pass kernel needs none.
+    void *words = nullptr;
+    if (use_split_count(a)) {
+        if (cudaMallocFromPoolAsync(&words, aggregate_scratch_bytes(a), ctx->pool, s) != cudaSuccess) {
+            cudaGetLastError();
+            words = nullptr;
+        }
+    } else if (a.clustered) {
+        spx_status st = ensure(ctx, &ctx->scratch, &ctx->scratch_bytes, aggregate_scratch_bytes(a), s, "aggregate");
+        if (st != SPX_OK)
+            return st;
+    }
+    cudaError_t e = launch_aggregate(a, a.clustered ? ctx->scratch : words, s, ctx->timing ? ctx->ev : nullptr);
+    if (words) {
+        const cudaError_t e2 = cudaFreeAsync(words, s);
+        e = e != cudaSuccess ? e : e2;
+    }
     if (e != cudaSuccess)
         return cuda_fail(ctx, e, "aggregate launch");
     if (ctx->timing && pts->n) {
@@ -1843,10 +1873,13 @@ spx_status spx_aggregate_host(spx_ctx *ctx, const int32_t *xy_host, uint64_t n, 
     const uint64_t kSlice = uint64_t(1) << (ctx->host_slice_set ? ctx->host_slice_log2 : 25);
     const uint64_t n_slices = (n + kSlice - 1) / kSlice;
     const size_t b_pts = kSlice * 8;
+    JoinLaunch sized{};
+    sized.n = n < kSlice ? n : kSlice;
     spx_status st;
     if ((st = ensure(ctx, &ctx->st_counts, &ctx->st_counts_b, size_t(ix->view.P) * 8 + 16, s, "aggregate_host")) !=
             SPX_OK ||
-        (st = ensure(ctx, &ctx->scratch, &ctx->scratch_bytes, kRing * b_pts + 256, s, "aggregate_host")) != SPX_OK)
+        (st = ensure(ctx, &ctx->scratch, &ctx->scratch_bytes, kRing * b_pts + aggregate_scratch_bytes(sized) + 256, s,
+                     "aggregate_host")) != SPX_OK)
         return st;
     while (ctx->slice_ev.size() < 2 * n_slices + 1) {
         cudaEvent_t e = nullptr;
@@ -1882,7 +1915,7 @@ spx_status spx_aggregate_host(spx_ctx *ctx, const int32_t *xy_host, uint64_t n, 
         if (e == cudaSuccess)
             e = cudaStreamWaitEvent(s, ev_in[k], 0);
         if (e == cudaSuccess)
-            e = launch_aggregate(a, nullptr, s);
+            e = launch_aggregate(a, ring + kRing * b_pts, s); // the slices are counted one after the other
         if (e == cudaSuccess)
             e = cudaEventRecord(ev_agg[k], s);
         if (e != cudaSuccess)

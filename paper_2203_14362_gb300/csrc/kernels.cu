@@ -981,7 +981,13 @@ __host__ __device__ constexpr size_t resolve_smem_head(int warps, bool sum, int 
 // from there: the points arrive while the chunk is resolved, and their loads
 // cost the L1 nothing.  A warp's last chunk, when it is not full, is loaded
 // with plain loads.
-template <int THREADS, bool SUM, bool TMA, bool R16>
+//
+// OUT says what is kept per point: kOut32 or kOut16 (a result of that width and
+// the chunk's pair total), or kOutCount (nothing but the bitmap: the count
+// aggregate, whose pass 1b only counts).
+constexpr int kOut32 = 0, kOut16 = 1, kOutCount = 2;
+
+template <int THREADS, bool SUM, bool TMA, int OUT>
 __global__ void __launch_bounds__(THREADS, SUM ? 1 : (TMA ? 6 : kResolveMinBlocks))
     k_resolve(const __grid_constant__ JoinLaunch a, uint32_t *pend, uint32_t nchunks, int use_hist)
 {
@@ -1113,8 +1119,8 @@ __global__ void __launch_bounds__(THREADS, SUM ? 1 : (TMA ? 6 : kResolveMinBlock
             }
             // one: the polygon; list: its first entry (narrow: none; rewritten
             // by pass 1b); empty: none
-            if (loc < npts) {
-                if (R16)
+            if (OUT != kOutCount && loc < npts) {
+                if (OUT == kOut16)
                     __stcg(reinterpret_cast<unsigned short *>(res16 + loc),
                            (unsigned short)(kind == kCellInsideOne ? pay : kRes16None));
                 else
@@ -1127,6 +1133,8 @@ __global__ void __launch_bounds__(THREADS, SUM ? 1 : (TMA ? 6 : kResolveMinBlock
             __stcg(pend + (uint64_t)ch * kWItems + lane, mask);
         n_pts += lane == 0 ? npts : 0u;
         n_pairs += total;
+        if (OUT == kOutCount)
+            continue;
         total = warp_sum32(total);
         if (lane == 0)
             a.tile_tot[ch] = total; // the chunk's total without its list points; pass 1b adds theirs
@@ -1140,7 +1148,7 @@ __global__ void __launch_bounds__(THREADS, SUM ? 1 : (TMA ? 6 : kResolveMinBlock
     add_stats(a.stats, n_pts, 0u, 0u, n_pairs);
 }
 
-template <bool FP32, bool R16>
+template <bool FP32, int OUT>
 __global__ void __launch_bounds__(kThreads, kWalkMinBlocks) k_walk(JoinLaunch a, uint32_t *pend, uint32_t nwords,
                                                                    uint32_t range)
 {
@@ -1162,7 +1170,7 @@ __global__ void __launch_bounds__(kThreads, kWalkMinBlocks) k_walk(JoinLaunch a,
         // cell resolved again
         uint32_t e0;
         bool lst = has;
-        if (R16) {
+        if (OUT != kOut32) {
             const uint32_t w = resolve(ix, (uint32_t)p.x, (uint32_t)p.y, keep); // a marked row's point is in the box
             e0 = w & kPayloadMask;
             lst = has && in_bounds((w >> 30) == kCellList, ix);
@@ -1170,9 +1178,9 @@ __global__ void __launch_bounds__(kThreads, kWalkMinBlocks) k_walk(JoinLaunch a,
             e0 = __ldcg(a.res + row);
         }
         uint32_t f = 0, c = 0;
-        uint64_t ids = 0; // R16 and a.aux: the first four polygons, 16 bits each
+        uint64_t ids = 0; // kOut16 and a.aux: the first four polygons, 16 bits each
         walk_list_wave<FP32>(ix, lst, e0, p.x, p.y, n_tests, n_esc, keep, s_par, [&](uint32_t q) {
-            if (R16 && c < 4)
+            if (OUT == kOut16 && c < 4)
                 ids |= (uint64_t)q << (16 * c);
             f = c ? f : q;
             ++c;
@@ -1180,8 +1188,8 @@ __global__ void __launch_bounds__(kThreads, kWalkMinBlocks) k_walk(JoinLaunch a,
                 atomicAdd(a.counts + q, 1ull);
         });
         n_pairs += c;
-        if (has) {
-            if (R16) {
+        if (OUT != kOutCount && has) {
+            if (OUT == kOut16) {
                 __stcg(reinterpret_cast<unsigned short *>(a.res) + row,
                        (unsigned short)(c == 0 ? kRes16None : c == 1 ? f : c));
                 // the row's bit stays set iff the point is in several polygons;
@@ -2213,10 +2221,10 @@ __global__ void __launch_bounds__(256) k_agg_cells(const unsigned long long *cel
 // Pass 1 of the join (1a resolve, 1b walk).  pend: 8 words per chunk (the
 // bitmap of the rows pass 1b tests).  mid (or null): an event recorded between
 // the two kernels.
-template <bool FP32>
-cudaError_t launch_pass1(const JoinLaunch &a, uint32_t *pend, cudaStream_t s, cudaEvent_t mid)
+template <bool FP32, int OUT>
+cudaError_t launch_pass1_as(const JoinLaunch &a, uint32_t *pend, cudaStream_t s, cudaEvent_t mid)
 {
-    static bool done_r[8][64] = {};
+    static bool done_r[4][64] = {};
     const uint64_t nchunks = (a.n + kWChunk - 1) / kWChunk;
     if (a.n >= (1ull << 32))
         return cudaErrorInvalidValue; // rows are 32-bit
@@ -2243,22 +2251,15 @@ cudaError_t launch_pass1(const JoinLaunch &a, uint32_t *pend, cudaStream_t s, cu
         return cudaGetLastError();
     };
     constexpr int WS = kResolveSumThreads / 32;
-    auto pass1a = [&](auto r16) -> cudaError_t {
-        constexpr bool R16 = decltype(r16)::value;
-        bool(*d)[64] = done_r + (R16 ? 4 : 0);
-        if (a.ix.use_sum) {
-            // beside the summary, shared memory holds one chunk buffer per warp
-            // at most, too shallow to hide a bulk copy: L2 prefetches instead
-            return launch(k_resolve<kResolveSumThreads, true, false, R16>, kResolveSumThreads,
-                          resolve_smem_head(WS, true, a.ix.sg, false), resolve_smem_head(WS, true, kSumLog2, false),
-                          d[2]);
-        }
+    if (a.ix.use_sum) {
+        // beside the summary, shared memory holds one chunk buffer per warp
+        // at most, too shallow to hide a bulk copy: L2 prefetches instead
+        e = launch(k_resolve<kResolveSumThreads, true, false, OUT>, kResolveSumThreads,
+                   resolve_smem_head(WS, true, a.ix.sg, false), resolve_smem_head(WS, true, kSumLog2, false), done_r[2]);
+    } else {
         const size_t head = kTmaPoints ? resolve_smem_head(kWarps, false, 0, true) : 0;
-        if (kTmaPoints)
-            return launch(k_resolve<kThreads, false, true, R16>, kThreads, head, head, d[3]);
-        return launch(k_resolve<kThreads, false, false, R16>, kThreads, head, head, d[0]);
-    };
-    e = a.narrow ? pass1a(std::true_type{}) : pass1a(std::false_type{});
+        e = launch(k_resolve<kThreads, false, kTmaPoints, OUT>, kThreads, head, head, done_r[3]);
+    }
     if (e != cudaSuccess) // pass 1b must not run on what an earlier call left in the scratch
         return e;
     if (mid)
@@ -2267,11 +2268,14 @@ cudaError_t launch_pass1(const JoinLaunch &a, uint32_t *pend, cudaStream_t s, cu
     const uint64_t nwords = nchunks * kWItems;
     const uint32_t range = walk_range(nwords);
     const uint64_t wblk = (nwords + uint64_t(kWarps) * range - 1) / (uint64_t(kWarps) * range);
-    if (a.narrow)
-        k_walk<FP32, true><<<unsigned(wblk), kThreads, 0, s>>>(a, pend, uint32_t(nwords), range);
-    else
-        k_walk<FP32, false><<<unsigned(wblk), kThreads, 0, s>>>(a, pend, uint32_t(nwords), range);
+    k_walk<FP32, OUT><<<unsigned(wblk), kThreads, 0, s>>>(a, pend, uint32_t(nwords), range);
     return cudaGetLastError();
+}
+
+template <bool FP32>
+cudaError_t launch_pass1(const JoinLaunch &a, uint32_t *pend, cudaStream_t s, cudaEvent_t mid)
+{
+    return a.narrow ? launch_pass1_as<FP32, kOut16>(a, pend, s, mid) : launch_pass1_as<FP32, kOut32>(a, pend, s, mid);
 }
 
 // Exclusive scan of n values in place; the total goes to *total.  part: at
@@ -3220,9 +3224,27 @@ static bool use_directory(const JoinLaunch &a)
     return a.clustered && a.cell_end && a.cluster_log2 >= a.ix.gc && a.cluster_log2 <= 13;
 }
 
+// A table in row order is counted by the join's pass 1 with nothing kept but the
+// row bitmap: the points of blocks that the summary resolves read no index
+// word, and the exact tests run in their own kernel instead of holding up the
+// streaming warps (100M points: 5000-cell map 1928 -> 530 us, 2000 cells 883 ->
+// 345, 64 queries 1020 -> 409, 256 stars 478 -> 305).  From 2M points on: at 2M
+// two launches cost as much as they save (2000 cells 25.8 one pass / 28.9, at 4M
+// 50.9 / 38.1).  Only with the summary: without it (a 40000-cell map, counts in
+// global memory) the one pass is as fast (2021 / 2068 us).
+constexpr uint64_t kSplitCountMin = uint64_t(1) << 21;
+bool use_split_count(const JoinLaunch &a) { return !a.clustered && a.ix.use_sum && a.n > kSplitCountMin; }
+
+static size_t split_count_bytes(uint64_t n)
+{
+    return n > kSplitCountMin ? size_t((n + kWChunk - 1) / kWChunk) * kWItems * 4 : 0;
+}
+
 size_t aggregate_scratch_bytes(const JoinLaunch &a)
 {
     const uint64_t nchunks = (a.n + kWChunk - 1) / kWChunk;
+    if (!a.clustered)
+        return split_count_bytes(a.n);
     return use_directory(a) ? size_t((nchunks + 31) / 32) * 4 + 16 : 16;
 }
 
@@ -3235,6 +3257,16 @@ cudaError_t launch_aggregate(const JoinLaunch &a, void *scratch, cudaStream_t s,
         return e;
     if (reinterpret_cast<uintptr_t>(a.pts) & 15)
         return cudaErrorMisalignedAddress;
+    if (scratch && use_split_count(a)) {
+        if (ev)
+            cudaEventRecord(ev[0], s);
+        uint32_t *pend = static_cast<uint32_t *>(scratch);
+        e = a.fp32 ? launch_pass1_as<true, kOutCount>(a, pend, s, nullptr)
+                   : launch_pass1_as<false, kOutCount>(a, pend, s, nullptr);
+        if (ev)
+            cudaEventRecord(ev[1], s);
+        return e;
+    }
     const int use_hist = a.ix.P <= (uint32_t)kHistMax ? 1 : 0;
     if (ev)
         cudaEventRecord(ev[0], s);

@@ -197,8 +197,11 @@ cudaError_t launch_join_count(const JoinLaunch &a, void *scratch, cudaStream_t s
 cudaError_t launch_join_write(const JoinLaunch &a, void *scratch, cudaStream_t s);
 cudaError_t launch_join_plain(const JoinLaunch &a, void *scratch, cudaStream_t s);
 // scratch: aggregate_scratch_bytes(a) bytes (the chunk bitmap of the directory
-// path; unused otherwise).  a.keep_counts: add to the counts instead of
-// zeroing them first.
+// path, the row bitmap of a table in row order), not shared with a launch that
+// may overlap this one; null with a table in row order: one pass without
+// scratch, slower.  a.keep_counts: add to the counts instead of zeroing them
+// first.  use_split_count: whether this launch would use the row bitmap.
+bool use_split_count(const JoinLaunch &a);
 size_t aggregate_scratch_bytes(const JoinLaunch &a);
 cudaError_t launch_aggregate(const JoinLaunch &a, void *scratch, cudaStream_t s, cudaEvent_t *ev = nullptr);
 
