@@ -53,10 +53,12 @@ struct PolysObj {
 
 struct IndexObj {
     uint64_t polys = 0;
-    int kind = 0;        // 0: polygons (view), 1: disks (dview), 2: buffered polygons (view and bview)
+    int kind = 0;        // 0: polygons (view), 1: disks (dview), 2: buffered polygons (view, nview, near)
     DiskView dview{};
-    BufferView bview{};
-    void *mem2 = nullptr; // buffered polygons: edge grid (cell offsets | polygons | segments | radii)
+    IndexView nview{};   // kind 2: the buffered polygons' own grid,
+    NearView near{};     // their radii and containment (view)
+    void *mem2 = nullptr; // buffered polygons: radii
+    void *mem3 = nullptr; // buffered polygons: their own grid (cells | fine | entries | edges | summary)
     IndexView view{};
     int fp32 = 1;
     void *mem = nullptr; // one allocation: cells | fine | entries | edges | cover | summary
@@ -316,42 +318,6 @@ spx_status disk_join_common(spx_ctx *ctx, PointsObj *pts, IndexObj *ix, uint32_t
     return report_total(ctx, s, a.total, cap, n_pairs, "join", "pairs");
 }
 
-BufferLaunch buffer_launch(spx_ctx *ctx, PointsObj *pts, IndexObj *ix)
-{
-    BufferLaunch a{};
-    a.ix = ix->view;
-    a.bv = ix->bview;
-    a.pts = reinterpret_cast<const int2 *>(pts->dev);
-    a.n = pts->n;
-    a.stats = ctx->aux->stats;
-    a.fp32 = ix->fp32;
-    return a;
-}
-
-// The buffered-polygon join: same contract as the polygon join.
-spx_status buffer_join_common(spx_ctx *ctx, PointsObj *pts, IndexObj *ix, uint32_t *pairs_dev, uint64_t cap,
-                              uint64_t *counts_dev, uint64_t *total_dev, uint64_t *n_pairs, void *stream)
-{
-    if (cap && !pairs_dev)
-        return fail(ctx, SPX_EINVAL, "join: pairs_dev is NULL with cap > 0");
-    if ((reinterpret_cast<uintptr_t>(pairs_dev) & 7) || (reinterpret_cast<uintptr_t>(counts_dev) & 7) ||
-        (reinterpret_cast<uintptr_t>(total_dev) & 7))
-        return fail(ctx, SPX_EINVAL, "join: output pointers must be 8-byte aligned");
-    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    spx_status st = ensure(ctx, &ctx->scratch, &ctx->scratch_bytes, buffer_scratch_bytes(pts->n), s, "join");
-    if (st != SPX_OK)
-        return st;
-    BufferLaunch a = buffer_launch(ctx, pts, ix);
-    a.pairs = reinterpret_cast<uint2 *>(pairs_dev);
-    a.cap = pairs_dev ? cap : 0;
-    a.counts = reinterpret_cast<unsigned long long *>(counts_dev);
-    a.total = total_dev ? reinterpret_cast<unsigned long long *>(total_dev) : (n_pairs ? &ctx->aux->total : nullptr);
-    cudaError_t e = launch_buffer_join(a, ctx->scratch, s);
-    if (e != cudaSuccess)
-        return cuda_fail(ctx, e, "join launch");
-    return report_total(ctx, s, a.total, cap, n_pairs, "join", "pairs");
-}
-
 spx_status join_common(spx_ctx *ctx, spx_points points, spx_index index, uint32_t *pairs_dev, uint64_t cap,
                        uint64_t *counts_dev, uint64_t *total_dev, uint64_t *n_pairs, void *stream, bool plain)
 {
@@ -367,20 +333,31 @@ spx_status join_common(spx_ctx *ctx, spx_points points, spx_index index, uint32_
         return fail(ctx, SPX_EINVAL, "join: a cell-clustered point table has no row order; use spx_aggregate");
     if (ix->kind == 1)
         return disk_join_common(ctx, pts, ix, pairs_dev, cap, counts_dev, total_dev, n_pairs, stream);
-    if (ix->kind == 2)
-        return buffer_join_common(ctx, pts, ix, pairs_dev, cap, counts_dev, total_dev, n_pairs, stream);
     if (cap && !pairs_dev)
         return fail(ctx, SPX_EINVAL, "join: pairs_dev is NULL with cap > 0");
     if ((reinterpret_cast<uintptr_t>(pairs_dev) & 7) || (reinterpret_cast<uintptr_t>(counts_dev) & 7) ||
         (reinterpret_cast<uintptr_t>(total_dev) & 7))
         return fail(ctx, SPX_EINVAL, "join: output pointers must be 8-byte aligned");
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+    const bool buffered = ix->kind == 2; // exact already: spx_join_plain takes the same path
+    plain = plain && !buffered;
     const size_t need = plain ? plain_scratch_bytes(pts->n) : join_scratch_bytes(pts->n);
-    spx_status st = ensure(ctx, &ctx->scratch, &ctx->scratch_bytes, need, s, "join");
+    // buffered polygons overlap: 8 B per point more let pass 1 keep a point's
+    // polygons for pass 3; a call goes without them where the scratch cannot grow
+    const size_t aux_at = (need + 15) & ~size_t(15), with_aux = aux_at + pts->n * 8;
+    bool aux = buffered && ix->nview.P <= kRes16MaxP && (ctx->scratch_bytes >= with_aux || !capturing(s));
+    spx_status st = ensure(ctx, &ctx->scratch, &ctx->scratch_bytes, aux ? with_aux : need, s, "join");
+    if (st == SPX_ENOMEM && aux) {
+        cudaGetLastError();
+        aux = false;
+        st = ensure(ctx, &ctx->scratch, &ctx->scratch_bytes, need, s, "join");
+    }
     if (st != SPX_OK)
         return st;
     JoinLaunch a{};
-    a.ix = ix->view;
+    a.ix = buffered ? ix->nview : ix->view;
+    a.near = ix->near;
+    a.aux = aux ? reinterpret_cast<uint64_t *>(static_cast<char *>(ctx->scratch) + aux_at) : nullptr;
     a.pts = reinterpret_cast<const int2 *>(pts->dev);
     a.n = pts->n;
     a.pairs = reinterpret_cast<uint2 *>(pairs_dev);
@@ -390,7 +367,7 @@ spx_status join_common(spx_ctx *ctx, spx_points points, spx_index index, uint32_
     a.err = &ctx->aux->err;
     a.stats = ctx->aux->stats;
     a.fp32 = ix->fp32;
-    const bool timed = ctx->timing && !plain;
+    const bool timed = ctx->timing && !plain && !buffered;
     cudaError_t e = plain ? launch_join_plain(a, ctx->scratch, s) : launch_join(a, ctx->scratch, s, timed ? ctx->ev : nullptr);
     if (e != cudaSuccess)
         return cuda_fail(ctx, e, "join launch");
@@ -723,8 +700,11 @@ void spx_destroy(spx_ctx *ctx)
         return;
     cudaSetDevice(ctx->device);
     cudaDeviceSynchronize();
-    for (auto &kv : ctx->indexes)
+    for (auto &kv : ctx->indexes) {
         cudaFree(kv.second->mem);
+        cudaFree(kv.second->mem2);
+        cudaFree(kv.second->mem3);
+    }
     for (auto &kv : ctx->points) {
         if (kv.second->owned)
             cudaFree(kv.second->dev);
@@ -1347,57 +1327,67 @@ spx_status spx_build_buffer_index(spx_ctx *ctx, spx_polys polys, const int32_t *
     auto up = [](size_t v) { return (v + 255) & ~size_t(255); };
     const uint32_t P = pg->P;
     const size_t n_items = he.item_q.size();
+    // kept: the radii; the edge grid only until the index over it is built
     const size_t b_off = he.cell_off.size() * 4, b_q = std::max<size_t>(n_items, 1) * 4,
-                 b_seg = std::max<size_t>(n_items, 1) * 16, b_r = std::max<size_t>(P, 1) * 4;
-    // the screen: cells with edges here, cells meeting a polygon by launch_buffer_mask
-    const uint64_t ncell = uint64_t(1) << (2 * g);
-    std::vector<uint32_t> mask(std::max<uint64_t>(ncell / 32, 1), 0u);
-    for (uint64_t c = 0; c < ncell; ++c)
-        if (he.cell_off[c + 1] > he.cell_off[c])
-            mask[c >> 5] |= 1u << (c & 31);
-    const size_t b_mask = mask.size() * 4;
-    const size_t total = up(b_off) + up(b_q) + up(b_seg) + up(b_r) + up(b_mask);
-    void *mem2 = nullptr;
-    if (cudaMalloc(&mem2, total) != cudaSuccess) {
+                 b_seg = std::max<size_t>(n_items, 1) * 16, total = std::max<size_t>(P, 1) * 4;
+    void *mem2 = nullptr, *tmp = nullptr;
+    NearIndexDev fx{};
+    auto drop = [&] {
+        cudaFree(tmp);
+        cudaFree(mem2);
+        cudaFree(fx.mem);
         cudaFree(ix->mem);
         pg->n_index--;
+    };
+    if (cudaMalloc(&mem2, total) != cudaSuccess || cudaMalloc(&tmp, up(b_off) + up(b_q) + up(b_seg)) != cudaSuccess) {
+        drop();
         return fail(ctx, SPX_ENOMEM, "build_buffer_index: cudaMalloc failed");
     }
-    char *m = static_cast<char *>(mem2), *p_q = m + up(b_off), *p_seg = p_q + up(b_q), *p_r = p_seg + up(b_seg),
-         *p_mask = p_r + up(b_r);
-    cudaError_t e = cudaMemcpy(m, he.cell_off.data(), b_off, cudaMemcpyHostToDevice);
+    char *p_r = static_cast<char *>(mem2), *p_off = static_cast<char *>(tmp), *p_q = p_off + up(b_off),
+         *p_seg = p_q + up(b_q);
+    cudaError_t e = cudaMemcpy(p_off, he.cell_off.data(), b_off, cudaMemcpyHostToDevice);
     if (e == cudaSuccess && n_items)
         e = cudaMemcpy(p_q, he.item_q.data(), n_items * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess && n_items)
         e = cudaMemcpy(p_seg, he.item_seg.data(), n_items * 16, cudaMemcpyHostToDevice);
     if (e == cudaSuccess && P)
         e = cudaMemcpy(p_r, r, size_t(P) * 4, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess)
-        e = cudaMemcpy(p_mask, mask.data(), b_mask, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess)
-        e = launch_buffer_mask(ix->view, reinterpret_cast<uint32_t *>(p_mask), g, nullptr);
-    if (e == cudaSuccess)
-        e = cudaDeviceSynchronize();
-    if (e != cudaSuccess) {
-        cudaFree(mem2);
-        cudaFree(ix->mem);
-        pg->n_index--;
-        return cuda_fail(ctx, e, "build_buffer_index upload");
+    if (e == cudaSuccess) {
+        const int built = build_near_index_device(ix->view, reinterpret_cast<uint32_t *>(p_off),
+                                                  reinterpret_cast<uint32_t *>(p_q), reinterpret_cast<int4 *>(p_seg),
+                                                  reinterpret_cast<int32_t *>(p_r), g, fx, e);
+        if (built == 1) {
+            drop();
+            return fail(ctx, SPX_EINVAL, "build_buffer_index: too many (cell, polygon) entries for 30-bit offsets; use "
+                                         "a coarser edge grid");
+        }
     }
+    if (e != cudaSuccess) {
+        drop();
+        return e == cudaErrorMemoryAllocation ? fail(ctx, SPX_ENOMEM, "build_buffer_index: cudaMalloc failed")
+                                              : cuda_fail(ctx, e, "build_buffer_index upload");
+    }
+    cudaFree(tmp);
     ix->kind = 2;
     ix->mem2 = mem2;
-    ix->bview.cell_off = reinterpret_cast<const uint32_t *>(m);
-    ix->bview.item_q = reinterpret_cast<const uint32_t *>(p_q);
-    ix->bview.item_seg = reinterpret_cast<const int4 *>(p_seg);
-    ix->bview.rad = reinterpret_cast<const int32_t *>(p_r);
-    ix->bview.mask = reinterpret_cast<const uint32_t *>(p_mask);
-    ix->bview.g = g;
-    ix->bview.sc = kBoxLog2 - g;
-    ix->bview.P = P;
-    ix->bview.n_items = n_items;
+    ix->mem3 = fx.mem;
+    GridParts gp{};
+    gp.cell = reinterpret_cast<char *>(fx.cell);
+    gp.ent = reinterpret_cast<char *>(fx.ent);
+    gp.fine = reinterpret_cast<char *>(fx.fine);
+    gp.edge = reinterpret_cast<char *>(fx.edge);
+    gp.sum = reinterpret_cast<char *>(fx.sum);
+    gp.n_ent = fx.n_ent;
+    gp.n_fine = fx.n_fine;
+    gp.n_edge = fx.n_edge;
+    gp.sum_resolved = fx.sum_resolved;
+    ix->nview = grid_view(gp, g, fx.sb, P);
+    ix->nview.err = &ctx->aux->err;
+    ix->near.rad = reinterpret_cast<const int32_t *>(p_r);
+    ix->near.in = ix->view;
     ix->info.edge_grid_log2 = g;
     ix->info.n_edge_items = n_items;
-    ix->info.device_bytes += total;
+    ix->info.device_bytes += total + fx.bytes;
     ix->info.build_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
     const uint64_t hb = make_handle(ctx, kTagIndex);
     ctx->indexes[hb] = std::move(ix);
@@ -1445,7 +1435,7 @@ spx_status spx_select(spx_ctx *ctx, spx_points points, spx_index index, uint32_t
         return fail(ctx, SPX_EINVAL, "select: offsets_dev is NULL, or ids_dev is NULL with cap > 0");
     if ((reinterpret_cast<uintptr_t>(offsets_dev) & 7) || (reinterpret_cast<uintptr_t>(ids_dev) & 3))
         return fail(ctx, SPX_EINVAL, "select: misaligned output pointer");
-    const uint32_t PQ = ix->kind == 1 ? ix->dview.Q : ix->kind == 2 ? ix->bview.P : ix->view.P;
+    const uint32_t PQ = ix->kind == 1 ? ix->dview.Q : ix->view.P;
     if (PQ > kSelectMaxQueries)
         return fail(ctx, SPX_EINVAL, "select: an index of " + std::to_string(PQ) +
                                          " queries; batched selection takes at most " +
@@ -1453,12 +1443,20 @@ spx_status spx_select(spx_ctx *ctx, spx_points points, spx_index index, uint32_t
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     if (ix->kind == 2) {
         // buffered polygons: points inside or within r of each polygon, ascending per polygon
-        spx_status st = ensure(ctx, &ctx->scratch, &ctx->scratch_bytes, buffer_select_scratch_bytes(pts->n, PQ, cap),
-                               s, "select");
+        spx_status st = ensure(ctx, &ctx->scratch, &ctx->scratch_bytes, select_scratch_bytes(pts->n, PQ, cap), s,
+                               "select");
         if (st != SPX_OK)
             return st;
+        JoinLaunch b{};
+        b.ix = ix->nview;
+        b.near = ix->near;
+        b.pts = reinterpret_cast<const int2 *>(pts->dev);
+        b.n = pts->n;
+        b.err = &ctx->aux->err;
+        b.stats = ctx->aux->stats;
+        b.fp32 = ix->fp32;
         unsigned long long *offs = reinterpret_cast<unsigned long long *>(offsets_dev);
-        cudaError_t e = launch_buffer_select(buffer_launch(ctx, pts, ix), ids_dev, cap, offs, ctx->scratch, s);
+        cudaError_t e = launch_select(b, ids_dev, cap, offs, ctx->scratch, s);
         if (e != cudaSuccess)
             return cuda_fail(ctx, e, "select launch");
         return report_total(ctx, s, offs + PQ, cap, n_ids, "select", "ids");
@@ -1547,14 +1545,10 @@ spx_status spx_aggregate(spx_ctx *ctx, spx_points points, spx_index index, uint6
         cudaError_t e = launch_disk_aggregate(d, reinterpret_cast<cudaStream_t>(stream));
         return e == cudaSuccess ? SPX_OK : cuda_fail(ctx, e, "aggregate launch");
     }
-    if (ix->kind == 2) { // counts do not depend on the point order: clustered tables too
-        BufferLaunch b = buffer_launch(ctx, pts, ix);
-        b.counts = reinterpret_cast<unsigned long long *>(counts_dev);
-        cudaError_t e = launch_buffer_aggregate(b, reinterpret_cast<cudaStream_t>(stream));
-        return e == cudaSuccess ? SPX_OK : cuda_fail(ctx, e, "aggregate launch");
-    }
+    const bool buffered = ix->kind == 2;
     JoinLaunch a{};
-    a.ix = ix->view;
+    a.ix = buffered ? ix->nview : ix->view;
+    a.near = ix->near;
     a.pts = reinterpret_cast<const int2 *>(pts->dev);
     a.n = pts->n;
     a.counts = reinterpret_cast<unsigned long long *>(counts_dev);
@@ -1574,19 +1568,20 @@ spx_status spx_aggregate(spx_ctx *ctx, spx_points points, spx_index index, uint6
             cudaGetLastError();
             words = nullptr;
         }
-    } else if (a.clustered) {
+    } else if (a.clustered && !buffered) {
         spx_status st = ensure(ctx, &ctx->scratch, &ctx->scratch_bytes, aggregate_scratch_bytes(a), s, "aggregate");
         if (st != SPX_OK)
             return st;
     }
-    cudaError_t e = launch_aggregate(a, a.clustered ? ctx->scratch : words, s, ctx->timing ? ctx->ev : nullptr);
+    cudaError_t e = launch_aggregate(a, a.clustered && !buffered ? ctx->scratch : words, s,
+                                     ctx->timing && !buffered ? ctx->ev : nullptr);
     if (words) {
         const cudaError_t e2 = cudaFreeAsync(words, s);
         e = e != cudaSuccess ? e : e2;
     }
     if (e != cudaSuccess)
         return cuda_fail(ctx, e, "aggregate launch");
-    if (ctx->timing && pts->n) {
+    if (ctx->timing && pts->n && !buffered) {
         SPX_CUDA(cudaEventSynchronize(ctx->ev[1]), "aggregate timing");
         float t = 0;
         cudaEventElapsedTime(&t, ctx->ev[0], ctx->ev[1]);
@@ -2156,6 +2151,7 @@ spx_status spx_free(spx_ctx *ctx, uint64_t handle)
             }
         cudaFree(ix->mem);
         cudaFree(ix->mem2);
+        cudaFree(ix->mem3);
         PolysObj *pg = lookup(ctx->polys, ix->polys);
         if (pg)
             pg->n_index--;

@@ -415,6 +415,85 @@ __device__ __forceinline__ uint32_t walk_list(const IndexView &ix, uint32_t e0, 
     return c;
 }
 
+// Is (px, py) within distance r of the closed segment v = (a, b)?  With
+// d = b - a, w = p - a and t = w . d: the distance is |w| when t <= 0, |p - b|
+// when t >= |d|^2, else |d x w| / |d|.  Coordinates lie in [0, 2^30], so every
+// product of two differences is below 2^60 in magnitude (int64 sums stay
+// exact); the last case compares (d x w)^2 with r^2 |d|^2 as 128-bit
+// products.  A zero-length edge takes the first case.
+__device__ __noinline__ bool seg_near_exact(const int4 &v, int px, int py, int64_t r)
+{
+    const int64_t dx = (int64_t)v.z - v.x, dy = (int64_t)v.w - v.y;
+    const int64_t wx = (int64_t)px - v.x, wy = (int64_t)py - v.y, rr = r * r;
+    const int64_t t = wx * dx + wy * dy;
+    if (t <= 0)
+        return wx * wx + wy * wy <= rr;
+    const int64_t dd = dx * dx + dy * dy;
+    if (t >= dd) {
+        const int64_t ux = (int64_t)px - v.z, uy = (int64_t)py - v.w;
+        return ux * ux + uy * uy <= rr;
+    }
+    const int64_t c = dx * wy - dy * wx;
+    const uint64_t ca = (uint64_t)(c < 0 ? -c : c);
+    const uint64_t lh = __umul64hi(ca, ca), ll = ca * ca;
+    const uint64_t rh = __umul64hi((uint64_t)rr, (uint64_t)dd), rl = (uint64_t)rr * (uint64_t)dd;
+    return lh < rh || (lh == rh && ll <= rl);
+}
+
+// The same with an FP32 filter.  Rounding a coordinate difference costs 2^-24
+// relative, so every product of two differences is within 3.01 x 2^-24 of its
+// value and a sum or difference of two within 4.1 x 2^-24 of the sum of their
+// magnitudes; r |d| (one conversion, half of |d|^2's error, two roundings)
+// within 5.2 x 2^-24.  Each comparison trusts FP32 only outside 2^-21 (8 x 2^-24)
+// of the magnitudes involved; the rest (near the radius, or near an end's
+// perpendicular) is decided exactly.
+template <bool FP32>
+__device__ __forceinline__ bool seg_near(const int4 &v, int px, int py, int r)
+{
+    if (FP32) {
+        constexpr float kE = 4.76837158203125e-07f; // 2^-21
+        const float dx = __int2float_rn(v.z - v.x), dy = __int2float_rn(v.w - v.y);
+        const float wx = __int2float_rn(px - v.x), wy = __int2float_rn(py - v.y), rf = __int2float_rn(r);
+        const float t1 = wx * dx, t2 = wy * dy, t = t1 + t2, et = kE * (fabsf(t1) + fabsf(t2));
+        const float dd = dx * dx + dy * dy, rr = rf * rf;
+        float a, b, m; // the point is near iff a <= b; m: the magnitudes compared
+        bool sure = true;
+        if (t < -et) {
+            a = wx * wx + wy * wy, b = rr, m = a + b;
+        } else if (t - dd > et + kE * dd) {
+            const float ux = __int2float_rn(px - v.z), uy = __int2float_rn(py - v.w);
+            a = ux * ux + uy * uy, b = rr, m = a + b;
+        } else {
+            sure = t > et && dd - t > et + kE * dd;
+            const float c1 = dx * wy, c2 = dy * wx;
+            a = fabsf(c1 - c2), b = rf * __fsqrt_rn(dd), m = fabsf(c1) + fabsf(c2) + b;
+        }
+        if (sure && fabsf(a - b) > kE * m)
+            return a < b;
+    }
+    return seg_near_exact(v, px, py, r);
+}
+
+// Does polygon q of its own index hold the in-box point (px, py)?
+template <bool FP32>
+__device__ __noinline__ bool poly_holds(const IndexView &ix, uint32_t q, int px, int py, uint32_t &tests, uint32_t &esc,
+                                        uint64_t pol)
+{
+    const uint32_t w = resolve(ix, (uint32_t)px, (uint32_t)py, pol), pay = w & kPayloadMask;
+    if ((w >> 30) == kCellInsideOne)
+        return pay == q;
+    if ((w >> 30) != kCellList)
+        return false;
+    for (uint64_t e = pay; in_bounds(e < ix.n_ent, ix); ++e) {
+        const uint4 en = ld_idx(ix.ent + e, pol);
+        if (en.x == q && in_bounds(!(en.w & kEntBoundary) || (uint64_t)en.y + en.z < ix.n_edge, ix))
+            return !(en.w & kEntBoundary) || row_parity<FP32>(ix.edge + en.y, en.z, px, py, tests, esc, pol);
+        if (en.x >= q || (en.w & kEntLast))
+            return false;
+    }
+    return false;
+}
+
 // The polygons of an entry list that contain a point, for the 32 lanes of a
 // converged warp at once, each lane with its own point (px, py) and list
 // (starting at entry e0; has = false: the lane takes part but has none).
@@ -429,9 +508,14 @@ __device__ __forceinline__ uint32_t walk_list(const IndexView &ix, uint32_t e0, 
 // sorted lists' early stop is not used (an edge that ends left of the point
 // counts nothing; recording where each list could stop measured slower).
 // s_par: kWaveWords words of shared memory owned by this warp.
-template <bool FP32, class F>
+// NEAR: the list is one of a buffered index (nv).  An edge hits when it comes
+// within its polygon's radius of the point, hits are ORed instead of XORed, and
+// a point that no edge hits asks the polygons' own index where the entry says
+// that the boundary may cross the cell.
+template <bool FP32, bool NEAR = false, class F>
 __device__ __forceinline__ void walk_list_wave(const IndexView &ix, bool has, uint32_t e0, int px, int py,
-                                               uint32_t &tests, uint32_t &esc, uint64_t pol, uint32_t *s_par, F f)
+                                               uint32_t &tests, uint32_t &esc, uint64_t pol, uint32_t *s_par, F f,
+                                               const NearView *nv = nullptr)
 {
     const int lane = threadIdx.x & 31;
     const uint4 *e = ix.ent + (has ? e0 : 0u);
@@ -454,6 +538,11 @@ __device__ __forceinline__ void walk_list_wave(const IndexView &ix, bool has, ui
         const uint32_t za = (more && (ea.w & kEntBoundary)) ? ea.z : 0u;
         const uint32_t zb = (hb && (eb.w & kEntBoundary)) ? eb.z : 0u;
         const uint32_t tot = za + zb;
+        int ra = 0, rb = 0; // NEAR: the entries' radii
+        if (NEAR) {
+            ra = za ? __ldg(nv->rad + ea.x) : 0;
+            rb = zb ? __ldg(nv->rad + eb.x) : 0;
+        }
         uint32_t pa = 0, pb = 0;
         if (__any_sync(kFull, tot != 0)) {
             uint32_t incl = tot;
@@ -470,7 +559,7 @@ __device__ __forceinline__ void walk_list_wave(const IndexView &ix, bool has, ui
             for (uint32_t base = 0; base < T; base += 64) {
                 int4 v[2];
                 uint32_t slot[2], own[2];
-                int ox[2], oy[2];
+                int ox[2], oy[2], rad[2];
                 bool act[2];
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
@@ -490,18 +579,33 @@ __device__ __forceinline__ void walk_list_wave(const IndexView &ix, bool has, ui
                     const uint32_t t = k - (oi - ot);
                     slot[h] = t >= oza ? 1u : 0u;
                     own[h] = o;
+                    if (NEAR) {
+                        const int r0 = __shfl_sync(kFull, ra, o), r1 = __shfl_sync(kFull, rb, o);
+                        rad[h] = slot[h] ? r1 : r0;
+                    }
                     const uint32_t ei = slot[h] ? oyb + (t - oza) : oya + t;
                     v[h] = act[h] ? ld_idx(ix.edge + ei, pol) : make_int4(0, 0, 0, 0); // a zero edge never straddles
                 }
 #pragma unroll
-                for (int h = 0; h < 2; ++h)
-                    if (act[h] && edge_cross<FP32>(v[h], ox[h], oy[h], tests, esc))
+                for (int h = 0; h < 2; ++h) {
+                    if (NEAR) {
+                        if (act[h] && seg_near<FP32>(v[h], ox[h], oy[h], rad[h]))
+                            atomicOr(s_par + 32 * slot[h] + own[h], 1u);
+                    } else if (act[h] && edge_cross<FP32>(v[h], ox[h], oy[h], tests, esc)) {
                         atomicXor(s_par + 32 * slot[h] + own[h], 1u);
+                    }
+                }
             }
             __syncwarp();
             pa = s_par[lane];
             pb = s_par[32 + lane];
             __syncwarp(); // s_par is rewritten by the next wave
+        }
+        if (NEAR) {
+            if (more && !pa && (ea.w & kEntCross))
+                pa = poly_holds<FP32>(nv->in, ea.x, px, py, tests, esc, pol);
+            if (hb && !pb && (eb.w & kEntCross))
+                pb = poly_holds<FP32>(nv->in, eb.x, px, py, tests, esc, pol);
         }
         if (more && (!(ea.w & kEntBoundary) || pa))
             f(ea.x);
@@ -567,6 +671,28 @@ __device__ __forceinline__ uint32_t point_count(const IndexView &ix, int px, int
         return 1;
     }
     return walk_list<FP32>(ix, w & kPayloadMask, px, py, first, tests, esc, pol);
+}
+
+// The number of buffered polygons that the in-box point (px, py) meets, by one
+// lane (points whose count does not fit their 32-bit result).
+template <bool FP32>
+__device__ __noinline__ uint32_t near_count(const IndexView &ix, const NearView &nv, int px, int py, uint64_t pol)
+{
+    const uint32_t w = resolve(ix, (uint32_t)px, (uint32_t)py, pol);
+    uint32_t n = 0, t = 0, s = 0;
+    if ((w >> 30) < kCellList)
+        return (w >> 30) == kCellInsideOne ? 1u : 0u;
+    for (uint64_t e = w & kPayloadMask; in_bounds(e < ix.n_ent, ix); ++e) {
+        const uint4 en = ld_idx(ix.ent + e, pol);
+        bool hit = !(en.w & kEntBoundary);
+        if (in_bounds(en.x < ix.P && (hit || (uint64_t)en.y + en.z < ix.n_edge), ix))
+            for (uint32_t k = 0; k < en.z && !hit; ++k)
+                hit = seg_near<FP32>(ld_idx(ix.edge + en.y + k, pol), px, py, __ldg(nv.rad + en.x));
+        n += hit || ((en.w & kEntCross) && poly_holds<FP32>(nv.in, en.x, px, py, t, s, pol)) ? 1u : 0u;
+        if (en.w & kEntLast)
+            break;
+    }
+    return n;
 }
 
 __device__ __forceinline__ unsigned long long warp_sum64(unsigned long long v)
@@ -1126,7 +1252,7 @@ __global__ void __launch_bounds__(THREADS, SUM ? 1 : (TMA ? 6 : kResolveMinBlock
                 else
                     __stcg(res + loc, kind == kCellEmpty ? kResNone : pay);
             }
-            const uint32_t bl = __ballot_sync(kFull, kind == kCellList);
+            const uint32_t bl = __ballot_sync(kFull, kind >= kCellList); // or kCellCoarseList
             mask = lane == j ? bl : mask;
         }
         if (lane < kWItems)
@@ -1148,17 +1274,31 @@ __global__ void __launch_bounds__(THREADS, SUM ? 1 : (TMA ? 6 : kResolveMinBlock
     add_stats(a.stats, n_pts, 0u, 0u, n_pairs);
 }
 
-template <bool FP32, int OUT>
-__global__ void __launch_bounds__(kThreads, kWalkMinBlocks) k_walk(JoinLaunch a, uint32_t *pend, uint32_t nwords,
+//
+// Up to kSmallHist polygons are counted in shared memory: where many points lie
+// in several polygons (overlapping queries) a global atomic per hit on a few
+// hundred counters was what this pass waited for (20M points x 256 buffered
+// queries: 1545 -> 185 us).
+constexpr uint32_t kSmallHist = 2048;
+
+template <bool FP32, int OUT, bool NEAR>
+__global__ void __launch_bounds__(kThreads, kWalkMinBlocks) k_walk(const __grid_constant__ JoinLaunch a, uint32_t *pend, uint32_t nwords,
                                                                    uint32_t range)
 {
     __shared__ uint32_t s_qa[kWarps * kWalkQueue];
     __shared__ uint32_t s_pa[kWarps * kWaveWords];
+    __shared__ uint32_t s_hist[kSmallHist];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t *s_q = s_qa + warp * kWalkQueue; // rows
     uint32_t *s_par = s_pa + warp * kWaveWords;
     const IndexView &ix = a.ix;
     const uint64_t keep = policy_evict_last();
+    const bool hist = a.counts && ix.P <= kSmallHist;
+    if (hist) {
+        for (uint32_t i = threadIdx.x; i < ix.P; i += kThreads)
+            s_hist[i] = 0;
+        __syncthreads();
+    }
     uint32_t n_tests = 0, n_esc = 0, n_pairs = 0;
     // walk the queued rows [0, m), m <= 32, one per lane
     auto walk = [&](uint32_t m) {
@@ -1173,20 +1313,20 @@ __global__ void __launch_bounds__(kThreads, kWalkMinBlocks) k_walk(JoinLaunch a,
         if (OUT != kOut32) {
             const uint32_t w = resolve(ix, (uint32_t)p.x, (uint32_t)p.y, keep); // a marked row's point is in the box
             e0 = w & kPayloadMask;
-            lst = has && in_bounds((w >> 30) == kCellList, ix);
+            lst = has && in_bounds((w >> 30) >= kCellList, ix);
         } else {
             e0 = __ldcg(a.res + row);
         }
         uint32_t f = 0, c = 0;
         uint64_t ids = 0; // kOut16 and a.aux: the first four polygons, 16 bits each
-        walk_list_wave<FP32>(ix, lst, e0, p.x, p.y, n_tests, n_esc, keep, s_par, [&](uint32_t q) {
+        walk_list_wave<FP32, NEAR>(ix, lst, e0, p.x, p.y, n_tests, n_esc, keep, s_par, [&](uint32_t q) {
             if (OUT == kOut16 && c < 4)
                 ids |= (uint64_t)q << (16 * c);
             f = c ? f : q;
             ++c;
             if (a.counts)
-                atomicAdd(a.counts + q, 1ull);
-        });
+                hist ? (void)atomicAdd(s_hist + q, 1u) : (void)atomicAdd(a.counts + q, 1ull);
+        }, &a.near);
         n_pairs += c;
         if (OUT != kOutCount && has) {
             if (OUT == kOut16) {
@@ -1255,6 +1395,12 @@ __global__ void __launch_bounds__(kThreads, kWalkMinBlocks) k_walk(JoinLaunch a,
     }
     if (qn)
         walk(qn);
+    if (hist) {
+        __syncthreads();
+        for (uint32_t i = threadIdx.x; i < ix.P; i += kThreads)
+            if (s_hist[i])
+                atomicAdd(a.counts + i, (unsigned long long)s_hist[i]);
+    }
     add_stats(a.stats, 0u, n_tests, n_esc, n_pairs);
 }
 
@@ -1268,9 +1414,8 @@ __global__ void __launch_bounds__(kThreads, kWalkMinBlocks) k_walk(JoinLaunch a,
 // + pass 3, 2000-cell map: 20k points 18.5 against 28.8 us, 500k 20.6 / 32.8,
 // 1M 32.8 / 39.0, 1.5M 39.0 / 39.1, 2M 53.7 / 43.1; the line is at 1M points.
 constexpr uint32_t kSmallChunks = 4096;
-constexpr uint32_t kSmallHist = 2048;
 
-template <bool FP32, bool R16>
+template <bool FP32, int OUT, bool NEAR>
 __global__ void __launch_bounds__(kThreads, 3) k_small(const __grid_constant__ JoinLaunch a, uint32_t *pend,
                                                        uint32_t nchunks, int use_hist)
 {
@@ -1323,11 +1468,11 @@ __global__ void __launch_bounds__(kThreads, 3) k_small(const __grid_constant__ J
 #pragma unroll
         for (int j = 0; j < kWItems; ++j) {
             const uint32_t kind = w[j] >> 30, loc = j * 32 + lane, pay = w[j] & kPayloadMask;
-            const bool one = kind == kCellInsideOne && in_bounds(pay < ix.P, ix), lst = kind == kCellList;
+            const bool one = kind == kCellInsideOne && in_bounds(pay < ix.P, ix), lst = kind >= kCellList;
             total += one ? 1u : 0u;
             count1(one, pay);
-            if (loc < npts && !lst) {
-                if (R16)
+            if (OUT != kOutCount && loc < npts && !lst) {
+                if (OUT == kOut16)
                     __stcg(res16 + loc, (unsigned short)(one ? pay : kRes16None));
                 else
                     __stcg(res + loc, one ? pay : kResNone);
@@ -1342,18 +1487,18 @@ __global__ void __launch_bounds__(kThreads, 3) k_small(const __grid_constant__ J
             const bool has = k0 + lane < qn;
             const uint4 it = s_q[has ? k0 + lane : k0]; // idle lanes walk nothing
             uint32_t f = 0, c = 0;
-            uint64_t ids = 0; // R16 and a.aux: the first four polygons, 16 bits each
-            walk_list_wave<FP32>(ix, has, it.z, (int)it.x, (int)it.y, n_tests, n_esc, keep, s_pa + warp * kWaveWords,
+            uint64_t ids = 0; // kOut16 and a.aux: the first four polygons, 16 bits each
+            walk_list_wave<FP32, NEAR>(ix, has, it.z, (int)it.x, (int)it.y, n_tests, n_esc, keep, s_pa + warp * kWaveWords,
                                  [&](uint32_t q) {
-                                     if (R16 && c < 4)
+                                     if (OUT == kOut16 && c < 4)
                                          ids |= (uint64_t)q << (16 * c);
                                      f = c ? f : q;
                                      ++c;
                                      count1(true, q);
-                                 });
+                                 }, &a.near);
             total += c;
-            if (has) {
-                if (R16) {
+            if (OUT != kOutCount && has) {
+                if (OUT == kOut16) {
                     __stcg(res16 + it.w, (unsigned short)(c == 0 ? kRes16None : c == 1 ? f : c));
                     if (c >= 2) {
                         atomicOr(s_m + (it.w >> 5), 1u << (it.w & 31));
@@ -1366,11 +1511,13 @@ __global__ void __launch_bounds__(kThreads, 3) k_small(const __grid_constant__ J
             }
         }
         __syncwarp();
-        if (lane < kWItems)
-            __stcg(pend + (uint64_t)ch * kWItems + lane, s_m[lane]);
-        const uint32_t t = warp_sum32(total);
-        if (lane == 0)
-            a.tile_tot[ch] = t;
+        if (OUT != kOutCount) {
+            if (lane < kWItems)
+                __stcg(pend + (uint64_t)ch * kWItems + lane, s_m[lane]);
+            const uint32_t t = warp_sum32(total);
+            if (lane == 0)
+                a.tile_tot[ch] = t;
+        }
     }
     if (hist) {
         __syncthreads();
@@ -1396,8 +1543,8 @@ constexpr size_t kEmitSmem = size_t(kWarps) * kWChunk * (sizeof(uint32_t) + size
 // With SELF (small tables, a warp per chunk) chunk_off holds the chunks' totals,
 // not their offsets: every CTA sums the totals before its first chunk itself
 // (at most 8 B x kSmallChunks from L2), which saves the scan's launch.
-template <bool FP32, bool R16, bool SELF>
-__global__ void __launch_bounds__(kThreads, 3) k_wemit(JoinLaunch a, const unsigned long long *chunk_off,
+template <bool FP32, bool R16, bool SELF, bool NEAR>
+__global__ void __launch_bounds__(kThreads, 3) k_wemit(const __grid_constant__ JoinLaunch a, const unsigned long long *chunk_off,
                                                        uint32_t nchunks, const uint32_t *pend)
 {
     __shared__ unsigned long long s_before[SELF ? kWarps : 1];
@@ -1474,7 +1621,8 @@ __global__ void __launch_bounds__(kThreads, 3) k_wemit(JoinLaunch a, const unsig
                     } else { // count not stored: count again
                         const int2 p = a.pts[base + loc];
                         uint32_t f = 0, t = 0, e = 0;
-                        c = point_count<FP32>(a.ix, p.x, p.y, f, t, e, keep);
+                        c = NEAR ? near_count<FP32>(a.ix, a.near, p.x, p.y, keep)
+                                 : point_count<FP32>(a.ix, p.x, p.y, f, t, e, keep);
                     }
                 }
                 uint32_t inc = c;
@@ -1522,12 +1670,12 @@ __global__ void __launch_bounds__(kThreads, 3) k_wemit(JoinLaunch a, const unsig
             const uint32_t pid = a.pid0 + (uint32_t)(base + loc);
             const uint32_t w = has ? resolve(a.ix, (uint32_t)p.x, (uint32_t)p.y, keep) : 0u;
             uint32_t t = 0, e = 0;
-            walk_list_wave<FP32>(a.ix, (w >> 30) == kCellList, w & kPayloadMask, p.x, p.y, t, e, keep, s_par,
+            walk_list_wave<FP32, NEAR>(a.ix, (w >> 30) >= kCellList, w & kPayloadMask, p.x, p.y, t, e, keep, s_par,
                                  [&](uint32_t q) {
                                      if (o < a.cap)
                                          __stcs(a.pairs + o, make_uint2(pid, q));
                                      ++o;
-                                 });
+                                 }, &a.near);
         }
         __syncwarp(); // the queue is rewritten by the next chunk
     }
@@ -1962,158 +2110,6 @@ __global__ void __launch_bounds__(kPlainThreads) k_plain_write(JoinLaunch a, con
     }
 }
 
-// ------------------------------------------------------- buffered polygons
-// Is (px, py) within distance r of the closed segment v = (a, b)?  With
-// d = b - a, w = p - a and t = w . d: the distance is |w| when t <= 0, |p - b|
-// when t >= |d|^2, else |d x w| / |d|.  Coordinates lie in [0, 2^30], so every
-// product of two differences is below 2^60 in magnitude (int64 sums stay
-// exact); the last case compares (d x w)^2 with r^2 |d|^2 as 128-bit
-// products.  A zero-length edge takes the first case.
-__device__ __forceinline__ bool seg_near(const int4 &v, int px, int py, int64_t r)
-{
-    const int64_t dx = (int64_t)v.z - v.x, dy = (int64_t)v.w - v.y;
-    const int64_t wx = (int64_t)px - v.x, wy = (int64_t)py - v.y, rr = r * r;
-    const int64_t t = wx * dx + wy * dy;
-    if (t <= 0)
-        return wx * wx + wy * wy <= rr;
-    const int64_t dd = dx * dx + dy * dy;
-    if (t >= dd) {
-        const int64_t ux = (int64_t)px - v.z, uy = (int64_t)py - v.w;
-        return ux * ux + uy * uy <= rr;
-    }
-    const int64_t c = dx * wy - dy * wx;
-    const uint64_t ca = (uint64_t)(c < 0 ? -c : c);
-    const uint64_t lh = __umul64hi(ca, ca), ll = ca * ca;
-    const uint64_t rh = __umul64hi((uint64_t)rr, (uint64_t)dd), rl = (uint64_t)rr * (uint64_t)dd;
-    return lh < rh || (lh == rh && ll <= rl);
-}
-
-// Calls f(q) for every buffered polygon q that the in-box point (px, py)
-// meets, ascending, and returns their number: the polygons that contain the
-// point (its polygon index's cell, ascending), merged with the polygons of its
-// edge-grid cell that have an edge within r[q] of it (the cell's items are
-// sorted by polygon, each polygon's edges together; a polygon that contains
-// the point needs no edge test).
-template <bool FP32, class F>
-__device__ __forceinline__ uint32_t buffer_point(const IndexView &ix, const BufferView &bv, int px, int py,
-                                                 uint32_t &tests, uint32_t &esc, uint64_t pol, F f)
-{
-    const uint32_t c = (((uint32_t)py >> bv.sc) << bv.g) | ((uint32_t)px >> bv.sc);
-    if (!((__ldg(bv.mask + (c >> 5)) >> (c & 31)) & 1u))
-        return 0u; // no edge near the cell, no polygon in it: a small L2-resident screen
-    uint32_t k = __ldg(bv.cell_off + c);
-    const uint32_t kend = __ldg(bv.cell_off + c + 1);
-    if (!in_bounds(k <= kend && kend <= bv.n_items, ix))
-        return 0u;
-    uint32_t n = 0;
-    // the cell's polygons below `bound` that have an edge within r (an item
-    // flagged kBufferFull: the polygon's r-region holds the whole cell)
-    auto near_below = [&](uint32_t bound) {
-        while (k < kend) {
-            const uint32_t raw = __ldg(bv.item_q + k), q = raw & ~kBufferFull;
-            if (q >= bound || !in_bounds(q < bv.P, ix))
-                break;
-            bool hit = (raw & kBufferFull) != 0;
-            if (hit) {
-                ++k;
-            } else {
-                const int64_t r = __ldg(bv.rad + q);
-                for (; k < kend && __ldg(bv.item_q + k) == q; ++k)
-                    hit = hit || seg_near(ld_idx(bv.item_seg + k, pol), px, py, r);
-            }
-            if (hit) {
-                f(q);
-                ++n;
-            }
-        }
-    };
-    auto inside = [&](uint32_t q) {
-        near_below(q);
-        while (k < kend && (__ldg(bv.item_q + k) & ~kBufferFull) == q) // met already: no test
-            ++k;
-        f(q);
-        ++n;
-    };
-    const uint32_t w = resolve(ix, (uint32_t)px, (uint32_t)py, pol);
-    const uint32_t kind = w >> 30, pay = w & kPayloadMask;
-    if (kind == kCellInsideOne && in_bounds(pay < ix.P, ix))
-        inside(pay);
-    else if (kind == kCellList && in_bounds((uint64_t)pay + 1 < ix.n_ent, ix))
-        walk_entries<FP32>(ix, ix.ent + pay, px, py, tests, esc, pol, inside);
-    near_below(0xffffffffu);
-    return n;
-}
-
-// Pass 1: per-point pair counts (kept for pass 2), per-polygon counts, and
-// the pair total of every 256-point block (block_cnt null: counts only).
-template <bool FP32>
-__global__ void __launch_bounds__(kPlainThreads) k_buf_count(BufferLaunch a, uint32_t *pt_cnt,
-                                                             unsigned long long *block_cnt)
-{
-    __shared__ uint32_t s_w[kPlainThreads / 32];
-    const uint64_t i = (uint64_t)blockIdx.x * kPlainThreads + threadIdx.x;
-    const uint64_t keep = policy_evict_last();
-    uint32_t c = 0, t = 0, e = 0;
-    if (i < a.n) {
-        const int2 p = a.pts[i];
-        if ((uint32_t)(p.x | p.y) < kBox)
-            c = buffer_point<FP32>(a.ix, a.bv, p.x, p.y, t, e, keep, [&](uint32_t q) {
-                if (a.counts)
-                    atomicAdd(a.counts + q, 1ull);
-            });
-        if (pt_cnt)
-            pt_cnt[i] = c;
-    }
-    add_stats(a.stats, i < a.n ? 1u : 0u, t, e, c);
-    if (!block_cnt)
-        return;
-    const uint32_t s = warp_sum32(c);
-    if ((threadIdx.x & 31) == 0)
-        s_w[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long b = 0;
-        for (int w = 0; w < kPlainThreads / 32; ++w)
-            b += s_w[w];
-        block_cnt[blockIdx.x] = b;
-    }
-}
-
-// Pass 2: each point's pairs at its block's scanned offset plus the counts
-// of the block's earlier points.
-template <bool FP32>
-__global__ void __launch_bounds__(kPlainThreads) k_buf_write(BufferLaunch a, const uint32_t *pt_cnt,
-                                                             const unsigned long long *block_off)
-{
-    __shared__ uint32_t s_w[kPlainThreads / 32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint64_t i = (uint64_t)blockIdx.x * kPlainThreads + threadIdx.x;
-    const uint32_t c = i < a.n ? pt_cnt[i] : 0u;
-    uint32_t inc = c;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t v = __shfl_up_sync(kFull, inc, o);
-        if (lane >= o)
-            inc += v;
-    }
-    if (lane == 31)
-        s_w[warp] = inc;
-    __syncthreads();
-    uint32_t wpre = 0;
-    for (int w = 0; w < warp; ++w)
-        wpre += s_w[w];
-    if (!c)
-        return;
-    unsigned long long o = block_off[blockIdx.x] + wpre + inc - c;
-    const int2 p = a.pts[i];
-    uint32_t t = 0, e = 0;
-    buffer_point<FP32>(a.ix, a.bv, p.x, p.y, t, e, policy_evict_last(), [&](uint32_t q) {
-        if (o < a.cap)
-            a.pairs[o] = make_uint2((uint32_t)i, q);
-        ++o;
-    });
-}
-
 // Opt a kernel in to the shared memory it needs (once per device).
 template <class K>
 cudaError_t smem_opt_in(K kernel, size_t bytes, bool (&done)[64])
@@ -2221,7 +2217,7 @@ __global__ void __launch_bounds__(256) k_agg_cells(const unsigned long long *cel
 // Pass 1 of the join (1a resolve, 1b walk).  pend: 8 words per chunk (the
 // bitmap of the rows pass 1b tests).  mid (or null): an event recorded between
 // the two kernels.
-template <bool FP32, int OUT>
+template <bool FP32, int OUT, bool NEAR>
 cudaError_t launch_pass1_as(const JoinLaunch &a, uint32_t *pend, cudaStream_t s, cudaEvent_t mid)
 {
     static bool done_r[4][64] = {};
@@ -2268,14 +2264,27 @@ cudaError_t launch_pass1_as(const JoinLaunch &a, uint32_t *pend, cudaStream_t s,
     const uint64_t nwords = nchunks * kWItems;
     const uint32_t range = walk_range(nwords);
     const uint64_t wblk = (nwords + uint64_t(kWarps) * range - 1) / (uint64_t(kWarps) * range);
-    k_walk<FP32, OUT><<<unsigned(wblk), kThreads, 0, s>>>(a, pend, uint32_t(nwords), range);
+    k_walk<FP32, OUT, NEAR><<<unsigned(wblk), kThreads, 0, s>>>(a, pend, uint32_t(nwords), range);
     return cudaGetLastError();
 }
 
-template <bool FP32>
-cudaError_t launch_pass1(const JoinLaunch &a, uint32_t *pend, cudaStream_t s, cudaEvent_t mid)
+// Calls f(fp32, near) with the launch's two switches as compile-time values.
+template <class F>
+cudaError_t with_switches(const JoinLaunch &a, F f)
 {
-    return a.narrow ? launch_pass1_as<FP32, kOut16>(a, pend, s, mid) : launch_pass1_as<FP32, kOut32>(a, pend, s, mid);
+    if (a.near.rad)
+        return a.fp32 ? f(std::true_type{}, std::true_type{}) : f(std::false_type{}, std::true_type{});
+    return a.fp32 ? f(std::true_type{}, std::false_type{}) : f(std::false_type{}, std::false_type{});
+}
+
+cudaError_t launch_pass1(const JoinLaunch &a, uint32_t *pend, cudaStream_t s, cudaEvent_t mid, bool count_only)
+{
+    return with_switches(a, [&](auto fp32, auto near) {
+        constexpr bool F = decltype(fp32)::value, N = decltype(near)::value;
+        return count_only ? launch_pass1_as<F, kOutCount, N>(a, pend, s, mid)
+               : a.narrow ? launch_pass1_as<F, kOut16, N>(a, pend, s, mid)
+                          : launch_pass1_as<F, kOut32, N>(a, pend, s, mid);
+    });
 }
 
 // Exclusive scan of n values in place; the total goes to *total.  part: at
@@ -3054,8 +3063,7 @@ static cudaError_t join_resolve_scan(const JoinLaunch &a, unsigned long long *pa
     if (nchunks == 0)
         return a.total ? cudaMemsetAsync(a.total, 0, sizeof(unsigned long long), s) : cudaSuccess;
     uint32_t *pend = reinterpret_cast<uint32_t *>(part);
-    cudaError_t e = a.fp32 ? launch_pass1<true>(a, pend, s, ev ? ev[0] : nullptr)
-                           : launch_pass1<false>(a, pend, s, ev ? ev[0] : nullptr);
+    cudaError_t e = launch_pass1(a, pend, s, ev ? ev[0] : nullptr, false);
     if (e != cudaSuccess)
         return e;
     if (ev)
@@ -3079,37 +3087,39 @@ cudaError_t launch_join_emit(const JoinLaunch &a, cudaStream_t s, const uint32_t
     if (a.narrow && !pend)
         return cudaErrorInvalidValue;
     const uint32_t nblk = (nchunks + kWarps - 1) / kWarps;
-    static bool done[4][64] = {};
-    auto emit = [&](auto kr, bool(&d)[64]) -> cudaError_t {
-        cudaError_t e = smem_opt_in(kr, kEmitSmem, d);
-        if (e != cudaSuccess)
-            return e;
-        kr<<<persistent_grid(kr, kThreads, kEmitSmem, nblk), kThreads, kEmitSmem, s>>>(a, a.tile_tot, nchunks, pend);
-        return cudaGetLastError();
-    };
-    if (a.narrow)
-        return a.fp32 ? emit(k_wemit<true, true, false>, done[2]) : emit(k_wemit<false, true, false>, done[3]);
-    return a.fp32 ? emit(k_wemit<true, false, false>, done[0]) : emit(k_wemit<false, false, false>, done[1]);
+    static bool done[8][64] = {};
+    return with_switches(a, [&](auto fp32, auto near) {
+        constexpr bool F = decltype(fp32)::value, N = decltype(near)::value;
+        auto emit = [&](auto kr, bool(&d)[64]) -> cudaError_t {
+            cudaError_t e = smem_opt_in(kr, kEmitSmem, d);
+            if (e != cudaSuccess)
+                return e;
+            kr<<<persistent_grid(kr, kThreads, kEmitSmem, nblk), kThreads, kEmitSmem, s>>>(a, a.tile_tot, nchunks, pend);
+            return cudaGetLastError();
+        };
+        return a.narrow ? emit(k_wemit<F, true, false, N>, done[F + 2 * N])
+                        : emit(k_wemit<F, false, false, N>, done[4 + F + 2 * N]);
+    });
 }
 
 // The join of a small table (at most kSmallChunks chunks, with an output): two
 // launches, k_small and k_wemit<SELF>.  ev as for launch_join.
-template <bool FP32, bool R16>
+template <bool FP32, bool R16, bool NEAR>
 static cudaError_t launch_small(const JoinLaunch &a, uint32_t *pend, cudaStream_t s, cudaEvent_t *ev)
 {
     static bool done[64] = {};
     const uint32_t nchunks = uint32_t((a.n + kWChunk - 1) / kWChunk), nblk = (nchunks + kWarps - 1) / kWarps;
     if (ev)
         cudaEventRecord(ev[0], s);
-    k_small<FP32, R16><<<nblk, kThreads, 0, s>>>(a, pend, nchunks, a.ix.P <= kSmallHist ? 1 : 0);
+    k_small<FP32, R16 ? kOut16 : kOut32, NEAR><<<nblk, kThreads, 0, s>>>(a, pend, nchunks, a.ix.P <= kSmallHist ? 1 : 0);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess)
-        e = smem_opt_in(k_wemit<FP32, R16, true>, kEmitSmem, done);
+        e = smem_opt_in(k_wemit<FP32, R16, true, NEAR>, kEmitSmem, done);
     if (e != cudaSuccess)
         return e;
     for (int k = 1; ev && k < 4; ++k)
         cudaEventRecord(ev[k], s);
-    k_wemit<FP32, R16, true><<<nblk, kThreads, kEmitSmem, s>>>(a, a.tile_tot, nchunks, pend);
+    k_wemit<FP32, R16, true, NEAR><<<nblk, kThreads, kEmitSmem, s>>>(a, a.tile_tot, nchunks, pend);
     return cudaGetLastError();
 }
 
@@ -3201,10 +3211,10 @@ cudaError_t launch_join(const JoinLaunch &a, void *scratch, cudaStream_t s, cuda
         if (a.counts && a.ix.P && !a.keep_counts)
             if ((e = cudaMemsetAsync(a.counts, 0, sizeof(unsigned long long) * a.ix.P, s)) != cudaSuccess)
                 return e;
-        if (b.narrow)
-            e = a.fp32 ? launch_small<true, true>(b, pend, s, ev) : launch_small<false, true>(b, pend, s, ev);
-        else
-            e = a.fp32 ? launch_small<true, false>(b, pend, s, ev) : launch_small<false, false>(b, pend, s, ev);
+        e = with_switches(b, [&](auto fp32, auto near) {
+            constexpr bool F = decltype(fp32)::value, N = decltype(near)::value;
+            return b.narrow ? launch_small<F, true, N>(b, pend, s, ev) : launch_small<F, false, N>(b, pend, s, ev);
+        });
         if (ev)
             cudaEventRecord(ev[4], s);
         return e;
@@ -3233,7 +3243,10 @@ static bool use_directory(const JoinLaunch &a)
 // 50.9 / 38.1).  Only with the summary: without it (a 40000-cell map, counts in
 // global memory) the one pass is as fast (2021 / 2068 us).
 constexpr uint64_t kSplitCountMin = uint64_t(1) << 21;
-bool use_split_count(const JoinLaunch &a) { return !a.clustered && a.ix.use_sum && a.n > kSplitCountMin; }
+bool use_split_count(const JoinLaunch &a)
+{
+    return a.n > kSplitCountMin && (a.near.rad || (!a.clustered && a.ix.use_sum));
+}
 
 static size_t split_count_bytes(uint64_t n)
 {
@@ -3243,7 +3256,7 @@ static size_t split_count_bytes(uint64_t n)
 size_t aggregate_scratch_bytes(const JoinLaunch &a)
 {
     const uint64_t nchunks = (a.n + kWChunk - 1) / kWChunk;
-    if (!a.clustered)
+    if (!a.clustered || a.near.rad)
         return split_count_bytes(a.n);
     return use_directory(a) ? size_t((nchunks + 31) / 32) * 4 + 16 : 16;
 }
@@ -3261,11 +3274,22 @@ cudaError_t launch_aggregate(const JoinLaunch &a, void *scratch, cudaStream_t s,
         if (ev)
             cudaEventRecord(ev[0], s);
         uint32_t *pend = static_cast<uint32_t *>(scratch);
-        e = a.fp32 ? launch_pass1_as<true, kOutCount>(a, pend, s, nullptr)
-                   : launch_pass1_as<false, kOutCount>(a, pend, s, nullptr);
+        e = launch_pass1(a, pend, s, nullptr, true);
         if (ev)
             cudaEventRecord(ev[1], s);
         return e;
+    }
+    if (a.near.rad) { // few points, or no scratch to have: one launch that keeps nothing
+        const uint64_t nchunks = (a.n + kWChunk - 1) / kWChunk;
+        if (a.n >= (1ull << 32))
+            return cudaErrorInvalidValue;
+        const unsigned nblk = unsigned((nchunks + kWarps - 1) / kWarps);
+        const int hist = a.ix.P <= kSmallHist ? 1 : 0;
+        if (a.fp32)
+            k_small<true, kOutCount, true><<<nblk, kThreads, 0, s>>>(a, nullptr, uint32_t(nchunks), hist);
+        else
+            k_small<false, kOutCount, true><<<nblk, kThreads, 0, s>>>(a, nullptr, uint32_t(nchunks), hist);
+        return cudaGetLastError();
     }
     const int use_hist = a.ix.P <= (uint32_t)kHistMax ? 1 : 0;
     if (ev)
@@ -3610,8 +3634,14 @@ cudaError_t launch_disk_select(const DiskLaunch &a, uint32_t *ids, uint64_t cap,
 }
 
 // ------------------------------------------------ buffered polygons: launchers
-__global__ void k_buf_mask(const uint32_t *cell, int gp, uint32_t *mask, int g)
+// Sets the bits of the cells of a 2^g grid that list items or meet a non-empty
+// coarse cell of the polygons' own index (2^gp).
+__global__ void k_buf_mask(const uint32_t *cell, int gp, const uint32_t *cell_off, uint32_t *mask, int g)
 {
+    const uint64_t nc = uint64_t(1) << (2 * g);
+    for (uint64_t c = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; c < nc; c += (uint64_t)gridDim.x * blockDim.x)
+        if (cell_off[c + 1] > cell_off[c])
+            atomicOr(mask + (c >> 5), 1u << (c & 31));
     const uint64_t n = uint64_t(1) << (2 * gp);
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
         if (!cell[i])
@@ -3631,95 +3661,331 @@ __global__ void k_buf_mask(const uint32_t *cell, int gp, uint32_t *mask, int g)
     }
 }
 
-cudaError_t launch_buffer_mask(const IndexView &ix, uint32_t *mask, int g, cudaStream_t s)
+static cudaError_t launch_buffer_mask(const IndexView &ix, const uint32_t *cell_off, uint32_t *mask, int g)
 {
     const uint64_t n = uint64_t(1) << (2 * ix.gc);
     const unsigned grid = unsigned(std::min<uint64_t>((n + 255) / 256, uint64_t(device_sm_count()) * 32));
-    k_buf_mask<<<grid, 256, 0, s>>>(ix.cell, ix.gc, mask, g);
+    k_buf_mask<<<grid, 256>>>(ix.cell, ix.gc, cell_off, mask, g);
     return cudaGetLastError();
 }
 
+// The index of buffered polygons (NearView) from the edge grid.  A cell's groups
+// (its polygons, ascending) are the union of the groups of items of its edge-grid
+// cell and of the polygons that hold its corner.  With S the side of the cell:
+//   whole   every point of the cell meets the polygon: the group is flagged
+//           kBufferFull, or one edge has the cell's four extreme points within r
+//           (the points within r of a segment are a convex set), or the polygon
+//           holds the corner and no edge's box meets the cell;
+//   cross   an edge's box meets the cell, so points of the cell may differ in
+//           being inside (an edge that passes between two points of the cell is
+//           listed there: the listing reaches every edge within r >= 0 of the
+//           box of the cell's points);
+//   edges   those within r + h + 2 of the cell's centre, h half its diagonal, in
+//           FP32 with the coordinate differences' rounding (2^-24 relative, a
+//           few of them) covered by 2^-18 of their sum;
+//   none    neither cross nor edges: no point of the cell meets the polygon.
+struct NearCell {
+    int x0, y0, S;
+};
 
-size_t buffer_scratch_bytes(uint64_t n)
+__device__ __forceinline__ bool edge_reaches(const int4 &v, const NearCell &c, int r)
 {
-    const uint64_t nb = (n + kPlainThreads - 1) / kPlainThreads;
-    return size_t(((n * 4 + 15) & ~uint64_t(15)) + (nb + scan_partials(nb) + 2) * 8 + 16);
+    const float dx = __int2float_rn(v.z - v.x), dy = __int2float_rn(v.w - v.y), m = 0.5f * __int2float_rn(c.S - 1);
+    const float wx = __int2float_rn(c.x0 - v.x) + m, wy = __int2float_rn(c.y0 - v.y) + m;
+    const float dd = dx * dx + dy * dy;
+    const float t = dd > 0.f ? fminf(1.f, fmaxf(0.f, (wx * dx + wy * dy) / dd)) : 0.f;
+    const float ex = wx - t * dx, ey = wy - t * dy;
+    const float reach = __int2float_rn(r) + 1.41421366f * m + 2.f;
+    const float slack = 3.814697265625e-06f * (fabsf(wx) + fabsf(wy) + fabsf(dx) + fabsf(dy) + reach); // 2^-18
+    return sqrtf(ex * ex + ey * ey) <= reach + slack;
 }
 
-cudaError_t launch_buffer_join(const BufferLaunch &a, void *scratch, cudaStream_t s)
+// Calls add(q, first item, end, flags) for every group of the cell but those
+// that no point meets: flags 0 for whole, else kEntBoundary and kEntCross.
+template <class F>
+__device__ __forceinline__ void near_groups(const IndexView &in, const uint32_t *item_q, const int4 *item_seg,
+                                            const int32_t *rad, uint32_t k, uint32_t kend, const NearCell &c, F add)
 {
-    if (a.n >= (1ull << 32))
-        return cudaErrorInvalidValue; // point ids are 32-bit
-    cudaError_t e = cudaSuccess;
-    if (a.counts && a.bv.P)
-        e = cudaMemsetAsync(a.counts, 0, sizeof(unsigned long long) * a.bv.P, s);
-    if (e != cudaSuccess)
-        return e;
-    if (a.n == 0)
-        return a.total ? cudaMemsetAsync(a.total, 0, sizeof(unsigned long long), s) : cudaSuccess;
-    const uint64_t nb = (a.n + kPlainThreads - 1) / kPlainThreads;
-    char *sc = static_cast<char *>(scratch);
-    uint32_t *pt_cnt = reinterpret_cast<uint32_t *>(sc);
-    unsigned long long *block = reinterpret_cast<unsigned long long *>(sc + ((a.n * 4 + 15) & ~uint64_t(15)));
-    unsigned long long *part = block + nb;
-    if (a.fp32)
-        k_buf_count<true><<<(unsigned)nb, kPlainThreads, 0, s>>>(a, pt_cnt, block);
-    else
-        k_buf_count<false><<<(unsigned)nb, kPlainThreads, 0, s>>>(a, pt_cnt, block);
-    if ((e = cudaGetLastError()) != cudaSuccess)
-        return e;
-    if ((e = launch_scan(block, nb, a.total, part, s)) != cudaSuccess)
-        return e;
-    if (!a.cap)
-        return cudaSuccess;
-    if (a.fp32)
-        k_buf_write<true><<<(unsigned)nb, kPlainThreads, 0, s>>>(a, pt_cnt, block);
-    else
-        k_buf_write<false><<<(unsigned)nb, kPlainThreads, 0, s>>>(a, pt_cnt, block);
-    return cudaGetLastError();
+    const int x1 = c.x0 + c.S - 1, y1 = c.y0 + c.S - 1;
+    auto group = [&](uint32_t q, bool holds) {
+        const uint32_t k0 = k;
+        if (item_q[k] & kBufferFull) {
+            ++k;
+            add(q, 0u, 0u, 0u);
+            return;
+        }
+        const int r = rad[q];
+        bool cross = false, reach = false, whole = false;
+        for (; k < kend && item_q[k] == q; ++k) {
+            const int4 v = item_seg[k];
+            cross = cross || (min(v.x, v.z) <= x1 && max(v.x, v.z) >= c.x0 && min(v.y, v.w) <= y1 && max(v.y, v.w) >= c.y0);
+            if (!whole && edge_reaches(v, c, r)) {
+                reach = true;
+                whole = seg_near<true>(v, c.x0, c.y0, r) && seg_near<true>(v, x1, c.y0, r) &&
+                        seg_near<true>(v, c.x0, y1, r) && seg_near<true>(v, x1, y1, r);
+            }
+        }
+        if (whole || (holds && !cross))
+            add(q, 0u, 0u, 0u);
+        else if (reach || cross)
+            add(q, k0, k, kEntBoundary | (cross ? kEntCross : 0u));
+    };
+    auto inside = [&](uint32_t q) {
+        while (k < kend && (item_q[k] & ~kBufferFull) < q)
+            group(item_q[k] & ~kBufferFull, false);
+        if (k < kend && (item_q[k] & ~kBufferFull) == q)
+            group(q, true);
+        else
+            add(q, 0u, 0u, 0u);
+    };
+    uint32_t t = 0, s = 0;
+    const uint64_t keep = policy_evict_last();
+    const uint32_t w = resolve(in, (uint32_t)c.x0, (uint32_t)c.y0, keep);
+    if ((w >> 30) == kCellInsideOne)
+        inside(w & kPayloadMask);
+    else if ((w >> 30) == kCellList)
+        walk_entries<false>(in, in.ent + (w & kPayloadMask), c.x0, c.y0, t, s, keep, inside);
+    while (k < kend)
+        group(item_q[k] & ~kBufferFull, false);
 }
 
-cudaError_t launch_buffer_aggregate(const BufferLaunch &a, cudaStream_t s)
+// Coarse level, a thread per cell.  COUNT: the cell's word (kinds kCellSub and
+// kCellCoarseList without their payload), its entries when it is a coarse list,
+// and 1 when it is split.  Else: the payloads and the coarse lists.
+template <bool COUNT>
+__global__ void __launch_bounds__(256) k_near_coarse(IndexView in, const uint32_t *cell_off, const uint32_t *item_q,
+                                                     const int4 *item_seg, const int32_t *rad, const uint32_t *mask,
+                                                     int g, unsigned long long *n_ent, unsigned long long *n_blk,
+                                                     uint32_t *cell, uint4 *ent)
 {
-    cudaError_t e = cudaMemsetAsync(a.counts, 0, sizeof(unsigned long long) * (a.bv.P ? a.bv.P : 1), s);
-    if (e != cudaSuccess || a.n == 0)
-        return e;
-    const uint64_t nb = (a.n + kPlainThreads - 1) / kPlainThreads;
-    if (nb >= (1ull << 31))
-        return cudaErrorInvalidValue;
-    if (a.fp32)
-        k_buf_count<true><<<(unsigned)nb, kPlainThreads, 0, s>>>(a, nullptr, nullptr);
-    else
-        k_buf_count<false><<<(unsigned)nb, kPlainThreads, 0, s>>>(a, nullptr, nullptr);
-    return cudaGetLastError();
+    const uint32_t ncell = 1u << (2 * g);
+    const int sh = kBoxLog2 - g;
+    for (uint32_t c = blockIdx.x * 256 + threadIdx.x; c < ncell; c += gridDim.x * 256) {
+        if (COUNT && !((mask[c >> 5] >> (c & 31)) & 1u)) {
+            n_ent[c] = n_blk[c] = 0;
+            cell[c] = 0u;
+            continue;
+        }
+        const uint32_t kind = COUNT ? 0u : cell[c] >> 30;
+        if (!COUNT && kind < kCellSub)
+            continue;
+        if (!COUNT && kind == kCellSub) {
+            cell[c] |= (uint32_t)n_blk[c];
+            continue;
+        }
+        const NearCell nc{int((c & ((1u << g) - 1)) << sh), int((c >> g) << sh), 1 << sh};
+        const uint64_t off = COUNT ? 0 : n_ent[c];
+        uint32_t n = 0, one = 0;
+        bool lists = false;
+        near_groups(in, item_q, item_seg, rad, cell_off[c], cell_off[c + 1], nc,
+                    [&](uint32_t q, uint32_t, uint32_t, uint32_t flags) {
+                        if (!COUNT)
+                            ent[off + n] = make_uint4(q, 0u, 0u, 0u);
+                        one = q;
+                        lists = lists || flags;
+                        ++n;
+                    });
+        if (COUNT) {
+            n_ent[c] = !lists && n > 1 ? n : 0;
+            n_blk[c] = lists ? 1 : 0;
+            cell[c] = lists ? kCellSub << 30 : n > 1 ? kCellCoarseList << 30 : n ? (kCellInsideOne << 30) | one : 0u;
+        } else {
+            ent[off + n - 1].w = kEntLast;
+            cell[c] |= uint32_t(off);
+        }
+    }
 }
 
-size_t buffer_select_scratch_bytes(uint64_t n, uint32_t P, uint64_t cap)
+// The cell of every block.
+__global__ void __launch_bounds__(256) k_near_blocks(uint32_t ncell, const uint32_t *cell,
+                                                     const unsigned long long *n_blk, uint32_t *blk_cell)
 {
-    return ((buffer_scratch_bytes(n) + 15) & ~size_t(15)) + 16 + cap * 8 + partition_scratch_bytes(cap, P);
+    for (uint32_t c = blockIdx.x * 256 + threadIdx.x; c < ncell; c += gridDim.x * 256)
+        if ((cell[c] >> 30) == kCellSub)
+            blk_cell[n_blk[c]] = c;
 }
 
-cudaError_t launch_buffer_select(const BufferLaunch &a, uint32_t *ids, uint64_t cap, unsigned long long *offsets,
-                                 void *scratch, cudaStream_t s)
+// Fine level, a thread per fine cell of every block.  COUNT: its word (a list's
+// without its offset), its entries and its edges; else the lists.
+template <bool COUNT>
+__global__ void __launch_bounds__(256) k_near_fine(IndexView in, const uint32_t *cell_off, const uint32_t *item_q,
+                                                   const int4 *item_seg, const int32_t *rad, int g, int sb,
+                                                   const uint32_t *blk_cell, uint64_t n_fine, unsigned long long *n_ent,
+                                                   unsigned long long *n_edge, uint64_t ent0, uint32_t *fine, uint4 *ent,
+                                                   int4 *edge)
 {
-    if (a.bv.P > (uint32_t)kSelMaxQ)
-        return cudaErrorInvalidValue;
-    char *sc = static_cast<char *>(scratch);
-    void *join_scratch = sc;
-    sc += (buffer_scratch_bytes(a.n) + 15) & ~size_t(15);
-    unsigned long long *total = reinterpret_cast<unsigned long long *>(sc);
-    sc += 16;
-    uint2 *pairs = reinterpret_cast<uint2 *>(sc);
-    sc += cap * 8;
-    BufferLaunch b = a;
-    b.pairs = pairs;
-    b.cap = cap;
-    b.counts = nullptr;
-    b.total = total;
-    cudaError_t e = launch_buffer_join(b, join_scratch, s);
-    if (e != cudaSuccess)
-        return e;
-    return launch_partition(pairs, total, cap, a.bv.P, ids, offsets, sc, s);
+    const int sh = kBoxLog2 - g, sf = sh - sb;
+    const uint32_t fm = (1u << sb) - 1;
+    for (uint64_t t = (uint64_t)blockIdx.x * 256 + threadIdx.x; t < n_fine; t += (uint64_t)gridDim.x * 256) {
+        if (!COUNT && (fine[t] >> 30) != kCellList)
+            continue;
+        const uint32_t c = blk_cell[t >> (2 * sb)], f = (uint32_t)t & ((1u << (2 * sb)) - 1);
+        const NearCell nc{int(((c & ((1u << g) - 1)) << sh) | ((f & fm) << sf)), int(((c >> g) << sh) | ((f >> sb) << sf)),
+                          1 << sf};
+        const uint64_t off = COUNT ? 0 : ent0 + n_ent[t], eoff = COUNT ? 0 : n_edge[t];
+        uint32_t n = 0, one = 0, ne = 0;
+        bool whole = false;
+        near_groups(in, item_q, item_seg, rad, cell_off[c], cell_off[c + 1], nc,
+                    [&](uint32_t q, uint32_t k0, uint32_t k1, uint32_t flags) {
+                        const uint32_t first = ne;
+                        for (uint32_t k = k0; k < k1; ++k) {
+                            const int4 v = item_seg[k];
+                            if (edge_reaches(v, nc, rad[q])) {
+                                if (!COUNT)
+                                    edge[eoff + ne] = v;
+                                ++ne;
+                            }
+                        }
+                        if (!COUNT)
+                            ent[off + n] = make_uint4(q, uint32_t(eoff + first), ne - first, flags);
+                        one = q;
+                        whole = !flags;
+                        ++n;
+                    });
+        if (COUNT) {
+            const bool lst = n > 1 || (n == 1 && !whole);
+            n_ent[t] = lst ? n : 0;
+            n_edge[t] = lst ? ne : 0;
+            fine[t] = lst ? kCellList << 30 : n ? (kCellInsideOne << 30) | one : 0u;
+        } else {
+            ent[off + n - 1].w |= kEntLast;
+            fine[t] = (kCellList << 30) | uint32_t(off);
+        }
+    }
+}
+
+// Block summary of the coarse words (an empty block, one polygon holding it, or
+// mixed), the number of blocks that are not mixed, and the sentinels.
+__global__ void __launch_bounds__(256) k_near_sum(int g, int sg, const uint32_t *cell, uint16_t *sum,
+                                                  unsigned long long *resolved, uint4 *ent_end, int4 *edge_end)
+{
+    const uint32_t nb = 1u << sg, sh = uint32_t(g - sg), t = blockIdx.x * 256 + threadIdx.x;
+    if (t < 4)
+        ent_end[t] = make_uint4(0u, 0u, 0u, kEntLast);
+    if (t == 0)
+        *edge_end = make_int4(0, 0, 0, 0);
+    if (t >= nb * nb)
+        return;
+    const uint32_t by = t / nb, bx = t % nb, w0 = cell[(uint64_t(by << sh) << g) | (bx << sh)];
+    bool same = (w0 >> 30) == kCellEmpty || ((w0 >> 30) == kCellInsideOne && (w0 & kPayloadMask) < kSumEmpty);
+    for (uint32_t cy = by << sh; same && cy < ((by + 1) << sh); ++cy)
+        for (uint32_t cx = bx << sh; same && cx < ((bx + 1) << sh); ++cx)
+            same = cell[(uint64_t(cy) << g) | cx] == w0;
+    sum[t] = uint16_t(!same ? kSumMixed : (w0 >> 30) == kCellEmpty ? kSumEmpty : (w0 & kPayloadMask));
+    if (same)
+        atomicAdd(resolved, 1ull);
+}
+
+int build_near_index_device(const IndexView &in, const uint32_t *cell_off, const uint32_t *item_q, const int4 *item_seg,
+                            const int32_t *rad, int g, NearIndexDev &out, cudaError_t &cerr)
+{
+    out = NearIndexDev{};
+    const uint32_t ncell = 1u << (2 * g);
+    const int sg = std::min(g, kSumLog2);
+    auto up = [](size_t v) { return (v + 255) & ~size_t(255); };
+    char *tmp = nullptr, *tmp2 = nullptr;
+    cudaError_t &e = cerr;
+    auto done = [&](int status) {
+        cudaFree(tmp);
+        cudaFree(tmp2);
+        if (status && out.mem) {
+            cudaFree(out.mem);
+            out.mem = nullptr;
+        }
+        return status;
+    };
+    auto blocks = [](uint64_t n) { return unsigned(std::min<uint64_t>((n + 255) / 256, uint64_t(device_sm_count()) * 32)); };
+    const size_t t_cnt = up(size_t(ncell) * 8), t_part = up((scan_partials(ncell) + 2) * 8),
+                 t_mask = up(std::max<size_t>(ncell / 8, 4)), b_cell = up(size_t(ncell) * 4),
+                 b_sum = up(std::max<size_t>(size_t(2) << (2 * sg), 16));
+    if ((e = cudaMalloc(&tmp, 2 * t_cnt + t_part + t_mask + 2 * b_cell + 256)) != cudaSuccess)
+        return done(2);
+    auto *n_ent = reinterpret_cast<unsigned long long *>(tmp);
+    auto *n_blk = reinterpret_cast<unsigned long long *>(tmp + t_cnt);
+    auto *part = reinterpret_cast<unsigned long long *>(tmp + 2 * t_cnt);
+    auto *mask = reinterpret_cast<uint32_t *>(tmp + 2 * t_cnt + t_part);
+    auto *word = reinterpret_cast<uint32_t *>(tmp + 2 * t_cnt + t_part + t_mask);
+    auto *blk_cell = reinterpret_cast<uint32_t *>(tmp + 2 * t_cnt + t_part + t_mask + b_cell);
+    // coarse entries, blocks, fine entries, fine edges, resolved summary blocks
+    auto *tot = reinterpret_cast<unsigned long long *>(tmp + 2 * t_cnt + t_part + t_mask + 2 * b_cell);
+    unsigned long long h[5] = {};
+    if ((e = cudaMemset(mask, 0, t_mask)) != cudaSuccess || (e = cudaMemset(tot, 0, sizeof(h))) != cudaSuccess ||
+        (e = launch_buffer_mask(in, cell_off, mask, g)) != cudaSuccess)
+        return done(2);
+    k_near_coarse<true><<<blocks(ncell), 256>>>(in, cell_off, item_q, item_seg, rad, mask, g, n_ent, n_blk, word, nullptr);
+    if ((e = cudaGetLastError()) != cudaSuccess || (e = launch_scan(n_ent, ncell, tot, part, nullptr)) != cudaSuccess ||
+        (e = launch_scan(n_blk, ncell, tot + 1, part, nullptr)) != cudaSuccess ||
+        (e = cudaMemcpy(h, tot, 16, cudaMemcpyDeviceToHost)) != cudaSuccess)
+        return done(2);
+    const uint64_t NB = h[1];
+    k_near_blocks<<<blocks(ncell), 256>>>(ncell, word, n_blk, blk_cell);
+    // 8 x 8 fine cells per split cell, fewer where that would be more than 2^27
+    // fine cells, or more entries or edges than their offsets can name
+    for (int sb = kMaxSubLog2;; --sb) {
+        const uint64_t nf = NB << (2 * sb);
+        if (sb && (nf > (uint64_t(1) << 27) || g + sb > kMaxFineLog2))
+            continue;
+        const size_t t_f = up(std::max<uint64_t>(nf, 1) * 8), t_fp = up((scan_partials(nf) + 2) * 8),
+                     t_fw = up(std::max<uint64_t>(nf, 1) * 4);
+        if ((e = cudaMalloc(&tmp2, 2 * t_f + t_fp + t_fw)) != cudaSuccess) {
+            if (!sb)
+                return done(2);
+            cudaGetLastError();
+            tmp2 = nullptr;
+            continue;
+        }
+        auto *f_ent = reinterpret_cast<unsigned long long *>(tmp2);
+        auto *f_edge = reinterpret_cast<unsigned long long *>(tmp2 + t_f);
+        auto *f_part = reinterpret_cast<unsigned long long *>(tmp2 + 2 * t_f);
+        auto *f_word = reinterpret_cast<uint32_t *>(tmp2 + 2 * t_f + t_fp);
+        if (NB) {
+            k_near_fine<true><<<blocks(nf), 256>>>(in, cell_off, item_q, item_seg, rad, g, sb, blk_cell, nf, f_ent, f_edge, 0,
+                                                   f_word, nullptr, nullptr);
+            if ((e = cudaGetLastError()) != cudaSuccess || (e = launch_scan(f_ent, nf, tot + 2, f_part, nullptr)) != cudaSuccess ||
+                (e = launch_scan(f_edge, nf, tot + 3, f_part, nullptr)) != cudaSuccess ||
+                (e = cudaMemcpy(h, tot, 32, cudaMemcpyDeviceToHost)) != cudaSuccess)
+                return done(2);
+        }
+        if (h[0] + h[2] + 4 > kPayloadMask || h[3] + 1 >= (1ull << 32)) {
+            if (!sb)
+                return done(1);
+            cudaFree(tmp2);
+            tmp2 = nullptr;
+            continue;
+        }
+        const size_t b_fine = t_fw, b_ent = up((h[0] + h[2] + 4) * sizeof(uint4)), b_edge = up((h[3] + 1) * sizeof(int4));
+        out.bytes = b_cell + b_fine + b_ent + b_edge + b_sum;
+        if ((e = cudaMalloc(&out.mem, out.bytes)) != cudaSuccess) {
+            out.mem = nullptr;
+            return done(2);
+        }
+        char *m = static_cast<char *>(out.mem);
+        out.cell = reinterpret_cast<uint32_t *>(m);
+        out.fine = reinterpret_cast<uint32_t *>(m + b_cell);
+        out.ent = reinterpret_cast<uint4 *>(m + b_cell + b_fine);
+        out.edge = reinterpret_cast<int4 *>(m + b_cell + b_fine + b_ent);
+        out.sum = reinterpret_cast<uint16_t *>(m + b_cell + b_fine + b_ent + b_edge);
+        out.sb = sb;
+        out.n_fine = std::max<uint64_t>(nf, 1);
+        out.n_ent = h[0] + h[2] + 4;
+        out.n_edge = h[3] + 1;
+        if ((e = cudaMemcpy(out.cell, word, size_t(ncell) * 4, cudaMemcpyDeviceToDevice)) != cudaSuccess ||
+            (e = cudaMemset(out.fine, 0, 4)) != cudaSuccess ||
+            (nf && (e = cudaMemcpy(out.fine, f_word, nf * 4, cudaMemcpyDeviceToDevice)) != cudaSuccess))
+            return done(2);
+        k_near_coarse<false><<<blocks(ncell), 256>>>(in, cell_off, item_q, item_seg, rad, mask, g, n_ent, n_blk, out.cell,
+                                                     out.ent);
+        if (NB)
+            k_near_fine<false><<<blocks(nf), 256>>>(in, cell_off, item_q, item_seg, rad, g, sb, blk_cell, nf, f_ent, f_edge,
+                                                    h[0], out.fine, out.ent, out.edge);
+        k_near_sum<<<((1u << (2 * sg)) + 255) / 256, 256>>>(g, sg, out.cell, out.sum, tot + 4, out.ent + (out.n_ent - 4),
+                                                            out.edge + h[3]);
+        if ((e = cudaGetLastError()) != cudaSuccess ||
+            (e = cudaMemcpy(h + 4, tot + 4, 8, cudaMemcpyDeviceToHost)) != cudaSuccess)
+            return done(2);
+        out.sum_resolved = double(h[4]) / double(uint64_t(1) << (2 * sg));
+        return done(0);
+    }
 }
 
 } // namespace spx

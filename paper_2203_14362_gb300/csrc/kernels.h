@@ -34,6 +34,21 @@ struct IndexView {
     uint64_t n_fine, n_ent, n_edge;
     unsigned *err;
 };
+// Buffered polygons (SPADE §4.2 distance canvases: a polygon plus a rounded
+// rectangle of radius r around each edge).  The index is an IndexView as ever,
+// but for three things.  A coarse word of kind kCellCoarseList names an entry
+// list itself (every polygon of the list holds the whole cell).  An entry's
+// edges are those that may come within the polygon's radius of a point of the
+// cell (kEntBoundary), not a crossing list.  kEntCross: the polygon's boundary
+// may also cross the cell, so that a point far from those edges still asks the
+// polygons' own index `in`.
+struct NearView {
+    const int32_t *rad; // P radii, each in [0, 2^30); null: not a buffered index
+    IndexView in;
+};
+constexpr uint32_t kEntCross = 4u;
+constexpr uint32_t kCellCoarseList = 3u;
+
 constexpr int kCoverLog2 = 8;
 constexpr int kSumLog2 = 8;
 constexpr uint32_t kSumMixed = 0xffffu;
@@ -78,48 +93,6 @@ cudaError_t launch_disk_aggregate(const DiskLaunch &a, cudaStream_t s);
 size_t disk_select_scratch_bytes(uint64_t n, uint32_t Q, uint64_t cap);
 cudaError_t launch_disk_select(const DiskLaunch &a, uint32_t *ids, uint64_t cap, unsigned long long *offsets,
                                void *scratch, cudaStream_t s);
-
-// Buffered polygons (SPADE §4.2 distance canvases: a polygon plus a rounded
-// rectangle of radius r around each edge): the polygon index answers
-// containment, an edge grid the distance part.
-struct BufferView {
-    const uint32_t *cell_off; // 4^g + 1 item offsets per edge-grid cell
-    const uint32_t *item_q;   // polygon of each item, ascending within a cell
-    const int4 *item_seg;     // the item's edge (ax, ay, bx, by)
-    const int32_t *rad;       // P radii, each in [0, 2^30)
-    const uint32_t *mask;     // a bit per cell: it lists edges or meets a non-empty cell of the polygon index
-    int g, sc;                // 2^g cells per side of 2^sc units
-    uint32_t P;
-    uint64_t n_items;
-};
-
-struct BufferLaunch {
-    IndexView ix; // the polygons' own index (containment)
-    BufferView bv;
-    const int2 *pts;
-    uint64_t n;
-    uint2 *pairs; // may be null when cap == 0
-    uint64_t cap;
-    unsigned long long *counts; // P entries or null; zeroed by the launchers
-    unsigned long long *total;  // device total or null
-    unsigned long long *stats;
-    int fp32;
-};
-
-// Buffered-polygon join: pairs (point, polygon) of the points inside the
-// polygon or within its radius of one of its edges, in (point, polygon)
-// order, counts, total; scratch: buffer_scratch_bytes(n).
-size_t buffer_scratch_bytes(uint64_t n);
-cudaError_t launch_buffer_join(const BufferLaunch &a, void *scratch, cudaStream_t s);
-// Counts only.
-cudaError_t launch_buffer_aggregate(const BufferLaunch &a, cudaStream_t s);
-// Per-polygon ascending point-id lists; scratch: buffer_select_scratch_bytes(n, P, cap).
-size_t buffer_select_scratch_bytes(uint64_t n, uint32_t P, uint64_t cap);
-// ORs into mask (a bit per cell of a 2^g grid) every cell that meets a
-// non-empty coarse cell of polygon index ix.
-cudaError_t launch_buffer_mask(const IndexView &ix, uint32_t *mask, int g, cudaStream_t s);
-cudaError_t launch_buffer_select(const BufferLaunch &a, uint32_t *ids, uint64_t cap, unsigned long long *offsets,
-                                 void *scratch, cudaStream_t s);
 
 // Device build of the disk index of Q disks (host array of (cx, cy, r, 0),
 // already checked) on a 2^g grid: the same cell words and entries as the host
@@ -177,7 +150,28 @@ struct JoinLaunch {
     // polygons (four 16-bit ids, ascending) of a point in two to four of
     // them, so that pass 3 writes its pairs without walking its list again
     uint64_t *aux;
+    NearView near; // near.rad set: ix is a buffered-polygon index
 };
+
+// The index of buffered polygons (NearView), built on the device from the host's
+// edge grid (cell_off, item_q, item_seg: CSR by cell of a 2^g grid, on the
+// device), the radii and the polygons' own index.  out.mem holds cells | fine |
+// entries | edges | summary and belongs to the caller.  Runs on the legacy
+// default stream, synchronises.  Returns 0; 1 when the entries exceed 30-bit
+// offsets; 2 on a CUDA error (in cerr).
+struct NearIndexDev {
+    void *mem;
+    size_t bytes;
+    uint32_t *cell, *fine;
+    uint4 *ent;
+    int4 *edge;
+    uint16_t *sum;
+    int sb;
+    uint64_t n_fine, n_ent, n_edge; // n_ent, n_edge with their sentinels
+    double sum_resolved;
+};
+int build_near_index_device(const IndexView &in, const uint32_t *cell_off, const uint32_t *item_q, const int4 *item_seg,
+                            const int32_t *rad, int g, NearIndexDev &out, cudaError_t &cerr);
 
 // Largest polygon count whose join keeps 16-bit per-point results.
 constexpr uint32_t kRes16MaxP = 0xfffeu;
