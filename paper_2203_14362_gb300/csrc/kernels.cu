@@ -1318,10 +1318,10 @@ __global__ void __launch_bounds__(kThreads, kWalkMinBlocks) k_walk(const __grid_
             e0 = __ldcg(a.res + row);
         }
         uint32_t f = 0, c = 0;
-        uint64_t ids = 0; // kOut16 and a.aux: the first four polygons, 16 bits each
+        uint64_t ids = 0; // kOut16 and a.aux: the first polygons, aux_bits each
         walk_list_wave<FP32, NEAR>(ix, lst, e0, p.x, p.y, n_tests, n_esc, keep, s_par, [&](uint32_t q) {
-            if (OUT == kOut16 && c < 4)
-                ids |= (uint64_t)q << (16 * c);
+            if (OUT == kOut16 && (c + 1) * a.aux_bits <= 64)
+                ids |= (uint64_t)q << (a.aux_bits * c);
             f = c ? f : q;
             ++c;
             if (a.counts)
@@ -1336,7 +1336,7 @@ __global__ void __launch_bounds__(kThreads, kWalkMinBlocks) k_walk(const __grid_
                 // only this warp reads or writes the bitmap words of its range
                 if (c < 2)
                     atomicAnd(pend + (row >> 5), ~(1u << (row & 31)));
-                else if (a.aux && c <= 4)
+                else if (a.aux && c * a.aux_bits <= 64)
                     __stcg(reinterpret_cast<unsigned long long *>(a.aux) + row, (unsigned long long)ids);
             } else {
                 __stcg(a.res + row, res_encode(c, f));
@@ -1410,7 +1410,7 @@ __global__ void __launch_bounds__(kThreads, kWalkMinBlocks) k_walk(const __grid_
 // not by bandwidth, and the persistent CTAs of pass 1a would copy the 128 KB
 // summary for a few chunks each.  CTA of kThreads, no barrier between its warps
 // but for the counters (a CTA's points counted in shared memory when P is at
-// most kSmallHist).  Whole join with k_wemit<SELF>, against pass 1a + 1b + scan
+// most kSmallHist).  Whole join with k_wemit16<SELF>, against pass 1a + 1b + scan
 // + pass 3, 2000-cell map: 20k points 18.5 against 28.8 us, 500k 20.6 / 32.8,
 // 1M 32.8 / 39.0, 1.5M 39.0 / 39.1, 2M 53.7 / 43.1; the line is at 1M points.
 constexpr uint32_t kSmallChunks = 4096;
@@ -1443,7 +1443,6 @@ __global__ void __launch_bounds__(kThreads, 3) k_small(const __grid_constant__ J
     if (ch < nchunks) {
         const uint64_t base = (uint64_t)ch * kWChunk;
         npts = (uint32_t)min((uint64_t)kWChunk, a.n - base);
-        uint32_t *res = a.res + base;
         unsigned short *res16 = reinterpret_cast<unsigned short *>(a.res) + base;
         int2 p[kWItems];
         uint32_t w[kWItems];
@@ -1471,12 +1470,8 @@ __global__ void __launch_bounds__(kThreads, 3) k_small(const __grid_constant__ J
             const bool one = kind == kCellInsideOne && in_bounds(pay < ix.P, ix), lst = kind >= kCellList;
             total += one ? 1u : 0u;
             count1(one, pay);
-            if (OUT != kOutCount && loc < npts && !lst) {
-                if (OUT == kOut16)
-                    __stcg(res16 + loc, (unsigned short)(one ? pay : kRes16None));
-                else
-                    __stcg(res + loc, one ? pay : kResNone);
-            }
+            if (OUT == kOut16 && loc < npts && !lst)
+                __stcg(res16 + loc, (unsigned short)(one ? pay : kRes16None));
             const uint32_t bl = __ballot_sync(kFull, lst);
             if (lst)
                 s_q[qn + __popc(bl & lanemask_lt())] = make_uint4((uint32_t)p[j].x, (uint32_t)p[j].y, pay, loc);
@@ -1487,26 +1482,22 @@ __global__ void __launch_bounds__(kThreads, 3) k_small(const __grid_constant__ J
             const bool has = k0 + lane < qn;
             const uint4 it = s_q[has ? k0 + lane : k0]; // idle lanes walk nothing
             uint32_t f = 0, c = 0;
-            uint64_t ids = 0; // kOut16 and a.aux: the first four polygons, 16 bits each
+            uint64_t ids = 0; // kOut16 and a.aux: the first polygons, aux_bits each
             walk_list_wave<FP32, NEAR>(ix, has, it.z, (int)it.x, (int)it.y, n_tests, n_esc, keep, s_pa + warp * kWaveWords,
                                  [&](uint32_t q) {
-                                     if (OUT == kOut16 && c < 4)
-                                         ids |= (uint64_t)q << (16 * c);
+                                     if (OUT == kOut16 && (c + 1) * a.aux_bits <= 64)
+                                         ids |= (uint64_t)q << (a.aux_bits * c);
                                      f = c ? f : q;
                                      ++c;
                                      count1(true, q);
                                  }, &a.near);
             total += c;
-            if (OUT != kOutCount && has) {
-                if (OUT == kOut16) {
-                    __stcg(res16 + it.w, (unsigned short)(c == 0 ? kRes16None : c == 1 ? f : c));
-                    if (c >= 2) {
-                        atomicOr(s_m + (it.w >> 5), 1u << (it.w & 31));
-                        if (a.aux && c <= 4)
-                            __stcg(reinterpret_cast<unsigned long long *>(a.aux) + base + it.w, (unsigned long long)ids);
-                    }
-                } else {
-                    __stcg(res + it.w, res_encode(c, f));
+            if (OUT == kOut16 && has) {
+                __stcg(res16 + it.w, (unsigned short)(c == 0 ? kRes16None : c == 1 ? f : c));
+                if (c >= 2) {
+                    atomicOr(s_m + (it.w >> 5), 1u << (it.w & 31));
+                    if (a.aux && c * a.aux_bits <= 64)
+                        __stcg(reinterpret_cast<unsigned long long *>(a.aux) + base + it.w, (unsigned long long)ids);
                 }
             }
         }
@@ -1539,15 +1530,11 @@ __global__ void __launch_bounds__(kThreads, 3) k_small(const __grid_constant__ J
 constexpr size_t kEmitSmem = size_t(kWarps) * kWChunk * (sizeof(uint32_t) + sizeof(unsigned long long)) +
                              size_t(kWarps) * kWaveWords * sizeof(uint32_t);
 
-//
-// With SELF (small tables, a warp per chunk) chunk_off holds the chunks' totals,
-// not their offsets: every CTA sums the totals before its first chunk itself
-// (at most 8 B x kSmallChunks from L2), which saves the scan's launch.
-template <bool FP32, bool R16, bool SELF, bool NEAR>
+// (k_wemit: 32-bit results, more than kRes16MaxP polygons.)
+template <bool FP32, bool NEAR>
 __global__ void __launch_bounds__(kThreads, 3) k_wemit(const __grid_constant__ JoinLaunch a, const unsigned long long *chunk_off,
-                                                       uint32_t nchunks, const uint32_t *pend)
+                                                       uint32_t nchunks)
 {
-    __shared__ unsigned long long s_before[SELF ? kWarps : 1];
     extern __shared__ __align__(16) unsigned char s_raw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     unsigned long long *s_o = reinterpret_cast<unsigned long long *>(s_raw) + warp * kWChunk;
@@ -1558,55 +1545,22 @@ __global__ void __launch_bounds__(kThreads, 3) k_wemit(const __grid_constant__ J
                       warp * kWaveWords; // words of walk_list_wave
     const uint64_t keep = policy_evict_last();
     const uint32_t nw = gridDim.x * kWarps;
-    unsigned long long before = 0; // SELF: the pairs before this warp's chunk
-    if (SELF) {
-        const uint32_t c0 = blockIdx.x * kWarps;
-        for (uint32_t i = threadIdx.x; i < c0; i += kThreads)
-            before += chunk_off[i];
-        before = warp_sum64(before);
-        if (lane == 0)
-            s_before[warp] = before;
-        __syncthreads();
-        before = 0;
-        for (int w = 0; w < kWarps; ++w)
-            before += s_before[w];
-        for (int w = 0; w < warp && c0 + w < nchunks; ++w)
-            before += chunk_off[c0 + w];
-        if (c0 + warp == nchunks - 1 && lane == 0 && a.total)
-            *a.total = before + chunk_off[nchunks - 1];
-    }
     for (uint32_t ch = blockIdx.x * kWarps + warp; ch < nchunks; ch += nw) {
         const uint64_t base = (uint64_t)ch * kWChunk;
         const uint32_t npts = (uint32_t)min((uint64_t)kWChunk, a.n - base);
-        unsigned long long run = SELF ? before : chunk_off[ch] + (a.pair_base ? *a.pair_base : 0ull);
-        uint32_t res[kWItems], mw = 0;
+        unsigned long long run = chunk_off[ch] + (a.pair_base ? *a.pair_base : 0ull);
+        uint32_t res[kWItems];
 #pragma unroll
         for (int j = 0; j < kWItems; ++j) {
             const uint32_t loc = j * 32 + lane;
-            if (R16) {
-                const uint16_t r = loc < npts ? __ldcs(reinterpret_cast<const unsigned short *>(a.res) + base + loc)
-                                              : kRes16None;
-                res[j] = r == kRes16None ? kResNone : r;
-            } else {
-                res[j] = loc < npts ? __ldcs(a.res + base + loc) : kResNone;
-            }
+            res[j] = loc < npts ? __ldcs(a.res + base + loc) : kResNone;
         }
-        if (R16 && lane < kWItems) // lane j: the bitmap word of round j (rows in several polygons)
-            mw = __ldcs(pend + (uint64_t)ch * kWItems + lane);
         uint32_t qn = 0;
 #pragma unroll
         for (int j = 0; j < kWItems; ++j) {
             const uint32_t loc = j * 32 + lane;
-            uint32_t r = res[j];
-            const uint32_t pid = a.pid0 + (uint32_t)(base + loc);
-            bool multi;
-            if (R16) {
-                multi = (__shfl_sync(kFull, mw, j) >> lane) & 1u;
-                if (multi) // the count; the polygons come from walking the list again
-                    r = kResMulti | kResCount;
-            } else {
-                multi = r != kResNone && (r & kResMulti);
-            }
+            const uint32_t r = res[j], pid = a.pid0 + (uint32_t)(base + loc);
+            const bool multi = r != kResNone && (r & kResMulti);
             uint32_t c = r == kResNone ? 0u : 1u, pre, tot;
             if (!__any_sync(kFull, multi)) {
                 const uint32_t bl = __ballot_sync(kFull, c != 0);
@@ -1614,9 +1568,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_wemit(const __grid_constant__ J
                 tot = __popc(bl);
             } else {
                 if (multi) {
-                    if (R16) {
-                        c = res[j];
-                    } else if (r & kResCount) {
+                    if (r & kResCount) {
                         c = (r >> 20) & 0x3ffu;
                     } else { // count not stored: count again
                         const int2 p = a.pts[base + loc];
@@ -1634,22 +1586,12 @@ __global__ void __launch_bounds__(kThreads, 3) k_wemit(const __grid_constant__ J
                 }
                 pre = inc - c;
                 tot = __shfl_sync(kFull, inc, 31);
-                // a point whose polygons pass 1b packed: written from them
-                const bool packed = R16 && multi && a.aux && c <= 4;
-                if (packed) {
-                    const unsigned long long ids = __ldcs(reinterpret_cast<const unsigned long long *>(a.aux) + base + loc);
-                    for (uint32_t t = 0; t < c; ++t)
-                        if (run + pre + t < a.cap)
-                            __stcs(a.pairs + run + pre + t, make_uint2(pid, uint32_t(ids >> (16 * t)) & 0xffffu));
-                }
-                const uint32_t bl = __ballot_sync(kFull, multi && !packed);
+                const uint32_t bl = __ballot_sync(kFull, multi);
                 if (multi) {
-                    if (!packed) {
-                        const uint32_t slot = qn + __popc(bl & lanemask_lt());
-                        s_q[slot] = loc;
-                        s_o[slot] = run + pre;
-                    }
-                    c = 0; // written above or from the queue
+                    const uint32_t slot = qn + __popc(bl & lanemask_lt());
+                    s_q[slot] = loc;
+                    s_o[slot] = run + pre;
+                    c = 0; // written from the queue
                 }
                 qn += __popc(bl);
             }
@@ -1678,6 +1620,176 @@ __global__ void __launch_bounds__(kThreads, 3) k_wemit(const __grid_constant__ J
                                  }, &a.near);
         }
         __syncwarp(); // the queue is rewritten by the next chunk
+    }
+}
+
+// Pass 3 with 16-bit results, lane-major: lane l owns rows 8l .. 8l + 7 of the
+// warp's chunk (one 16-byte load of results and one byte of the row bitmap,
+// loaded a chunk ahead), so one warp scan of the lanes' pair counts gives every
+// row its place, where the row-major form above scans once per round of 32 rows
+// that holds a point in several polygons.  The chunk's pairs are put together in
+// shared memory and written out as whole lines (lanes' own stretches are 64
+// bytes apart).  Points in several polygons are queued and taken 32 at a time, so
+// that a chunk waits once for their packed words (a wait per row of a lane was
+// most of this kernel: 8 dependent round trips a chunk); those that pass 1b could
+// not pack have their lists walked by the warp.  A chunk of more than kEmitStage pairs is written
+// straight to its place.  500M points x 256 queries (17 % of the points in one or
+// more): 2.77 -> 1.19 ms; 100M x 2000 cells (a pair per point): 204 -> 175 us for
+// 1.0 GB, where a plain fill of its 0.8 GB takes 105; 20M x 256 buffered queries:
+// 232 -> 72 us.
+//
+// With SELF (small tables, a warp per chunk) chunk_off holds the chunks' totals,
+// not their offsets: every CTA sums the totals before its first chunk itself
+// (at most 8 B x kSmallChunks from L2), which saves the scan's launch.
+constexpr uint32_t kEmitStage = 512;
+__host__ __device__ constexpr uint32_t stage_at(uint32_t i) { return i + (i >> 3); } // eight pairs per lane: no bank conflict
+constexpr size_t kEmit16Warp = (stage_at(kEmitStage) * 8 + size_t(kWChunk) * 8 + kWaveWords * 4 + 15) & ~size_t(15);
+constexpr size_t kEmit16Smem = kWarps * kEmit16Warp;
+static_assert(kWItems == 8, "a lane's rows: one 16-byte load of 2-byte results");
+
+template <bool FP32, bool SELF, bool NEAR>
+__global__ void __launch_bounds__(kThreads, NEAR ? 3 : 4) k_wemit16(const __grid_constant__ JoinLaunch a,
+                                                         const unsigned long long *chunk_off, uint32_t nchunks,
+                                                         const uint32_t *pend)
+{
+    __shared__ unsigned long long s_before[SELF ? kWarps : 1];
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint2 *s_st = reinterpret_cast<uint2 *>(s_raw + warp * kEmit16Warp);
+    uint2 *s_q = s_st + stage_at(kEmitStage); // (row | count << 8, place in the chunk's pairs)
+    uint32_t *s_par = reinterpret_cast<uint32_t *>(s_q + kWChunk);
+    const uint64_t keep = policy_evict_last();
+    const uint32_t nw = gridDim.x * kWarps, r0 = 8u * (uint32_t)lane;
+    const unsigned short *res = reinterpret_cast<const unsigned short *>(a.res);
+    const uint8_t *bits = reinterpret_cast<const uint8_t *>(pend);
+    unsigned long long before = 0; // SELF: the pairs before this warp's chunk
+    if (SELF) {
+        const uint32_t c0 = blockIdx.x * kWarps;
+        for (uint32_t i = threadIdx.x; i < c0; i += kThreads)
+            before += chunk_off[i];
+        before = warp_sum64(before);
+        if (lane == 0)
+            s_before[warp] = before;
+        __syncthreads();
+        before = 0;
+        for (int w = 0; w < kWarps; ++w)
+            before += s_before[w];
+        for (int w = 0; w < warp && c0 + w < nchunks; ++w)
+            before += chunk_off[c0 + w];
+        if (c0 + warp == nchunks - 1 && lane == 0 && a.total)
+            *a.total = before + chunk_off[nchunks - 1];
+    }
+    uint32_t nr[4], nm = 0; // the next chunk's results (two per word) and bitmap byte
+    unsigned long long noff = 0;
+    auto fetch = [&](uint32_t ch) {
+        const uint64_t base = (uint64_t)ch * kWChunk;
+        const uint32_t npts = ch < nchunks ? (uint32_t)min((uint64_t)kWChunk, a.n - base) : 0u;
+        if (r0 + 8 <= npts) {
+            const uint4 u = __ldcs(reinterpret_cast<const uint4 *>(res + base + r0));
+            nr[0] = u.x, nr[1] = u.y, nr[2] = u.z, nr[3] = u.w;
+        } else { // the table's ragged end
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const uint32_t lo = r0 + 2 * k < npts ? __ldcs(res + base + r0 + 2 * k) : kRes16None;
+                const uint32_t hi = r0 + 2 * k + 1 < npts ? __ldcs(res + base + r0 + 2 * k + 1) : kRes16None;
+                nr[k] = lo | hi << 16;
+            }
+        }
+        nm = ch < nchunks ? __ldcs(bits + (uint64_t)ch * 32 + lane) : 0u;
+        if (!SELF)
+            noff = ch < nchunks ? chunk_off[ch] : 0ull;
+    };
+    const unsigned long long pb = a.pair_base ? *a.pair_base : 0ull;
+    fetch(blockIdx.x * kWarps + warp);
+    for (uint32_t ch = blockIdx.x * kWarps + warp; ch < nchunks; ch += nw) {
+        const uint64_t base = (uint64_t)ch * kWChunk;
+        const uint32_t m = nm, pid0 = a.pid0 + (uint32_t)base + r0;
+        const unsigned long long run = SELF ? before : noff + pb;
+        uint32_t r[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            r[k] = k & 1 ? nr[k >> 1] >> 16 : nr[k >> 1] & 0xffffu;
+        if (!SELF)
+            fetch(ch + nw);
+        // pairs of this lane's rows, and (upper half) its rows in several polygons
+        unsigned long long mine = 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const bool multi = (m >> k) & 1u;
+            mine += multi ? r[k] : r[k] != kRes16None ? 1u : 0u;
+            mine += (unsigned long long)multi << 32;
+        }
+        uint32_t at, tot, slot = 0, qn = 0;
+        if (!__any_sync(kFull, m != 0)) {
+            uint32_t inc = (uint32_t)mine;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t v = __shfl_up_sync(kFull, inc, o);
+                if (lane >= o)
+                    inc += v;
+            }
+            tot = __shfl_sync(kFull, inc, 31);
+            at = inc - (uint32_t)mine;
+        } else {
+            unsigned long long inc = mine;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned long long v = __shfl_up_sync(kFull, inc, o);
+                if (lane >= o)
+                    inc += v;
+            }
+            const unsigned long long t = __shfl_sync(kFull, inc, 31);
+            tot = (uint32_t)t;
+            qn = uint32_t(t >> 32);
+            at = uint32_t(inc - mine);
+            slot = uint32_t((inc - mine) >> 32);
+        }
+        if (tot == 0)
+            continue;
+        const bool staged = tot <= kEmitStage;
+        auto put = [&](uint32_t place, uint32_t pid, uint32_t q) {
+            if (staged)
+                s_st[stage_at(place)] = make_uint2(pid, q);
+            else if (run + place < a.cap)
+                __stcs(a.pairs + run + place, make_uint2(pid, q));
+        };
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            if ((m >> k) & 1u) {
+                s_q[slot++] = make_uint2((r0 + k) | r[k] << 8, at);
+                at += r[k];
+            } else if (r[k] != kRes16None) {
+                put(at++, pid0 + k, r[k]);
+            }
+        }
+        __syncwarp();
+        for (uint32_t k0 = 0; k0 < qn; k0 += 32) {
+            const bool has = k0 + lane < qn;
+            const uint2 it = s_q[has ? k0 + lane : 0];
+            const uint32_t row = it.x & 0xffu, c = it.x >> 8, pid = a.pid0 + (uint32_t)base + row;
+            const bool packed = a.aux && c * a.aux_bits <= 64;
+            uint32_t place = it.y;
+            if (has && packed) {
+                unsigned long long ids = __ldcs(reinterpret_cast<const unsigned long long *>(a.aux) + base + row);
+                for (uint32_t t = 0; t < c; ++t, ids >>= a.aux_bits)
+                    put(place++, pid, uint32_t(ids) & ((1u << a.aux_bits) - 1u));
+            }
+            const bool walk = has && !packed; // the whole warp walks these points' lists together
+            if (!__any_sync(kFull, walk))
+                continue;
+            const int2 p = walk ? a.pts[base + row] : make_int2(0, 0);
+            const uint32_t w = walk ? resolve(a.ix, (uint32_t)p.x, (uint32_t)p.y, keep) : 0u;
+            uint32_t t = 0, e = 0;
+            walk_list_wave<FP32, NEAR>(a.ix, (w >> 30) >= kCellList, w & kPayloadMask, p.x, p.y, t, e, keep, s_par,
+                                       [&](uint32_t q) { put(place++, pid, q); }, &a.near);
+        }
+        if (staged) {
+            __syncwarp();
+            const uint32_t n_out = run >= a.cap ? 0u : (uint32_t)min((unsigned long long)tot, a.cap - run);
+            for (uint32_t i = lane; i < n_out; i += 32)
+                __stcs(a.pairs + run + i, s_st[stage_at(i)]);
+        }
+        __syncwarp(); // the queue and the stage are rewritten by the next chunk
     }
 }
 
@@ -3088,38 +3200,41 @@ cudaError_t launch_join_emit(const JoinLaunch &a, cudaStream_t s, const uint32_t
         return cudaErrorInvalidValue;
     const uint32_t nblk = (nchunks + kWarps - 1) / kWarps;
     static bool done[8][64] = {};
-    return with_switches(a, [&](auto fp32, auto near) {
+    return with_switches(a, [&](auto fp32, auto near) -> cudaError_t {
         constexpr bool F = decltype(fp32)::value, N = decltype(near)::value;
-        auto emit = [&](auto kr, bool(&d)[64]) -> cudaError_t {
-            cudaError_t e = smem_opt_in(kr, kEmitSmem, d);
-            if (e != cudaSuccess)
-                return e;
-            kr<<<persistent_grid(kr, kThreads, kEmitSmem, nblk), kThreads, kEmitSmem, s>>>(a, a.tile_tot, nchunks, pend);
-            return cudaGetLastError();
-        };
-        return a.narrow ? emit(k_wemit<F, true, false, N>, done[F + 2 * N])
-                        : emit(k_wemit<F, false, false, N>, done[4 + F + 2 * N]);
+        auto kn = k_wemit16<F, false, N>;
+        auto kw = k_wemit<F, N>;
+        const cudaError_t e = a.narrow ? smem_opt_in(kn, kEmit16Smem, done[F + 2 * N])
+                                       : smem_opt_in(kw, kEmitSmem, done[4 + F + 2 * N]);
+        if (e != cudaSuccess)
+            return e;
+        if (a.narrow)
+            kn<<<persistent_grid(kn, kThreads, kEmit16Smem, nblk), kThreads, kEmit16Smem, s>>>(a, a.tile_tot, nchunks, pend);
+        else
+            kw<<<persistent_grid(kw, kThreads, kEmitSmem, nblk), kThreads, kEmitSmem, s>>>(a, a.tile_tot, nchunks);
+        return cudaGetLastError();
     });
 }
 
-// The join of a small table (at most kSmallChunks chunks, with an output): two
-// launches, k_small and k_wemit<SELF>.  ev as for launch_join.
-template <bool FP32, bool R16, bool NEAR>
+// The join of a small table (at most kSmallChunks chunks, 16-bit results, with an
+// output): two
+// launches, k_small and k_wemit16<SELF>.  ev as for launch_join.
+template <bool FP32, bool NEAR>
 static cudaError_t launch_small(const JoinLaunch &a, uint32_t *pend, cudaStream_t s, cudaEvent_t *ev)
 {
     static bool done[64] = {};
     const uint32_t nchunks = uint32_t((a.n + kWChunk - 1) / kWChunk), nblk = (nchunks + kWarps - 1) / kWarps;
     if (ev)
         cudaEventRecord(ev[0], s);
-    k_small<FP32, R16 ? kOut16 : kOut32, NEAR><<<nblk, kThreads, 0, s>>>(a, pend, nchunks, a.ix.P <= kSmallHist ? 1 : 0);
+    k_small<FP32, kOut16, NEAR><<<nblk, kThreads, 0, s>>>(a, pend, nchunks, a.ix.P <= kSmallHist ? 1 : 0);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess)
-        e = smem_opt_in(k_wemit<FP32, R16, true, NEAR>, kEmitSmem, done);
+        e = smem_opt_in(k_wemit16<FP32, true, NEAR>, kEmit16Smem, done);
     if (e != cudaSuccess)
         return e;
     for (int k = 1; ev && k < 4; ++k)
         cudaEventRecord(ev[k], s);
-    k_wemit<FP32, R16, true, NEAR><<<nblk, kThreads, kEmitSmem, s>>>(a, a.tile_tot, nchunks, pend);
+    k_wemit16<FP32, true, NEAR><<<nblk, kThreads, kEmit16Smem, s>>>(a, a.tile_tot, nchunks, pend);
     return cudaGetLastError();
 }
 
@@ -3168,6 +3283,9 @@ static unsigned long long *join_layout(JoinLaunch &b, void *scratch)
     // 16-bit results when every polygon id and every point's polygon count
     // fit (the row bitmap in part stays in place until pass 3)
     b.narrow = b.ix.P <= kRes16MaxP ? 1 : 0;
+    b.aux_bits = 8;
+    while ((1u << b.aux_bits) < b.ix.P && b.aux_bits < 16)
+        ++b.aux_bits;
     return b.tile_tot + (b.n + kWChunk - 1) / kWChunk;
 }
 
@@ -3203,7 +3321,7 @@ cudaError_t launch_join_write(const JoinLaunch &a, void *scratch, cudaStream_t s
 cudaError_t launch_join(const JoinLaunch &a, void *scratch, cudaStream_t s, cudaEvent_t *ev)
 {
     cudaError_t e;
-    if (a.n && (a.n + kWChunk - 1) / kWChunk <= kSmallChunks && a.cap && !a.pair_base) {
+    if (a.n && (a.n + kWChunk - 1) / kWChunk <= kSmallChunks && a.cap && !a.pair_base && a.ix.P <= kRes16MaxP) {
         if (reinterpret_cast<uintptr_t>(a.pts) & 15)
             return cudaErrorMisalignedAddress;
         JoinLaunch b = a;
@@ -3213,7 +3331,7 @@ cudaError_t launch_join(const JoinLaunch &a, void *scratch, cudaStream_t s, cuda
                 return e;
         e = with_switches(b, [&](auto fp32, auto near) {
             constexpr bool F = decltype(fp32)::value, N = decltype(near)::value;
-            return b.narrow ? launch_small<F, true, N>(b, pend, s, ev) : launch_small<F, false, N>(b, pend, s, ev);
+            return launch_small<F, N>(b, pend, s, ev);
         });
         if (ev)
             cudaEventRecord(ev[4], s);

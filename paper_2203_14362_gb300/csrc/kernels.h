@@ -147,9 +147,11 @@ struct JoinLaunch {
     // words (the index has at most kRes16MaxP polygons)
     int narrow;
     // with narrow results, or null: a word per point where pass 1b packs the
-    // polygons (four 16-bit ids, ascending) of a point in two to four of
-    // them, so that pass 3 writes its pairs without walking its list again
+    // polygons (ascending, aux_bits each, set by the launchers: 8 bits for up to
+    // 256 polygons, 10 for 1024) of a point in as many of them as the word
+    // holds, so that pass 3 writes its pairs without walking its list again
     uint64_t *aux;
+    int aux_bits;
     NearView near; // near.rad set: ix is a buffered-polygon index
 };
 
