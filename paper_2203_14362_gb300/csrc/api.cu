@@ -61,7 +61,9 @@ struct IndexObj {
     void *mem3 = nullptr; // buffered polygons: their own grid (cells | fine | entries | edges | summary)
     IndexView view{};
     int fp32 = 1;
+    bool pooled = false; // mem is from the ctx's pool (else cudaMalloc)
     void *mem = nullptr; // one allocation: cells | fine | entries | edges | cover | summary
+    LocalLists local{};  // kinds 0 and 2: the local lists of view, and what they replaced
     uint64_t n_fine = 0, n_ent = 0, n_edge = 0; // words / entries / edges of a polygon index, sentinels included
     spx_index_info info{};
 };
@@ -75,7 +77,9 @@ struct Aux {
 };
 
 constexpr size_t kPinnedBytes = 128;
-constexpr uint64_t kPoolKeep = uint64_t(64) << 20; // the row bitmap of 512M points
+// of the pool's memory, what stays with the ctx between calls: the temporaries of
+// a query-time index of some thousand cells, the row bitmap of 8G points
+constexpr uint64_t kPoolKeep = uint64_t(1) << 30;
 
 } // namespace
 
@@ -87,7 +91,7 @@ struct spx_ctx {
     std::map<uint64_t, std::unique_ptr<PolysObj>> polys;
     std::map<uint64_t, std::unique_ptr<IndexObj>> indexes;
     Aux *aux = nullptr;
-    cudaMemPool_t pool = nullptr; // stream-ordered scratch of the row-order count, at most kPoolKeep kept between calls
+    cudaMemPool_t pool = nullptr; // stream-ordered memory: scratch of the counts, index builds on the device
     char *pinned = nullptr; // kPinnedBytes of host memory: a call's status and total come back here
     void *scratch = nullptr;
     size_t scratch_bytes = 0;
@@ -152,6 +156,30 @@ bool capturing(cudaStream_t s)
     return st != cudaStreamCaptureStatusNone;
 }
 
+// cudaMalloc; when there is no memory, what the ctx's pool keeps is given back
+// and the allocation tried once more.
+cudaError_t dev_alloc(spx_ctx *ctx, void **p, size_t bytes)
+{
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        cudaStreamSynchronize(ctx->stream);
+        cudaMemPoolTrimTo(ctx->pool, 0);
+        e = cudaMalloc(p, bytes);
+    }
+    return e;
+}
+
+void free_index_memory(spx_ctx *ctx, IndexObj &ix)
+{
+    ix.pooled ? cudaFreeAsync(ix.mem, ctx->stream) : cudaFree(ix.mem);
+    if (ix.local.mem)
+        cudaFreeAsync(ix.local.mem, ctx->stream);
+    cudaFree(ix.mem2);
+    cudaFree(ix.mem3);
+    ix.mem = ix.mem2 = ix.mem3 = ix.local.mem = nullptr;
+}
+
 // Grow a device buffer (never while the stream is being captured).
 spx_status ensure(spx_ctx *ctx, void **buf, size_t *have, size_t need, cudaStream_t s, const char *what)
 {
@@ -173,7 +201,7 @@ spx_status ensure(spx_ctx *ctx, void **buf, size_t *have, size_t need, cudaStrea
             cudaGraphExecDestroy(kv.second);
         ctx->select_graphs.clear();
     }
-    cudaError_t e = cudaMalloc(buf, sz);
+    cudaError_t e = dev_alloc(ctx, buf, sz);
     if (e != cudaSuccess)
         return fail(ctx, SPX_ENOMEM, std::string(what) + ": cudaMalloc failed: " + cudaGetErrorString(e));
     *have = sz;
@@ -479,6 +507,18 @@ spx_status register_grid_index(spx_ctx *ctx, spx_polys polys, std::unique_ptr<In
     inf.build_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
     inf.sum_resolved = gp.sum_resolved;
     inf.use_sum = ix->view.use_sum;
+    const cudaError_t e = build_local_lists(ix->view, reinterpret_cast<uint4 *>(gp.ent), ix->local, ctx->stream, ctx->pool);
+    if (e != cudaSuccess) {
+        free_index_memory(ctx, *ix);
+        return cuda_fail(ctx, e, "build_index: local edge lists");
+    }
+    if (ix->local.mem) {
+        ix->view.loc = ix->local.loc;
+        ix->view.loc_bit = kLocalEdge;
+        ix->view.n_loc = ix->local.n_loc;
+        inf.device_bytes += ix->local.bytes;
+        inf.build_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
+    }
     pg->n_index++;
     const uint64_t h = make_handle(ctx, kTagIndex);
     ctx->indexes[h] = std::move(ix);
@@ -521,7 +561,7 @@ spx_status build_index_impl(spx_ctx *ctx, spx_polys polys, const spx_index_param
         return SPX_OK;
     }
     auto ix = std::make_unique<IndexObj>();
-    if (cudaMalloc(&ix->mem, total) != cudaSuccess)
+    if (dev_alloc(ctx, &ix->mem, total) != cudaSuccess)
         return fail(ctx, SPX_ENOMEM, "build_index: cudaMalloc of " + std::to_string(total) + " bytes failed");
     char *m = static_cast<char *>(ix->mem);
     char *p_cell = m, *p_fine = p_cell + up(b_cell), *p_ent = p_fine + up(b_fine), *p_edge = p_ent + up(b_ent),
@@ -700,11 +740,9 @@ void spx_destroy(spx_ctx *ctx)
         return;
     cudaSetDevice(ctx->device);
     cudaDeviceSynchronize();
-    for (auto &kv : ctx->indexes) {
-        cudaFree(kv.second->mem);
-        cudaFree(kv.second->mem2);
-        cudaFree(kv.second->mem3);
-    }
+    for (auto &kv : ctx->indexes)
+        free_index_memory(ctx, *kv.second);
+    cudaStreamSynchronize(ctx->stream);
     for (auto &kv : ctx->points) {
         if (kv.second->owned)
             cudaFree(kv.second->dev);
@@ -762,7 +800,7 @@ spx_status spx_load_points(spx_ctx *ctx, const int32_t *xy, uint64_t n, int xy_i
                 return fail(ctx, SPX_EINVAL, "load_points: coordinate " + std::to_string(xy[i]) + " at point " +
                                                  std::to_string(i / 2) + " outside [0, 2^30)");
         void *d = nullptr;
-        if (cudaMalloc(&d, n ? n * 8 : 16) != cudaSuccess)
+        if (dev_alloc(ctx, &d, n ? n * 8 : 16) != cudaSuccess)
             return fail(ctx, SPX_ENOMEM, "load_points: cudaMalloc failed");
         const cudaError_t e = n ? cudaMemcpy(d, xy, n * 8, cudaMemcpyHostToDevice) : cudaSuccess;
         if (e != cudaSuccess) {
@@ -795,14 +833,14 @@ spx_status spx_cluster_points(spx_ctx *ctx, spx_points points, int grid_log2, sp
     p->owned = true;
     p->cluster_log2 = c;
     void *d = nullptr, *scratch = nullptr;
-    if (cudaMalloc(&d, src->n ? src->n * 8 : 16) != cudaSuccess)
+    if (dev_alloc(ctx, &d, src->n ? src->n * 8 : 16) != cudaSuccess)
         return fail(ctx, SPX_ENOMEM, "cluster_points: cudaMalloc of the copy failed");
-    if (cudaMalloc(&scratch, cluster_scratch_bytes(c)) != cudaSuccess) {
+    if (dev_alloc(ctx, &scratch, cluster_scratch_bytes(c)) != cudaSuccess) {
         cudaFree(d);
         return fail(ctx, SPX_ENOMEM, "cluster_points: cudaMalloc of the cell counters failed");
     }
     const size_t bins = (size_t(1) << (2 * c)) + 1;
-    if (cudaMalloc(reinterpret_cast<void **>(&p->cell_end), bins * 8) != cudaSuccess) {
+    if (dev_alloc(ctx, reinterpret_cast<void **>(&p->cell_end), bins * 8) != cudaSuccess) {
         cudaFree(d);
         cudaFree(scratch);
         return fail(ctx, SPX_ENOMEM, "cluster_points: cudaMalloc of the cell directory failed");
@@ -904,7 +942,11 @@ spx_status spx_build_index_device(spx_ctx *ctx, spx_polys polys, const spx_index
     GridIndexDev d{};
     const char *why = nullptr;
     cudaError_t e = cudaSuccess;
-    const int st = build_grid_index_device(pg->xy.data(), pg->off.data(), pg->P, g, sb, d, why, e);
+    // temporaries and the index itself from the ctx's pool, in the order of its
+    // stream: an index built, used and freed per query reuses its memory (20
+    // allocations and frees were half of a query-time build of 1000 cells)
+    const int st = build_grid_index_device(pg->xy.data(), pg->off.data(), pg->P, g, sb, d, why, e, ctx->stream, ctx->pool);
+    cudaDeviceSynchronize(); // as documented
     if (st == 1)
         return fail(ctx, SPX_EINVAL, std::string("build_index_device: ") + why);
     if (st != 0)
@@ -912,6 +954,7 @@ spx_status spx_build_index_device(spx_ctx *ctx, spx_polys polys, const spx_index
                                               : cuda_fail(ctx, e, "build_index_device");
     auto ix = std::make_unique<IndexObj>();
     ix->mem = d.mem;
+    ix->pooled = true;
     return register_grid_index(ctx, polys, std::move(ix), d.bytes, g, sb, prm.fp32_filter, device_parts(d), t0, out);
 }
 
@@ -935,6 +978,14 @@ spx_status spx_index_arrays(spx_ctx *ctx, spx_index index, uint32_t *coarse, uin
         SPX_CUDA(cudaMemcpy(fine, ix->view.fine, sizes[1] * 4, cudaMemcpyDeviceToHost), "index_arrays fine");
     if (entries)
         SPX_CUDA(cudaMemcpy(entries, ix->view.ent, sizes[2] * 16, cudaMemcpyDeviceToHost), "index_arrays entries");
+    if (entries && ix->local.n_undo) { // as built: entries with a local list get their row list back
+        std::vector<uint32_t> undo(ix->local.n_undo * 4);
+        SPX_CUDA(cudaMemcpy(undo.data(), ix->local.undo, undo.size() * 4, cudaMemcpyDeviceToHost), "index_arrays entries");
+        for (size_t k = 0; k < undo.size(); k += 4) {
+            entries[4 * size_t(undo[k]) + 1] = undo[k + 1];
+            entries[4 * size_t(undo[k]) + 2] = undo[k + 2];
+        }
+    }
     if (edges)
         SPX_CUDA(cudaMemcpy(edges, ix->view.edge, sizes[3] * 16, cudaMemcpyDeviceToHost), "index_arrays edges");
     return SPX_OK;
@@ -999,7 +1050,7 @@ spx_status spx_autotune(spx_ctx *ctx, spx_points points, spx_polys polys, const 
     sized.n = m;
     sized.clustered = pts->cluster_log2 ? 1 : 0; // the strided sample keeps the table's order
     void *mem = nullptr;
-    if (cudaMalloc(&mem, b_sample + 2 * b_counts + aggregate_scratch_bytes(sized) + 256) != cudaSuccess)
+    if (dev_alloc(ctx, &mem, b_sample + 2 * b_counts + aggregate_scratch_bytes(sized) + 256) != cudaSuccess)
         return fail(ctx, SPX_ENOMEM, "autotune: cudaMalloc of the sample failed");
     std::unique_ptr<void, decltype(&cudaFree)> mem_guard(mem, &cudaFree);
     int2 *sample = static_cast<int2 *>(mem);
@@ -1219,7 +1270,7 @@ spx_status spx_build_disk_index(spx_ctx *ctx, const int32_t *cxy, const int32_t 
                  b_cover = cover.size() * 4;
     const size_t total = up(b_cell) + up(b_ent) + up(b_disk) + up(b_cover);
     void *mem = nullptr;
-    if (cudaMalloc(&mem, total) != cudaSuccess)
+    if (dev_alloc(ctx, &mem, total) != cudaSuccess)
         return fail(ctx, SPX_ENOMEM, "build_disk_index: cudaMalloc failed");
     char *m = static_cast<char *>(mem), *p_ent = m + up(b_cell), *p_disk = p_ent + up(b_ent),
          *p_cover = p_disk + up(b_disk);
@@ -1336,10 +1387,10 @@ spx_status spx_build_buffer_index(spx_ctx *ctx, spx_polys polys, const int32_t *
         cudaFree(tmp);
         cudaFree(mem2);
         cudaFree(fx.mem);
-        cudaFree(ix->mem);
+        free_index_memory(ctx, *ix);
         pg->n_index--;
     };
-    if (cudaMalloc(&mem2, total) != cudaSuccess || cudaMalloc(&tmp, up(b_off) + up(b_q) + up(b_seg)) != cudaSuccess) {
+    if (dev_alloc(ctx, &mem2, total) != cudaSuccess || dev_alloc(ctx, &tmp, up(b_off) + up(b_q) + up(b_seg)) != cudaSuccess) {
         drop();
         return fail(ctx, SPX_ENOMEM, "build_buffer_index: cudaMalloc failed");
     }
@@ -1559,22 +1610,16 @@ spx_status spx_aggregate(spx_ctx *ctx, spx_points points, spx_index index, uint6
     a.cell_end = pts->cell_end;
     a.cluster_log2 = pts->cluster_log2;
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    // a table in row order takes its scratch from the ctx's pool, in stream
-    // order: counts on several streams, or beside a join, share nothing.  When
-    // there is none to have, the one-pass kernel needs none.
+    // the scratch comes from the ctx's pool, in stream order: counts on several
+    // streams, or beside a join, share nothing.  When there is none to have, the
+    // one-pass kernels need none.
     void *words = nullptr;
-    if (use_split_count(a)) {
-        if (cudaMallocFromPoolAsync(&words, aggregate_scratch_bytes(a), ctx->pool, s) != cudaSuccess) {
-            cudaGetLastError();
-            words = nullptr;
-        }
-    } else if (a.clustered && !buffered) {
-        spx_status st = ensure(ctx, &ctx->scratch, &ctx->scratch_bytes, aggregate_scratch_bytes(a), s, "aggregate");
-        if (st != SPX_OK)
-            return st;
+    const size_t need = use_split_count(a) || use_directory(a) ? aggregate_scratch_bytes(a) : 0;
+    if (need && cudaMallocFromPoolAsync(&words, need, ctx->pool, s) != cudaSuccess) {
+        cudaGetLastError();
+        words = nullptr;
     }
-    cudaError_t e = launch_aggregate(a, a.clustered && !buffered ? ctx->scratch : words, s,
-                                     ctx->timing && !buffered ? ctx->ev : nullptr);
+    cudaError_t e = launch_aggregate(a, words, s, ctx->timing && !buffered ? ctx->ev : nullptr);
     if (words) {
         const cudaError_t e2 = cudaFreeAsync(words, s);
         e = e != cudaSuccess ? e : e2;
@@ -2149,9 +2194,7 @@ spx_status spx_free(spx_ctx *ctx, uint64_t handle)
             } else {
                 ++it;
             }
-        cudaFree(ix->mem);
-        cudaFree(ix->mem2);
-        cudaFree(ix->mem3);
+        free_index_memory(ctx, *ix);
         PolysObj *pg = lookup(ctx->polys, ix->polys);
         if (pg)
             pg->n_index--;

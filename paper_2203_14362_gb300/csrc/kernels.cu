@@ -234,6 +234,17 @@ __device__ __forceinline__ bool in_bounds(bool ok, const IndexView &ix)
 #endif
 }
 
+// An entry's edges: in the row lists, or (kLocalEdge) in the local ones.
+__device__ __forceinline__ const int4 *edge_at(const IndexView &ix, uint32_t y)
+{
+    return (y & ix.loc_bit) ? ix.loc + (y & ~kLocalEdge) : ix.edge + y;
+}
+__device__ __forceinline__ bool edges_ok(const IndexView &ix, const uint4 &en)
+{
+    return !(en.w & kEntBoundary) ||
+           ((en.y & ix.loc_bit) ? (uint64_t)(en.y & ~kLocalEdge) + en.z <= ix.n_loc : (uint64_t)en.y + en.z < ix.n_edge);
+}
+
 __device__ __forceinline__ uint32_t coarse_word(const IndexView &ix, uint32_t px, uint32_t py, uint64_t pol)
 {
     return ld_idx(ix.cell + (((py >> ix.sc) << ix.gc) | (px >> ix.sc)), pol);
@@ -284,7 +295,7 @@ __device__ __forceinline__ uint32_t entry_in(const IndexView &ix, const uint4 &e
     for (int j = 0; j < 4; ++j)
         par ^= edge_cross<FP32>(v[j], px, py, tests, esc);
     if (en.z > 4 && max(v[3].x, v[3].z) > px)
-        par ^= row_parity<FP32>(ix.edge + en.y + 4, en.z - 4, px, py, tests, esc, pol);
+        par ^= row_parity<FP32>(edge_at(ix, en.y) + 4, en.z - 4, px, py, tests, esc, pol);
     return par;
 }
 
@@ -307,7 +318,7 @@ __device__ __forceinline__ void walk_entries(const IndexView &ix, const uint4 *e
 #pragma unroll
         for (int k = 0; k < B; ++k)
             if ((k == 0 || !(en[0].w & kEntLast)) &&
-                !in_bounds(en[k].x < ix.P && (!(en[k].w & kEntBoundary) || (uint64_t)en[k].y + en[k].z < ix.n_edge),
+                !in_bounds(en[k].x < ix.P && edges_ok(ix, en[k]),
                            ix))
                 return;
         // entries of this list among the B: up to and including the first LAST
@@ -325,7 +336,7 @@ __device__ __forceinline__ void walk_entries(const IndexView &ix, const uint4 *e
             const uint32_t nk = ((live >> k) & 1u) && (en[k].w & kEntBoundary) ? min(en[k].z, 4u) : 0u;
 #pragma unroll
             for (int j = 0; j < 4; ++j)
-                v[k][j] = ld_idx(ix.edge + ((uint32_t)j < nk ? en[k].y + j : 0u), pol);
+                v[k][j] = ld_idx((uint32_t)j < nk ? edge_at(ix, en[k].y) + j : ix.edge, pol);
 #pragma unroll
             for (int j = 0; j < 4; ++j)
                 if ((uint32_t)j >= nk)
@@ -366,8 +377,8 @@ __device__ __forceinline__ uint32_t walk_list(const IndexView &ix, uint32_t e0, 
     const uint4 *e = ix.ent + e0;
     const uint4 en0 = ld_idx(e, pol), en1 = ld_idx(e + 1, pol);
     const bool two = !(en0.w & kEntLast);
-    if (!in_bounds(en0.x < ix.P && (!(en0.w & kEntBoundary) || (uint64_t)en0.y + en0.z < ix.n_edge) &&
-                       (!two || (en1.x < ix.P && (!(en1.w & kEntBoundary) || (uint64_t)en1.y + en1.z < ix.n_edge))),
+    if (!in_bounds(en0.x < ix.P && edges_ok(ix, en0) &&
+                       (!two || (en1.x < ix.P && edges_ok(ix, en1))),
                    ix))
         return 0u;
     const uint32_t n0 = (en0.w & kEntBoundary) ? min(en0.z, 4u) : 0u;
@@ -375,8 +386,8 @@ __device__ __forceinline__ uint32_t walk_list(const IndexView &ix, uint32_t e0, 
     int4 v0[4], v1[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        v0[j] = ld_idx(ix.edge + ((uint32_t)j < n0 ? en0.y + j : 0u), pol);
-        v1[j] = ld_idx(ix.edge + ((uint32_t)j < n1 ? en1.y + j : 0u), pol);
+        v0[j] = ld_idx((uint32_t)j < n0 ? edge_at(ix, en0.y) + j : ix.edge, pol);
+        v1[j] = ld_idx((uint32_t)j < n1 ? edge_at(ix, en1.y) + j : ix.edge, pol);
     }
     uint32_t p0 = 0, p1 = 0;
 #pragma unroll
@@ -388,9 +399,9 @@ __device__ __forceinline__ uint32_t walk_list(const IndexView &ix, uint32_t e0, 
     }
     // lists longer than four edges: the rest, in row order
     if ((en0.w & kEntBoundary) && en0.z > 4 && max(v0[3].x, v0[3].z) > px)
-        p0 ^= row_parity<FP32, RW>(ix.edge + en0.y + 4, en0.z - 4, px, py, tests, esc, pol);
+        p0 ^= row_parity<FP32, RW>(edge_at(ix, en0.y) + 4, en0.z - 4, px, py, tests, esc, pol);
     if (two && (en1.w & kEntBoundary) && en1.z > 4 && max(v1[3].x, v1[3].z) > px)
-        p1 ^= row_parity<FP32, RW>(ix.edge + en1.y + 4, en1.z - 4, px, py, tests, esc, pol);
+        p1 ^= row_parity<FP32, RW>(edge_at(ix, en1.y) + 4, en1.z - 4, px, py, tests, esc, pol);
     const uint32_t in0 = (en0.w & kEntBoundary) ? p0 : 1u;
     const uint32_t in1 = two ? ((en1.w & kEntBoundary) ? p1 : 1u) : 0u;
     uint32_t c = in0 + in1;
@@ -401,9 +412,9 @@ __device__ __forceinline__ uint32_t walk_list(const IndexView &ix, uint32_t e0, 
             if (!in_bounds((uint64_t)(q - ix.ent) < ix.n_ent, ix))
                 break;
             const uint4 en = ld_idx(q, pol);
-            if (!in_bounds(en.x < ix.P && (!(en.w & kEntBoundary) || (uint64_t)en.y + en.z < ix.n_edge), ix))
+            if (!in_bounds(en.x < ix.P && edges_ok(ix, en), ix))
                 break;
-            if (!(en.w & kEntBoundary) || row_parity<FP32>(ix.edge + en.y, en.z, px, py, tests, esc, pol)) {
+            if (!(en.w & kEntBoundary) || row_parity<FP32>(edge_at(ix, en.y), en.z, px, py, tests, esc, pol)) {
                 if (!c)
                     first = en.x;
                 ++c;
@@ -486,8 +497,8 @@ __device__ __noinline__ bool poly_holds(const IndexView &ix, uint32_t q, int px,
         return false;
     for (uint64_t e = pay; in_bounds(e < ix.n_ent, ix); ++e) {
         const uint4 en = ld_idx(ix.ent + e, pol);
-        if (en.x == q && in_bounds(!(en.w & kEntBoundary) || (uint64_t)en.y + en.z < ix.n_edge, ix))
-            return !(en.w & kEntBoundary) || row_parity<FP32>(ix.edge + en.y, en.z, px, py, tests, esc, pol);
+        if (en.x == q && in_bounds(edges_ok(ix, en), ix))
+            return !(en.w & kEntBoundary) || row_parity<FP32>(edge_at(ix, en.y), en.z, px, py, tests, esc, pol);
         if (en.x >= q || (en.w & kEntLast))
             return false;
     }
@@ -526,9 +537,9 @@ __device__ __forceinline__ void walk_list_wave(const IndexView &ix, bool has, ui
         uint4 ea = more ? ld_idx(e, pol) : make_uint4(0, 0, 0, kEntLast);
         const uint4 eb0 = more ? ld_idx(e + 1, pol) : make_uint4(0, 0, 0, kEntLast);
         const bool hb0 = more && !(ea.w & kEntLast);
-        if (more && !in_bounds(ea.x < ix.P && (!(ea.w & kEntBoundary) || (uint64_t)ea.y + ea.z < ix.n_edge) &&
+        if (more && !in_bounds(ea.x < ix.P && edges_ok(ix, ea) &&
                                    (!hb0 || (eb0.x < ix.P &&
-                                             (!(eb0.w & kEntBoundary) || (uint64_t)eb0.y + eb0.z < ix.n_edge))),
+                                             edges_ok(ix, eb0))),
                                ix)) {
             more = false; // this lane's list ends here
             ea = make_uint4(0, 0, 0, kEntLast);
@@ -584,7 +595,7 @@ __device__ __forceinline__ void walk_list_wave(const IndexView &ix, bool has, ui
                         rad[h] = slot[h] ? r1 : r0;
                     }
                     const uint32_t ei = slot[h] ? oyb + (t - oza) : oya + t;
-                    v[h] = act[h] ? ld_idx(ix.edge + ei, pol) : make_int4(0, 0, 0, 0); // a zero edge never straddles
+                    v[h] = act[h] ? ld_idx(edge_at(ix, ei), pol) : make_int4(0, 0, 0, 0); // a zero edge never straddles
                 }
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
@@ -919,14 +930,9 @@ constexpr int kWQueue = kWChunk;        // list points queued per warp: a whole 
 // per warp: the queue, then the words of walk_list_wave
 constexpr size_t kWarpSmem = size_t(kWarps) * (kWQueue * sizeof(uint4) + kWaveWords * sizeof(uint32_t));
 
-// With DIR (a cell-clustered table and its directory, the directory grid at
-// least as fine as the coarse grid), k_agg_cells has already counted every
-// point of a coarse cell INSIDE one polygon from the cell's row range, and
-// marked the chunks that hold points of mixed coarse cells: the others are
-// skipped unread, and INSIDE coarse words count nothing here.
-template <bool FP32, bool CLUSTERED, bool DIR = false>
+template <bool FP32, bool CLUSTERED>
 __global__ void __launch_bounds__(kThreads, SPX_WARP_MIN_BLOCKS)
-    k_warp(JoinLaunch a, uint32_t nchunks, int use_hist, const uint32_t *chunk_mask)
+    k_warp(JoinLaunch a, uint32_t nchunks, int use_hist)
 {
     extern __shared__ __align__(16) unsigned char s_raw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -954,8 +960,6 @@ __global__ void __launch_bounds__(kThreads, SPX_WARP_MIN_BLOCKS)
     };
     const uint32_t nw = gridDim.x * kWarps;
     for (uint32_t ch = blockIdx.x * kWarps + warp; ch < nchunks; ch += nw) {
-        if (DIR && !((chunk_mask[ch >> 5] >> (ch & 31)) & 1u))
-            continue; // no point of a mixed coarse cell here
         const uint64_t base = (uint64_t)ch * kWChunk;
         const uint32_t npts = (uint32_t)min((uint64_t)kWChunk, a.n - base);
         int2 p[kWItems];
@@ -964,17 +968,13 @@ __global__ void __launch_bounds__(kThreads, SPX_WARP_MIN_BLOCKS)
         for (int j = 0; j < kWItems; ++j) {
             const uint32_t loc = j * 32 + lane;
             p[j] = loc < npts ? __ldcs(a.pts + base + loc) : make_int2(-1, -1);
-            n_pts += (!DIR && loc < npts) ? 1u : 0u;
+            n_pts += loc < npts ? 1u : 0u;
         }
 #pragma unroll
         for (int j = 0; j < kWItems; ++j) {
             const bool ok = (unsigned)p[j].x < kBox && (unsigned)p[j].y < kBox;
             const uint32_t cw = coarse_word(ix, ok ? (uint32_t)p[j].x : 0u, ok ? (uint32_t)p[j].y : 0u, keep);
             w[j] = ok ? cw : 0u;
-            if (DIR) { // INSIDE and empty coarse cells were counted from the directory
-                n_pts += ok && (cw >> 30) == kCellSub ? 1u : 0u;
-                w[j] = (cw >> 30) == kCellSub ? w[j] : 0u;
-            }
         }
 #pragma unroll
         for (int j = 0; j < kWItems; ++j) {
@@ -1053,14 +1053,14 @@ __global__ void __launch_bounds__(kThreads, SPX_WARP_MIN_BLOCKS)
 #endif
 constexpr int kResolveMinBlocks = SPX_RESOLVE_MIN_BLOCKS;
 #ifndef SPX_WALK_MIN_BLOCKS
-#define SPX_WALK_MIN_BLOCKS 3
+#define SPX_WALK_MIN_BLOCKS 4
 #endif
 constexpr int kWalkMinBlocks = SPX_WALK_MIN_BLOCKS;
-constexpr int kWalkQueue = 64; // < 32 rows carried over + one gather step of 32
 #ifndef SPX_WALK_BATCH
 #define SPX_WALK_BATCH 4
 #endif
-constexpr int kWalkBatch = SPX_WALK_BATCH;
+constexpr int kWalkBatch = SPX_WALK_BATCH; // rounds of rows resolved at a time
+constexpr int kWalkQueue = 32 * (kWalkBatch + 1); // < 32 carried over + a batch; or a batch less one + a gather step
 // A warp's range: short enough that a small table's words fill the chip twice
 // over (1M points: 61 warps of 512 words took 20.3 us, 977 of 32 take 7.5; 3M:
 // 22.7 -> 14.0), at most 512 (100M points: within 2 us from 256 to 1024).
@@ -1281,15 +1281,26 @@ __global__ void __launch_bounds__(THREADS, SUM ? 1 : (TMA ? 6 : kResolveMinBlock
 // queries: 1545 -> 185 us).
 constexpr uint32_t kSmallHist = 2048;
 
-template <bool FP32, int OUT, bool NEAR>
-__global__ void __launch_bounds__(kThreads, kWalkMinBlocks) k_walk(const __grid_constant__ JoinLaunch a, uint32_t *pend, uint32_t nwords,
-                                                                   uint32_t range)
+// The rows go through two queues of the warp.  Rows are resolved kWalkBatch rounds
+// of 32 at a time (their points, then their coarse words, then their fine words:
+// three round trips for 128 rows instead of for 32), and those with a list are
+// walked 32 at a time (500M points x 256 queries 4.54 -> 4.39 ms at 72 registers and
+// three CTAs per SM; with local edge lists 2.7 ms at 64 registers and four).
+//
+// With ALL (the count aggregate over a cell directory) a marked row is any row
+// of a mixed coarse cell: rows that its fine cell resolves are counted here.
+template <bool FP32, int OUT, bool NEAR, bool ALL>
+__global__ void __launch_bounds__(kThreads, NEAR ? 3 : kWalkMinBlocks) k_walk(const __grid_constant__ JoinLaunch a, uint32_t *pend,
+                                                                   uint32_t nwords)
 {
+    static_assert(!ALL || OUT == kOutCount, "ALL keeps nothing per row");
     __shared__ uint32_t s_qa[kWarps * kWalkQueue];
+    __shared__ uint4 s_la[kWarps * kWalkQueue];
     __shared__ uint32_t s_pa[kWarps * kWaveWords];
     __shared__ uint32_t s_hist[kSmallHist];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t *s_q = s_qa + warp * kWalkQueue; // rows
+    uint32_t *s_q = s_qa + warp * kWalkQueue; // rows to resolve
+    uint4 *s_l = s_la + warp * kWalkQueue;    // (x, y, first entry, row) to walk
     uint32_t *s_par = s_pa + warp * kWaveWords;
     const IndexView &ix = a.ix;
     const uint64_t keep = policy_evict_last();
@@ -1299,34 +1310,33 @@ __global__ void __launch_bounds__(kThreads, kWalkMinBlocks) k_walk(const __grid_
             s_hist[i] = 0;
         __syncthreads();
     }
-    uint32_t n_tests = 0, n_esc = 0, n_pairs = 0;
-    // walk the queued rows [0, m), m <= 32, one per lane
+    uint32_t n_tests = 0, n_esc = 0, n_pairs = 0, n_pts = 0, qn = 0, ln = 0;
+    // ALL: neighbouring rows mostly share a polygon (a clustered table): one
+    // atomic per distinct polygon of the warp
+    auto count_warp = [&](bool has, uint32_t q) {
+        if (hist)
+            hist_add_warp(s_hist, has, q);
+        else
+            global_add_warp(a.counts, has, q);
+    };
+    // walks the last m <= 32 queued lists, one per lane
     auto walk = [&](uint32_t m) {
-        __syncwarp();
         const bool has = (uint32_t)lane < m;
-        const uint32_t row = s_q[has ? lane : 0]; // idle lanes load lane 0's row and walk nothing
-        const int2 p = a.pts[row];
-        // the list's first entry: stored by pass 1a, or (narrow results) the
-        // cell resolved again
-        uint32_t e0;
-        bool lst = has;
-        if (OUT != kOut32) {
-            const uint32_t w = resolve(ix, (uint32_t)p.x, (uint32_t)p.y, keep); // a marked row's point is in the box
-            e0 = w & kPayloadMask;
-            lst = has && in_bounds((w >> 30) >= kCellList, ix);
-        } else {
-            e0 = __ldcg(a.res + row);
-        }
+        const uint4 it = s_l[ln - m + (has ? lane : 0)]; // idle lanes walk nothing
+        ln -= m;
+        const uint32_t row = it.w;
         uint32_t f = 0, c = 0;
         uint64_t ids = 0; // kOut16 and a.aux: the first polygons, aux_bits each
-        walk_list_wave<FP32, NEAR>(ix, lst, e0, p.x, p.y, n_tests, n_esc, keep, s_par, [&](uint32_t q) {
+        walk_list_wave<FP32, NEAR>(ix, has, it.z, (int)it.x, (int)it.y, n_tests, n_esc, keep, s_par, [&](uint32_t q) {
             if (OUT == kOut16 && (c + 1) * a.aux_bits <= 64)
                 ids |= (uint64_t)q << (a.aux_bits * c);
             f = c ? f : q;
             ++c;
-            if (a.counts)
+            if (a.counts && !(ALL && c == 1))
                 hist ? (void)atomicAdd(s_hist + q, 1u) : (void)atomicAdd(a.counts + q, 1ull);
         }, &a.near);
+        if (ALL)
+            count_warp(c >= 1, f);
         n_pairs += c;
         if (OUT != kOutCount && has) {
             if (OUT == kOut16) {
@@ -1346,29 +1356,77 @@ __global__ void __launch_bounds__(kThreads, kWalkMinBlocks) k_walk(const __grid_
         }
         __syncwarp(); // the queue is rewritten after the round
     };
-    constexpr int B = kWalkBatch; // bitmap words per lane per step, the next step's loaded ahead
-    const uint64_t w0 = ((uint64_t)blockIdx.x * kWarps + warp) * range;
-    const uint64_t w1 = min((uint64_t)nwords, w0 + range);
-    uint32_t qn = 0;
-    uint32_t nxt[B];
+    // resolves the last m <= 32 B queued rows, B per lane, and walks what fills rounds
+    constexpr int B = kWalkBatch;
+    auto take = [&](uint32_t m) {
+        __syncwarp();
+        qn -= m;
+        uint32_t row[B], w[B];
+        int2 p[B];
 #pragma unroll
-    for (int k = 0; k < B; ++k)
-        nxt[k] = w0 + k * 32 + lane < w1 ? __ldcs(pend + w0 + k * 32 + lane) : 0u;
-    for (uint64_t wb = w0; wb < w1; wb += 32 * B) {
-        uint32_t cur[B];
+        for (int u = 0; u < B; ++u) {
+            const uint32_t k = u * 32 + lane;
+            row[u] = s_q[qn + (k < m ? k : 0)]; // idle lanes repeat the first row and add nothing
+            p[u] = a.pts[row[u]];
+        }
+        // the list's first entry: stored by pass 1a (32-bit results), else the
+        // cell resolved again; a marked row's point is in the box
 #pragma unroll
-        for (int k = 0; k < B; ++k) {
+        for (int u = 0; u < B; ++u)
+            w[u] = OUT == kOut32 ? (kCellList << 30) | __ldcg(a.res + row[u])
+                                 : coarse_word(ix, (uint32_t)p[u].x, (uint32_t)p[u].y, keep);
+        if (OUT != kOut32) {
+#pragma unroll
+            for (int u = 0; u < B; ++u)
+                if ((w[u] >> 30) == kCellSub)
+                    w[u] = fine_word(ix, w[u], (uint32_t)p[u].x, (uint32_t)p[u].y, keep);
+        }
+#pragma unroll
+        for (int u = 0; u < B; ++u) {
+            const bool has = u * 32 + lane < m;
+            const uint32_t kind = w[u] >> 30, pay = w[u] & kPayloadMask;
+            const bool lst = has && kind >= kCellList;
+            if (ALL) {
+                const bool one = has && kind == kCellInsideOne && in_bounds(pay < ix.P, ix);
+                count_warp(one, pay);
+                n_pairs += one ? 1u : 0u;
+            } else {
+                in_bounds(!has || lst, ix);
+            }
+            const uint32_t bl = __ballot_sync(kFull, lst);
+            if (lst)
+                s_l[ln + __popc(bl & lanemask_lt())] = make_uint4((uint32_t)p[u].x, (uint32_t)p[u].y, pay, row[u]);
+            ln += __popc(bl);
+        }
+        __syncwarp();
+        while (ln >= 32)
+            walk(32);
+    };
+    // this warp's words: every nw-th group of 32, so that a run of marked rows (a
+    // clustered table) is shared out; a lane per word, BW groups loaded ahead
+    constexpr int BW = 4;
+    const uint64_t nw = (uint64_t)gridDim.x * kWarps, g0 = (uint64_t)blockIdx.x * kWarps + warp;
+    auto load = [&](uint64_t g) { return g * 32 + lane < nwords ? __ldcs(pend + g * 32 + lane) : 0u; };
+    uint32_t nxt[BW];
+#pragma unroll
+    for (int k = 0; k < BW; ++k)
+        nxt[k] = load(g0 + k * nw);
+    for (uint64_t g = g0; g * 32 < nwords; g += BW * nw) {
+        uint32_t cur[BW];
+#pragma unroll
+        for (int k = 0; k < BW; ++k) {
             cur[k] = nxt[k];
-            const uint64_t wn = wb + 32 * B + k * 32 + lane;
-            nxt[k] = wn < w1 ? __ldcs(pend + wn) : 0u;
+            nxt[k] = load(g + (BW + k) * nw);
         }
 #pragma unroll 1
-        for (int k = 0; k < B; ++k) { // not unrolled: one copy of the walk
-            const uint64_t wi = wb + k * 32 + lane;
+        for (int k = 0; k < BW; ++k) { // not unrolled: one copy of the walk
+            const uint64_t wi = (g + k * nw) * 32 + lane;
             uint32_t m = cur[0];
 #pragma unroll
-            for (int t = 0; t + 1 < B; ++t)
+            for (int t = 0; t + 1 < BW; ++t)
                 cur[t] = cur[t + 1];
+            if (ALL)
+                n_pts += __popc(m);
             while (__any_sync(kFull, m != 0)) {
                 const bool has = m != 0;
                 const uint32_t b = (uint32_t)__ffs(m) - 1u;
@@ -1377,31 +1435,33 @@ __global__ void __launch_bounds__(kThreads, kWalkMinBlocks) k_walk(const __grid_
                 if (has) {
                     const uint32_t row = (uint32_t)(wi * 32 + b);
                     s_q[qn + __popc(bl & lanemask_lt())] = row;
-                    prefetch_l2(a.pts + row); // loaded when its round is walked
+                    prefetch_l2(a.pts + row); // loaded when its round is resolved
                 }
                 qn += __popc(bl);
-                if (qn >= 32) {
-                    walk(32);
-                    const uint32_t rem = qn - 32; // move the rest (< 32) to the front
-                    const uint32_t it = (uint32_t)lane < rem ? s_q[32 + lane] : 0u;
-                    __syncwarp();
-                    if ((uint32_t)lane < rem)
-                        s_q[lane] = it;
-                    qn = rem;
-                    __syncwarp();
-                }
+                if (qn >= 32 * B)
+                    take(32 * B);
             }
         }
     }
     if (qn)
-        walk(qn);
+        take(qn);
+    if (ln)
+        walk(ln);
     if (hist) {
         __syncthreads();
         for (uint32_t i = threadIdx.x; i < ix.P; i += kThreads)
             if (s_hist[i])
                 atomicAdd(a.counts + i, (unsigned long long)s_hist[i]);
     }
-    add_stats(a.stats, 0u, n_tests, n_esc, n_pairs);
+    add_stats(a.stats, n_pts, n_tests, n_esc, n_pairs);
+}
+
+template <bool FP32, int OUT, bool NEAR, bool ALL = false>
+cudaError_t launch_walk(const JoinLaunch &a, uint32_t *pend, cudaStream_t s)
+{
+    const uint64_t nwords = (a.n + kWChunk - 1) / kWChunk * kWItems, per_cta = uint64_t(kWarps) * walk_range(nwords);
+    k_walk<FP32, OUT, NEAR, ALL><<<unsigned((nwords + per_cta - 1) / per_cta), kThreads, 0, s>>>(a, pend, uint32_t(nwords));
+    return cudaGetLastError();
 }
 
 // Pass 1 of a small table in one launch: a warp per 256-point chunk resolves its
@@ -2249,70 +2309,100 @@ int persistent_grid(K kernel, int threads, size_t smem, uint32_t ntiles)
     return grid;
 }
 
-template <bool FP32, bool CLUSTERED, bool DIR = false>
-cudaError_t launch_warp_kernel(const JoinLaunch &a, int use_hist, cudaStream_t s, const uint32_t *chunk_mask = nullptr)
+template <bool FP32, bool CLUSTERED>
+cudaError_t launch_warp_kernel(const JoinLaunch &a, int use_hist, cudaStream_t s)
 {
     static bool done[64] = {};
     const uint64_t nchunks = (a.n + kWChunk - 1) / kWChunk;
     if (nchunks >= (1ull << 32))
         return cudaErrorInvalidValue;
     const size_t smem = kWarpSmem + (use_hist ? sizeof(uint32_t) * a.ix.P : 0);
-    auto kern = k_warp<FP32, CLUSTERED, DIR>;
+    auto kern = k_warp<FP32, CLUSTERED>;
     cudaError_t e = smem_opt_in(kern, kWarpSmem + sizeof(uint32_t) * kHistMax, done);
     if (e != cudaSuccess)
         return e;
     const uint32_t nblk = uint32_t((nchunks + kWarps - 1) / kWarps);
-    kern<<<persistent_grid(kern, kThreads, smem, nblk), kThreads, smem, s>>>(a, uint32_t(nchunks), use_hist,
-                                                                             chunk_mask);
+    kern<<<persistent_grid(kern, kThreads, smem, nblk), kThreads, smem, s>>>(a, uint32_t(nchunks), use_hist);
     return cudaGetLastError();
 }
 
-// The directory stage of the count aggregate over a cell-clustered table:
-// a thread per cell of the directory grid (2^c, c >= g).  A cell inside a
-// coarse cell INSIDE one polygon adds its whole row range to that polygon
-// (its points need not be read); an empty one adds nothing; one in a mixed
-// coarse cell marks the 256-point chunks its range touches, for k_warp<DIR>.
-// The points of the cells counted here, and of the bin outside the box, go
-// into the scanned-points counter.
+// The directory stage of the count aggregate over a cell-clustered table: a
+// lane per cell of the directory grid (2^c, c >= g), kDirCells cells at a time.
+// A cell inside a coarse cell INSIDE one polygon adds its whole row range to
+// that polygon (its points need not be read); an empty one adds nothing; one in
+// a mixed coarse cell marks its rows in the bitmap, for k_walk<ALL>.  The points
+// of the cells counted here, and of the bin outside the box, go into the
+// scanned-points counter.  The stage reads 8 B per cell and a coarse word per
+// cell with points, kDirCells independent loads of each per lane; rows are 32-bit
+// (2^26 cells, 500M points: 500 us with 64-bit rows and one cell per lane at a
+// time, DIRUS so).
+constexpr int kDirCells = 4;
 __global__ void __launch_bounds__(256) k_agg_cells(const unsigned long long *cell_end, int c, IndexView ix,
-                                                   unsigned long long *counts, uint32_t *chunk_mask,
+                                                   unsigned long long *counts, uint32_t *rows,
                                                    unsigned long long *stats)
 {
-    const uint32_t ncell = 1u << (2 * c);
+    const uint32_t ncell = 1u << (2 * c), lane = threadIdx.x & 31;
     const int sh = c - ix.gc;
     unsigned long long done_pts = 0;
-    for (uint32_t k0 = blockIdx.x * 256 + (threadIdx.x & ~31u); k0 < ncell; k0 += gridDim.x * 256) {
-        const uint32_t k = k0 + (threadIdx.x & 31);
-        const bool in = k < ncell;
-        const unsigned long long s0 = in && k ? cell_end[k - 1] : 0ull, s1 = in ? cell_end[k] : 0ull;
-        const bool has = s1 > s0;
-        uint32_t w = 0;
-        if (has) {
-            const uint32_t cx = k & ((1u << c) - 1), cy = k >> c;
-            w = ix.cell[((cy >> sh) << ix.gc) | (cx >> sh)];
+    for (uint32_t k0 = (blockIdx.x * 256 + (threadIdx.x & ~31u)) * kDirCells; k0 < ncell; k0 += gridDim.x * 256 * kDirCells) {
+        uint32_t s0[kDirCells], s1[kDirCells], w[kDirCells]; // a cell's rows [s0, s1) and its coarse word
+#pragma unroll
+        for (int j = 0; j < kDirCells; ++j) {
+            const uint32_t k = k0 + 32 * j + lane;
+            s1[j] = k < ncell ? (uint32_t)cell_end[k] : 0u;
         }
-        const uint32_t kind = w >> 30, q = w & kPayloadMask;
-        const bool one = has && kind == kCellInsideOne && in_bounds(q < ix.P, ix);
-        done_pts += has && kind != kCellSub ? s1 - s0 : 0ull;
-        // counts: one atomic for the warp when its cells share the polygon
-        const uint32_t m = __ballot_sync(kFull, one);
-        if (m) {
-            const uint32_t qmin = __reduce_min_sync(kFull, one ? q : 0xffffffffu);
-            const uint32_t qmax = __reduce_max_sync(kFull, one ? q : 0u);
-            if (qmin == qmax) {
-                const unsigned long long t = warp_sum64(one ? s1 - s0 : 0ull);
-                if ((int)(threadIdx.x & 31) == __ffs(m) - 1)
-                    atomicAdd(counts + qmin, t);
-            } else if (one) {
-                atomicAdd(counts + q, s1 - s0);
+        uint32_t last = k0 ? (uint32_t)cell_end[k0 - 1] : 0u;
+#pragma unroll
+        for (int j = 0; j < kDirCells; ++j) {
+            const uint32_t up = __shfl_up_sync(kFull, s1[j], 1);
+            s0[j] = lane ? up : last;
+            last = __shfl_sync(kFull, s1[j], 31);
+            const uint32_t k = k0 + 32 * j + lane;
+            w[j] = 0;
+            if (s1[j] > s0[j])
+                w[j] = ix.cell[(((k >> c) >> sh) << ix.gc) | ((k & ((1u << c) - 1u)) >> sh)];
+        }
+#pragma unroll
+        for (int j = 0; j < kDirCells; ++j) {
+            const uint32_t num = s1[j] > s0[j] ? s1[j] - s0[j] : 0u;
+            const uint32_t kind = w[j] >> 30, q = w[j] & kPayloadMask;
+            const bool sub = kind == kCellSub; // a cell without points has w = 0
+            const bool one = kind == kCellInsideOne && in_bounds(q < ix.P, ix);
+            done_pts += sub ? 0u : num;
+            // counts: one atomic for the warp when its cells share the polygon
+            const uint32_t m = __ballot_sync(kFull, one);
+            if (m) {
+                const uint32_t q0 = __shfl_sync(kFull, q, __ffs(m) - 1);
+                if (!__any_sync(kFull, one && q != q0)) {
+                    const uint32_t t = __reduce_add_sync(kFull, one ? num : 0u); // rows: below 2^32 in all
+                    if ((int)lane == __ffs(m) - 1)
+                        atomicAdd(counts + q0, (unsigned long long)t);
+                } else if (one) {
+                    atomicAdd(counts + q, (unsigned long long)num);
+                }
             }
-        }
-        if (has && kind == kCellSub) {
-            const uint64_t c0 = s0 / kWChunk, c1 = (s1 - 1) / kWChunk;
-            for (uint64_t wd = c0 >> 5; wd <= (c1 >> 5); ++wd) {
-                const uint64_t lo = max(c0, wd << 5), hi = min(c1, (wd << 5) + 31);
-                const uint32_t bits = (hi - lo == 31) ? 0xffffffffu : (((1u << (hi - lo + 1)) - 1u) << (lo & 31));
-                atomicOr(chunk_mask + wd, bits);
+            if (!__any_sync(kFull, sub))
+                continue;
+            // rows of a cell in a mixed coarse cell; ranges over two words by the warp
+            const uint32_t r0 = s0[j], r1 = sub ? s1[j] - 1 : s0[j];
+            auto mark = [&](uint32_t wd, uint32_t a, uint32_t z) {
+                const uint32_t lo = wd == (a >> 5) ? a & 31u : 0u, hi = wd == (z >> 5) ? z & 31u : 31u;
+                if (hi - lo == 31)
+                    rows[wd] = 0xffffffffu; // no other cell's rows here
+                else
+                    atomicOr(rows + wd, (0xffffffffu >> (31 - (hi - lo))) << lo);
+            };
+            const bool wide = (r1 >> 5) - (r0 >> 5) > 1;
+            if (sub && !wide) {
+                mark(r0 >> 5, r0, r1);
+                if ((r1 >> 5) != (r0 >> 5))
+                    mark(r1 >> 5, r0, r1);
+            }
+            for (uint32_t todo = __ballot_sync(kFull, sub && wide); todo; todo &= todo - 1) {
+                const int src = __ffs(todo) - 1;
+                const uint32_t a = __shfl_sync(kFull, r0, src), z = __shfl_sync(kFull, r1, src);
+                for (uint32_t wd = (a >> 5) + lane; wd <= (z >> 5); wd += 32)
+                    mark(wd, a, z);
             }
         }
     }
@@ -2320,7 +2410,7 @@ __global__ void __launch_bounds__(256) k_agg_cells(const unsigned long long *cel
     if (blockIdx.x == 0 && threadIdx.x == 0)
         done_pts += cell_end[ncell] - cell_end[ncell - 1];
     done_pts = warp_sum64(done_pts);
-    if ((threadIdx.x & 31) == 0 && done_pts) {
+    if (lane == 0 && done_pts) {
         atomicAdd(stats + kStatPoints, done_pts);
         atomicAdd(stats + kStatDirPoints, done_pts);
     }
@@ -2372,12 +2462,7 @@ cudaError_t launch_pass1_as(const JoinLaunch &a, uint32_t *pend, cudaStream_t s,
         return e;
     if (mid)
         cudaEventRecord(mid, s);
-    // pass 1b: a warp per `range` bitmap words, as many CTAs as that takes
-    const uint64_t nwords = nchunks * kWItems;
-    const uint32_t range = walk_range(nwords);
-    const uint64_t wblk = (nwords + uint64_t(kWarps) * range - 1) / (uint64_t(kWarps) * range);
-    k_walk<FP32, OUT, NEAR><<<unsigned(wblk), kThreads, 0, s>>>(a, pend, uint32_t(nwords), range);
-    return cudaGetLastError();
+    return launch_walk<FP32, OUT, NEAR>(a, pend, s); // pass 1b
 }
 
 // Calls f(fp32, near) with the launch's two switches as compile-time values.
@@ -3250,6 +3335,259 @@ cudaError_t launch_sum_u64(unsigned long long *dst, const unsigned long long *x,
     return cudaGetLastError();
 }
 
+// ------------------------------------------------------ local edge lists
+// A fine cell of side S at (x0, y0) and the row list of one of its polygons.  An
+// edge takes part in the cell's tests through its part over the integer rows
+// [y0, y0 + S - 1], and that part is, for the cell's points,
+//   left   never crossed by a rightward ray: dropped;
+//   right  crossed by every ray of a row it straddles, whatever the point's x:
+//          only the parity of such edges per row matters, a step function of y;
+//   near   neither for certain: kept.
+// The ends of the part come from FP32 with 2^-18 of the magnitudes (and 4 units)
+// as margin, 64 times what its few roundings cost; an edge whose own x range is
+// right of the cell needs no arithmetic.  The step function is written as edges
+// at x = 2^30, right of every point: one over all rows when it is odd at y0, and
+// one from t up for every y = t where it changes.  A vertex between two right
+// edges changes it twice, so the changes are the few vertices where a chain
+// passes from right to near or left.
+constexpr uint32_t kLocalMin = 8;   // shorter lists stay
+constexpr uint32_t kLocalMean = 8;  // mean edges per list from which an index gets local lists
+constexpr int kLocalTurns = 8;      // changes of parity a cell may record; else the list stays
+
+struct LocalCell {
+    int x0, y0, S;
+};
+
+// 0 left or without a row, 1 near, 2 right
+__device__ __forceinline__ int edge_side(const int4 &v, const LocalCell &c)
+{
+    const int ylo = max(c.y0, min(v.y, v.w)), yhi = min(c.y0 + c.S, max(v.y, v.w)) - 1;
+    if (ylo > yhi)
+        return 0; // straddles no integer row of the cell
+    if (min(v.x, v.z) >= c.x0 + c.S)
+        return 2;
+    const float ax = __int2float_rn(v.x - c.x0), dx = __int2float_rn(v.z - v.x);
+    const float slope = dx / __int2float_rn(v.w - v.y);
+    const float xa = ax + slope * __int2float_rn(ylo - v.y), xb = ax + slope * __int2float_rn(yhi - v.y);
+    const float margin = 4.f + 3.814697265625e-06f * (fabsf(ax) + fabsf(dx)); // 2^-18
+    if (fminf(xa, xb) - margin >= __int2float_rn(c.S))
+        return 2;
+    return fmaxf(xa, xb) + margin < 0.f ? 0 : 1;
+}
+
+// What the list of entry en becomes in cell c: its number of edges, and the
+// changes of parity (turn[0 .. nt), odd: the parity at y0); or en.z when it stays.
+__device__ __forceinline__ uint32_t local_size(const IndexView &ix, const uint4 &en, const LocalCell &c,
+                                               int (&turn)[kLocalTurns], int &nt, uint32_t &odd)
+{
+    nt = 0;
+    odd = 0;
+    if (!(en.w & kEntBoundary) || en.z < kLocalMin)
+        return en.z;
+    uint32_t near = 0;
+    for (uint32_t k = 0; k < en.z; ++k) {
+        const int4 v = ix.edge[en.y + k];
+        const int side = edge_side(v, c);
+        near += side == 1 ? 1u : 0u;
+        if (side != 2)
+            continue;
+        odd ^= (v.y > c.y0) != (v.w > c.y0) ? 1u : 0u;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int y = h ? v.w : v.y;
+            if (y <= c.y0 || y >= c.y0 + c.S)
+                continue;
+            int at = -1;
+            for (int i = 0; i < nt; ++i)
+                at = turn[i] == y ? i : at;
+            if (at >= 0)
+                turn[at] = turn[--nt];
+            else if (nt < kLocalTurns)
+                turn[nt++] = y;
+            else
+                return en.z;
+        }
+    }
+    const uint32_t size = near + odd + (uint32_t)nt;
+    return size * 4 <= en.z * 3 ? size : en.z;
+}
+
+// A lane per fine cell.  COUNT: totals[0..1] += local edges, changed entries.
+// Else: the lists and the records of the changed entries, at places that each
+// warp takes from totals[0..1] (zeroed), in no particular order.
+template <bool COUNT>
+__global__ void __launch_bounds__(256) k_local(IndexView ix, const uint32_t *blk_cell, uint64_t n_words,
+                                               unsigned long long *totals, uint4 *ent, int4 *loc, uint4 *undo)
+{
+    const int lane = threadIdx.x & 31;
+    unsigned long long all_loc = 0, all_ent = 0;
+    for (uint64_t t0 = (uint64_t)blockIdx.x * 256 + (threadIdx.x & ~31u); t0 < n_words; t0 += (uint64_t)gridDim.x * 256) {
+        const uint64_t t = t0 + lane;
+        const uint32_t w = t < n_words ? ix.fine[t] : 0u;
+        const bool lst = (w >> 30) == kCellList;
+        if (!__any_sync(kFull, lst))
+            continue;
+        LocalCell c{0, 0, 1 << ix.sf};
+        if (lst) {
+            const uint32_t cw = blk_cell[t >> (2 * ix.sb)], f = (uint32_t)t & ((1u << (2 * ix.sb)) - 1);
+            c.x0 = int(((cw & ((1u << ix.gc) - 1)) << ix.sc) | ((f & ((1u << ix.sb) - 1)) << ix.sf));
+            c.y0 = int(((cw >> ix.gc) << ix.sc) | ((f >> ix.sb) << ix.sf));
+        }
+        int turn[kLocalTurns], nt;
+        uint32_t odd, n_loc = 0, n_ent = 0;
+        bool more = lst;
+        for (uint64_t e = w & kPayloadMask; more; ++e) {
+            const uint4 en = ent[e];
+            const uint32_t size = local_size(ix, en, c, turn, nt, odd);
+            n_loc += size < en.z ? size : 0u;
+            n_ent += size < en.z ? 1u : 0u;
+            more = !(en.w & kEntLast);
+        }
+        all_loc += n_loc;
+        all_ent += n_ent;
+        if (COUNT || !__any_sync(kFull, n_ent != 0))
+            continue;
+        unsigned long long inc = ((unsigned long long)n_ent << 40) | n_loc;
+        const unsigned long long mine = inc;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long v = __shfl_up_sync(kFull, inc, o);
+            if (lane >= o)
+                inc += v;
+        }
+        constexpr unsigned long long kLow = (1ull << 40) - 1;
+        unsigned long long at_loc = 0, at_ent = 0;
+        if (lane == 31) {
+            at_loc = atomicAdd(totals, inc & kLow);
+            at_ent = atomicAdd(totals + 1, inc >> 40);
+        }
+        at_loc = __shfl_sync(kFull, at_loc, 31) + ((inc - mine) & kLow);
+        at_ent = __shfl_sync(kFull, at_ent, 31) + ((inc - mine) >> 40);
+        more = n_ent != 0;
+        for (uint64_t e = w & kPayloadMask; more; ++e) {
+            const uint4 en = ent[e];
+            more = !(en.w & kEntLast);
+            const uint32_t size = local_size(ix, en, c, turn, nt, odd);
+            if (size >= en.z)
+                continue;
+            undo[at_ent++] = make_uint4((uint32_t)e, en.y, en.z, 0u);
+            int4 *d = loc + at_loc;
+            const int far = int(kBox);
+            if (odd)
+                *d++ = make_int4(far, c.y0, far, c.y0 + c.S);
+            for (int i = 0; i < nt; ++i)
+                *d++ = make_int4(far, turn[i], far, c.y0 + c.S);
+            for (uint32_t k = 0; k < en.z; ++k) { // in the list's order: right ends descending
+                const int4 v = ix.edge[en.y + k];
+                if (edge_side(v, c) == 1)
+                    *d++ = v;
+            }
+            ent[e].y = kLocalEdge | (uint32_t)at_loc;
+            ent[e].z = size;
+            at_loc += size;
+        }
+    }
+    if (COUNT) {
+        all_loc = warp_sum64(all_loc), all_ent = warp_sum64(all_ent);
+        if (lane == 0) {
+            atomicAdd(totals, all_loc);
+            atomicAdd(totals + 1, all_ent);
+        }
+    }
+}
+
+// totals[0..1] += the edges that the entries list, and the entries that list any.
+__global__ void __launch_bounds__(256) k_list_edges(const uint4 *ent, uint64_t n, unsigned long long *totals)
+{
+    unsigned long long z = 0, b = 0;
+    for (uint64_t i = (uint64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (uint64_t)gridDim.x * 256) {
+        const uint4 en = ent[i];
+        const bool bnd = en.w & kEntBoundary;
+        z += bnd ? en.z : 0u;
+        b += bnd ? 1u : 0u;
+    }
+    z = warp_sum64(z), b = warp_sum64(b);
+    if ((threadIdx.x & 31) == 0) {
+        atomicAdd(totals, z);
+        atomicAdd(totals + 1, b);
+    }
+}
+
+// The cell of every block.
+__global__ void __launch_bounds__(256) k_blk_cell(uint32_t ncell, const uint32_t *cell, uint32_t *blk_cell)
+{
+    for (uint32_t c = blockIdx.x * 256 + threadIdx.x; c < ncell; c += gridDim.x * 256)
+        if ((cell[c] >> 30) == kCellSub)
+            blk_cell[cell[c] & kPayloadMask] = c;
+}
+
+cudaError_t build_local_lists(const IndexView &view, uint4 *ent, LocalLists &out, cudaStream_t s, cudaMemPool_t pool)
+{
+    out = LocalLists{};
+    const uint64_t n_blk = view.n_fine >> (2 * view.sb), n_words = n_blk << (2 * view.sb);
+    if (!n_words || view.n_edge >= kLocalEdge || view.n_ent >= (1ull << 32))
+        return cudaSuccess;
+    auto blocks = [](uint64_t n) { return unsigned(std::min<uint64_t>((n + 255) / 256, uint64_t(device_sm_count()) * 32)); };
+    const size_t b_blk = (n_blk * 4 + 255) & ~size_t(255);
+    void *tmp = nullptr;
+    unsigned long long h[4] = {};
+    cudaError_t e = cudaMallocFromPoolAsync(&tmp, b_blk + sizeof(h), pool, s);
+    if (e != cudaSuccess) { // the index works without them
+        cudaGetLastError();
+        return cudaSuccess;
+    }
+    auto done = [&](cudaError_t err) {
+        cudaFreeAsync(tmp, s);
+        if (err != cudaSuccess && out.mem) {
+            cudaFreeAsync(out.mem, s);
+            out = LocalLists{};
+        }
+        return err;
+    };
+    uint32_t *blk_cell = static_cast<uint32_t *>(tmp);
+    auto *totals = reinterpret_cast<unsigned long long *>(static_cast<char *>(tmp) + b_blk);
+    auto read = [&](int n) {
+        const cudaError_t x = cudaMemcpyAsync(h, totals, n * 8, cudaMemcpyDeviceToHost, s);
+        return x != cudaSuccess ? x : cudaStreamSynchronize(s);
+    };
+    if ((e = cudaMemsetAsync(totals, 0, sizeof(h), s)) != cudaSuccess)
+        return done(e);
+    k_list_edges<<<blocks(view.n_ent), 256, 0, s>>>(ent, view.n_ent, totals + 2);
+    if ((e = cudaGetLastError()) != cudaSuccess || (e = read(4)) != cudaSuccess)
+        return done(e);
+    // Lists of four edges (maps of 500 to 5000 cells with about 500 vertices each)
+    // gain nothing: 2000 cells, walk 81 us without, 92 with, and the build costs
+    // 2 ms.  40 (queries of up to 5000 vertices) or 15 (40000 cells of up to 10000):
+    // the walk of 500M points x 256 queries 4.39 -> 2.74 ms.
+    if (h[2] < kLocalMean * h[3])
+        return done(cudaSuccess);
+    const uint32_t ncell = 1u << (2 * view.gc);
+    k_blk_cell<<<blocks(ncell), 256, 0, s>>>(ncell, view.cell, blk_cell);
+    k_local<true><<<blocks(n_words), 256, 0, s>>>(view, blk_cell, n_words, totals, ent, nullptr, nullptr);
+    if ((e = cudaGetLastError()) != cudaSuccess || (e = read(2)) != cudaSuccess)
+        return done(e);
+    if (h[0] >= kLocalEdge || !h[1])
+        return done(cudaSuccess);
+    out.bytes = (h[0] + h[1] + 1) * 16;
+    if (cudaMallocFromPoolAsync(&out.mem, out.bytes, pool, s) != cudaSuccess) {
+        out = LocalLists{};
+        cudaGetLastError();
+        return done(cudaSuccess);
+    }
+    int4 *loc = static_cast<int4 *>(out.mem);
+    uint4 *undo = reinterpret_cast<uint4 *>(loc + h[0]);
+    out.loc = loc;
+    out.undo = undo;
+    out.n_loc = h[0];
+    out.n_undo = h[1];
+    if ((e = cudaMemsetAsync(totals, 0, 16, s)) != cudaSuccess)
+        return done(e);
+    k_local<false><<<blocks(n_words), 256, 0, s>>>(view, blk_cell, n_words, totals, ent, loc, undo);
+    if ((e = cudaGetLastError()) != cudaSuccess || (e = cudaStreamSynchronize(s)) != cudaSuccess)
+        return done(e);
+    return done(cudaSuccess);
+}
+
 int device_sm_count()
 {
     int dev = 0;
@@ -3347,7 +3685,7 @@ cudaError_t launch_join(const JoinLaunch &a, void *scratch, cudaStream_t s, cuda
     return cudaSuccess;
 }
 
-static bool use_directory(const JoinLaunch &a)
+bool use_directory(const JoinLaunch &a)
 {
     return a.clustered && a.cell_end && a.cluster_log2 >= a.ix.gc && a.cluster_log2 <= 13;
 }
@@ -3373,10 +3711,9 @@ static size_t split_count_bytes(uint64_t n)
 
 size_t aggregate_scratch_bytes(const JoinLaunch &a)
 {
-    const uint64_t nchunks = (a.n + kWChunk - 1) / kWChunk;
-    if (!a.clustered || a.near.rad)
-        return split_count_bytes(a.n);
-    return use_directory(a) ? size_t((nchunks + 31) / 32) * 4 + 16 : 16;
+    return use_directory(a) && !a.near.rad ? size_t((a.n + kWChunk - 1) / kWChunk) * kWItems * 4
+           : !a.clustered || a.near.rad    ? split_count_bytes(a.n)
+                                           : 0;
 }
 
 cudaError_t launch_aggregate(const JoinLaunch &a, void *scratch, cudaStream_t s, cudaEvent_t *ev)
@@ -3412,19 +3749,18 @@ cudaError_t launch_aggregate(const JoinLaunch &a, void *scratch, cudaStream_t s,
     const int use_hist = a.ix.P <= (uint32_t)kHistMax ? 1 : 0;
     if (ev)
         cudaEventRecord(ev[0], s);
-    if (use_directory(a)) {
-        // cells INSIDE one polygon counted from the directory, then the chunks of mixed cells
-        uint32_t *mask = static_cast<uint32_t *>(scratch);
-        const uint64_t nchunks = (a.n + kWChunk - 1) / kWChunk;
-        if ((e = cudaMemsetAsync(mask, 0, size_t((nchunks + 31) / 32) * 4, s)) != cudaSuccess)
+    if (use_directory(a) && scratch) {
+        // cells INSIDE one polygon counted from the directory, then the rows of mixed cells
+        uint32_t *rows = static_cast<uint32_t *>(scratch);
+        if ((e = cudaMemsetAsync(rows, 0, aggregate_scratch_bytes(a), s)) != cudaSuccess)
             return e;
         const uint64_t ncell = uint64_t(1) << (2 * a.cluster_log2);
-        const unsigned grid = unsigned(std::min<uint64_t>((ncell + 255) / 256, uint64_t(device_sm_count()) * 16));
-        k_agg_cells<<<grid, 256, 0, s>>>(a.cell_end, a.cluster_log2, a.ix, a.counts, mask, a.stats);
+        const unsigned grid = unsigned(std::min<uint64_t>((ncell + 256 * kDirCells - 1) / (256 * kDirCells), uint64_t(device_sm_count()) * 16));
+        k_agg_cells<<<grid, 256, 0, s>>>(a.cell_end, a.cluster_log2, a.ix, a.counts, rows, a.stats);
         if ((e = cudaGetLastError()) != cudaSuccess)
             return e;
-        e = a.fp32 ? launch_warp_kernel<true, true, true>(a, use_hist, s, mask)
-                   : launch_warp_kernel<false, true, true>(a, use_hist, s, mask);
+        e = a.fp32 ? launch_walk<true, kOutCount, false, true>(a, rows, s)
+                   : launch_walk<false, kOutCount, false, true>(a, rows, s);
     } else if (a.clustered)
         e = a.fp32 ? launch_warp_kernel<true, true>(a, use_hist, s) : launch_warp_kernel<false, true>(a, use_hist, s);
     else

@@ -29,11 +29,19 @@ struct IndexView {
     int ssh;              // summary shift: 30 - sg
     int sg;               // summary grid log2
     int use_sum;          // the summary resolves enough of the box to be worth its shared memory
+    // local edge lists of long entries (build_local_lists): an entry whose y has
+    // the bit loc_bit (kLocalEdge, or 0 without such lists) set names its edges in
+    // loc, at y without that bit, instead of in edge
+    const int4 *loc;
+    uint32_t loc_bit;
+    uint64_t n_loc;
     // array sizes (sentinels included) and the error word, for the bounds
     // checks of a build with SPX_BOUNDS_CHECK
     uint64_t n_fine, n_ent, n_edge;
     unsigned *err;
 };
+constexpr uint32_t kLocalEdge = 0x80000000u;
+
 // Buffered polygons (SPADE §4.2 distance canvases: a polygon plus a rounded
 // rectangle of radius r around each edge).  The index is an IndexView as ever,
 // but for three things.  A coarse word of kind kCellCoarseList names an entry
@@ -155,6 +163,24 @@ struct JoinLaunch {
     NearView near; // near.rad set: ix is a buffered-polygon index
 };
 
+// Shortens the edge lists of a built polygon index where they are long, in place
+// (ent is view.ent): an entry's row list, which runs to the far side of its
+// polygon, becomes the list of the edges that can cross the row inside its fine
+// cell, and of one edge beyond the box per change of parity that the others make
+// along the cell's rows.  Every point of the cell crosses the new list as often,
+// modulo 2, as the old one.  out.mem (the lists, then a record (entry, y, z, 0)
+// per changed entry) belongs to the caller, who frees it with cudaFreeAsync; null
+// where the lists are short anyway, or there is no memory.  Memory from `pool`, in
+// the order of stream s, which is synchronised.
+struct LocalLists {
+    void *mem;
+    size_t bytes;
+    const int4 *loc;
+    const uint4 *undo;
+    uint64_t n_loc, n_undo;
+};
+cudaError_t build_local_lists(const IndexView &view, uint4 *ent, LocalLists &out, cudaStream_t s, cudaMemPool_t pool);
+
 // The index of buffered polygons (NearView), built on the device from the host's
 // edge grid (cell_off, item_q, item_seg: CSR by cell of a 2^g grid, on the
 // device), the radii and the polygons' own index.  out.mem holds cells | fine |
@@ -192,11 +218,11 @@ cudaError_t launch_join(const JoinLaunch &a, void *scratch, cudaStream_t s, cuda
 cudaError_t launch_join_count(const JoinLaunch &a, void *scratch, cudaStream_t s, cudaEvent_t *ev = nullptr);
 cudaError_t launch_join_write(const JoinLaunch &a, void *scratch, cudaStream_t s);
 cudaError_t launch_join_plain(const JoinLaunch &a, void *scratch, cudaStream_t s);
-// scratch: aggregate_scratch_bytes(a) bytes (the chunk bitmap of the directory
-// path, the row bitmap of a table in row order), not shared with a launch that
-// may overlap this one; null with a table in row order: one pass without
-// scratch, slower.  a.keep_counts: add to the counts instead of zeroing them
-// first.  use_split_count: whether this launch would use the row bitmap.
+// scratch: aggregate_scratch_bytes(a) bytes (a bitmap over the rows), not shared
+// with a launch that may overlap this one, or null: one pass without scratch,
+// slower.  a.keep_counts: add to the counts instead of zeroing them first.
+// use_split_count, use_directory: whether this launch would use the bitmap.
+bool use_directory(const JoinLaunch &a);
 bool use_split_count(const JoinLaunch &a);
 size_t aggregate_scratch_bytes(const JoinLaunch &a);
 cudaError_t launch_aggregate(const JoinLaunch &a, void *scratch, cudaStream_t s, cudaEvent_t *ev = nullptr);
