@@ -33,41 +33,43 @@ struct PBox {
     int32_t fx0, fx1, fy0, fy1; // fine columns and rows
 };
 
-__device__ __forceinline__ long long fdiv(long long a, long long b) // floor(a / b), b > 0
-{
-    const long long q = a / b;
-    return (a % b != 0 && a < 0) ? q - 1 : q;
-}
-__device__ __forceinline__ long long cdiv(long long a, long long b) // ceil(a / b), b > 0
-{
-    const long long q = a / b;
-    return (a % b != 0 && a > 0) ? q + 1 : q;
-}
-// x of the line through a -> b at height Y, as floor and ceil (exact rationals)
-__device__ __forceinline__ void line_x(long long ax, long long ay, long long bx, long long by, long long Y,
-                                       long long &fl, long long &ce)
-{
-    long long num = (bx - ax) * (Y - ay), den = by - ay;
-    if (den < 0) {
-        num = -num;
-        den = -den;
+// floor and ceil of v / 2^sh
+__device__ __forceinline__ long long fshr(long long v, int sh) { return v >> sh; }
+__device__ __forceinline__ long long cshr(long long v, int sh) { return -((-v) >> sh); }
+
+// The edge a -> b (not horizontal), for x of its line at heights Y between its
+// ends as floor and ceil (exact rationals).  The quotient is at most 2^30 in
+// magnitude: an FP32 estimate is within 2^9 of it (2^-22 relative), a second one
+// of the exact remainder within 0.51, and one step makes it the floor.  A 64-bit
+// division costs four times as much, and k_ib_mark needs one per row.
+struct EdgeLine {
+    long long ax, ay, dx; // dx: signed so that (Y - ay) dx / den is the x offset
+    int den;              // |by - ay|
+    float inv;
+    __device__ __forceinline__ EdgeLine(int2 a, int2 b)
+        : ax(a.x), ay(a.y), dx(b.y > a.y ? (long long)b.x - a.x : (long long)a.x - b.x), den(abs(b.y - a.y)),
+          inv(1.f / (float)den)
+    {
     }
-    fl = ax + fdiv(num, den);
-    ce = ax + cdiv(num, den);
-}
-// The edge a -> b straddles the corner row at height y0: the corners (x0, y0)
-// left of its crossing x* are those with x0 <= ceil(x*) - 1; the largest such
-// cell column of side S.
-__device__ __forceinline__ long long corner_col(long long ax, long long ay, long long bx, long long by, long long y0,
-                                                long long S)
-{
-    long long num = (bx - ax) * (y0 - ay), den = by - ay;
-    if (den < 0) {
-        num = -num;
-        den = -den;
+    __device__ __forceinline__ void at(long long Y, long long &fl, long long &ce) const
+    {
+        const long long num = dx * (Y - ay);
+        long long q = __float2ll_rn(__ll2float_rn(num) * inv);
+        long long r = num - q * den;
+        const int q1 = __float2int_rn(__ll2float_rn(r) * inv);
+        q += q1;
+        r -= (long long)q1 * den;
+        if (r < 0) {
+            --q;
+            r += den;
+        } else if (r >= den) {
+            ++q;
+            r -= den;
+        }
+        fl = ax + q;
+        ce = fl + (r > 0 ? 1 : 0);
     }
-    return fdiv(ax + cdiv(num, den) - 1, S);
-}
+};
 
 // the polygon owning vertex (and edge) i: the largest q with off[q] <= i
 __device__ __forceinline__ uint32_t owner(const uint64_t *off, uint32_t P, uint64_t i)
@@ -181,42 +183,45 @@ __global__ void __launch_bounds__(kT) k_ib_mark(const int2 *v, const uint64_t *o
         if (ay == by) {
             // a horizontal edge meets the open squares of its row unless it lies on a row border
             const long long lo = min(ax, bx), hi = max(ax, bx);
-            if (ay % Sc != 0)
-                mark_c(ay >> sc, fdiv(lo, Sc), cdiv(hi, Sc) - 1);
-            if (ay % Sf != 0)
-                mark_f(ay >> sf, fdiv(lo, Sf), cdiv(hi, Sf) - 1);
+            if (ay & (Sc - 1))
+                mark_c(ay >> sc, fshr(lo, sc), cshr(hi, sc) - 1);
+            if (ay & (Sf - 1))
+                mark_f(ay >> sf, fshr(lo, sf), cshr(hi, sf) - 1);
             continue; // never straddles a corner row, in no row list
         }
+        const EdgeLine line(pa, pb);
         const long long lo_y = min(ay, by), hi_y = max(ay, by);
-        for (long long row = max(lo_y >> sc, (long long)b.cy0), r1 = min(cdiv(hi_y, Sc) - 1, (long long)b.cy1);
-             row <= r1; ++row) {
+        // The rows of the edge, bottom up, x at each row border taken once.  A row
+        // that starts on the edge (lo_y <= y0 = row S < hi_y) has its corner row
+        // there: the corners (x0, y0) left of the crossing x* are those with x0 <=
+        // ceil(x*) - 1, and the largest such cell column takes the toggle.
+        {
+            const long long r0 = max(lo_y >> sc, (long long)b.cy0), r1 = min(cshr(hi_y, sc) - 1, (long long)b.cy1);
             long long fa, ca, fb, cb;
-            line_x(ax, ay, bx, by, max(lo_y, row * Sc), fa, ca);
-            line_x(ax, ay, bx, by, min(hi_y, (row + 1) * Sc), fb, cb);
-            mark_c(row, fdiv(min(fa, fb), Sc), cdiv(max(ca, cb), Sc) - 1);
+            if (r0 <= r1)
+                line.at(max(lo_y, r0 * Sc), fa, ca);
+            for (long long row = r0; row <= r1; ++row, fa = fb, ca = cb) {
+                line.at(min(hi_y, (row + 1) * Sc), fb, cb);
+                mark_c(row, fshr(min(fa, fb), sc), cshr(max(ca, cb), sc) - 1);
+                const long long kx = fshr(ca - 1, sc);
+                if (row * Sc >= lo_y && kx >= b.cx0)
+                    atomicXor(cflip + cbase + (row - b.cy0) * wc + (min(kx, (long long)b.cx1) - b.cx0), 1u);
+            }
         }
-        // coarse corner rows y0 = cy Sc with lo_y <= y0 < hi_y
-        for (long long cy = max(cdiv(lo_y, Sc), (long long)b.cy0), c1 = min(cdiv(hi_y, Sc) - 1, (long long)b.cy1);
-             cy <= c1; ++cy) {
-            const long long kx = corner_col(ax, ay, bx, by, cy * Sc, Sc);
-            if (kx >= b.cx0)
-                atomicXor(cflip + cbase + (cy - b.cy0) * wc + (min(kx, (long long)b.cx1) - b.cx0), 1u);
-        }
-        for (long long fr = max(lo_y >> sf, (long long)b.fy0), r1 = min(cdiv(hi_y, Sf) - 1, (long long)b.fy1);
-             fr <= r1; ++fr) {
-            atomicAdd(rcnt + froff[q] + (fr - b.fy0), 1u);
+        {
+            const long long r0 = max(lo_y >> sf, (long long)b.fy0), r1 = min(cshr(hi_y, sf) - 1, (long long)b.fy1);
             long long fa, ca, fb, cb;
-            line_x(ax, ay, bx, by, max(lo_y, fr * Sf), fa, ca);
-            line_x(ax, ay, bx, by, min(hi_y, (fr + 1) * Sf), fb, cb);
-            mark_f(fr, fdiv(min(fa, fb), Sf), cdiv(max(ca, cb), Sf) - 1);
-        }
-        // fine corner rows
-        for (long long fy = max(cdiv(lo_y, Sf), (long long)b.fy0), f1 = min(cdiv(hi_y, Sf) - 1, (long long)b.fy1);
-             fy <= f1; ++fy) {
-            const long long kf = corner_col(ax, ay, bx, by, fy * Sf, Sf);
-            if (kf >= b.fx0) {
-                const long long col = min(kf, (long long)b.fx1) - b.fx0;
-                atomicXor(fflip + fwoff[q] + (fy - b.fy0) * wwords + (col >> 5), 1u << (col & 31));
+            if (r0 <= r1)
+                line.at(max(lo_y, r0 * Sf), fa, ca);
+            for (long long fr = r0; fr <= r1; ++fr, fa = fb, ca = cb) {
+                atomicAdd(rcnt + froff[q] + (fr - b.fy0), 1u);
+                line.at(min(hi_y, (fr + 1) * Sf), fb, cb);
+                mark_f(fr, fshr(min(fa, fb), sf), cshr(max(ca, cb), sf) - 1);
+                const long long kf = fshr(ca - 1, sf);
+                if (fr * Sf >= lo_y && kf >= b.fx0) {
+                    const long long col = min(kf, (long long)b.fx1) - b.fx0;
+                    atomicXor(fflip + fwoff[q] + (fr - b.fy0) * wwords + (col >> 5), 1u << (col & 31));
+                }
             }
         }
     }
@@ -367,7 +372,6 @@ __global__ void __launch_bounds__(kT) k_ib_lists(const int2 *v, const uint64_t *
                                                  uint32_t *rcur, unsigned long long *keys)
 {
     const int sf = kBoxLog2 - g - sb;
-    const long long Sf = 1ll << sf;
     for (uint64_t i = blockIdx.x * (uint64_t)kT + threadIdx.x; i < V; i += (uint64_t)gridDim.x * kT) {
         const uint32_t q = owner(off, P, i);
         const PBox b = box[q];
@@ -380,7 +384,7 @@ __global__ void __launch_bounds__(kT) k_ib_lists(const int2 *v, const uint64_t *
         const long long lo_y = min(pa.y, pb.y), hi_y = max(pa.y, pb.y);
         const unsigned long long key =
             ((unsigned long long)(0x7FFFFFFF - max(pa.x, pb.x)) << 32) | (unsigned long long)(i - off[q]);
-        for (long long fr = max(lo_y >> sf, (long long)b.fy0), r1 = min(cdiv(hi_y, Sf) - 1, (long long)b.fy1);
+        for (long long fr = max(lo_y >> sf, (long long)b.fy0), r1 = min(cshr(hi_y, sf) - 1, (long long)b.fy1);
              fr <= r1; ++fr) {
             const uint64_t ri = froff[q] + (fr - b.fy0);
             if (rlen[ri])
