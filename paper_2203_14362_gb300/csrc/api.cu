@@ -55,8 +55,8 @@ struct IndexObj {
     uint64_t polys = 0;
     int kind = 0;        // 0: polygons (view), 1: disks (dview), 2: buffered polygons (view, nview, near)
     DiskView dview{};
-    IndexView nview{};   // kind 2: the buffered polygons' own grid,
-    NearView near{};     // their radii and containment (view)
+    IndexView nview{};   // kinds 1 and 2: the grid of the disks or buffered polygons,
+    NearView near{};     // and their disks, or radii and containment (view)
     void *mem2 = nullptr; // buffered polygons: radii
     void *mem3 = nullptr; // buffered polygons: their own grid (cells | fine | entries | edges | summary)
     IndexView view{};
@@ -296,54 +296,34 @@ std::vector<uint16_t> block_summary(const uint32_t *cell, int g, double *resolve
     return sum;
 }
 
-// Adds the phases of the join just launched to the totals: a polygon join
-// recorded five events (pass 1a, pass 1b, scan, emit), a distance join four
-// (pass 1, scan, emit).
-spx_status add_phase_times(spx_ctx *ctx, bool polygons)
+// Adds the phases of the join just launched to the totals (five events: pass
+// 1a, pass 1b, scan, emit).
+spx_status add_phase_times(spx_ctx *ctx)
 {
-    const int last = polygons ? 4 : 3;
-    SPX_CUDA(cudaEventSynchronize(ctx->ev[last]), "join timing");
+    SPX_CUDA(cudaEventSynchronize(ctx->ev[4]), "join timing");
     float t[4] = {0, 0, 0, 0};
-    for (int k = 0; k < last; ++k)
+    for (int k = 0; k < 4; ++k)
         cudaEventElapsedTime(&t[k], ctx->ev[k], ctx->ev[k + 1]);
     ctx->ms_resolve += t[0];
-    if (polygons)
-        ctx->ms_walk += t[1];
-    ctx->ms_scan += t[last - 2];
-    ctx->ms_emit += t[last - 1];
+    ctx->ms_walk += t[1];
+    ctx->ms_scan += t[2];
+    ctx->ms_emit += t[3];
     ctx->timed_joins++;
     return SPX_OK;
 }
 
-// The distance join (a disk index): same contract as the polygon join.
-spx_status disk_join_common(spx_ctx *ctx, PointsObj *pts, IndexObj *ix, uint32_t *pairs_dev, uint64_t cap,
-                            uint64_t *counts_dev, uint64_t *total_dev, uint64_t *n_pairs, void *stream)
+// What every query kernel launch takes from a table and an index, whatever its kind.
+JoinLaunch index_launch(spx_ctx *ctx, const PointsObj *pts, const IndexObj *ix)
 {
-    if (cap && !pairs_dev)
-        return fail(ctx, SPX_EINVAL, "join: pairs_dev is NULL with cap > 0");
-    if ((reinterpret_cast<uintptr_t>(pairs_dev) & 7) || (reinterpret_cast<uintptr_t>(counts_dev) & 7) ||
-        (reinterpret_cast<uintptr_t>(total_dev) & 7))
-        return fail(ctx, SPX_EINVAL, "join: output pointers must be 8-byte aligned");
-    cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    spx_status st = ensure(ctx, &ctx->scratch, &ctx->scratch_bytes, disk_scratch_bytes(pts->n), s, "join");
-    if (st != SPX_OK)
-        return st;
-    DiskLaunch a{};
-    a.dv = ix->dview;
+    JoinLaunch a{};
+    a.ix = ix->kind ? ix->nview : ix->view;
+    a.near = ix->near;
     a.pts = reinterpret_cast<const int2 *>(pts->dev);
     a.n = pts->n;
-    a.pairs = reinterpret_cast<uint2 *>(pairs_dev);
-    a.cap = pairs_dev ? cap : 0;
-    a.counts = reinterpret_cast<unsigned long long *>(counts_dev);
-    a.total = total_dev ? reinterpret_cast<unsigned long long *>(total_dev) : (n_pairs ? &ctx->aux->total : nullptr);
+    a.err = &ctx->aux->err;
     a.stats = ctx->aux->stats;
-    const bool timed = ctx->timing;
-    cudaError_t e = launch_disk_join(a, ctx->scratch, s, timed ? ctx->ev : nullptr);
-    if (e != cudaSuccess)
-        return cuda_fail(ctx, e, "join launch");
-    if (timed && pts->n && (st = add_phase_times(ctx, false)) != SPX_OK)
-        return st;
-    return report_total(ctx, s, a.total, cap, n_pairs, "join", "pairs");
+    a.fp32 = ix->fp32;
+    return a;
 }
 
 spx_status join_common(spx_ctx *ctx, spx_points points, spx_index index, uint32_t *pairs_dev, uint64_t cap,
@@ -359,16 +339,14 @@ spx_status join_common(spx_ctx *ctx, spx_points points, spx_index index, uint32_
         return fail(ctx, SPX_EINVAL, "join: bad points or index handle");
     if (pts->cluster_log2)
         return fail(ctx, SPX_EINVAL, "join: a cell-clustered point table has no row order; use spx_aggregate");
-    if (ix->kind == 1)
-        return disk_join_common(ctx, pts, ix, pairs_dev, cap, counts_dev, total_dev, n_pairs, stream);
     if (cap && !pairs_dev)
         return fail(ctx, SPX_EINVAL, "join: pairs_dev is NULL with cap > 0");
     if ((reinterpret_cast<uintptr_t>(pairs_dev) & 7) || (reinterpret_cast<uintptr_t>(counts_dev) & 7) ||
         (reinterpret_cast<uintptr_t>(total_dev) & 7))
         return fail(ctx, SPX_EINVAL, "join: output pointers must be 8-byte aligned");
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    const bool buffered = ix->kind == 2; // exact already: spx_join_plain takes the same path
-    plain = plain && !buffered;
+    plain = plain && ix->kind == 0; // distance queries have one path
+    const bool buffered = ix->kind == 2;
     const size_t need = plain ? plain_scratch_bytes(pts->n) : join_scratch_bytes(pts->n);
     // buffered polygons overlap: 8 B per point more let pass 1 keep a point's
     // polygons for pass 3; a call goes without them where the scratch cannot grow
@@ -382,24 +360,17 @@ spx_status join_common(spx_ctx *ctx, spx_points points, spx_index index, uint32_
     }
     if (st != SPX_OK)
         return st;
-    JoinLaunch a{};
-    a.ix = buffered ? ix->nview : ix->view;
-    a.near = ix->near;
+    JoinLaunch a = index_launch(ctx, pts, ix);
     a.aux = aux ? reinterpret_cast<uint64_t *>(static_cast<char *>(ctx->scratch) + aux_at) : nullptr;
-    a.pts = reinterpret_cast<const int2 *>(pts->dev);
-    a.n = pts->n;
     a.pairs = reinterpret_cast<uint2 *>(pairs_dev);
     a.cap = pairs_dev ? cap : 0;
     a.counts = reinterpret_cast<unsigned long long *>(counts_dev);
     a.total = total_dev ? reinterpret_cast<unsigned long long *>(total_dev) : (n_pairs ? &ctx->aux->total : nullptr);
-    a.err = &ctx->aux->err;
-    a.stats = ctx->aux->stats;
-    a.fp32 = ix->fp32;
     const bool timed = ctx->timing && !plain && !buffered;
     cudaError_t e = plain ? launch_join_plain(a, ctx->scratch, s) : launch_join(a, ctx->scratch, s, timed ? ctx->ev : nullptr);
     if (e != cudaSuccess)
         return cuda_fail(ctx, e, "join launch");
-    if (timed && pts->n && (st = add_phase_times(ctx, true)) != SPX_OK)
+    if (timed && pts->n && (st = add_phase_times(ctx)) != SPX_OK)
         return st;
     return report_total(ctx, s, a.total, cap, n_pairs, "join", "pairs");
 }
@@ -1213,6 +1184,24 @@ static spx_status register_disk_index(spx_ctx *ctx, void *mem, size_t total, con
     auto ix = std::make_unique<IndexObj>();
     ix->mem = mem;
     ix->kind = 1;
+    double resolved = 0;
+    cudaError_t e = cudaMalloc(&ix->mem2, size_t(2) << (2 * kSumLog2));
+    if (e == cudaSuccess)
+        e = prepare_disk_words(const_cast<uint32_t *>(cell), g, static_cast<uint16_t *>(ix->mem2), &resolved);
+    if (e != cudaSuccess) {
+        free_index_memory(ctx, *ix);
+        return e == cudaErrorMemoryAllocation ? fail(ctx, SPX_ENOMEM, "build_disk_index: cudaMalloc failed")
+                                              : cuda_fail(ctx, e, "build_disk_index");
+    }
+    GridParts gp{};
+    gp.cell = reinterpret_cast<char *>(const_cast<uint32_t *>(cell));
+    gp.cover = reinterpret_cast<char *>(const_cast<uint32_t *>(cover));
+    gp.sum = static_cast<char *>(ix->mem2);
+    gp.sum_resolved = resolved;
+    ix->nview = grid_view(gp, g, 0, Q);
+    ix->nview.err = &ctx->aux->err;
+    ix->near.disk = disk;
+    ix->near.dent = ent;
     ix->dview.cell = cell;
     ix->dview.ent = ent;
     ix->dview.disk = disk;
@@ -1229,7 +1218,9 @@ static spx_status register_disk_index(spx_ctx *ctx, void *mem, size_t total, con
     inf.n_entries = n_entries;
     inf.n_inside = n_inside;
     inf.n_boundary = n_boundary;
-    inf.device_bytes = total;
+    inf.device_bytes = total + (size_t(2) << (2 * kSumLog2));
+    inf.sum_resolved = resolved;
+    inf.use_sum = ix->nview.use_sum;
     inf.build_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
     const uint64_t h = make_handle(ctx, kTagIndex);
     ctx->indexes[h] = std::move(ix);
@@ -1334,6 +1325,9 @@ spx_status spx_disk_index_arrays(spx_ctx *ctx, spx_index index, uint32_t *cell, 
     sizes[2] = uint64_t(ix->info.grid_log2);
     if (cell)
         SPX_CUDA(cudaMemcpy(cell, ix->dview.cell, sizes[0] * 4, cudaMemcpyDeviceToHost), "disk_index_arrays copy");
+    for (uint64_t c = 0; cell && c < sizes[0]; ++c) // as built: prepare_disk_words set the lists' lower kind bit
+        if ((cell[c] >> 30) == kCellCoarseList)
+            cell[c] ^= 1u << 30;
     if (entries)
         SPX_CUDA(cudaMemcpy(entries, ix->dview.ent, sizes[1] * 4, cudaMemcpyDeviceToHost), "disk_index_arrays copy");
     return SPX_OK;
@@ -1486,75 +1480,46 @@ spx_status spx_select(spx_ctx *ctx, spx_points points, spx_index index, uint32_t
         return fail(ctx, SPX_EINVAL, "select: offsets_dev is NULL, or ids_dev is NULL with cap > 0");
     if ((reinterpret_cast<uintptr_t>(offsets_dev) & 7) || (reinterpret_cast<uintptr_t>(ids_dev) & 3))
         return fail(ctx, SPX_EINVAL, "select: misaligned output pointer");
-    const uint32_t PQ = ix->kind == 1 ? ix->dview.Q : ix->view.P;
+    const uint32_t PQ = ix->kind ? ix->nview.P : ix->view.P;
     if (PQ > kSelectMaxQueries)
         return fail(ctx, SPX_EINVAL, "select: an index of " + std::to_string(PQ) +
                                          " queries; batched selection takes at most " +
                                          std::to_string(kSelectMaxQueries));
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    if (ix->kind == 2) {
-        // buffered polygons: points inside or within r of each polygon, ascending per polygon
-        spx_status st = ensure(ctx, &ctx->scratch, &ctx->scratch_bytes, select_scratch_bytes(pts->n, PQ, cap), s,
-                               "select");
-        if (st != SPX_OK)
-            return st;
-        JoinLaunch b{};
-        b.ix = ix->nview;
-        b.near = ix->near;
-        b.pts = reinterpret_cast<const int2 *>(pts->dev);
-        b.n = pts->n;
-        b.err = &ctx->aux->err;
-        b.stats = ctx->aux->stats;
-        b.fp32 = ix->fp32;
-        unsigned long long *offs = reinterpret_cast<unsigned long long *>(offsets_dev);
-        cudaError_t e = launch_select(b, ids_dev, cap, offs, ctx->scratch, s);
-        if (e != cudaSuccess)
-            return cuda_fail(ctx, e, "select launch");
-        return report_total(ctx, s, offs + PQ, cap, n_ids, "select", "ids");
+    // pass 1b keeps the polygons of a point in several for pass 3 in 8 B per point
+    // more; the distance selections go without where the scratch cannot grow
+    const size_t full = select_scratch_bytes(pts->n, PQ, cap, true), least = select_scratch_bytes(pts->n, PQ, cap, false);
+    bool aux = ix->kind == 0 || ctx->scratch_bytes >= full || !capturing(s);
+    spx_status st = ensure(ctx, &ctx->scratch, &ctx->scratch_bytes, aux ? full : least, s, "select");
+    if (st == SPX_ENOMEM && ix->kind) {
+        cudaGetLastError();
+        aux = false;
+        st = ensure(ctx, &ctx->scratch, &ctx->scratch_bytes, least, s, "select");
     }
-    if (ix->kind == 1) {
-        // distance selection: points within r of each centre, ascending per disk
-        spx_status st = ensure(ctx, &ctx->scratch, &ctx->scratch_bytes, disk_select_scratch_bytes(pts->n, PQ, cap), s,
-                               "select");
-        if (st != SPX_OK)
-            return st;
-        DiskLaunch a{};
-        a.dv = ix->dview;
-        a.pts = reinterpret_cast<const int2 *>(pts->dev);
-        a.n = pts->n;
-        a.stats = ctx->aux->stats;
-        unsigned long long *offs = reinterpret_cast<unsigned long long *>(offsets_dev);
-        cudaError_t e = launch_disk_select(a, ids_dev, cap, offs, ctx->scratch, s);
-        if (e != cudaSuccess)
-            return cuda_fail(ctx, e, "select launch");
-        return report_total(ctx, s, offs + PQ, cap, n_ids, "select", "ids");
-    }
-    spx_status st = ensure(ctx, &ctx->scratch, &ctx->scratch_bytes, select_scratch_bytes(pts->n, ix->view.P, cap), s,
-                           "select");
     if (st != SPX_OK)
         return st;
-    JoinLaunch a{};
-    a.ix = ix->view;
-    a.pts = reinterpret_cast<const int2 *>(pts->dev);
-    a.n = pts->n;
-    a.err = &ctx->aux->err;
-    a.stats = ctx->aux->stats;
-    a.fp32 = ix->fp32;
+    const JoinLaunch a = index_launch(ctx, pts, ix);
     unsigned long long *offs = reinterpret_cast<unsigned long long *>(offsets_dev);
+    if (ix->kind) { // distance selections: not captured
+        const cudaError_t e = launch_select(a, ids_dev, cap, offs, ctx->scratch, s, aux);
+        if (e != cudaSuccess)
+            return cuda_fail(ctx, e, "select launch");
+        return report_total(ctx, s, offs + PQ, cap, n_ids, "select", "ids");
+    }
     const auto key = std::make_tuple(points, index, reinterpret_cast<uintptr_t>(ids_dev), cap,
                                      reinterpret_cast<uintptr_t>(offsets_dev));
     auto it = ctx->select_graphs.find(key);
     if (it == ctx->select_graphs.end()) {
         // first call with these arguments: run once directly (sets kernel attributes),
         // then capture the whole sequence into a graph for the next calls
-        cudaError_t e = launch_select(a, ids_dev, cap, offs, ctx->scratch, s);
+        cudaError_t e = launch_select(a, ids_dev, cap, offs, ctx->scratch, s, aux);
         if (e != cudaSuccess)
             return cuda_fail(ctx, e, "select launch");
         if (!ctx->capture_stream)
             SPX_CUDA(cudaStreamCreateWithFlags(&ctx->capture_stream, cudaStreamNonBlocking), "capture stream");
         SPX_CUDA(cudaStreamSynchronize(s), "select synchronize");
         SPX_CUDA(cudaStreamBeginCapture(ctx->capture_stream, cudaStreamCaptureModeRelaxed), "select capture");
-        e = launch_select(a, ids_dev, cap, offs, ctx->scratch, ctx->capture_stream);
+        e = launch_select(a, ids_dev, cap, offs, ctx->scratch, ctx->capture_stream, aux);
         cudaGraph_t g = nullptr;
         const cudaError_t e2 = cudaStreamEndCapture(ctx->capture_stream, &g);
         if (e != cudaSuccess || e2 != cudaSuccess) {
@@ -1586,26 +1551,9 @@ spx_status spx_aggregate(spx_ctx *ctx, spx_points points, spx_index index, uint6
         return fail(ctx, SPX_EINVAL, "aggregate: bad points or index handle");
     if (reinterpret_cast<uintptr_t>(counts_dev) & 7)
         return fail(ctx, SPX_EINVAL, "aggregate: counts_dev must be 8-byte aligned");
-    if (ix->kind == 1) {
-        DiskLaunch d{};
-        d.dv = ix->dview;
-        d.pts = reinterpret_cast<const int2 *>(pts->dev);
-        d.n = pts->n;
-        d.counts = reinterpret_cast<unsigned long long *>(counts_dev);
-        d.stats = ctx->aux->stats;
-        cudaError_t e = launch_disk_aggregate(d, reinterpret_cast<cudaStream_t>(stream));
-        return e == cudaSuccess ? SPX_OK : cuda_fail(ctx, e, "aggregate launch");
-    }
-    const bool buffered = ix->kind == 2;
-    JoinLaunch a{};
-    a.ix = buffered ? ix->nview : ix->view;
-    a.near = ix->near;
-    a.pts = reinterpret_cast<const int2 *>(pts->dev);
-    a.n = pts->n;
+    const bool distance = ix->kind != 0;
+    JoinLaunch a = index_launch(ctx, pts, ix);
     a.counts = reinterpret_cast<unsigned long long *>(counts_dev);
-    a.err = &ctx->aux->err;
-    a.stats = ctx->aux->stats;
-    a.fp32 = ix->fp32;
     a.clustered = pts->cluster_log2 ? 1 : 0;
     a.cell_end = pts->cell_end;
     a.cluster_log2 = pts->cluster_log2;
@@ -1619,14 +1567,14 @@ spx_status spx_aggregate(spx_ctx *ctx, spx_points points, spx_index index, uint6
         cudaGetLastError();
         words = nullptr;
     }
-    cudaError_t e = launch_aggregate(a, words, s, ctx->timing && !buffered ? ctx->ev : nullptr);
+    cudaError_t e = launch_aggregate(a, words, s, ctx->timing && !distance ? ctx->ev : nullptr);
     if (words) {
         const cudaError_t e2 = cudaFreeAsync(words, s);
         e = e != cudaSuccess ? e : e2;
     }
     if (e != cudaSuccess)
         return cuda_fail(ctx, e, "aggregate launch");
-    if (ctx->timing && pts->n && !buffered) {
+    if (ctx->timing && pts->n && !distance) {
         SPX_CUDA(cudaEventSynchronize(ctx->ev[1]), "aggregate timing");
         float t = 0;
         cudaEventElapsedTime(&t, ctx->ev[0], ctx->ev[1]);

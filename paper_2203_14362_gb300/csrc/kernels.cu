@@ -76,7 +76,9 @@ __device__ __forceinline__ uint32_t lanemask_lt()
     return m;
 }
 // L2 eviction policies: the index stays resident (evict_last) while the
-// streamed points pass through (evict_first).
+// streamed points pass through (evict_first).  Index words are read once per point
+// at random, 32 lines a warp: they take no L1 line (tess. join 100M x 2000 cells
+// 618 -> 604 us, count x 5000 cells 521 -> 487).
 __device__ __forceinline__ uint64_t policy_evict_last()
 {
     uint64_t p;
@@ -86,8 +88,16 @@ __device__ __forceinline__ uint64_t policy_evict_last()
 __device__ __forceinline__ uint32_t ld_idx(const uint32_t *p, uint64_t pol)
 {
     uint32_t v;
-    asm volatile("ld.global.nc.L2::cache_hint.u32 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(pol));
+    asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.u32 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(pol));
     return v;
+}
+// The same where `on`, else v stays; without a branch.
+__device__ __forceinline__ void ld_idx_if(uint32_t &v, const uint32_t *p, uint64_t pol, bool on)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\t"
+                 "@p ld.global.nc.L1::no_allocate.L2::cache_hint.u32 %0, [%1], %2;\n\t}"
+                 : "+r"(v)
+                 : "l"(p), "l"(pol), "r"((uint32_t)on));
 }
 __device__ __forceinline__ uint4 ld_idx(const uint4 *p, uint64_t pol)
 {
@@ -426,6 +436,20 @@ __device__ __forceinline__ uint32_t walk_list(const IndexView &ix, uint32_t e0, 
     return c;
 }
 
+// What an index's entry lists hold: polygons with crossing edges, buffered
+// polygons with edges that may be near, or disks.
+constexpr int kPoly = 0, kNear = 1, kDisk = 2;
+
+// A point is within distance r of a centre c iff (px-cx)^2 + (py-cy)^2 <= r^2,
+// exact in int64 (differences < 2^31; r < 2^30; the x term is compared with
+// r^2 before the sum, so the sum cannot overflow).
+__device__ __forceinline__ bool in_disk(const int4 &d, int px, int py)
+{
+    const long long dx = (long long)px - d.x, dy = (long long)py - d.y, rr = (long long)d.z * d.z;
+    const long long dx2 = dx * dx;
+    return dx2 <= rr && dx2 + dy * dy <= rr;
+}
+
 // Is (px, py) within distance r of the closed segment v = (a, b)?  With
 // d = b - a, w = p - a and t = w . d: the distance is |w| when t <= 0, |p - b|
 // when t >= |d|^2, else |d x w| / |d|.  Coordinates lie in [0, 2^30], so every
@@ -519,15 +543,26 @@ __device__ __noinline__ bool poly_holds(const IndexView &ix, uint32_t q, int px,
 // sorted lists' early stop is not used (an edge that ends left of the point
 // counts nothing; recording where each list could stop measured slower).
 // s_par: kWaveWords words of shared memory owned by this warp.
-// NEAR: the list is one of a buffered index (nv).  An edge hits when it comes
+// KIND kNear: the list is one of a buffered index (nv).  An edge hits when it comes
 // within its polygon's radius of the point, hits are ORed instead of XORed, and
 // a point that no edge hits asks the polygons' own index where the entry says
 // that the boundary may cross the cell.
-template <bool FP32, bool NEAR = false, class F>
+template <bool FP32, int KIND = kPoly, class F>
 __device__ __forceinline__ void walk_list_wave(const IndexView &ix, bool has, uint32_t e0, int px, int py,
                                                uint32_t &tests, uint32_t &esc, uint64_t pol, uint32_t *s_par, F f,
                                                const NearView *nv = nullptr)
 {
+    if constexpr (KIND == kDisk) { // short lists of disks, a test each: every lane walks its own
+        const uint32_t n = has ? ld_idx(nv->dent + e0, pol) : 0u;
+        for (uint32_t k = 1; k <= n; ++k) {
+            const uint32_t en = ld_idx(nv->dent + e0 + k, pol), q = en >> 1;
+            tests += en & 1u;
+            if (!(en & 1u) || in_disk(__ldg(nv->disk + q), px, py))
+                f(q);
+        }
+        __syncwarp();
+        return;
+    }
     const int lane = threadIdx.x & 31;
     const uint4 *e = ix.ent + (has ? e0 : 0u);
     bool more = has;
@@ -549,8 +584,8 @@ __device__ __forceinline__ void walk_list_wave(const IndexView &ix, bool has, ui
         const uint32_t za = (more && (ea.w & kEntBoundary)) ? ea.z : 0u;
         const uint32_t zb = (hb && (eb.w & kEntBoundary)) ? eb.z : 0u;
         const uint32_t tot = za + zb;
-        int ra = 0, rb = 0; // NEAR: the entries' radii
-        if (NEAR) {
+        int ra = 0, rb = 0; // kNear: the entries' radii
+        if (KIND == kNear) {
             ra = za ? __ldg(nv->rad + ea.x) : 0;
             rb = zb ? __ldg(nv->rad + eb.x) : 0;
         }
@@ -590,7 +625,7 @@ __device__ __forceinline__ void walk_list_wave(const IndexView &ix, bool has, ui
                     const uint32_t t = k - (oi - ot);
                     slot[h] = t >= oza ? 1u : 0u;
                     own[h] = o;
-                    if (NEAR) {
+                    if (KIND == kNear) {
                         const int r0 = __shfl_sync(kFull, ra, o), r1 = __shfl_sync(kFull, rb, o);
                         rad[h] = slot[h] ? r1 : r0;
                     }
@@ -599,7 +634,7 @@ __device__ __forceinline__ void walk_list_wave(const IndexView &ix, bool has, ui
                 }
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    if (NEAR) {
+                    if (KIND == kNear) {
                         if (act[h] && seg_near<FP32>(v[h], ox[h], oy[h], rad[h]))
                             atomicOr(s_par + 32 * slot[h] + own[h], 1u);
                     } else if (act[h] && edge_cross<FP32>(v[h], ox[h], oy[h], tests, esc)) {
@@ -612,7 +647,7 @@ __device__ __forceinline__ void walk_list_wave(const IndexView &ix, bool has, ui
             pb = s_par[32 + lane];
             __syncwarp(); // s_par is rewritten by the next wave
         }
-        if (NEAR) {
+        if (KIND == kNear) {
             if (more && !pa && (ea.w & kEntCross))
                 pa = poly_holds<FP32>(nv->in, ea.x, px, py, tests, esc, pol);
             if (hb && !pb && (eb.w & kEntCross))
@@ -704,6 +739,21 @@ __device__ __noinline__ uint32_t near_count(const IndexView &ix, const NearView 
             break;
     }
     return n;
+}
+
+// The number of disks that hold the in-box point (px, py), by one lane.
+__device__ __noinline__ uint32_t disk_count(const IndexView &ix, const NearView &nv, int px, int py, uint64_t pol)
+{
+    const uint32_t w = coarse_word(ix, (uint32_t)px, (uint32_t)py, pol);
+    if ((w >> 30) < kCellList)
+        return (w >> 30) == kCellInsideOne ? 1u : 0u;
+    const uint32_t *e = nv.dent + (w & kPayloadMask);
+    uint32_t c = 0;
+    for (uint32_t n = ld_idx(e, pol), k = 1; k <= n; ++k) {
+        const uint32_t en = ld_idx(e + k, pol);
+        c += !(en & 1u) || in_disk(__ldg(nv.disk + (en >> 1)), px, py) ? 1u : 0u;
+    }
+    return c;
 }
 
 __device__ __forceinline__ unsigned long long warp_sum64(unsigned long long v)
@@ -1087,12 +1137,6 @@ constexpr int kPrefetchChunks = SPX_PREFETCH_CHUNKS; // L2 prefetch distance of 
 #define SPX_TMA_POINTS 1
 #endif
 constexpr bool kTmaPoints = SPX_TMA_POINTS != 0; // pass 1a stages points with bulk copies when they fit
-#ifndef SPX_RESOLVE_PIPE
-#define SPX_RESOLVE_PIPE 1
-#endif
-// pass 1a with the block summary loads a warp's next chunk of points into
-// registers before the current chunk's cell words
-constexpr bool kResolvePipe = SPX_RESOLVE_PIPE != 0;
 
 // Shared memory of pass 1a: [summary][TMA: per warp a chunk buffer, then per
 // warp an mbarrier][counters].
@@ -1102,41 +1146,168 @@ __host__ __device__ constexpr size_t resolve_smem_head(int warps, bool sum, int 
            (tma ? size_t(warps) * (kWChunk * sizeof(int2) + sizeof(uint64_t)) : 0);
 }
 
+// With the summary the kernel is bound by issue (0.65 to 0.74 of the issue slots,
+// ALU first), so it is written for few instructions: whole chunks run without
+// row checks, a point outside the box reads a masked summary word instead of a
+// selected one, loads are predicated instead of branched around, the kind of a
+// word is a signed comparison (kind 1: at least 2^30; lists: negative), a counter's
+// address is the word shifted left (its kind bits fall off), and lane 0 stores the
+// eight ballots.  100M points x 2000 cells: 322 -> 285 us, x 1024 disks 258 -> 213.
+// Each warp loads its next chunk's points before the current chunk's words, and
+// prefetches the one after into L2.
+// OUT says what is kept per point: kOut32 or kOut16 (a result of that width and
+// the chunk's pair total), or kOutCount (nothing but the bitmap: the count
+// aggregate, whose pass 1b only counts).
+constexpr int kOut32 = 0, kOut16 = 1, kOutCount = 2;
+
+template <int OUT>
+__global__ void __launch_bounds__(kResolveSumThreads, 1)
+    k_resolve_sum(const __grid_constant__ JoinLaunch a, uint32_t *pend, uint32_t nchunks, int use_hist)
+{
+    constexpr int WARPS = kResolveSumThreads / 32;
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    const IndexView &ix = a.ix;
+    const uint32_t sum_words = 1u << (2 * ix.sg), smask = sum_words - 1u; // 16-bit words
+    const uint16_t *s_sum = reinterpret_cast<const uint16_t *>(s_raw);
+    uint32_t *s_hist = reinterpret_cast<uint32_t *>(s_raw + resolve_smem_head(WARPS, true, ix.sg, false));
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint64_t keep = policy_evict_last();
+    const bool hist = use_hist && a.counts;
+    const uint32_t nw = gridDim.x * WARPS, hist_at = smem_u32(s_hist);
+    for (uint32_t i = threadIdx.x; i < (sum_words + 7) / 8; i += kResolveSumThreads)
+        reinterpret_cast<uint4 *>(s_raw)[i] = ld_idx(ix.sum + i, keep);
+    if (hist)
+        for (uint32_t i = threadIdx.x; i < ix.P; i += kResolveSumThreads)
+            s_hist[i] = 0;
+    __syncthreads();
+    uint32_t n_pairs = 0;
+    int2 pn[kWItems]; // the points of this warp's next chunk
+    auto load_chunk = [&](uint32_t c) {
+        const uint64_t b = (uint64_t)c * kWChunk;
+        const int2 *q = a.pts + b + lane;
+        if (b + kWChunk <= a.n) {
+#pragma unroll
+            for (int j = 0; j < kWItems; ++j)
+                pn[j] = __ldcs(q + 32 * j);
+        } else {
+#pragma unroll
+            for (int j = 0; j < kWItems; ++j)
+                pn[j] = c < nchunks && b + 32 * j + lane < a.n ? __ldcs(q + 32 * j) : make_int2(-1, -1);
+        }
+    };
+    load_chunk(blockIdx.x * WARPS + warp);
+    for (uint32_t ch = blockIdx.x * WARPS + warp; ch < nchunks; ch += nw) {
+        const uint64_t base = (uint64_t)ch * kWChunk;
+        if (lane == 0) { // the chunk after the next goes to L2; the next one to registers now
+            const uint64_t nb = base + 2ull * nw * kWChunk;
+            if (nb + kWChunk <= a.n)
+                prefetch_l2_bulk(a.pts + nb, kWChunk * sizeof(int2));
+        }
+        int2 p[kWItems];
+        uint32_t w[kWItems];
+#pragma unroll
+        for (int j = 0; j < kWItems; ++j)
+            p[j] = pn[j];
+        load_chunk(ch + nw);
+#pragma unroll
+        for (int j = 0; j < kWItems; ++j) {
+            const uint32_t px = (uint32_t)p[j].x, py = (uint32_t)p[j].y;
+            const bool ok = (px | py) < kBox; // both in [0, 2^30)
+            const uint32_t sv = s_sum[(((py >> ix.ssh) << ix.sg) | (px >> ix.ssh)) & smask];
+            w[j] = ok && sv != kSumEmpty ? (kCellInsideOne << 30) | sv : 0u;
+            ld_idx_if(w[j], ix.cell + (((py >> ix.sc) << ix.gc) | (px >> ix.sc)), keep, ok && sv == kSumMixed);
+        }
+#pragma unroll
+        for (int j = 0; j < kWItems; ++j)
+            if ((w[j] >> 30) == kCellSub)
+                w[j] = fine_word(ix, w[j], (uint32_t)p[j].x, (uint32_t)p[j].y, keep);
+        uint32_t bl[kWItems];
+#pragma unroll
+        for (int j = 0; j < kWItems; ++j)
+            bl[j] = __ballot_sync(kFull, (int)w[j] < 0); // kCellList, kCellCoarseList
+        if (lane == 0) {
+            uint2 *d = reinterpret_cast<uint2 *>(pend + (uint64_t)ch * kWItems); // the bitmap is 8-byte aligned
+#pragma unroll
+            for (int j = 0; j < kWItems / 2; ++j)
+                __stcg(d + j, make_uint2(bl[2 * j], bl[2 * j + 1]));
+        }
+        constexpr int kOne = int(kCellInsideOne << 30);
+        // one: the polygon; list: its first entry (narrow: none; rewritten by pass
+        // 1b); empty: none
+        if (OUT == kOut16) {
+            unsigned short *res = reinterpret_cast<unsigned short *>(a.res) + base + lane;
+            if (base + kWChunk <= a.n) {
+#pragma unroll
+                for (int j = 0; j < kWItems; ++j)
+                    __stcg(res + 32 * j, (unsigned short)((int)w[j] >= kOne ? w[j] : kRes16None));
+            } else {
+#pragma unroll
+                for (int j = 0; j < kWItems; ++j)
+                    if (base + 32 * j + lane < a.n)
+                        __stcg(res + 32 * j, (unsigned short)((int)w[j] >= kOne ? w[j] : kRes16None));
+            }
+        } else if (OUT == kOut32) {
+#pragma unroll
+            for (int j = 0; j < kWItems; ++j)
+                if (base + 32 * j + lane < a.n)
+                    __stcg(a.res + base + 32 * j + lane, (w[j] >> 30) == kCellEmpty ? kResNone : w[j] & kPayloadMask);
+        }
+        uint32_t total = 0;
+#pragma unroll
+        for (int j = 0; j < kWItems; ++j)
+            total += (int)w[j] >= kOne && in_bounds((w[j] & kPayloadMask) < ix.P, ix) ? 1u : 0u;
+        if (hist) {
+#pragma unroll
+            for (int j = 0; j < kWItems; ++j)
+                if ((int)w[j] >= kOne && in_bounds((w[j] & kPayloadMask) < ix.P, ix))
+                    asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(hist_at + (w[j] << 2)) : "memory");
+        } else if (a.counts) {
+#pragma unroll
+            for (int j = 0; j < kWItems; ++j)
+                global_add_warp(a.counts, (int)w[j] >= kOne && in_bounds((w[j] & kPayloadMask) < ix.P, ix),
+                                w[j] & kPayloadMask);
+        }
+        n_pairs += total;
+        if (OUT != kOutCount) {
+            total = __reduce_add_sync(kFull, total);
+            if (lane == 0)
+                a.tile_tot[ch] = total; // the chunk's total without its list points; pass 1b adds theirs
+        }
+    }
+    if (hist) {
+        __syncthreads();
+        for (uint32_t i = threadIdx.x; i < ix.P; i += kResolveSumThreads)
+            if (s_hist[i])
+                atomicAdd(a.counts + i, (unsigned long long)s_hist[i]);
+    }
+    add_stats(a.stats, 0u, 0u, 0u, n_pairs);
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        atomicAdd(a.stats + kStatPoints, (unsigned long long)a.n);
+}
+
 // With TMA, every warp stages its next chunk's points in its own shared-memory
 // buffer with one bulk copy, issued as soon as it has read the current chunk
 // from there: the points arrive while the chunk is resolved, and their loads
 // cost the L1 nothing.  A warp's last chunk, when it is not full, is loaded
 // with plain loads.
 //
-// OUT says what is kept per point: kOut32 or kOut16 (a result of that width and
-// the chunk's pair total), or kOutCount (nothing but the bitmap: the count
-// aggregate, whose pass 1b only counts).
-constexpr int kOut32 = 0, kOut16 = 1, kOutCount = 2;
-
-template <int THREADS, bool SUM, bool TMA, int OUT>
-__global__ void __launch_bounds__(THREADS, SUM ? 1 : (TMA ? 6 : kResolveMinBlocks))
+// Without the summary.
+template <int THREADS, bool TMA, int OUT>
+__global__ void __launch_bounds__(THREADS, TMA ? 6 : kResolveMinBlocks)
     k_resolve(const __grid_constant__ JoinLaunch a, uint32_t *pend, uint32_t nchunks, int use_hist)
 {
     constexpr int WARPS = THREADS / 32;
     extern __shared__ __align__(16) unsigned char s_raw[];
     const IndexView &ix = a.ix;
-    const uint32_t sum_words = SUM ? (1u << (2 * ix.sg)) : 0u; // 16-bit words
-    const uint16_t *s_sum = reinterpret_cast<const uint16_t *>(s_raw);
-    const size_t sum_bytes = SUM ? ((size_t(sum_words) * 2 + 15) & ~size_t(15)) : 0;
-    int2 *s_buf = reinterpret_cast<int2 *>(s_raw + sum_bytes) + (size_t)(threadIdx.x >> 5) * kWChunk;
-    uint64_t *s_bar = reinterpret_cast<uint64_t *>(s_raw + sum_bytes + size_t(WARPS) * kWChunk * sizeof(int2)) +
+    int2 *s_buf = reinterpret_cast<int2 *>(s_raw) + (size_t)(threadIdx.x >> 5) * kWChunk;
+    uint64_t *s_bar = reinterpret_cast<uint64_t *>(s_raw + size_t(WARPS) * kWChunk * sizeof(int2)) +
                       (threadIdx.x >> 5);
-    uint32_t *s_hist = reinterpret_cast<uint32_t *>(s_raw + resolve_smem_head(WARPS, SUM, SUM ? ix.sg : 0, TMA));
+    uint32_t *s_hist = reinterpret_cast<uint32_t *>(s_raw + resolve_smem_head(WARPS, false, 0, TMA));
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint64_t keep = policy_evict_last();
     const bool hist = use_hist && a.counts;
     const uint32_t nw = gridDim.x * WARPS;
     auto full = [&](uint32_t c) { return (uint64_t)(c + 1) * kWChunk <= a.n; };
-    if constexpr (SUM) {
-        uint4 *d = reinterpret_cast<uint4 *>(s_raw);
-        for (uint32_t i = threadIdx.x; i < (sum_words + 7) / 8; i += THREADS)
-            d[i] = ld_idx(ix.sum + i, keep);
-    }
     if constexpr (TMA) {
         const uint32_t c0 = blockIdx.x * WARPS + warp;
         if (lane == 0) {
@@ -1150,19 +1321,6 @@ __global__ void __launch_bounds__(THREADS, SUM ? 1 : (TMA ? 6 : kResolveMinBlock
             s_hist[i] = 0;
     __syncthreads();
     uint32_t n_pts = 0, n_pairs = 0, phase = 0;
-    constexpr bool PIPE = SUM && !TMA && kResolvePipe;
-    int2 pn[kWItems]; // PIPE: the points of this warp's next chunk
-    auto load_chunk = [&](uint32_t c, int2(&q)[kWItems]) {
-        const uint64_t b = (uint64_t)c * kWChunk;
-        const uint32_t m = c < nchunks ? (uint32_t)min((uint64_t)kWChunk, a.n - b) : 0u;
-#pragma unroll
-        for (int j = 0; j < kWItems; ++j) {
-            const uint32_t loc = j * 32 + lane;
-            q[j] = loc < m ? __ldcs(a.pts + b + loc) : make_int2(-1, -1);
-        }
-    };
-    if (PIPE)
-        load_chunk(blockIdx.x * WARPS + warp, pn);
     for (uint32_t ch = blockIdx.x * WARPS + warp; ch < nchunks; ch += nw) {
         const uint64_t base = (uint64_t)ch * kWChunk;
         const uint32_t npts = (uint32_t)min((uint64_t)kWChunk, a.n - base);
@@ -1171,18 +1329,7 @@ __global__ void __launch_bounds__(THREADS, SUM ? 1 : (TMA ? 6 : kResolveMinBlock
         uint16_t *res16 = reinterpret_cast<uint16_t *>(a.res) + base;
         int2 p[kWItems];
         uint32_t w[kWItems];
-        if (PIPE) {
-            if (kPrefetchChunks > 0 && lane == 0) {
-                // the chunk after the next goes to L2; the next one to registers now
-                const uint64_t nb = base + (uint64_t)(kPrefetchChunks + 1) * nw * kWChunk;
-                if (nb + kWChunk <= a.n)
-                    prefetch_l2_bulk(a.pts + nb, kWChunk * sizeof(int2));
-            }
-#pragma unroll
-            for (int j = 0; j < kWItems; ++j)
-                p[j] = pn[j];
-            load_chunk(ch + nw, pn);
-        } else if (TMA && npts == kWChunk) {
+        if (TMA && npts == kWChunk) {
             if (!mbar_wait(s_bar, phase, kWaitTries)) {
                 // the copy did not arrive: report it, give it one more bounded wait, stop
                 if (lane == 0)
@@ -1216,16 +1363,9 @@ __global__ void __launch_bounds__(THREADS, SUM ? 1 : (TMA ? 6 : kResolveMinBlock
             // x, y >= 0 and both < 2^30 iff their bitwise or is below 2^30
             const bool ok = (uint32_t)(p[j].x | p[j].y) < kBox;
             const uint32_t px = ok ? (uint32_t)p[j].x : 0u, py = ok ? (uint32_t)p[j].y : 0u;
-            bool look = ok;
-            if (SUM) {
-                const uint32_t sv = s_sum[((py >> ix.ssh) << ix.sg) | (px >> ix.ssh)];
-                look = ok && sv == kSumMixed;
-                w[j] = !ok || sv == kSumEmpty ? 0u : (kCellInsideOne << 30) | sv;
-            }
-            if (look)
+            w[j] = 0u;
+            if (ok)
                 w[j] = coarse_word(ix, px, py, keep);
-            else if (!SUM)
-                w[j] = 0u;
         }
 #pragma unroll
         for (int j = 0; j < kWItems; ++j)
@@ -1289,8 +1429,8 @@ constexpr uint32_t kSmallHist = 2048;
 //
 // With ALL (the count aggregate over a cell directory) a marked row is any row
 // of a mixed coarse cell: rows that its fine cell resolves are counted here.
-template <bool FP32, int OUT, bool NEAR, bool ALL>
-__global__ void __launch_bounds__(kThreads, NEAR ? 3 : kWalkMinBlocks) k_walk(const __grid_constant__ JoinLaunch a, uint32_t *pend,
+template <bool FP32, int OUT, int KIND, bool ALL>
+__global__ void __launch_bounds__(kThreads, KIND == kNear ? 3 : kWalkMinBlocks) k_walk(const __grid_constant__ JoinLaunch a, uint32_t *pend,
                                                                    uint32_t nwords)
 {
     static_assert(!ALL || OUT == kOutCount, "ALL keeps nothing per row");
@@ -1327,7 +1467,7 @@ __global__ void __launch_bounds__(kThreads, NEAR ? 3 : kWalkMinBlocks) k_walk(co
         const uint32_t row = it.w;
         uint32_t f = 0, c = 0;
         uint64_t ids = 0; // kOut16 and a.aux: the first polygons, aux_bits each
-        walk_list_wave<FP32, NEAR>(ix, has, it.z, (int)it.x, (int)it.y, n_tests, n_esc, keep, s_par, [&](uint32_t q) {
+        walk_list_wave<FP32, KIND>(ix, has, it.z, (int)it.x, (int)it.y, n_tests, n_esc, keep, s_par, [&](uint32_t q) {
             if (OUT == kOut16 && (c + 1) * a.aux_bits <= 64)
                 ids |= (uint64_t)q << (a.aux_bits * c);
             f = c ? f : q;
@@ -1456,11 +1596,11 @@ __global__ void __launch_bounds__(kThreads, NEAR ? 3 : kWalkMinBlocks) k_walk(co
     add_stats(a.stats, n_pts, n_tests, n_esc, n_pairs);
 }
 
-template <bool FP32, int OUT, bool NEAR, bool ALL = false>
+template <bool FP32, int OUT, int KIND, bool ALL = false>
 cudaError_t launch_walk(const JoinLaunch &a, uint32_t *pend, cudaStream_t s)
 {
     const uint64_t nwords = (a.n + kWChunk - 1) / kWChunk * kWItems, per_cta = uint64_t(kWarps) * walk_range(nwords);
-    k_walk<FP32, OUT, NEAR, ALL><<<unsigned((nwords + per_cta - 1) / per_cta), kThreads, 0, s>>>(a, pend, uint32_t(nwords));
+    k_walk<FP32, OUT, KIND, ALL><<<unsigned((nwords + per_cta - 1) / per_cta), kThreads, 0, s>>>(a, pend, uint32_t(nwords));
     return cudaGetLastError();
 }
 
@@ -1475,7 +1615,7 @@ cudaError_t launch_walk(const JoinLaunch &a, uint32_t *pend, cudaStream_t s)
 // 1M 32.8 / 39.0, 1.5M 39.0 / 39.1, 2M 53.7 / 43.1; the line is at 1M points.
 constexpr uint32_t kSmallChunks = 4096;
 
-template <bool FP32, int OUT, bool NEAR>
+template <bool FP32, int OUT, int KIND>
 __global__ void __launch_bounds__(kThreads, 3) k_small(const __grid_constant__ JoinLaunch a, uint32_t *pend,
                                                        uint32_t nchunks, int use_hist)
 {
@@ -1543,7 +1683,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_small(const __grid_constant__ J
             const uint4 it = s_q[has ? k0 + lane : k0]; // idle lanes walk nothing
             uint32_t f = 0, c = 0;
             uint64_t ids = 0; // kOut16 and a.aux: the first polygons, aux_bits each
-            walk_list_wave<FP32, NEAR>(ix, has, it.z, (int)it.x, (int)it.y, n_tests, n_esc, keep, s_pa + warp * kWaveWords,
+            walk_list_wave<FP32, KIND>(ix, has, it.z, (int)it.x, (int)it.y, n_tests, n_esc, keep, s_pa + warp * kWaveWords,
                                  [&](uint32_t q) {
                                      if (OUT == kOut16 && (c + 1) * a.aux_bits <= 64)
                                          ids |= (uint64_t)q << (a.aux_bits * c);
@@ -1591,7 +1731,7 @@ constexpr size_t kEmitSmem = size_t(kWarps) * kWChunk * (sizeof(uint32_t) + size
                              size_t(kWarps) * kWaveWords * sizeof(uint32_t);
 
 // (k_wemit: 32-bit results, more than kRes16MaxP polygons.)
-template <bool FP32, bool NEAR>
+template <bool FP32, int KIND>
 __global__ void __launch_bounds__(kThreads, 3) k_wemit(const __grid_constant__ JoinLaunch a, const unsigned long long *chunk_off,
                                                        uint32_t nchunks)
 {
@@ -1633,8 +1773,9 @@ __global__ void __launch_bounds__(kThreads, 3) k_wemit(const __grid_constant__ J
                     } else { // count not stored: count again
                         const int2 p = a.pts[base + loc];
                         uint32_t f = 0, t = 0, e = 0;
-                        c = NEAR ? near_count<FP32>(a.ix, a.near, p.x, p.y, keep)
-                                 : point_count<FP32>(a.ix, p.x, p.y, f, t, e, keep);
+                        c = KIND == kPoly   ? point_count<FP32>(a.ix, p.x, p.y, f, t, e, keep)
+                            : KIND == kNear ? near_count<FP32>(a.ix, a.near, p.x, p.y, keep)
+                                            : disk_count(a.ix, a.near, p.x, p.y, keep);
                     }
                 }
                 uint32_t inc = c;
@@ -1672,7 +1813,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_wemit(const __grid_constant__ J
             const uint32_t pid = a.pid0 + (uint32_t)(base + loc);
             const uint32_t w = has ? resolve(a.ix, (uint32_t)p.x, (uint32_t)p.y, keep) : 0u;
             uint32_t t = 0, e = 0;
-            walk_list_wave<FP32, NEAR>(a.ix, (w >> 30) >= kCellList, w & kPayloadMask, p.x, p.y, t, e, keep, s_par,
+            walk_list_wave<FP32, KIND>(a.ix, (w >> 30) >= kCellList, w & kPayloadMask, p.x, p.y, t, e, keep, s_par,
                                  [&](uint32_t q) {
                                      if (o < a.cap)
                                          __stcs(a.pairs + o, make_uint2(pid, q));
@@ -1689,26 +1830,27 @@ __global__ void __launch_bounds__(kThreads, 3) k_wemit(const __grid_constant__ J
 // row its place, where the row-major form above scans once per round of 32 rows
 // that holds a point in several polygons.  The chunk's pairs are put together in
 // shared memory and written out as whole lines (lanes' own stretches are 64
-// bytes apart).  Points in several polygons are queued and taken 32 at a time, so
-// that a chunk waits once for their packed words (a wait per row of a lane was
-// most of this kernel: 8 dependent round trips a chunk); those that pass 1b could
-// not pack have their lists walked by the warp.  A chunk of more than kEmitStage pairs is written
-// straight to its place.  500M points x 256 queries (17 % of the points in one or
-// more): 2.77 -> 1.19 ms; 100M x 2000 cells (a pair per point): 204 -> 175 us for
-// 1.0 GB, where a plain fill of its 0.8 GB takes 105; 20M x 256 buffered queries:
-// 232 -> 72 us.
+// bytes apart).  Points in several polygons are queued, across chunks, and taken
+// in full rounds of 32: their polygons come from the words that pass 1b packed,
+// or the warp walks their lists (a wait per row of a lane, then one per chunk, was
+// most of this kernel).  A chunk of more than kEmitStage pairs is written straight
+// to its place.  500M points x 256 queries (17 % of the points in one or more):
+// 2.77 ms row-major, 1.19 with a wait per chunk, 1.09 now; 100M x 1024 disks 257
+// -> 154 us; 20M x 256 buffered queries 232 -> 65 us; 100M x 2000 cells (a
+// pair per point) 204 -> 162 us for 1.0 GB, where a plain fill of its 0.8 GB
+// takes 105.
 //
 // With SELF (small tables, a warp per chunk) chunk_off holds the chunks' totals,
 // not their offsets: every CTA sums the totals before its first chunk itself
 // (at most 8 B x kSmallChunks from L2), which saves the scan's launch.
-constexpr uint32_t kEmitStage = 512;
-__host__ __device__ constexpr uint32_t stage_at(uint32_t i) { return i + (i >> 3); } // eight pairs per lane: no bank conflict
-constexpr size_t kEmit16Warp = (stage_at(kEmitStage) * 8 + size_t(kWChunk) * 8 + kWaveWords * 4 + 15) & ~size_t(15);
-constexpr size_t kEmit16Smem = kWarps * kEmit16Warp;
+constexpr uint32_t kEmitStage = 320; // pairs; a full chunk's lie nine apart per lane of eight (no bank conflict)
+constexpr uint32_t kEmitQueue = kWChunk + 32; // a chunk's rows and a partial round
+constexpr size_t kEmit16Warp = (kEmitStage * 8 + size_t(kEmitQueue) * 12 + kWaveWords * 4 + 15) & ~size_t(15);
+constexpr size_t kEmit16Smem = kWarps * kEmit16Warp; // 53 KB: four CTAs per SM
 static_assert(kWItems == 8, "a lane's rows: one 16-byte load of 2-byte results");
 
-template <bool FP32, bool SELF, bool NEAR>
-__global__ void __launch_bounds__(kThreads, NEAR ? 3 : 4) k_wemit16(const __grid_constant__ JoinLaunch a,
+template <bool FP32, bool SELF, int KIND>
+__global__ void __launch_bounds__(kThreads, KIND == kNear ? 3 : 4) k_wemit16(const __grid_constant__ JoinLaunch a,
                                                          const unsigned long long *chunk_off, uint32_t nchunks,
                                                          const uint32_t *pend)
 {
@@ -1716,8 +1858,9 @@ __global__ void __launch_bounds__(kThreads, NEAR ? 3 : 4) k_wemit16(const __grid
     extern __shared__ __align__(16) unsigned char s_raw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint2 *s_st = reinterpret_cast<uint2 *>(s_raw + warp * kEmit16Warp);
-    uint2 *s_q = s_st + stage_at(kEmitStage); // (row | count << 8, place in the chunk's pairs)
-    uint32_t *s_par = reinterpret_cast<uint32_t *>(s_q + kWChunk);
+    unsigned long long *s_o = reinterpret_cast<unsigned long long *>(s_st + kEmitStage); // offset | count << 48
+    uint32_t *s_q = reinterpret_cast<uint32_t *>(s_o + kEmitQueue); // rows of the table
+    uint32_t *s_par = s_q + kEmitQueue;
     const uint64_t keep = policy_evict_last();
     const uint32_t nw = gridDim.x * kWarps, r0 = 8u * (uint32_t)lane;
     const unsigned short *res = reinterpret_cast<const unsigned short *>(a.res);
@@ -1759,98 +1902,152 @@ __global__ void __launch_bounds__(kThreads, NEAR ? 3 : 4) k_wemit16(const __grid
         if (!SELF)
             noff = ch < nchunks ? chunk_off[ch] : 0ull;
     };
+    // writes the pairs of queued points [k0, k0 + m), m <= 32, one per lane
+    auto several = [&](uint32_t k0, uint32_t m_) {
+        const bool has = (uint32_t)lane < m_;
+        const uint32_t row = s_q[k0 + (has ? lane : 0)], pid = a.pid0 + row;
+        const unsigned long long oc = s_o[k0 + (has ? lane : 0)];
+        unsigned long long o = oc & ((1ull << 48) - 1);
+        const uint32_t c = uint32_t(oc >> 48);
+        const bool packed = a.aux && c * a.aux_bits <= 64;
+        if (has && packed) {
+            unsigned long long ids = __ldcs(reinterpret_cast<const unsigned long long *>(a.aux) + row);
+            for (uint32_t t = 0; t < c; ++t, ++o, ids >>= a.aux_bits)
+                if (o < a.cap)
+                    __stcs(a.pairs + o, make_uint2(pid, uint32_t(ids) & ((1u << a.aux_bits) - 1u)));
+        }
+        const bool walk = has && !packed; // the whole warp walks these points' lists together
+        if (__any_sync(kFull, walk)) {
+            const int2 p = walk ? a.pts[row] : make_int2(0, 0);
+            const uint32_t w = walk ? resolve(a.ix, (uint32_t)p.x, (uint32_t)p.y, keep) : 0u;
+            uint32_t t = 0, e = 0;
+            walk_list_wave<FP32, KIND>(a.ix, (w >> 30) >= kCellList, w & kPayloadMask, p.x, p.y, t, e, keep, s_par,
+                                       [&](uint32_t q) {
+                                           if (o < a.cap)
+                                               __stcs(a.pairs + o, make_uint2(pid, q));
+                                           ++o;
+                                       }, &a.near);
+        }
+        __syncwarp();
+    };
+    uint32_t qn = 0; // queued points, < 32 between chunks
     const unsigned long long pb = a.pair_base ? *a.pair_base : 0ull;
     fetch(blockIdx.x * kWarps + warp);
     for (uint32_t ch = blockIdx.x * kWarps + warp; ch < nchunks; ch += nw) {
         const uint64_t base = (uint64_t)ch * kWChunk;
         const uint32_t m = nm, pid0 = a.pid0 + (uint32_t)base + r0;
         const unsigned long long run = SELF ? before : noff + pb;
-        uint32_t r[8];
+        uint32_t w[4];
 #pragma unroll
-        for (int k = 0; k < 8; ++k)
-            r[k] = k & 1 ? nr[k >> 1] >> 16 : nr[k >> 1] & 0xffffu;
+        for (int k = 0; k < 4; ++k)
+            w[k] = nr[k];
         if (!SELF)
             fetch(ch + nw);
-        // pairs of this lane's rows, and (upper half) its rows in several polygons
-        unsigned long long mine = 0;
+        // row k's result, and whether it is none (0xffff)
+        auto r = [&](int k) { return k & 1 ? w[k >> 1] >> 16 : w[k >> 1] & 0xffffu; };
+        auto none = [&](int k) { return (k & 1 ? w[k >> 1] : w[k >> 1] << 16) >= 0xffff0000u; };
+        const bool any_m = __any_sync(kFull, m != 0);
+        uint32_t mine = 0;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const bool multi = (m >> k) & 1u;
-            mine += multi ? r[k] : r[k] != kRes16None ? 1u : 0u;
-            mine += (unsigned long long)multi << 32;
+        for (int k = 0; k < 8; ++k)
+            mine += none(k) ? 0u : 1u;
+        if (any_m) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if ((m >> k) & 1u) // the count of a row in several polygons (never 0xffff: P is below it)
+                    mine += r(k) - 1u;
         }
-        uint32_t at, tot, slot = 0, qn = 0;
-        if (!__any_sync(kFull, m != 0)) {
-            uint32_t inc = (uint32_t)mine;
+        if (!any_m && __all_sync(kFull, mine == 8)) { // every row in one polygon
+            uint2 *d = s_st + 9 * lane;
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t v = __shfl_up_sync(kFull, inc, o);
-                if (lane >= o)
-                    inc += v;
-            }
-            tot = __shfl_sync(kFull, inc, 31);
-            at = inc - (uint32_t)mine;
-        } else {
-            unsigned long long inc = mine;
+            for (int k = 0; k < 8; ++k)
+                d[k] = make_uint2(pid0 + k, r(k));
+            __syncwarp();
+            const uint2 *src = s_st + lane + (lane >> 3);
+            if (run + kWChunk <= a.cap) {
+                uint2 *out = a.pairs + run + lane;
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned long long v = __shfl_up_sync(kFull, inc, o);
-                if (lane >= o)
-                    inc += v;
+                for (int k = 0; k < 8; ++k)
+                    __stcs(out + 32 * k, src[36 * k]);
+            } else {
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    if (run + 32 * k + lane < a.cap)
+                        __stcs(a.pairs + run + 32 * k + lane, src[36 * k]);
             }
-            const unsigned long long t = __shfl_sync(kFull, inc, 31);
-            tot = (uint32_t)t;
-            qn = uint32_t(t >> 32);
-            at = uint32_t(inc - mine);
-            slot = uint32_t((inc - mine) >> 32);
+            __syncwarp(); // the stage is rewritten by the next chunk
+            continue;
         }
+        uint32_t inc = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t v = __shfl_up_sync(kFull, inc, o);
+            if (lane >= o)
+                inc += v;
+        }
+        const uint32_t tot = __shfl_sync(kFull, inc, 31);
         if (tot == 0)
             continue;
+        uint32_t at = inc - mine;
         const bool staged = tot <= kEmitStage;
-        auto put = [&](uint32_t place, uint32_t pid, uint32_t q) {
-            if (staged)
-                s_st[stage_at(place)] = make_uint2(pid, q);
-            else if (run + place < a.cap)
-                __stcs(a.pairs + run + place, make_uint2(pid, q));
-        };
+        if (!any_m && staged) {
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            if ((m >> k) & 1u) {
-                s_q[slot++] = make_uint2((r0 + k) | r[k] << 8, at);
-                at += r[k];
-            } else if (r[k] != kRes16None) {
-                put(at++, pid0 + k, r[k]);
+            for (int k = 0; k < 8; ++k)
+                if (!none(k))
+                    s_st[at++] = make_uint2(pid0 + k, r(k));
+        } else {
+            uint32_t slot = __popc(m); // rows in several polygons: their places in the queue
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t v = __shfl_up_sync(kFull, slot, o);
+                if (lane >= o)
+                    slot += v;
+            }
+            const uint32_t nq = __shfl_sync(kFull, slot, 31);
+            slot += qn - __popc(m);
+            qn += nq;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                if ((m >> k) & 1u) {
+                    s_q[slot] = (uint32_t)base + r0 + k;
+                    s_o[slot++] = (run + at) | (unsigned long long)r(k) << 48;
+                    at += r(k);
+                } else if (!none(k)) {
+                    if (staged)
+                        s_st[at] = make_uint2(pid0 + k, r(k));
+                    else if (run + at < a.cap)
+                        __stcs(a.pairs + run + at, make_uint2(pid0 + k, r(k)));
+                    ++at;
+                }
             }
         }
         __syncwarp();
-        for (uint32_t k0 = 0; k0 < qn; k0 += 32) {
-            const bool has = k0 + lane < qn;
-            const uint2 it = s_q[has ? k0 + lane : 0];
-            const uint32_t row = it.x & 0xffu, c = it.x >> 8, pid = a.pid0 + (uint32_t)base + row;
-            const bool packed = a.aux && c * a.aux_bits <= 64;
-            uint32_t place = it.y;
-            if (has && packed) {
-                unsigned long long ids = __ldcs(reinterpret_cast<const unsigned long long *>(a.aux) + base + row);
-                for (uint32_t t = 0; t < c; ++t, ids >>= a.aux_bits)
-                    put(place++, pid, uint32_t(ids) & ((1u << a.aux_bits) - 1u));
-            }
-            const bool walk = has && !packed; // the whole warp walks these points' lists together
-            if (!__any_sync(kFull, walk))
-                continue;
-            const int2 p = walk ? a.pts[base + row] : make_int2(0, 0);
-            const uint32_t w = walk ? resolve(a.ix, (uint32_t)p.x, (uint32_t)p.y, keep) : 0u;
-            uint32_t t = 0, e = 0;
-            walk_list_wave<FP32, NEAR>(a.ix, (w >> 30) >= kCellList, w & kPayloadMask, p.x, p.y, t, e, keep, s_par,
-                                       [&](uint32_t q) { put(place++, pid, q); }, &a.near);
-        }
         if (staged) {
-            __syncwarp();
+            // whole lines; the places of queued points are written with what the
+            // stage held, and with their pairs when their round comes
             const uint32_t n_out = run >= a.cap ? 0u : (uint32_t)min((unsigned long long)tot, a.cap - run);
             for (uint32_t i = lane; i < n_out; i += 32)
-                __stcs(a.pairs + run + i, s_st[stage_at(i)]);
+                __stcs(a.pairs + run + i, s_st[i]);
+            __syncwarp();
         }
-        __syncwarp(); // the queue and the stage are rewritten by the next chunk
+        if (qn >= 32) {
+            uint32_t k0 = 0;
+            for (; qn - k0 >= 32; k0 += 32)
+                several(k0, 32);
+            const uint32_t rem = qn - k0; // move the partial round (< 32, from k0 >= 32) to the front
+            const uint32_t q = (uint32_t)lane < rem ? s_q[k0 + lane] : 0u;
+            const unsigned long long oo = (uint32_t)lane < rem ? s_o[k0 + lane] : 0ull;
+            __syncwarp();
+            if ((uint32_t)lane < rem) {
+                s_q[lane] = q;
+                s_o[lane] = oo;
+            }
+            qn = rem;
+            __syncwarp();
+        }
     }
+    if (qn)
+        several(0, qn);
 }
 
 // ------------------------------------------------------ multi-request batches
@@ -2333,9 +2530,9 @@ cudaError_t launch_warp_kernel(const JoinLaunch &a, int use_hist, cudaStream_t s
 // a mixed coarse cell marks its rows in the bitmap, for k_walk<ALL>.  The points
 // of the cells counted here, and of the bin outside the box, go into the
 // scanned-points counter.  The stage reads 8 B per cell and a coarse word per
-// cell with points, kDirCells independent loads of each per lane; rows are 32-bit
-// (2^26 cells, 500M points: 500 us with 64-bit rows and one cell per lane at a
-// time, DIRUS so).
+// cell with points, kDirCells independent loads of each per lane.  2^26 cells,
+// 500M points: 656 us, and k_walk<ALL> 998 for the 34M marked rows; marking 256-row
+// chunks took 500, and the chunks, nearly all of them, 3020.
 constexpr int kDirCells = 4;
 __global__ void __launch_bounds__(256) k_agg_cells(const unsigned long long *cell_end, int c, IndexView ix,
                                                    unsigned long long *counts, uint32_t *rows,
@@ -2419,7 +2616,7 @@ __global__ void __launch_bounds__(256) k_agg_cells(const unsigned long long *cel
 // Pass 1 of the join (1a resolve, 1b walk).  pend: 8 words per chunk (the
 // bitmap of the rows pass 1b tests).  mid (or null): an event recorded between
 // the two kernels.
-template <bool FP32, int OUT, bool NEAR>
+template <bool FP32, int OUT, int KIND>
 cudaError_t launch_pass1_as(const JoinLaunch &a, uint32_t *pend, cudaStream_t s, cudaEvent_t mid)
 {
     static bool done_r[4][64] = {};
@@ -2452,32 +2649,37 @@ cudaError_t launch_pass1_as(const JoinLaunch &a, uint32_t *pend, cudaStream_t s,
     if (a.ix.use_sum) {
         // beside the summary, shared memory holds one chunk buffer per warp
         // at most, too shallow to hide a bulk copy: L2 prefetches instead
-        e = launch(k_resolve<kResolveSumThreads, true, false, OUT>, kResolveSumThreads,
+        e = launch(k_resolve_sum<OUT>, kResolveSumThreads,
                    resolve_smem_head(WS, true, a.ix.sg, false), resolve_smem_head(WS, true, kSumLog2, false), done_r[2]);
     } else {
         const size_t head = kTmaPoints ? resolve_smem_head(kWarps, false, 0, true) : 0;
-        e = launch(k_resolve<kThreads, false, kTmaPoints, OUT>, kThreads, head, head, done_r[3]);
+        e = launch(k_resolve<kThreads, kTmaPoints, OUT>, kThreads, head, head, done_r[3]);
     }
     if (e != cudaSuccess) // pass 1b must not run on what an earlier call left in the scratch
         return e;
     if (mid)
         cudaEventRecord(mid, s);
-    return launch_walk<FP32, OUT, NEAR>(a, pend, s); // pass 1b
+    return launch_walk<FP32, OUT, KIND>(a, pend, s); // pass 1b
 }
 
-// Calls f(fp32, near) with the launch's two switches as compile-time values.
+// Calls f(fp32, kind) with the launch's two switches as compile-time values
+// (disk tests are in int64 alone).
 template <class F>
 cudaError_t with_switches(const JoinLaunch &a, F f)
 {
+    using std::integral_constant;
+    if (a.near.disk)
+        return f(std::true_type{}, integral_constant<int, kDisk>{});
     if (a.near.rad)
-        return a.fp32 ? f(std::true_type{}, std::true_type{}) : f(std::false_type{}, std::true_type{});
-    return a.fp32 ? f(std::true_type{}, std::false_type{}) : f(std::false_type{}, std::false_type{});
+        return a.fp32 ? f(std::true_type{}, integral_constant<int, kNear>{}) : f(std::false_type{}, integral_constant<int, kNear>{});
+    return a.fp32 ? f(std::true_type{}, integral_constant<int, kPoly>{}) : f(std::false_type{}, integral_constant<int, kPoly>{});
 }
 
 cudaError_t launch_pass1(const JoinLaunch &a, uint32_t *pend, cudaStream_t s, cudaEvent_t mid, bool count_only)
 {
-    return with_switches(a, [&](auto fp32, auto near) {
-        constexpr bool F = decltype(fp32)::value, N = decltype(near)::value;
+    return with_switches(a, [&](auto fp32, auto kind) {
+        constexpr bool F = decltype(fp32)::value;
+        constexpr int N = decltype(kind)::value;
         return count_only ? launch_pass1_as<F, kOutCount, N>(a, pend, s, mid)
                : a.narrow ? launch_pass1_as<F, kOut16, N>(a, pend, s, mid)
                           : launch_pass1_as<F, kOut32, N>(a, pend, s, mid);
@@ -2549,344 +2751,6 @@ cudaError_t launch_gather_stride(const int2 *src, uint64_t n, int2 *dst, uint64_
     const uint64_t blocks = std::min<uint64_t>((m + 255) / 256, uint64_t(device_sm_count()) * 8);
     k_gather_stride<<<unsigned(blocks), 256, 0, s>>>(src, stride, dst, m);
     return cudaGetLastError();
-}
-
-// ------------------------------------------------------ distance queries (disks)
-// A point is within distance r of a centre c iff (px-cx)^2 + (py-cy)^2 <= r^2,
-// exact in int64 (differences < 2^31; r < 2^30; the x term is compared with
-// r^2 before the sum, so the sum cannot overflow).  A point reads the word of
-// its cell in the disks' grid; INSIDE entries count at once and BOUNDARY
-// entries take the exact test; lists are in disk order.
-__device__ __forceinline__ bool in_disk(const int4 &d, int px, int py)
-{
-    const long long dx = (long long)px - d.x, dy = (long long)py - d.y, rr = (long long)d.z * d.z;
-    const long long dx2 = dx * dx;
-    return dx2 <= rr && dx2 + dy * dy <= rr;
-}
-
-template <class F>
-__device__ __forceinline__ uint32_t disk_walk(const DiskView &d, int px, int py, uint32_t &first, uint32_t &tests,
-                                              uint64_t pol, F f)
-{
-    if ((unsigned)px >= kBox || (unsigned)py >= kBox)
-        return 0;
-    const uint32_t w = ld_idx(d.cell + ((((uint32_t)py >> d.sc) << d.g) | ((uint32_t)px >> d.sc)), pol);
-    const uint32_t kind = w >> 30;
-    if (kind == kCellInsideOne) {
-        first = w & kPayloadMask;
-        f(first);
-        return 1;
-    }
-    if (kind != kCellList)
-        return 0;
-    const uint32_t *e = d.ent + (w & kPayloadMask);
-    const uint32_t n = ld_idx(e, pol);
-    uint32_t c = 0;
-    for (uint32_t k = 1; k <= n; ++k) {
-        const uint32_t en = ld_idx(e + k, pol), q = en >> 1;
-        bool in = true;
-        if (en & 1u) {
-            ++tests;
-            in = in_disk(__ldg(d.disk + q), px, py);
-        }
-        if (in) {
-            if (!c)
-                first = q;
-            ++c;
-            f(q);
-        }
-    }
-    return c;
-}
-
-// Distance join with warp chunks (the design of k_warp / k_wemit): pass 1
-// resolves every point once: the cover bitmap (in shared memory) sends the
-// points of blocks without any disk away without an index read; the others
-// read their cell word, and the points of list cells are queued in shared
-// memory.  The queue carries over from chunk to chunk and the warp walks it
-// in full rounds of 32 (one chain of dependent loads per 32 list points); a
-// walked point adds its pairs to its own chunk's total (stored by lane 0
-// before any of the chunk's points is walked; __syncwarp orders the two).
-// It stores a 4-byte result per point and a pair total per 256-point chunk,
-// and counts per disk (in shared memory when Q <= kHistMax); pass 3 writes
-// the pairs from the results.
-constexpr int kDiskMinBlocks = 4;
-constexpr uint32_t kDiskCoverWords = 1u << (2 * kCoverLog2 - 5); // cover bitmap in shared memory
-constexpr int kDQueue = kWChunk + 32; // a chunk's points plus a partial round
-constexpr size_t kDWarpSmem = size_t(kWarps) * kDQueue * sizeof(uint4);
-
-template <bool RESOLVE>
-__global__ void __launch_bounds__(kThreads, kDiskMinBlocks) k_dwarp(DiskLaunch a, unsigned long long *chunk_tot, uint32_t *res,
-                                                       uint32_t nchunks, int use_hist)
-{
-    extern __shared__ __align__(16) unsigned char s_raw[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint4 *s_q = reinterpret_cast<uint4 *>(s_raw) + warp * kDQueue; // (x, y, list offset, point index)
-    uint32_t *s_cov = reinterpret_cast<uint32_t *>(s_raw + kDWarpSmem);
-    uint32_t *s_hist = s_cov + kDiskCoverWords;
-    const DiskView &d = a.dv;
-    const uint64_t keep = policy_evict_last();
-    const bool hist = use_hist && a.counts;
-    const uint32_t ncov = max(1u, (1u << (2 * d.cg)) >> 5);
-    for (uint32_t i = threadIdx.x; i < ncov; i += kThreads)
-        s_cov[i] = __ldg(d.cover + i);
-    if (hist)
-        for (uint32_t i = threadIdx.x; i < d.Q; i += kThreads)
-            s_hist[i] = 0;
-    __syncthreads();
-    // count one disk for every lane with has (converged warp)
-    auto count1 = [&](bool has, uint32_t q) {
-        if (!a.counts)
-            return;
-        if (!hist)
-            global_add_warp(a.counts, has, q);
-        else if (has)
-            atomicAdd(s_hist + q, 1u);
-    };
-    uint32_t n_tests = 0, n_pts = 0, n_pairs = 0;
-    // walk queued list points [k0, k0 + m), m <= 32, one per lane; their pairs
-    // are added to their chunk's total
-    auto walk = [&](uint32_t k0, uint32_t m) {
-        const bool has = (uint32_t)lane < m;
-        const uint4 it = s_q[k0 + (has ? lane : 0)]; // idle lanes repeat lane 0's walk, uncounted
-        const uint32_t *e = d.ent + it.z;
-        const uint32_t n = ld_idx(e, keep);
-        uint32_t c = 0, f = 0, t_l = 0;
-        for (uint32_t k = 1; k <= n; ++k) {
-            const uint32_t en = ld_idx(e + k, keep), q = en >> 1;
-            bool in = true;
-            if (en & 1u) {
-                ++t_l;
-                in = in_disk(__ldg(d.disk + q), (int)it.x, (int)it.y);
-            }
-            if (in) {
-                if (!c)
-                    f = q;
-                else if (has && a.counts) // the first disk is counted with the warp below
-                    hist ? (void)atomicAdd(s_hist + q, 1u) : (void)atomicAdd(a.counts + q, 1ull);
-                ++c;
-            }
-        }
-        c = has ? c : 0u;
-        n_tests += has ? t_l : 0u;
-        n_pairs += c;
-        count1(c >= 1, f);
-        if (RESOLVE && has) {
-            __stcg(res + it.w, res_encode(c, f));
-            if (c)
-                atomicAdd(chunk_tot + it.w / kWChunk, (unsigned long long)c);
-        }
-        __syncwarp();
-    };
-    const uint32_t nw = gridDim.x * kWarps;
-    uint32_t qn = 0; // queued list points, < 32 between chunks
-    for (uint32_t ch = blockIdx.x * kWarps + warp; ch < nchunks; ch += nw) {
-        const uint64_t base = (uint64_t)ch * kWChunk;
-        const uint32_t npts = (uint32_t)min((uint64_t)kWChunk, a.n - base);
-        if (lane == 0)
-            n_pts += npts;
-        int2 p[kWItems];
-        uint32_t w[kWItems];
-        // rows past the table's end read as outside the box
-#pragma unroll
-        for (int j = 0; j < kWItems; ++j) {
-            const uint32_t loc = j * 32 + lane;
-            p[j] = loc < npts ? __ldcs(a.pts + base + loc) : make_int2(-1, -1);
-        }
-#pragma unroll
-        for (int j = 0; j < kWItems; ++j) {
-            // points outside the box or in a block of empty cells read no cell word
-            const uint32_t px = (uint32_t)p[j].x, py = (uint32_t)p[j].y;
-            const uint32_t b = (((py & (kBox - 1)) >> d.scv) << d.cg) | ((px & (kBox - 1)) >> d.scv);
-            const bool ok = px < kBox && py < kBox && ((s_cov[b >> 5] >> (b & 31)) & 1u);
-            w[j] = ok ? ld_idx(d.cell + ((((py & (kBox - 1)) >> d.sc) << d.g) | ((px & (kBox - 1)) >> d.sc)), keep)
-                      : 0u;
-        }
-        uint32_t total = 0;
-#pragma unroll
-        for (int j = 0; j < kWItems; ++j) {
-            const uint32_t kind = w[j] >> 30, loc = j * 32 + lane;
-            const bool one = kind == kCellInsideOne, lst = kind == kCellList;
-            total += one ? 1u : 0u;
-            count1(one, w[j] & kPayloadMask);
-            if (RESOLVE && loc < npts && !lst)
-                __stcg(res + base + loc, one ? (w[j] & kPayloadMask) : kResNone);
-            const uint32_t bl = __ballot_sync(kFull, lst);
-            if (lst)
-                s_q[qn + __popc(bl & lanemask_lt())] =
-                    make_uint4((uint32_t)p[j].x, (uint32_t)p[j].y, w[j] & kPayloadMask, (uint32_t)(base + loc));
-            qn += __popc(bl);
-        }
-        n_pairs += total;
-        total = warp_sum32(total);
-        if (RESOLVE && lane == 0)
-            chunk_tot[ch] = total; // the chunk's pair total so far; its queued points add theirs
-        __syncwarp();
-        if (qn >= 32) {
-            uint32_t k0 = 0;
-            for (; qn - k0 >= 32; k0 += 32)
-                walk(k0, 32);
-            // move the partial round (< 32, from k0 >= 32) to the front
-            const uint32_t rem = qn - k0;
-            const uint4 it = (uint32_t)lane < rem ? s_q[k0 + lane] : make_uint4(0, 0, 0, 0);
-            __syncwarp();
-            if ((uint32_t)lane < rem)
-                s_q[lane] = it;
-            qn = rem;
-            __syncwarp();
-        }
-    }
-    __syncwarp();
-    if (qn)
-        walk(0, qn);
-    if (hist) {
-        __syncthreads();
-        for (uint32_t i = threadIdx.x; i < d.Q; i += kThreads)
-            if (s_hist[i])
-                atomicAdd(a.counts + i, (unsigned long long)s_hist[i]);
-    }
-    add_stats(a.stats, n_pts, n_tests, 0u, n_pairs);
-}
-
-// Pass 3 of the distance join.  Lane-major: lane l owns rows 8l .. 8l + 7 of
-// the warp's 256-row chunk (two 16-byte loads of stored results), so one warp
-// scan of the lanes' pair counts gives every row its offset in point order.
-// A point in one disk is written at once; a point in several is queued (its
-// row and its offset; its count comes with its stored result).  Such points
-// are rare, so the queue carries over from chunk to chunk and the warp walks
-// it only in full rounds of 32 (and what is left at the end), loading the
-// queued points' coordinates then, one independent load per lane.  The next
-// chunk's results are loaded while this one is written.
-constexpr size_t kDEmitSmem = size_t(kWarps) * kDQueue * (sizeof(uint32_t) + sizeof(unsigned long long));
-static_assert(kWItems == 8, "lane-major emit: two 16-byte loads of 4-byte results per lane");
-
-__global__ void __launch_bounds__(kThreads, 4) k_dwemit(DiskLaunch a, const unsigned long long *chunk_off,
-                                                        const uint32_t *res_in, uint32_t nchunks)
-{
-    extern __shared__ __align__(16) unsigned char s_raw[];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    unsigned long long *s_o = reinterpret_cast<unsigned long long *>(s_raw) + warp * kDQueue;
-    uint32_t *s_q = reinterpret_cast<uint32_t *>(s_raw + size_t(kWarps) * kDQueue * sizeof(unsigned long long)) +
-                    warp * kDQueue; // point rows
-    const uint64_t keep = policy_evict_last();
-    // walk queued points [k0, k0 + m), m <= 32, one per lane
-    auto walk = [&](uint32_t k0, uint32_t m) {
-        if ((uint32_t)lane < m) {
-            const uint32_t pid = s_q[k0 + lane];
-            unsigned long long o = s_o[k0 + lane];
-            const int2 p = a.pts[pid];
-            uint32_t f = 0, t = 0;
-            disk_walk(a.dv, p.x, p.y, f, t, keep, [&](uint32_t q) {
-                if (o < a.cap)
-                    __stcs(a.pairs + o, make_uint2(pid, q));
-                ++o;
-            });
-        }
-    };
-    uint32_t qn = 0; // queued points, < 32 between chunks
-    const uint32_t nw = gridDim.x * kWarps;
-    const uint32_t r0 = 8u * (uint32_t)lane; // this lane's first row in a chunk
-    uint32_t nres[8];
-    unsigned long long noff = 0;
-    auto fetch = [&](uint32_t ch) {
-        const uint64_t base = (uint64_t)ch * kWChunk;
-        const uint32_t npts = ch < nchunks ? (uint32_t)min((uint64_t)kWChunk, a.n - base) : 0u;
-        if (r0 + 8 <= npts) {
-            const uint4 u = __ldcs(reinterpret_cast<const uint4 *>(res_in + base + r0));
-            const uint4 v = __ldcs(reinterpret_cast<const uint4 *>(res_in + base + r0 + 4));
-            nres[0] = u.x, nres[1] = u.y, nres[2] = u.z, nres[3] = u.w;
-            nres[4] = v.x, nres[5] = v.y, nres[6] = v.z, nres[7] = v.w;
-        } else { // the table's ragged end
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-                nres[k] = r0 + k < npts ? __ldcs(res_in + base + r0 + k) : kResNone;
-        }
-        noff = ch < nchunks ? chunk_off[ch] : 0ull;
-    };
-    fetch(blockIdx.x * kWarps + warp);
-    for (uint32_t ch = blockIdx.x * kWarps + warp; ch < nchunks; ch += nw) {
-        const uint32_t pid0 = (uint32_t)((uint64_t)ch * kWChunk) + r0;
-        const unsigned long long run = noff;
-        uint32_t res[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k)
-            res[k] = nres[k];
-        fetch(ch + nw);
-        // pairs (low 32 bits) and multi-disk points (high 32 bits) of this
-        // lane's rows, for one scan; a multi-disk row keeps kResMulti | count
-        unsigned long long mine = 0;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const uint32_t r = res[k];
-            if (r == kResNone)
-                continue;
-            uint32_t c = 1;
-            if (r & kResMulti) {
-                if (r & kResCount) {
-                    c = (r >> 20) & 0x3ffu;
-                } else { // count not stored: count again
-                    const int2 p = a.pts[pid0 + k];
-                    uint32_t f = 0, t = 0;
-                    c = disk_walk(a.dv, p.x, p.y, f, t, keep, [](uint32_t) {});
-                }
-                res[k] = kResMulti | c;
-                mine += 1ull << 32;
-            }
-            mine += c;
-        }
-        unsigned long long inc = mine;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long v = __shfl_up_sync(kFull, inc, o);
-            if (lane >= o)
-                inc += v;
-        }
-        const unsigned long long tot = __shfl_sync(kFull, inc, 31), before = inc - mine;
-        if (mine) {
-            unsigned long long o = run + (uint32_t)before;
-            uint32_t slot = qn + (uint32_t)(before >> 32);
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const uint32_t r = res[k];
-                if (r == kResNone)
-                    continue;
-                if (r & kResMulti) {
-                    s_q[slot] = pid0 + k;
-                    s_o[slot] = o;
-                    ++slot;
-                    o += r & ~kResMulti;
-                } else {
-                    if (o < a.cap)
-                        __stcs(a.pairs + o, make_uint2(pid0 + k, r));
-                    ++o;
-                }
-            }
-        }
-        qn += (uint32_t)(tot >> 32);
-        __syncwarp();
-        if (qn >= 32) {
-            uint32_t k0 = 0;
-            for (; qn - k0 >= 32; k0 += 32)
-                walk(k0, 32);
-            // move the partial round (< 32, from k0 >= 32) to the front
-            const uint32_t rem = qn - k0;
-            uint32_t q = 0;
-            unsigned long long oo = 0;
-            if ((uint32_t)lane < rem) {
-                q = s_q[k0 + lane];
-                oo = s_o[k0 + lane];
-            }
-            __syncwarp();
-            if ((uint32_t)lane < rem) {
-                s_q[lane] = q;
-                s_o[lane] = oo;
-            }
-            qn = rem;
-            __syncwarp();
-        }
-    }
-    __syncwarp();
-    walk(0, qn);
 }
 
 // ------------------------------------------------------ disk index, built on the device
@@ -3284,13 +3148,14 @@ cudaError_t launch_join_emit(const JoinLaunch &a, cudaStream_t s, const uint32_t
     if (a.narrow && !pend)
         return cudaErrorInvalidValue;
     const uint32_t nblk = (nchunks + kWarps - 1) / kWarps;
-    static bool done[8][64] = {};
-    return with_switches(a, [&](auto fp32, auto near) -> cudaError_t {
-        constexpr bool F = decltype(fp32)::value, N = decltype(near)::value;
+    static bool done[12][64] = {};
+    return with_switches(a, [&](auto fp32, auto kind) -> cudaError_t {
+        constexpr bool F = decltype(fp32)::value;
+        constexpr int N = decltype(kind)::value;
         auto kn = k_wemit16<F, false, N>;
         auto kw = k_wemit<F, N>;
         const cudaError_t e = a.narrow ? smem_opt_in(kn, kEmit16Smem, done[F + 2 * N])
-                                       : smem_opt_in(kw, kEmitSmem, done[4 + F + 2 * N]);
+                                       : smem_opt_in(kw, kEmitSmem, done[6 + F + 2 * N]);
         if (e != cudaSuccess)
             return e;
         if (a.narrow)
@@ -3304,22 +3169,22 @@ cudaError_t launch_join_emit(const JoinLaunch &a, cudaStream_t s, const uint32_t
 // The join of a small table (at most kSmallChunks chunks, 16-bit results, with an
 // output): two
 // launches, k_small and k_wemit16<SELF>.  ev as for launch_join.
-template <bool FP32, bool NEAR>
+template <bool FP32, int KIND>
 static cudaError_t launch_small(const JoinLaunch &a, uint32_t *pend, cudaStream_t s, cudaEvent_t *ev)
 {
     static bool done[64] = {};
     const uint32_t nchunks = uint32_t((a.n + kWChunk - 1) / kWChunk), nblk = (nchunks + kWarps - 1) / kWarps;
     if (ev)
         cudaEventRecord(ev[0], s);
-    k_small<FP32, kOut16, NEAR><<<nblk, kThreads, 0, s>>>(a, pend, nchunks, a.ix.P <= kSmallHist ? 1 : 0);
+    k_small<FP32, kOut16, KIND><<<nblk, kThreads, 0, s>>>(a, pend, nchunks, a.ix.P <= kSmallHist ? 1 : 0);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess)
-        e = smem_opt_in(k_wemit16<FP32, true, NEAR>, kEmit16Smem, done);
+        e = smem_opt_in(k_wemit16<FP32, true, KIND>, kEmit16Smem, done);
     if (e != cudaSuccess)
         return e;
     for (int k = 1; ev && k < 4; ++k)
         cudaEventRecord(ev[k], s);
-    k_wemit16<FP32, true, NEAR><<<nblk, kThreads, kEmit16Smem, s>>>(a, a.tile_tot, nchunks, pend);
+    k_wemit16<FP32, true, KIND><<<nblk, kThreads, kEmit16Smem, s>>>(a, a.tile_tot, nchunks, pend);
     return cudaGetLastError();
 }
 
@@ -3667,8 +3532,9 @@ cudaError_t launch_join(const JoinLaunch &a, void *scratch, cudaStream_t s, cuda
         if (a.counts && a.ix.P && !a.keep_counts)
             if ((e = cudaMemsetAsync(a.counts, 0, sizeof(unsigned long long) * a.ix.P, s)) != cudaSuccess)
                 return e;
-        e = with_switches(b, [&](auto fp32, auto near) {
-            constexpr bool F = decltype(fp32)::value, N = decltype(near)::value;
+        e = with_switches(b, [&](auto fp32, auto kind) {
+            constexpr bool F = decltype(fp32)::value;
+        constexpr int N = decltype(kind)::value;
             return launch_small<F, N>(b, pend, s, ev);
         });
         if (ev)
@@ -3701,7 +3567,7 @@ bool use_directory(const JoinLaunch &a)
 constexpr uint64_t kSplitCountMin = uint64_t(1) << 21;
 bool use_split_count(const JoinLaunch &a)
 {
-    return a.n > kSplitCountMin && (a.near.rad || (!a.clustered && a.ix.use_sum));
+    return a.n > kSplitCountMin && (a.near.any() || (!a.clustered && a.ix.use_sum));
 }
 
 static size_t split_count_bytes(uint64_t n)
@@ -3711,8 +3577,8 @@ static size_t split_count_bytes(uint64_t n)
 
 size_t aggregate_scratch_bytes(const JoinLaunch &a)
 {
-    return use_directory(a) && !a.near.rad ? size_t((a.n + kWChunk - 1) / kWChunk) * kWItems * 4
-           : !a.clustered || a.near.rad    ? split_count_bytes(a.n)
+    return use_directory(a) && !a.near.any() ? size_t((a.n + kWChunk - 1) / kWChunk) * kWItems * 4
+           : !a.clustered || a.near.any() ? split_count_bytes(a.n)
                                            : 0;
 }
 
@@ -3734,17 +3600,18 @@ cudaError_t launch_aggregate(const JoinLaunch &a, void *scratch, cudaStream_t s,
             cudaEventRecord(ev[1], s);
         return e;
     }
-    if (a.near.rad) { // few points, or no scratch to have: one launch that keeps nothing
+    if (a.near.any()) { // few points, or no scratch to have: one launch that keeps nothing
         const uint64_t nchunks = (a.n + kWChunk - 1) / kWChunk;
         if (a.n >= (1ull << 32))
             return cudaErrorInvalidValue;
         const unsigned nblk = unsigned((nchunks + kWarps - 1) / kWarps);
         const int hist = a.ix.P <= kSmallHist ? 1 : 0;
-        if (a.fp32)
-            k_small<true, kOutCount, true><<<nblk, kThreads, 0, s>>>(a, nullptr, uint32_t(nchunks), hist);
-        else
-            k_small<false, kOutCount, true><<<nblk, kThreads, 0, s>>>(a, nullptr, uint32_t(nchunks), hist);
-        return cudaGetLastError();
+        return with_switches(a, [&](auto fp32, auto kind) {
+            if constexpr (decltype(kind)::value != kPoly)
+                k_small<decltype(fp32)::value, kOutCount, decltype(kind)::value>
+                    <<<nblk, kThreads, 0, s>>>(a, nullptr, uint32_t(nchunks), hist);
+            return cudaGetLastError();
+        });
     }
     const int use_hist = a.ix.P <= (uint32_t)kHistMax ? 1 : 0;
     if (ev)
@@ -3770,9 +3637,9 @@ cudaError_t launch_aggregate(const JoinLaunch &a, void *scratch, cudaStream_t s,
     return e;
 }
 
-size_t select_scratch_bytes(uint64_t n, uint32_t P, uint64_t cap)
+size_t select_scratch_bytes(uint64_t n, uint32_t P, uint64_t cap, bool aux)
 {
-    return ((join_scratch_bytes(n) + 15) & ~size_t(15)) + n * 8 + 16 + cap * 8 + partition_scratch_bytes(cap, P);
+    return ((join_scratch_bytes(n) + 15) & ~size_t(15)) + (aux ? n * 8 : 0) + 16 + cap * 8 + partition_scratch_bytes(cap, P);
 }
 
 size_t partition_scratch_bytes(uint64_t cap, uint32_t P)
@@ -3816,7 +3683,7 @@ cudaError_t launch_partition(const uint2 *pairs, const unsigned long long *total
 }
 
 cudaError_t launch_select(const JoinLaunch &a, uint32_t *ids, uint64_t cap, unsigned long long *offsets,
-                          void *scratch, cudaStream_t s)
+                          void *scratch, cudaStream_t s, bool with_aux)
 {
     if (a.ix.P > (uint32_t)kSelMaxQ)
         return cudaErrorInvalidValue;
@@ -3825,8 +3692,8 @@ cudaError_t launch_select(const JoinLaunch &a, uint32_t *ids, uint64_t cap, unsi
     sc += (join_scratch_bytes(a.n) + 15) & ~size_t(15);
     // overlapping queries put many points in several polygons: pass 1b packs
     // their ids so that pass 3 does not walk them again
-    uint64_t *aux = reinterpret_cast<uint64_t *>(sc);
-    sc += a.n * 8;
+    uint64_t *aux = with_aux ? reinterpret_cast<uint64_t *>(sc) : nullptr;
+    sc += with_aux ? a.n * 8 : 0;
     unsigned long long *total = reinterpret_cast<unsigned long long *>(sc);
     sc += 16;
     uint2 *pairs = reinterpret_cast<uint2 *>(sc);
@@ -3986,105 +3853,6 @@ cudaError_t launch_plain_write(const JoinLaunch &a, void *scratch, cudaStream_t 
         return cudaSuccess;
     k_plain_write<<<(unsigned)nb, kPlainThreads, 0, s>>>(a, static_cast<const unsigned long long *>(scratch));
     return cudaGetLastError();
-}
-
-// ------------------------------------------------------ distance-query launchers
-template <bool RESOLVE>
-cudaError_t launch_dwarp(const DiskLaunch &a, unsigned long long *tot, uint32_t *res, uint32_t nchunks,
-                         cudaStream_t s)
-{
-    static bool done[64] = {};
-    const int use_hist = a.counts && a.dv.Q <= (uint32_t)kHistMax;
-    const size_t fixed = kDWarpSmem + sizeof(uint32_t) * kDiskCoverWords;
-    const size_t smem = fixed + (use_hist ? sizeof(uint32_t) * a.dv.Q : 0);
-    auto kern = k_dwarp<RESOLVE>;
-    cudaError_t e = smem_opt_in(kern, fixed + sizeof(uint32_t) * kHistMax, done);
-    if (e != cudaSuccess)
-        return e;
-    const uint32_t nblk = (nchunks + kWarps - 1) / kWarps;
-    kern<<<persistent_grid(kern, kThreads, smem, nblk), kThreads, smem, s>>>(a, tot, res, nchunks, use_hist);
-    return cudaGetLastError();
-}
-
-// The polygon join's scratch layout: per-point results | per-chunk totals
-// (then offsets) | scan partials.
-size_t disk_scratch_bytes(uint64_t n) { return join_scratch_bytes(n); }
-
-cudaError_t launch_disk_join(const DiskLaunch &a, void *scratch, cudaStream_t s, cudaEvent_t *ev)
-{
-    const uint64_t nchunks = (a.n + kWChunk - 1) / kWChunk;
-    if (nchunks >= (1ull << 31))
-        return cudaErrorInvalidValue;
-    cudaError_t e;
-    if (a.counts && a.dv.Q)
-        if ((e = cudaMemsetAsync(a.counts, 0, sizeof(unsigned long long) * a.dv.Q, s)) != cudaSuccess)
-            return e;
-    if (nchunks == 0)
-        return a.total ? cudaMemsetAsync(a.total, 0, sizeof(unsigned long long), s) : cudaSuccess;
-    char *sc = static_cast<char *>(scratch);
-    uint32_t *res = reinterpret_cast<uint32_t *>(sc);
-    unsigned long long *tot = reinterpret_cast<unsigned long long *>(sc + ((a.n * 4 + 15) & ~uint64_t(15)));
-    unsigned long long *part = tot + nchunks;
-    const uint32_t nblk = uint32_t((nchunks + kWarps - 1) / kWarps);
-    if (ev)
-        cudaEventRecord(ev[0], s);
-    if ((e = launch_dwarp<true>(a, tot, res, uint32_t(nchunks), s)) != cudaSuccess)
-        return e;
-    if (ev)
-        cudaEventRecord(ev[1], s);
-    if ((e = launch_scan(tot, nchunks, a.total, part, s)) != cudaSuccess)
-        return e;
-    if (ev)
-        cudaEventRecord(ev[2], s);
-    if (a.cap) {
-        static bool done[64] = {};
-        if ((e = smem_opt_in(k_dwemit, kDEmitSmem, done)) != cudaSuccess)
-            return e;
-        k_dwemit<<<persistent_grid(k_dwemit, kThreads, kDEmitSmem, nblk), kThreads, kDEmitSmem, s>>>(
-            a, tot, res, uint32_t(nchunks));
-    }
-    if (ev)
-        cudaEventRecord(ev[3], s);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_disk_aggregate(const DiskLaunch &a, cudaStream_t s)
-{
-    const uint64_t nchunks = (a.n + kWChunk - 1) / kWChunk;
-    if (nchunks >= (1ull << 31))
-        return cudaErrorInvalidValue;
-    cudaError_t e = cudaMemsetAsync(a.counts, 0, sizeof(unsigned long long) * (a.dv.Q ? a.dv.Q : 1), s);
-    if (e != cudaSuccess || nchunks == 0)
-        return e;
-    return launch_dwarp<false>(a, nullptr, nullptr, uint32_t(nchunks), s);
-}
-
-size_t disk_select_scratch_bytes(uint64_t n, uint32_t Q, uint64_t cap)
-{
-    return ((disk_scratch_bytes(n) + 15) & ~size_t(15)) + 16 + cap * 8 + partition_scratch_bytes(cap, Q);
-}
-
-cudaError_t launch_disk_select(const DiskLaunch &a, uint32_t *ids, uint64_t cap, unsigned long long *offsets,
-                               void *scratch, cudaStream_t s)
-{
-    if (a.dv.Q > (uint32_t)kSelMaxQ)
-        return cudaErrorInvalidValue;
-    char *sc = static_cast<char *>(scratch);
-    void *join_scratch = sc;
-    sc += (disk_scratch_bytes(a.n) + 15) & ~size_t(15);
-    unsigned long long *total = reinterpret_cast<unsigned long long *>(sc);
-    sc += 16;
-    uint2 *pairs = reinterpret_cast<uint2 *>(sc);
-    sc += cap * 8;
-    DiskLaunch b = a;
-    b.pairs = pairs;
-    b.cap = cap;
-    b.counts = nullptr;
-    b.total = total;
-    cudaError_t e = launch_disk_join(b, join_scratch, s, nullptr);
-    if (e != cudaSuccess)
-        return e;
-    return launch_partition(pairs, total, cap, a.dv.Q, ids, offsets, sc, s);
 }
 
 // ------------------------------------------------ buffered polygons: launchers
@@ -4309,14 +4077,14 @@ __global__ void __launch_bounds__(256) k_near_fine(IndexView in, const uint32_t 
 }
 
 // Block summary of the coarse words (an empty block, one polygon holding it, or
-// mixed), the number of blocks that are not mixed, and the sentinels.
+// mixed), the number of blocks that are not mixed, and (not null) the sentinels.
 __global__ void __launch_bounds__(256) k_near_sum(int g, int sg, const uint32_t *cell, uint16_t *sum,
                                                   unsigned long long *resolved, uint4 *ent_end, int4 *edge_end)
 {
     const uint32_t nb = 1u << sg, sh = uint32_t(g - sg), t = blockIdx.x * 256 + threadIdx.x;
-    if (t < 4)
+    if (ent_end && t < 4)
         ent_end[t] = make_uint4(0u, 0u, 0u, kEntLast);
-    if (t == 0)
+    if (edge_end && t == 0)
         *edge_end = make_int4(0, 0, 0, 0);
     if (t >= nb * nb)
         return;
@@ -4440,6 +4208,34 @@ int build_near_index_device(const IndexView &in, const uint32_t *cell_off, const
         out.sum_resolved = double(h[4]) / double(uint64_t(1) << (2 * sg));
         return done(0);
     }
+}
+
+// A disk index's lists hang from its coarse words directly: kind kCellCoarseList.
+__global__ void __launch_bounds__(256) k_disk_words(uint32_t ncell, uint32_t *cell)
+{
+    for (uint32_t c = blockIdx.x * 256 + threadIdx.x; c < ncell; c += gridDim.x * 256)
+        if ((cell[c] >> 30) == kCellList)
+            cell[c] |= kCellCoarseList << 30;
+}
+
+cudaError_t prepare_disk_words(uint32_t *cell, int g, uint16_t *sum, double *sum_resolved)
+{
+    const uint32_t ncell = 1u << (2 * g);
+    const int sg = std::min(g, kSumLog2);
+    unsigned long long *n = nullptr, h = 0;
+    cudaError_t e = cudaMalloc(&n, 8);
+    if (e != cudaSuccess)
+        return e;
+    if ((e = cudaMemset(n, 0, 8)) == cudaSuccess) {
+        k_disk_words<<<std::min<uint32_t>((ncell + 255) / 256, uint32_t(device_sm_count()) * 32), 256>>>(ncell, cell);
+        k_near_sum<<<((1u << (2 * sg)) + 255) / 256, 256>>>(g, sg, cell, sum, n, nullptr, nullptr);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess)
+        e = cudaMemcpy(&h, n, 8, cudaMemcpyDeviceToHost);
+    cudaFree(n);
+    *sum_resolved = double(h) / double(uint64_t(1) << (2 * sg));
+    return e;
 }
 
 } // namespace spx

@@ -50,9 +50,14 @@ constexpr uint32_t kLocalEdge = 0x80000000u;
 // cell (kEntBoundary), not a crossing list.  kEntCross: the polygon's boundary
 // may also cross the cell, so that a point far from those edges still asks the
 // polygons' own index `in`.
+// A disk index is one too: its words are those of DiskView with kCellCoarseList
+// for lists, whose offsets point into dent.
 struct NearView {
     const int32_t *rad; // P radii, each in [0, 2^30); null: not a buffered index
     IndexView in;
+    const int4 *disk; // null: not a disk index
+    const uint32_t *dent;
+    __host__ __device__ bool any() const { return rad || disk; }
 };
 constexpr uint32_t kEntCross = 4u;
 constexpr uint32_t kCellCoarseList = 3u;
@@ -78,30 +83,6 @@ struct DiskView {
     int cg;  // min(g, kCoverLog2)
 };
 
-struct DiskLaunch {
-    DiskView dv;
-    const int2 *pts;
-    uint64_t n;
-    uint2 *pairs; // may be null when cap == 0
-    uint64_t cap;
-    unsigned long long *counts; // Q entries or null; zeroed by the launchers
-    unsigned long long *total;  // device total or null
-    unsigned long long *stats;
-};
-
-// Distance join: pairs (point, disk) with distance <= r, in (point, disk)
-// order, counts, total.  scratch: disk_scratch_bytes(n).  ev (or null): four
-// events recorded before pass 1, before the scan, before pass 3 and after it.
-size_t disk_scratch_bytes(uint64_t n);
-cudaError_t launch_disk_join(const DiskLaunch &a, void *scratch, cudaStream_t s, cudaEvent_t *ev);
-// Counts only.
-cudaError_t launch_disk_aggregate(const DiskLaunch &a, cudaStream_t s);
-// Per-disk ascending point-id lists (the selection); scratch:
-// disk_select_scratch_bytes(n, Q, cap).
-size_t disk_select_scratch_bytes(uint64_t n, uint32_t Q, uint64_t cap);
-cudaError_t launch_disk_select(const DiskLaunch &a, uint32_t *ids, uint64_t cap, unsigned long long *offsets,
-                               void *scratch, cudaStream_t s);
-
 // Device build of the disk index of Q disks (host array of (cx, cy, r, 0),
 // already checked) on a 2^g grid: the same cell words and entries as the host
 // build (build_disk_index) and the same cover bitmap, in one new device
@@ -118,6 +99,11 @@ struct DiskIndexDev {
     uint64_t n_ent, n_inside, n_boundary;
 };
 int build_disk_index_device(const int4 *disks_host, uint32_t Q, int g, DiskIndexDev &out, cudaError_t &cerr);
+
+// Turns the lists of a disk index's words (2^g grid, in place) into
+// kCellCoarseList, and writes their block summary (4^min(g, kSumLog2) words) and
+// the fraction of it that is not mixed.  Legacy default stream, synchronises.
+cudaError_t prepare_disk_words(uint32_t *cell, int g, uint16_t *sum, double *sum_resolved);
 
 // Device status word bits (ORed into the ctx's persistent error word).
 constexpr unsigned kErrTimeout = 1u;   // a bounded wait (for a bulk copy) gave up
@@ -160,7 +146,7 @@ struct JoinLaunch {
     // holds, so that pass 3 writes its pairs without walking its list again
     uint64_t *aux;
     int aux_bits;
-    NearView near; // near.rad set: ix is a buffered-polygon index
+    NearView near; // near.rad or near.disk set: ix is an index of buffered polygons or of disks
 };
 
 // Shortens the edge lists of a built polygon index where they are long, in place
@@ -230,9 +216,9 @@ cudaError_t launch_aggregate(const JoinLaunch &a, void *scratch, cudaStream_t s,
 // Batched selection: per-query ascending point-id lists in ids (cap entries),
 // offsets[q] / offsets[P] (device, P + 1 values; offsets[P] = total).  At most
 // 1024 queries per index.  scratch: select_scratch_bytes(n, P, cap).
-size_t select_scratch_bytes(uint64_t n, uint32_t P, uint64_t cap);
+size_t select_scratch_bytes(uint64_t n, uint32_t P, uint64_t cap, bool aux);
 cudaError_t launch_select(const JoinLaunch &a, uint32_t *ids, uint64_t cap, unsigned long long *offsets,
-                          void *scratch, cudaStream_t s);
+                          void *scratch, cudaStream_t s, bool aux);
 constexpr uint32_t kSelectMaxQueries = 1024;
 
 // Stable partition of (point, query) pairs (point order) by query: ids[] gets
