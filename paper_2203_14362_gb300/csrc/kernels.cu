@@ -776,6 +776,19 @@ __device__ __forceinline__ void add_stats(unsigned long long *stats, uint32_t pt
     }
 }
 
+template <class K>
+int persistent_grid(K kernel, int threads, size_t smem, uint32_t ntiles)
+{
+    int per_sm = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
+    if (per_sm < 1)
+        per_sm = 1;
+    int grid = per_sm * device_sm_count();
+    if ((uint32_t)grid > ntiles)
+        grid = (int)ntiles;
+    return grid;
+}
+
 // ------------------------------------------------------- plain comparison join
 // Exact int64 only; one thread per point; pass 1 counts per 256-point block,
 // a one-block scan makes block offsets, pass 2 recounts and writes.  Counts by
@@ -1109,19 +1122,9 @@ constexpr int kWalkMinBlocks = SPX_WALK_MIN_BLOCKS;
 #ifndef SPX_WALK_BATCH
 #define SPX_WALK_BATCH 4
 #endif
+constexpr uint32_t kWalkGroups = 16;
 constexpr int kWalkBatch = SPX_WALK_BATCH; // rounds of rows resolved at a time
 constexpr int kWalkQueue = 32 * (kWalkBatch + 1); // < 32 carried over + a batch; or a batch less one + a gather step
-// A warp's range: short enough that a small table's words fill the chip twice
-// over (1M points: 61 warps of 512 words took 20.3 us, 977 of 32 take 7.5; 3M:
-// 22.7 -> 14.0), at most 512 (100M points: within 2 us from 256 to 1024).
-constexpr int kWalkRangeMax = 512, kWalkRangeMin = 32; // bitmap words (of 32 rows) per warp of pass 1b
-uint32_t walk_range(uint64_t nwords)
-{
-    const uint64_t warps = 2ull * kWalkMinBlocks * kWarps * uint64_t(device_sm_count());
-    const uint64_t r = (nwords / warps + 31) & ~uint64_t(31); // whole steps of a lane per word
-    return uint32_t(std::min<uint64_t>(std::max<uint64_t>(r, kWalkRangeMin), kWalkRangeMax));
-}
-
 // With the block summary (SUM), a CTA of 1024 threads (one per SM) first
 // copies the summary into shared memory; a point whose block is empty or
 // INSIDE one polygon is resolved there and reads no index word.  Random
@@ -1599,8 +1602,17 @@ __global__ void __launch_bounds__(kThreads, KIND == kNear ? 3 : kWalkMinBlocks) 
 template <bool FP32, int OUT, int KIND, bool ALL = false>
 cudaError_t launch_walk(const JoinLaunch &a, uint32_t *pend, cudaStream_t s)
 {
-    const uint64_t nwords = (a.n + kWChunk - 1) / kWChunk * kWItems, per_cta = uint64_t(kWarps) * walk_range(nwords);
-    k_walk<FP32, OUT, KIND, ALL><<<unsigned((nwords + per_cta - 1) / per_cta), kThreads, 0, s>>>(a, pend, uint32_t(nwords));
+    // a warp per group of 32 words, shared out by stride over what the chip holds
+    // at once (1M points: 61 warps of 512 words took 20.3 us, 977 of 32 take 7.5;
+    // 100M x 2000 cells: 1.8 waves 87 us, one 74), or over up to six times as many
+    // while a warp keeps kWalkGroups groups, which evens out long walks (500M x 256
+    // queries: one wave 3.15 ms, six 2.95)
+    const uint64_t nwords = (a.n + kWChunk - 1) / kWChunk * kWItems;
+    auto kern = k_walk<FP32, OUT, KIND, ALL>;
+    const uint32_t nblk = uint32_t((nwords + 32 * kWarps - 1) / (32 * kWarps));
+    const uint32_t wave = (uint32_t)persistent_grid(kern, kThreads, 0, nblk);
+    const uint32_t waves = std::min(std::max(nblk / (wave * kWalkGroups), 1u), 6u);
+    kern<<<std::min(nblk, wave * waves), kThreads, 0, s>>>(a, pend, uint32_t(nwords));
     return cudaGetLastError();
 }
 
@@ -2280,7 +2292,7 @@ constexpr int kSuperTileMax = 32768, kSuperTileMin = 1024;
 constexpr int kSelMaxQ = 1024;            // queries per index (shared-memory counters)
 constexpr int kPartTile = 4096;           // pairs that k_part_emit orders in shared memory at a time
 constexpr int kPartRounds = kPartTile / kThreads; // rounds of 32 pairs per warp and tile
-static_assert(kSelMaxQ == 4 * kThreads, "k_part_emit: four queries per thread");
+static_assert(kSelMaxQ == 4 * kThreads, "k_part_emit: at most four queries per thread");
 
 uint32_t super_tile(uint64_t cap)
 {
@@ -2337,7 +2349,8 @@ __global__ void __launch_bounds__(kThreads, 4) k_part_emit(const uint2 *__restri
     uint16_t *s_qy = reinterpret_cast<uint16_t *>(s_id + kPartTile);          // and their queries
     uint16_t *s_wc = s_qy + kPartTile;                                        // kWarps x P counts, then places
     __shared__ uint32_t s_wsum[kWarps];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, bits = 32 - __clz(P - 1); // of a query (P = 1: none)
+    const int kq = (P + kThreads - 1) / kThreads;
     const unsigned long long n = min(*total, (unsigned long long)cap); // pairs past cap were not written
     const uint64_t base = (uint64_t)blockIdx.x * tile;
     if (base >= n)
@@ -2364,7 +2377,15 @@ __global__ void __launch_bounds__(kThreads, 4) k_part_emit(const uint2 *__restri
             if (r * 32 >= span)
                 break;
             const bool has = w0 + r * 32 + lane < w1;
-            const uint32_t q = pr[r].y, peers = __match_any_sync(kFull, q);
+            // the lanes of the same query, from a vote per bit of it (a match per
+            // round, and 64 threads summing the warps' counts of 256 queries, took 827 us
+            // of 84M ids, this 610)
+            const uint32_t q = pr[r].y;
+            uint32_t peers = __ballot_sync(kFull, has);
+            for (int b = 0; b < bits; ++b) {
+                const uint32_t v = __ballot_sync(kFull, (q >> b) & 1u);
+                peers &= (q >> b) & 1u ? v : ~v;
+            }
             const uint32_t before = has ? wc[q] : 0u;
             __syncwarp();
             if (has && lane == __ffs(peers) - 1)
@@ -2374,12 +2395,12 @@ __global__ void __launch_bounds__(kThreads, 4) k_part_emit(const uint2 *__restri
         }
         __syncthreads();
         // 2. places: queries in order, within a query the warps in order
-        uint32_t c4[4], mine = 0;
+        uint32_t c4[4], mine = 0; // kq queries per thread
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const uint32_t q = threadIdx.x * 4 + k;
+            const uint32_t q = threadIdx.x * kq + k;
             c4[k] = 0;
-            if (q < P)
+            if (k < kq && q < P)
                 for (int w = 0; w < kWarps; ++w)
                     c4[k] += s_wc[w * P + q];
             mine += c4[k];
@@ -2399,8 +2420,8 @@ __global__ void __launch_bounds__(kThreads, 4) k_part_emit(const uint2 *__restri
             at += s_wsum[w];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const uint32_t q = threadIdx.x * 4 + k;
-            if (q < P) {
+            const uint32_t q = threadIdx.x * kq + k;
+            if (k < kq && q < P) {
                 s_off[q] = s_run[q] - at; // modulo 2^64: a place of the query is at or above `at`
                 s_run[q] += c4[k];
                 for (int w = 0; w < kWarps; ++w) {
@@ -2491,19 +2512,6 @@ cudaError_t smem_opt_in(K kernel, size_t bytes, bool (&done)[64])
     if (e == cudaSuccess && dev < 64)
         done[dev] = true;
     return e;
-}
-
-template <class K>
-int persistent_grid(K kernel, int threads, size_t smem, uint32_t ntiles)
-{
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem);
-    if (per_sm < 1)
-        per_sm = 1;
-    int grid = per_sm * device_sm_count();
-    if ((uint32_t)grid > ntiles)
-        grid = (int)ntiles;
-    return grid;
 }
 
 template <bool FP32, bool CLUSTERED>
