@@ -1628,7 +1628,7 @@ cudaError_t launch_walk(const JoinLaunch &a, uint32_t *pend, cudaStream_t s)
 constexpr uint32_t kSmallChunks = 4096;
 
 template <bool FP32, int OUT, int KIND>
-__global__ void __launch_bounds__(kThreads, 3) k_small(const __grid_constant__ JoinLaunch a, uint32_t *pend,
+__global__ void __launch_bounds__(kThreads, KIND == kNear ? 3 : 4) k_small(const __grid_constant__ JoinLaunch a, uint32_t *pend,
                                                        uint32_t nchunks, int use_hist)
 {
     __shared__ uint4 s_qa[kWarps * kWChunk]; // (x, y, first entry, row in the chunk)
