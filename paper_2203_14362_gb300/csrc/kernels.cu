@@ -2542,89 +2542,103 @@ cudaError_t launch_warp_kernel(const JoinLaunch &a, int use_hist, cudaStream_t s
     return cudaGetLastError();
 }
 
-// The directory stage of the count aggregate over a cell-clustered table: a
-// lane per cell of the directory grid (2^c, c >= g), kDirCells cells at a time.
-// A cell inside a coarse cell INSIDE one polygon adds its whole row range to
-// that polygon (its points need not be read); an empty one adds nothing; one in
-// a mixed coarse cell marks its rows in the bitmap, for k_walk<ALL>.  The points
-// of the cells counted here, and of the bin outside the box, go into the
-// scanned-points counter.  The stage reads 8 B per cell and a coarse word per
-// cell with points, kDirCells independent loads of each per lane.  2^26 cells,
-// 500M points: 656 us, and k_walk<ALL> 998 for the 34M marked rows; marking 256-row
-// chunks took 500, and the chunks, nearly all of them, 3020.
+// The directory stage of the count aggregate over a cell-clustered table (2^c
+// grid, c >= g).  A cell inside a coarse cell INSIDE one polygon adds its whole row
+// range to that polygon (its points need not be read); an empty one adds nothing;
+// one in a mixed coarse cell marks its rows in the bitmap, for k_walk<ALL>.  The
+// points of the cells counted here, and of the bin outside the box, go into the
+// scanned-points counter.  A warp takes strips of 32 columns and kDirRows rows, a
+// lane per column, kDirCells rows at a time: going down its column a lane stays in
+// one polygon for many rows and adds to that polygon's counter when it leaves it.
+// (32 neighbouring cells of a row mostly hold two polygons, and an atomic per cell
+// was two thirds of this stage: 2^26 cells and 40000 polygons, 656 -> 331 us; the
+// marks are most of the rest.)
 constexpr int kDirCells = 4;
+constexpr uint32_t kDirRows = 64;
 __global__ void __launch_bounds__(256) k_agg_cells(const unsigned long long *cell_end, int c, IndexView ix,
                                                    unsigned long long *counts, uint32_t *rows,
                                                    unsigned long long *stats)
 {
-    const uint32_t ncell = 1u << (2 * c), lane = threadIdx.x & 31;
+    const uint32_t side = 1u << c, lane = threadIdx.x & 31;
+    const uint32_t strips = (side + 31) / 32, bands = (side + kDirRows - 1) / kDirRows;
     const int sh = c - ix.gc;
     unsigned long long done_pts = 0;
-    for (uint32_t k0 = (blockIdx.x * 256 + (threadIdx.x & ~31u)) * kDirCells; k0 < ncell; k0 += gridDim.x * 256 * kDirCells) {
-        uint32_t s0[kDirCells], s1[kDirCells], w[kDirCells]; // a cell's rows [s0, s1) and its coarse word
+    for (uint32_t u = blockIdx.x * 8 + (threadIdx.x >> 5); u < strips * bands; u += gridDim.x * 8) {
+        const uint32_t x = (u % strips) * 32 + lane, y0 = (u / strips) * kDirRows, y1 = min(side, y0 + kDirRows);
+        uint32_t cur_q = 0, cur_n = 0; // this lane's polygon and its points so far
+        for (uint32_t yb = y0; yb < y1; yb += kDirCells) {
+            uint32_t s0[kDirCells], s1[kDirCells], w[kDirCells]; // a cell's rows [s0, s1) and its coarse word
 #pragma unroll
-        for (int j = 0; j < kDirCells; ++j) {
-            const uint32_t k = k0 + 32 * j + lane;
-            s1[j] = k < ncell ? (uint32_t)cell_end[k] : 0u;
-        }
-        uint32_t last = k0 ? (uint32_t)cell_end[k0 - 1] : 0u;
+            for (int j = 0; j < kDirCells; ++j) {
+                const uint32_t k = ((yb + j) << c) + x;
+                const bool in = x < side && yb + j < y1;
+                s1[j] = in ? (uint32_t)cell_end[k] : 0u;
+                s0[j] = in && lane == 0 && k ? (uint32_t)cell_end[k - 1] : 0u;
+            }
 #pragma unroll
-        for (int j = 0; j < kDirCells; ++j) {
-            const uint32_t up = __shfl_up_sync(kFull, s1[j], 1);
-            s0[j] = lane ? up : last;
-            last = __shfl_sync(kFull, s1[j], 31);
-            const uint32_t k = k0 + 32 * j + lane;
-            w[j] = 0;
-            if (s1[j] > s0[j])
-                w[j] = ix.cell[(((k >> c) >> sh) << ix.gc) | ((k & ((1u << c) - 1u)) >> sh)];
-        }
+            for (int j = 0; j < kDirCells; ++j) {
+                const uint32_t up = __shfl_up_sync(kFull, s1[j], 1);
+                s0[j] = lane ? up : s0[j];
+                w[j] = 0;
+                if (s1[j] > s0[j])
+                    w[j] = ix.cell[(((yb + j) >> sh) << ix.gc) | (x >> sh)];
+            }
 #pragma unroll
-        for (int j = 0; j < kDirCells; ++j) {
-            const uint32_t num = s1[j] > s0[j] ? s1[j] - s0[j] : 0u;
-            const uint32_t kind = w[j] >> 30, q = w[j] & kPayloadMask;
-            const bool sub = kind == kCellSub; // a cell without points has w = 0
-            const bool one = kind == kCellInsideOne && in_bounds(q < ix.P, ix);
-            done_pts += sub ? 0u : num;
-            // counts: one atomic for the warp when its cells share the polygon
-            const uint32_t m = __ballot_sync(kFull, one);
-            if (m) {
-                const uint32_t q0 = __shfl_sync(kFull, q, __ffs(m) - 1);
-                if (!__any_sync(kFull, one && q != q0)) {
-                    const uint32_t t = __reduce_add_sync(kFull, one ? num : 0u); // rows: below 2^32 in all
-                    if ((int)lane == __ffs(m) - 1)
-                        atomicAdd(counts + q0, (unsigned long long)t);
-                } else if (one) {
-                    atomicAdd(counts + q, (unsigned long long)num);
+            for (int j = 0; j < kDirCells; ++j) {
+                const uint32_t num = s1[j] > s0[j] ? s1[j] - s0[j] : 0u;
+                const uint32_t kind = w[j] >> 30, q = w[j] & kPayloadMask;
+                const bool sub = kind == kCellSub; // a cell without points has w = 0
+                done_pts += sub ? 0u : num;
+                if (kind == kCellInsideOne && in_bounds(q < ix.P, ix)) {
+                    if (q != cur_q) {
+                        if (cur_n)
+                            atomicAdd(counts + cur_q, (unsigned long long)cur_n);
+                        cur_q = q;
+                        cur_n = 0;
+                    }
+                    cur_n += num;
+                }
+                if (!__any_sync(kFull, sub))
+                    continue;
+                // rows of a cell in a mixed coarse cell; ranges over two words by the warp
+                const uint32_t r0 = s0[j], r1 = sub ? s1[j] - 1 : s0[j];
+                auto mark = [&](uint32_t wd, uint32_t a, uint32_t z) {
+                    const uint32_t lo = wd == (a >> 5) ? a & 31u : 0u, hi = wd == (z >> 5) ? z & 31u : 31u;
+                    if (hi - lo == 31)
+                        rows[wd] = 0xffffffffu; // no other cell's rows here
+                    else
+                        atomicOr(rows + wd, (0xffffffffu >> (31 - (hi - lo))) << lo);
+                };
+                const bool wide = (r1 >> 5) - (r0 >> 5) > 1;
+                if (sub && !wide) {
+                    mark(r0 >> 5, r0, r1);
+                    if ((r1 >> 5) != (r0 >> 5))
+                        mark(r1 >> 5, r0, r1);
+                }
+                for (uint32_t todo = __ballot_sync(kFull, sub && wide); todo; todo &= todo - 1) {
+                    const int src = __ffs(todo) - 1;
+                    const uint32_t a = __shfl_sync(kFull, r0, src), z = __shfl_sync(kFull, r1, src);
+                    for (uint32_t wd = (a >> 5) + lane; wd <= (z >> 5); wd += 32)
+                        mark(wd, a, z);
                 }
             }
-            if (!__any_sync(kFull, sub))
-                continue;
-            // rows of a cell in a mixed coarse cell; ranges over two words by the warp
-            const uint32_t r0 = s0[j], r1 = sub ? s1[j] - 1 : s0[j];
-            auto mark = [&](uint32_t wd, uint32_t a, uint32_t z) {
-                const uint32_t lo = wd == (a >> 5) ? a & 31u : 0u, hi = wd == (z >> 5) ? z & 31u : 31u;
-                if (hi - lo == 31)
-                    rows[wd] = 0xffffffffu; // no other cell's rows here
-                else
-                    atomicOr(rows + wd, (0xffffffffu >> (31 - (hi - lo))) << lo);
-            };
-            const bool wide = (r1 >> 5) - (r0 >> 5) > 1;
-            if (sub && !wide) {
-                mark(r0 >> 5, r0, r1);
-                if ((r1 >> 5) != (r0 >> 5))
-                    mark(r1 >> 5, r0, r1);
-            }
-            for (uint32_t todo = __ballot_sync(kFull, sub && wide); todo; todo &= todo - 1) {
-                const int src = __ffs(todo) - 1;
-                const uint32_t a = __shfl_sync(kFull, r0, src), z = __shfl_sync(kFull, r1, src);
-                for (uint32_t wd = (a >> 5) + lane; wd <= (z >> 5); wd += 32)
-                    mark(wd, a, z);
+        }
+        // the strip's last polygons: one atomic where the lanes share theirs
+        const uint32_t m = __ballot_sync(kFull, cur_n != 0);
+        if (m) {
+            const uint32_t q0 = __shfl_sync(kFull, cur_q, __ffs(m) - 1);
+            if (!__any_sync(kFull, cur_n && cur_q != q0)) {
+                const uint32_t t = __reduce_add_sync(kFull, cur_n); // rows: below 2^32 in all
+                if ((int)lane == __ffs(m) - 1)
+                    atomicAdd(counts + q0, (unsigned long long)t);
+            } else if (cur_n) {
+                atomicAdd(counts + cur_q, (unsigned long long)cur_n);
             }
         }
     }
     // the bin of points outside the box: in no polygon
     if (blockIdx.x == 0 && threadIdx.x == 0)
-        done_pts += cell_end[ncell] - cell_end[ncell - 1];
+        done_pts += cell_end[(size_t(1) << (2 * c))] - cell_end[(size_t(1) << (2 * c)) - 1];
     __shared__ unsigned long long s_done;
     if (threadIdx.x == 0)
         s_done = 0ull;
@@ -3647,8 +3661,8 @@ cudaError_t launch_aggregate(const JoinLaunch &a, void *scratch, cudaStream_t s,
         uint32_t *rows = static_cast<uint32_t *>(scratch);
         if ((e = cudaMemsetAsync(rows, 0, aggregate_scratch_bytes(a), s)) != cudaSuccess)
             return e;
-        const uint64_t ncell = uint64_t(1) << (2 * a.cluster_log2);
-        const unsigned grid = unsigned(std::min<uint64_t>((ncell + 256 * kDirCells - 1) / (256 * kDirCells), uint64_t(device_sm_count()) * 16));
+        const uint32_t side = 1u << a.cluster_log2, units = ((side + 31) / 32) * ((side + kDirRows - 1) / kDirRows);
+        const unsigned grid = std::min((units + 7) / 8, uint32_t(device_sm_count()) * 8);
         k_agg_cells<<<grid, 256, 0, s>>>(a.cell_end, a.cluster_log2, a.ix, a.counts, rows, a.stats);
         if ((e = cudaGetLastError()) != cudaSuccess)
             return e;
