@@ -1403,6 +1403,10 @@ spx_status spx_build_buffer_index(spx_ctx *ctx, spx_polys polys, const int32_t *
                                                   reinterpret_cast<int32_t *>(p_r), g, fx, e);
         if (built == 1) {
             drop();
+            // the offsets of a cell's entries have 30 bits; a coarser grid has
+            // fewer entries and gives the same answers
+            if (g > 1)
+                return spx_build_buffer_index(ctx, polys, r, g - 1, fp32_filter, out);
             return fail(ctx, SPX_EINVAL, "build_buffer_index: too many (cell, polygon) entries for 30-bit offsets; use "
                                          "a coarser edge grid");
         }

@@ -4219,7 +4219,12 @@ int build_near_index_device(const IndexView &in, const uint32_t *cell_off, const
         out.bytes = b_cell + b_fine + b_ent + b_edge + b_sum;
         if ((e = cudaMalloc(&out.mem, out.bytes)) != cudaSuccess) {
             out.mem = nullptr;
-            return done(2);
+            if (!sb)
+                return done(2);
+            cudaGetLastError();
+            cudaFree(tmp2);
+            tmp2 = nullptr;
+            continue;
         }
         char *m = static_cast<char *>(out.mem);
         out.cell = reinterpret_cast<uint32_t *>(m);
