@@ -95,7 +95,8 @@ spx_status spx_load_points(spx_ctx *ctx, const int32_t *xy, uint64_t n, int xy_i
  * is no finer than the clustering grid counts every cell that lies in a
  * coarse cell INSIDE one polygon from its range, without reading its points,
  * and reads only the points of cells in mixed coarse cells (§5.3: the blocks a
- * query needs).  Only spx_aggregate takes a clustered table -- per-polygon
+ * query needs; a bit per point of scratch from the ctx's pool, or without memory
+ * for it the whole copy).  Only spx_aggregate takes a clustered table -- per-polygon
  * counts do not depend on the order of the points; the join, the selection
  * and the server reject it with SPX_EINVAL (their outputs are keyed by row).
  * grid_log2 in [1, 13], 0 = 12.  Device memory: 8 B per point for the copy
@@ -141,7 +142,9 @@ typedef struct {
  * lower-left corner is inside.  params may be NULL (defaults: automatic grid,
  * FP32 filter on, sub_log2 3).  The index is built on the host (all cores) and
  * copied to the device; the polygon handle must stay alive while the index is
- * used.
+ * used.  Where the fine cells' edge lists are long (eight edges or more on
+ * average), the device also holds shorter lists local to the cells
+ * (device_bytes counts them; without memory for them the index works without).
  */
 spx_status spx_build_index(spx_ctx *ctx, spx_polys polys, const spx_index_params *params, spx_index *out);
 
@@ -155,9 +158,10 @@ spx_status spx_build_index(spx_ctx *ctx, spx_polys polys, const spx_index_params
  * the arrays are byte for byte those of spx_build_index with the same
  * parameters.  Same arguments, results and limits as spx_build_index.
  * Synchronous (the legacy default stream; the device is synchronised).
- * Temporary device memory is allocated and freed inside the call.  Errors:
- * SPX_EINVAL (bad handle or parameters, an index-format limit exceeded),
- * SPX_ENOMEM, SPX_ECUDA.
+ * Temporary device memory, and the index's own, come from a pool of the ctx,
+ * which keeps up to 4 GiB between calls (given back when another allocation of
+ * the ctx fails, and by spx_destroy).  Errors: SPX_EINVAL (bad handle or
+ * parameters, an index-format limit exceeded), SPX_ENOMEM, SPX_ECUDA.
  */
 spx_status spx_build_index_device(spx_ctx *ctx, spx_polys polys, const spx_index_params *params, spx_index *out);
 
@@ -251,19 +255,20 @@ spx_status spx_index_info_get(spx_ctx *ctx, spx_index index, spx_index_info *out
  * of its edges taken as a closed segment (a ring of one vertex: a disk),
  * decided exactly (int64, and 128-bit products for the distance to an edge's
  * interior).  The index holds the polygons' own grid index (automatic grid,
- * fp32_filter as given) and an edge grid of 2^grid_log2 cells per side
- * (0: cells of about a quarter of the median radius, or of the median edge
- * length when the radii are 0, clamped to 5..12) that lists, per cell, the
- * edges whose r-neighbourhood may reach it, by polygon; a polygon whose
- * r-region holds the whole cell keeps one flagged item and its points need
- * no test, and a bitmap of the cells that list edges or meet a polygon lets
- * the other points leave after one lookup.
+ * fp32_filter as given, which also filters the distance tests) and a grid of
+ * 2^grid_log2 cells per side (0: cells of about a quarter of the median radius,
+ * or of the median edge length when the radii are 0, clamped to 5..12), split
+ * into fine cells where needed, whose cells are empty, held whole by one
+ * polygon's region, or list their polygons: whole, or with the edges whose
+ * r-neighbourhood may reach the cell.
  * The returned index serves spx_join (pairs (point id, polygon id) in that
  * order, one per pair, counts per polygon), spx_select (at most 1024
  * polygons) and spx_aggregate; the other calls refuse it.  r: P host values,
  * copied.  The polygon handle must stay alive while the index is used.
  * Errors: SPX_EINVAL (bad handle, a radius out of range, grid_log2 outside
- * 0..12, an edge grid too large for 32-bit offsets), SPX_ENOMEM, SPX_ECUDA.
+ * 0..12, an edge grid too large for 32-bit offsets), SPX_ENOMEM, SPX_ECUDA.  A
+ * grid with more than 2^30 (cell, polygon) entries is built a level coarser
+ * (edge_grid_log2 of spx_index_info).
  */
 spx_status spx_build_buffer_index(spx_ctx *ctx, spx_polys polys, const int32_t *r, int grid_log2, int fp32_filter,
                                   spx_index *out);
@@ -275,7 +280,7 @@ typedef struct {
     int grid_max;           /* largest grid_log2 tried (default 13) */
     int reps;               /* timed launches per candidate, the fastest kept (default 5) */
     int fp32_filter;        /* filter setting of every candidate and of the result: 1 (default) or 0 */
-    uint64_t max_index_bytes; /* skip candidates whose index would exceed this (default 4 GiB) */
+    uint64_t max_index_bytes; /* skip candidates whose index (local lists aside) would exceed this (default 4 GiB) */
     int reserved[4];        /* must be zero */
 } spx_tune_params;
 
@@ -395,7 +400,9 @@ spx_status spx_join_plain_static(spx_ctx *ctx, spx_points points, spx_index inde
 /*
  * Count aggregation without materialising the join (§5.2 "Spatial
  * Aggregations", the plan for point data): counts_dev[q] (uint64, P entries,
- * device) = number of points inside polygon q.
+ * device) = number of points inside polygon q.  Large tables take a bit per point
+ * of scratch in the stream's order (none shared with other calls; a slower pass
+ * without it when there is no memory).
  */
 spx_status spx_aggregate(spx_ctx *ctx, spx_points points, spx_index index, uint64_t *counts_dev, void *stream);
 

@@ -15,15 +15,16 @@
 // from FP32 when |d_f| > 2^-21 (|t1| + |t2|) (forward error bound of the FP32
 // evaluation with a factor-2 margin), else from an exact int64 recomputation.
 //
-// The join is a cached two-pass Map (§5.1).  Pass 1 (k_warp) is persistent
-// and barrier-free: every warp takes its own 256-point chunks, resolves the
-// coarse and fine words of all its points with independent loads, queues the
-// few points whose fine cell holds an entry list in a per-warp shared-memory
-// queue and walks them 32 at a time, so the edge loops run converged; it
-// stores a 4-byte result per point and a pair total per chunk.  A device-wide
-// scan turns the totals into offsets, and pass 3 (k_wemit) writes each
-// chunk's pairs in point order.  The count aggregate is pass 1 alone.  Serving
-// batches (k_multi) and the selection partition (k_part_*) follow.
+// The join is a cached two-pass Map (§5.1), the same for polygons, buffered
+// polygons and disks.  Pass 1a (k_resolve_sum; k_resolve without the block
+// summary) is persistent and barrier-free: every warp takes its own 256-point
+// chunks, resolves their cells, stores a result per point (2 bytes up to 65534
+// polygons, else 4) and marks the rows whose cell holds an entry list; pass 1b
+// (k_walk) walks those lists 32 rows at a time.  A device-wide scan turns the
+// chunks' pair totals into offsets, and pass 3 (k_wemit16; k_wemit for 4-byte
+// results) writes each chunk's pairs in point order.  Small tables take one
+// pass-1 kernel (k_small).  The count aggregate is pass 1 alone, or k_warp.
+// Serving batches (k_multi) and the selection partition (k_part_*) follow.
 #include "kernels.h"
 #include "spx_internal.h"
 
@@ -3280,22 +3281,15 @@ __device__ __forceinline__ int edge_side(const int4 &v, const LocalCell &c)
     return fmaxf(xa, xb) + margin < 0.f ? 0 : 1;
 }
 
-// What the list of entry en becomes in cell c: its number of edges, and the
-// changes of parity (turn[0 .. nt), odd: the parity at y0); or en.z when it stays.
-__device__ __forceinline__ uint32_t local_size(const IndexView &ix, const uint4 &en, const LocalCell &c,
-                                               int (&turn)[kLocalTurns], int &nt, uint32_t &odd)
-{
-    nt = 0;
-    odd = 0;
-    if (!(en.w & kEntBoundary) || en.z < kLocalMin)
-        return en.z;
-    uint32_t near = 0;
-    for (uint32_t k = 0; k < en.z; ++k) {
-        const int4 v = ix.edge[en.y + k];
-        const int side = edge_side(v, c);
-        near += side == 1 ? 1u : 0u;
-        if (side != 2)
-            continue;
+// The parity of the right edges over the rows of a cell: at y0 (odd), and the y
+// where it changes.  add() is false when there are more changes than fit.
+struct LocalTurns {
+    int turn[kLocalTurns];
+    int nt = 0;
+    uint32_t odd = 0;
+
+    __device__ __forceinline__ bool add(const int4 &v, const LocalCell &c)
+    {
         odd ^= (v.y > c.y0) != (v.w > c.y0) ? 1u : 0u;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
@@ -3310,111 +3304,190 @@ __device__ __forceinline__ uint32_t local_size(const IndexView &ix, const uint4 
             else if (nt < kLocalTurns)
                 turn[nt++] = y;
             else
-                return en.z;
+                return false;
         }
+        return true;
     }
-    const uint32_t size = near + odd + (uint32_t)nt;
-    return size * 4 <= en.z * 3 ? size : en.z;
+};
+
+// The long lists and their cells: x entry, y and z the cell's corner, w what
+// k_local_size finds (kLocalChanged | changes << 27 | parity << 26 | kept edges; 0: stays).
+// Few cells hold one, and seldom two lanes of a warp, so the lists are gathered
+// first and then taken a lane each, four edges loaded at a time: 256 queries at
+// g = 13 take 1.5 (gathering) + 3.9 + 3.7 ms; with the lists walked where they were
+// found, a lane per cell, counting and writing took 4.8 + 12.4 ms.
+constexpr uint32_t kLocalChanged = 1u << 31;
+constexpr uint32_t kLocalMaxList = 1u << 26;
+
+__device__ __forceinline__ bool local_takes(const uint4 &en)
+{
+    return (en.w & kEntBoundary) && en.z >= kLocalMin && en.z < kLocalMaxList;
 }
 
-// A lane per fine cell.  COUNT: totals[0..1] += local edges, changed entries.
-// Else: the lists and the records of the changed entries, at places that each
-// warp takes from totals[0..1] (zeroed), in no particular order.
-template <bool COUNT>
-__global__ void __launch_bounds__(256) k_local(IndexView ix, const uint32_t *blk_cell, uint64_t n_words,
-                                               unsigned long long *totals, uint4 *ent, int4 *loc, uint4 *undo)
+// Edges k .. k + kLocalLoads - 1 of the list (past its end, the last one).
+constexpr uint32_t kLocalLoads = 4;
+
+__device__ __forceinline__ void load_list(const IndexView &ix, const uint4 &en, uint32_t k, int4 (&v)[kLocalLoads])
+{
+#pragma unroll
+    for (uint32_t u = 0; u < kLocalLoads; ++u)
+        v[u] = ix.edge[en.y + min(k + u, en.z - 1)];
+}
+
+// A lane per fine cell; *n_items counts (zeroed), in no particular order.
+__global__ void __launch_bounds__(256) k_local_items(IndexView ix, const uint32_t *blk_cell, uint64_t n_words, const uint4 *ent,
+                                                     unsigned long long *n_items, uint64_t cap, uint4 *items)
 {
     const int lane = threadIdx.x & 31;
-    unsigned long long all_loc = 0, all_ent = 0;
     for (uint64_t t0 = (uint64_t)blockIdx.x * 256 + (threadIdx.x & ~31u); t0 < n_words; t0 += (uint64_t)gridDim.x * 256) {
         const uint64_t t = t0 + lane;
         const uint32_t w = t < n_words ? ix.fine[t] : 0u;
         const bool lst = (w >> 30) == kCellList;
-        if (!__any_sync(kFull, lst))
-            continue;
-        LocalCell c{0, 0, 1 << ix.sf};
-        if (lst) {
-            const uint32_t cw = blk_cell[t >> (2 * ix.sb)], f = (uint32_t)t & ((1u << (2 * ix.sb)) - 1);
-            c.x0 = int(((cw & ((1u << ix.gc) - 1)) << ix.sc) | ((f & ((1u << ix.sb) - 1)) << ix.sf));
-            c.y0 = int(((cw >> ix.gc) << ix.sc) | ((f >> ix.sb) << ix.sf));
-        }
-        int turn[kLocalTurns], nt;
-        uint32_t odd, n_loc = 0, n_ent = 0;
+        uint32_t mine = 0;
         bool more = lst;
         for (uint64_t e = w & kPayloadMask; more; ++e) {
             const uint4 en = ent[e];
-            const uint32_t size = local_size(ix, en, c, turn, nt, odd);
-            n_loc += size < en.z ? size : 0u;
-            n_ent += size < en.z ? 1u : 0u;
+            mine += local_takes(en) ? 1u : 0u;
             more = !(en.w & kEntLast);
         }
-        all_loc += n_loc;
-        all_ent += n_ent;
-        if (COUNT || !__any_sync(kFull, n_ent != 0))
+        if (!__any_sync(kFull, mine != 0))
             continue;
-        unsigned long long inc = ((unsigned long long)n_ent << 40) | n_loc;
-        const unsigned long long mine = inc;
+        uint32_t inc = mine;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long v = __shfl_up_sync(kFull, inc, o);
-            if (lane >= o)
-                inc += v;
+            const uint32_t v = __shfl_up_sync(kFull, inc, o);
+            inc += lane >= o ? v : 0u;
         }
-        constexpr unsigned long long kLow = (1ull << 40) - 1;
-        unsigned long long at_loc = 0, at_ent = 0;
-        if (lane == 31) {
-            at_loc = atomicAdd(totals, inc & kLow);
-            at_ent = atomicAdd(totals + 1, inc >> 40);
-        }
-        at_loc = __shfl_sync(kFull, at_loc, 31) + ((inc - mine) & kLow);
-        at_ent = __shfl_sync(kFull, at_ent, 31) + ((inc - mine) >> 40);
-        more = n_ent != 0;
+        unsigned long long at = 0;
+        if (lane == 31)
+            at = atomicAdd(n_items, (unsigned long long)inc);
+        at = __shfl_sync(kFull, at, 31) + (inc - mine);
+        if (!mine)
+            continue;
+        const uint32_t cw = blk_cell[t >> (2 * ix.sb)], f = (uint32_t)t & ((1u << (2 * ix.sb)) - 1);
+        const uint32_t x0 = ((cw & ((1u << ix.gc) - 1)) << ix.sc) | ((f & ((1u << ix.sb) - 1)) << ix.sf);
+        const uint32_t y0 = ((cw >> ix.gc) << ix.sc) | ((f >> ix.sb) << ix.sf);
+        more = true;
         for (uint64_t e = w & kPayloadMask; more; ++e) {
             const uint4 en = ent[e];
             more = !(en.w & kEntLast);
-            const uint32_t size = local_size(ix, en, c, turn, nt, odd);
-            if (size >= en.z)
-                continue;
-            undo[at_ent++] = make_uint4((uint32_t)e, en.y, en.z, 0u);
-            int4 *d = loc + at_loc;
-            const int far = int(kBox);
-            if (odd)
-                *d++ = make_int4(far, c.y0, far, c.y0 + c.S);
-            for (int i = 0; i < nt; ++i)
-                *d++ = make_int4(far, turn[i], far, c.y0 + c.S);
-            for (uint32_t k = 0; k < en.z; ++k) { // in the list's order: right ends descending
-                const int4 v = ix.edge[en.y + k];
-                if (edge_side(v, c) == 1)
-                    *d++ = v;
-            }
-            ent[e].y = kLocalEdge | (uint32_t)at_loc;
-            ent[e].z = size;
-            at_loc += size;
-        }
-    }
-    if (COUNT) {
-        all_loc = warp_sum64(all_loc), all_ent = warp_sum64(all_ent);
-        if (lane == 0) {
-            atomicAdd(totals, all_loc);
-            atomicAdd(totals + 1, all_ent);
+            if (local_takes(en) && at < cap)
+                items[at++] = make_uint4((uint32_t)e, x0, y0, 0u);
         }
     }
 }
 
-// totals[0..1] += the edges that the entries list, and the entries that list any.
+// A lane per long list: items[].w, and totals[0..1] += local edges, changed lists.
+__global__ void __launch_bounds__(256) k_local_size(IndexView ix, const uint4 *ent, uint64_t n, uint4 *items,
+                                                    unsigned long long *totals)
+{
+    unsigned long long all_loc = 0, all_ent = 0;
+    for (uint64_t i = (uint64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (uint64_t)gridDim.x * 256) {
+        const uint4 it = items[i];
+        const uint4 en = ent[it.x];
+        const LocalCell c{int(it.y), int(it.z), 1 << ix.sf};
+        LocalTurns tn;
+        uint32_t near = 0;
+        bool fits = true;
+        for (uint32_t k = 0; k < en.z && fits; k += kLocalLoads) {
+            int4 v[kLocalLoads];
+            load_list(ix, en, k, v);
+#pragma unroll
+            for (uint32_t u = 0; u < kLocalLoads; ++u) {
+                const int side = k + u < en.z ? edge_side(v[u], c) : 0;
+                near += side == 1 ? 1u : 0u;
+                fits = fits && (side != 2 || tn.add(v[u], c));
+            }
+        }
+        const uint32_t size = near + tn.odd + (uint32_t)tn.nt;
+        if (fits && size * 4 <= en.z * 3) {
+            items[i].w = kLocalChanged | ((uint32_t)tn.nt << 27) | (tn.odd << 26) | near;
+            all_loc += size;
+            ++all_ent;
+        }
+    }
+    all_loc = warp_sum64(all_loc), all_ent = warp_sum64(all_ent);
+    if ((threadIdx.x & 31) == 0 && all_ent) {
+        atomicAdd(totals, all_loc);
+        atomicAdd(totals + 1, all_ent);
+    }
+}
+
+// A lane per long list: writes the changed ones and their records, at places that
+// each warp takes from totals[0..1] (zeroed), in no particular order.
+__global__ void __launch_bounds__(256) k_local_write(IndexView ix, uint4 *ent, uint64_t n, const uint4 *items,
+                                                     unsigned long long *totals, int4 *loc, uint4 *undo)
+{
+    const int lane = threadIdx.x & 31;
+    for (uint64_t i0 = (uint64_t)blockIdx.x * 256 + (threadIdx.x & ~31u); i0 < n; i0 += (uint64_t)gridDim.x * 256) {
+        const uint64_t i = i0 + lane;
+        const uint4 it = i < n ? items[i] : make_uint4(0u, 0u, 0u, 0u);
+        const bool take = it.w & kLocalChanged;
+        const uint32_t nt = (it.w >> 27) & 15u, odd = (it.w >> 26) & 1u;
+        const uint32_t size = take ? (it.w & (kLocalMaxList - 1)) + odd + nt : 0u;
+        const uint32_t b = __ballot_sync(kFull, take);
+        if (!b)
+            continue;
+        unsigned long long inc = size;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long v = __shfl_up_sync(kFull, inc, o);
+            inc += lane >= o ? v : 0ull;
+        }
+        unsigned long long at_loc = 0, at_ent = 0;
+        if (lane == 31) {
+            at_loc = atomicAdd(totals, inc);
+            at_ent = atomicAdd(totals + 1, (unsigned long long)__popc(b));
+        }
+        at_loc = __shfl_sync(kFull, at_loc, 31) + inc - size;
+        at_ent = __shfl_sync(kFull, at_ent, 31) + __popc(b & lanemask_lt());
+        if (!take)
+            continue;
+        const uint4 en = ent[it.x];
+        const LocalCell c{int(it.y), int(it.z), 1 << ix.sf};
+        LocalTurns tn;
+        int4 *d = loc + at_loc + odd + nt;
+        for (uint32_t k = 0; k < en.z; k += kLocalLoads) { // in the list's order: right ends descending
+            int4 v[kLocalLoads];
+            load_list(ix, en, k, v);
+#pragma unroll
+            for (uint32_t u = 0; u < kLocalLoads; ++u) {
+                const int side = k + u < en.z ? edge_side(v[u], c) : 0;
+                if (side == 1)
+                    *d++ = v[u];
+                else if (side == 2)
+                    tn.add(v[u], c);
+            }
+        }
+        const int far = int(kBox);
+        d = loc + at_loc;
+        if (odd)
+            *d++ = make_int4(far, c.y0, far, c.y0 + c.S);
+        for (uint32_t k = 0; k < nt; ++k)
+            *d++ = make_int4(far, tn.turn[k], far, c.y0 + c.S);
+        undo[at_ent] = make_uint4(it.x, en.y, en.z, 0u);
+        ent[it.x].y = kLocalEdge | (uint32_t)at_loc;
+        ent[it.x].z = size;
+    }
+}
+
+// totals[0..2] += the edges that the entries list, the entries that list any, and
+// the long lists among them.
 __global__ void __launch_bounds__(256) k_list_edges(const uint4 *ent, uint64_t n, unsigned long long *totals)
 {
-    unsigned long long z = 0, b = 0;
+    unsigned long long z = 0, b = 0, l = 0;
     for (uint64_t i = (uint64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (uint64_t)gridDim.x * 256) {
         const uint4 en = ent[i];
         const bool bnd = en.w & kEntBoundary;
         z += bnd ? en.z : 0u;
         b += bnd ? 1u : 0u;
+        l += local_takes(en) ? 1u : 0u;
     }
-    z = warp_sum64(z), b = warp_sum64(b);
+    z = warp_sum64(z), b = warp_sum64(b), l = warp_sum64(l);
     if ((threadIdx.x & 31) == 0) {
         atomicAdd(totals, z);
         atomicAdd(totals + 1, b);
+        atomicAdd(totals + 2, l);
     }
 }
 
@@ -3434,14 +3507,16 @@ cudaError_t build_local_lists(const IndexView &view, uint4 *ent, LocalLists &out
         return cudaSuccess;
     auto blocks = [](uint64_t n) { return unsigned(std::min<uint64_t>((n + 255) / 256, uint64_t(device_sm_count()) * 32)); };
     const size_t b_blk = (n_blk * 4 + 255) & ~size_t(255);
-    void *tmp = nullptr;
-    unsigned long long h[4] = {};
+    void *tmp = nullptr, *tmp2 = nullptr;
+    unsigned long long h[6] = {}; // local edges, changed lists, edges, lists, long lists, items
     cudaError_t e = cudaMallocFromPoolAsync(&tmp, b_blk + sizeof(h), pool, s);
     if (e != cudaSuccess) { // the index works without them
         cudaGetLastError();
         return cudaSuccess;
     }
     auto done = [&](cudaError_t err) {
+        if (tmp2)
+            cudaFreeAsync(tmp2, s);
         cudaFreeAsync(tmp, s);
         if (err != cudaSuccess && out.mem) {
             cudaFreeAsync(out.mem, s);
@@ -3458,17 +3533,30 @@ cudaError_t build_local_lists(const IndexView &view, uint4 *ent, LocalLists &out
     if ((e = cudaMemsetAsync(totals, 0, sizeof(h), s)) != cudaSuccess)
         return done(e);
     k_list_edges<<<blocks(view.n_ent), 256, 0, s>>>(ent, view.n_ent, totals + 2);
-    if ((e = cudaGetLastError()) != cudaSuccess || (e = read(4)) != cudaSuccess)
+    if ((e = cudaGetLastError()) != cudaSuccess || (e = read(5)) != cudaSuccess)
         return done(e);
     // Lists of four edges (maps of 500 to 5000 cells with about 500 vertices each)
     // gain nothing: 2000 cells, walk 81 us without, 92 with, and the build costs
     // 2 ms.  40 (queries of up to 5000 vertices) or 15 (40000 cells of up to 10000):
     // the walk of 500M points x 256 queries 4.39 -> 2.74 ms.
-    if (h[2] < kLocalMean * h[3])
+    if (h[2] < kLocalMean * h[3] || !h[4])
         return done(cudaSuccess);
+    if (cudaMallocFromPoolAsync(&tmp2, h[4] * 16, pool, s) != cudaSuccess) {
+        tmp2 = nullptr;
+        cudaGetLastError();
+        return done(cudaSuccess);
+    }
+    uint4 *items = static_cast<uint4 *>(tmp2);
+    const uint64_t cap = h[4];
     const uint32_t ncell = 1u << (2 * view.gc);
     k_blk_cell<<<blocks(ncell), 256, 0, s>>>(ncell, view.cell, blk_cell);
-    k_local<true><<<blocks(n_words), 256, 0, s>>>(view, blk_cell, n_words, totals, ent, nullptr, nullptr);
+    k_local_items<<<blocks(n_words), 256, 0, s>>>(view, blk_cell, n_words, ent, totals + 5, cap, items);
+    if ((e = cudaGetLastError()) != cudaSuccess || (e = read(6)) != cudaSuccess)
+        return done(e);
+    const uint64_t n_items = std::min<uint64_t>(h[5], cap);
+    if (!n_items)
+        return done(cudaSuccess);
+    k_local_size<<<blocks(n_items), 256, 0, s>>>(view, ent, n_items, items, totals);
     if ((e = cudaGetLastError()) != cudaSuccess || (e = read(2)) != cudaSuccess)
         return done(e);
     if (h[0] >= kLocalEdge || !h[1])
@@ -3487,7 +3575,7 @@ cudaError_t build_local_lists(const IndexView &view, uint4 *ent, LocalLists &out
     out.n_undo = h[1];
     if ((e = cudaMemsetAsync(totals, 0, 16, s)) != cudaSuccess)
         return done(e);
-    k_local<false><<<blocks(n_words), 256, 0, s>>>(view, blk_cell, n_words, totals, ent, loc, undo);
+    k_local_write<<<blocks(n_items), 256, 0, s>>>(view, ent, n_items, items, totals, loc, undo);
     if ((e = cudaGetLastError()) != cudaSuccess || (e = cudaStreamSynchronize(s)) != cudaSuccess)
         return done(e);
     return done(cudaSuccess);
