@@ -40,12 +40,12 @@ L2_BYTES = 129 * 1024 * 1024
 # results), scaled per point, keyed by the index's (grid_log2, sub_log2); only
 # valid for those kernel versions and the default workload.  A missing entry:
 # not captured.
-RESOLVE_TRAFFIC_BYTES_PER_POINT = {(12, 3): {"k_resolve": (272.762368e6 + 30.259712e6) / 20e6,
-                                             "k_walk": (62.574336e6 + 1.225728e6) / 20e6,
-                                             "k_wemit": (43.166720e6 + 98.548992e6) / 20e6}}
-# The same for the distance join's pass 1 (k_dwarp<resolve>), from one capture
-# of a 20M-point run of the 1024-disk workload at its default grid (g = 12).
-DISK_RESOLVE_TRAFFIC_BYTES_PER_POINT = (167.498496e6 + 25.302784e6) / 20e6
+RESOLVE_TRAFFIC_BYTES_PER_POINT = {(12, 3): {"k_resolve_sum": (268.1e6 + 29.26e6) / 20e6,
+                                             "k_walk": (61.11e6 + 1.40e6) / 20e6,
+                                             "k_wemit16": (43.18e6 + 100.5e6) / 20e6}}
+# The same for the distance join's pass 1a, from one capture of a 20M-point run
+# of the 1024-disk workload at its default grid (g = 12).
+DISK_RESOLVE_TRAFFIC_BYTES_PER_POINT = (164.3e6 + 6.44e6) / 20e6
 SERVE_SEED = 0x2203143620 + 4  # request indexes of the serving measurement
 
 
@@ -221,13 +221,13 @@ def sum_counts_over_ranks(counts, world: int):
 
 
 def join_launches(n: int, plain: bool, dist: bool = False) -> int:
-    """Kernels one spx_join launches: pass 1 (two kernels; the distance join:
-    one), the scan (one kernel up to 32768 values, else three), pass 3
-    (256-point chunks; plain: 256-point blocks and the one-block scan)."""
-    if plain:
+    """Kernels one spx_join launches: pass 1 (two kernels), the scan (one
+    kernel up to 32768 values, else three), pass 3 (256-point chunks; plain:
+    256-point blocks and the one-block scan); up to 4096 chunks, two in all."""
+    if plain and not dist:
         return 3
     chunks = (n + 255) // 256
-    return (2 if dist else 3) + (1 if chunks <= 4 * 8192 else 3)
+    return 2 if chunks <= 4096 else 3 + (1 if chunks <= 4 * 8192 else 3)
 
 
 def shard_start(rank: int, n_per_rank: int) -> int:
@@ -489,14 +489,12 @@ def run_spx(args, world, rank, local):
         dom, dom_ms, dom_bytes = "plain join (3 kernels)", ms, step_bytes
     else:
         cand = {"resolve": (phase_ms["resolve"], 8 * N + 8 * P + idx_bytes),
-                "emit": (phase_ms["emit"], 8 * n_pairs)}
-        if not dist:  # pass 1b re-reads what pass 1a read: no algorithmic bytes of its own
-            cand["walk"] = (phase_ms["walk"], 0)
+                "emit": (phase_ms["emit"], 8 * n_pairs),
+                "walk": (phase_ms["walk"], 0)}  # pass 1b re-reads what pass 1a read: no algorithmic bytes of its own
         key = max(cand, key=lambda k: cand[k][0])
         dom_ms, dom_bytes = cand[key]
-        names = {"resolve": "k_dwarp<resolve> (distance join pass 1)" if dist else "k_resolve (join pass 1a)",
-                 "walk": "k_walk (join pass 1b: exact tests)",
-                 "emit": "k_dwemit (distance join pass 3)" if dist else "k_wemit (join pass 3)"}
+        names = {"resolve": "k_resolve_sum (join pass 1a)" if info["use_sum"] else "k_resolve (join pass 1a)",
+                 "walk": "k_walk (join pass 1b: exact tests)", "emit": "k_wemit16 (join pass 3)"}
         dom = names[key]
     achieved = dom_bytes / (dom_ms * 1e-3) / 1e9
     traffic = args.traffic
@@ -504,7 +502,7 @@ def run_spx(args, world, rank, local):
             and (info["grid_log2"], info["sub_log2"]) in RESOLVE_TRAFFIC_BYTES_PER_POINT):
         per_pt = RESOLVE_TRAFFIC_BYTES_PER_POINT[(info["grid_log2"], info["sub_log2"])].get(dom.split(" ")[0])
         traffic = None if per_pt is None else per_pt * N
-    if traffic is None and dist and info["grid_log2"] == 12 and dom.startswith("k_dwarp"):
+    if traffic is None and dist and info["grid_log2"] == 12 and dom.startswith("k_resolve_sum"):
         traffic = DISK_RESOLVE_TRAFFIC_BYTES_PER_POINT * N
     out = None
     if rank == 0:
@@ -519,9 +517,8 @@ def run_spx(args, world, rank, local):
                 "workload": args.workload, "desc": desc, "points_per_gpu": N, "polygons": P,
                 "vertices": 0 if dist else int(v.shape[0]), "pairs": int(n_pairs), "grid_log2": info["grid_log2"],
                 "sub_log2": info["sub_log2"], "fp32_filter": bool(args.fp32),
-                "kernel": ("distance join: resolve (k_dwarp) + scan + emit (k_dwemit)" if dist else
-                           "plain two-pass" if args.plain else
-                           "resolve (k_resolve) + exact tests (k_walk) + scan + emit (k_wemit): cached two-pass Map"),
+                "kernel": ("plain two-pass" if args.plain and not dist else
+                           "resolve (k_resolve_sum) + exact tests (k_walk) + scan + emit (k_wemit16): cached two-pass Map"),
                 "index_build_ms": round(info["build_ms"], 1), "index_device_bytes": int(info["device_bytes"]),
                 "index_build_on_device_ms": None if device_build_ms is None else round(device_build_ms, 2),
                 "l2": "inputs larger than L2 (points 8 B x N + pairs 8 B x N >> 129 MB); no flush",
@@ -965,10 +962,10 @@ def count_measure(args, world, rank, local, torch, steps, warmup, n_override, e2
                    "l2": "inputs larger than L2 (32 GB of points); no flush"},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                      "traffic": None, "peak_source": f"{peak_kind} hbm_gbs",
-                     "kernel": ("k_agg_cells + k_warp<aggregate, directory>" if n_dir else "k_warp<aggregate>"),
+                     "kernel": ("k_agg_cells + k_walk<rows of mixed cells>" if n_dir else "k_warp<aggregate>"),
                      "kernel_ms": k_ms, "algorithmic_bytes_per_launch": int(alg),
                      "points_read": int(N - n_dir), "points_from_directory": int(n_dir)},
-        "cpu_baseline": cpu, "e2e": e2e_out, "gpu_launches": steps, "clocks": clk,
+        "cpu_baseline": cpu, "e2e": e2e_out, "gpu_launches": steps * (2 if n_dir else 1), "clocks": clk,
     }
     pr.close()
     eng.free(ih)
@@ -1140,10 +1137,10 @@ def buffer_measure(args, world, rank, local, torch, steps, warmup, n_override):
                    "l2": "inputs larger than L2 (0.8 GB of points); no flush"},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": None, "peak_source": f"{peak_kind} hbm_gbs",
-                     "kernel": "whole buffered join (k_buf_count, scan, k_buf_write)",
+                     "kernel": "whole buffered join (k_resolve_sum, k_walk, scan, k_wemit16)",
                      "algorithmic_bytes_per_launch": int(alg)},
         "cpu_baseline": cpu, "e2e": None, "clocks": clk,
-        "gpu_launches": steps * (2 + (1 if -(-N // 256) <= 4 * 8192 else 3)),
+        "gpu_launches": steps * join_launches(N, False),
     }
     eng.free(ih)
     eng.free(gh)
