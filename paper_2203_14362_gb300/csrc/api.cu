@@ -158,6 +158,13 @@ bool capturing(cudaStream_t s)
     return st != cudaStreamCaptureStatusNone;
 }
 
+// What the ctx's pool keeps goes back to the device.
+void give_back(spx_ctx *ctx)
+{
+    cudaStreamSynchronize(ctx->stream);
+    cudaMemPoolTrimTo(ctx->pool, 0);
+}
+
 // cudaMalloc; when there is no memory, what the ctx's pool keeps is given back
 // and the allocation tried once more.
 cudaError_t dev_alloc(spx_ctx *ctx, void **p, size_t bytes)
@@ -165,8 +172,7 @@ cudaError_t dev_alloc(spx_ctx *ctx, void **p, size_t bytes)
     cudaError_t e = cudaMalloc(p, bytes);
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();
-        cudaStreamSynchronize(ctx->stream);
-        cudaMemPoolTrimTo(ctx->pool, 0);
+        give_back(ctx);
         e = cudaMalloc(p, bytes);
     }
     return e;
@@ -607,6 +613,7 @@ spx_status served_data(spx_ctx *ctx, spx_points points, const spx_index *indexes
         return fail(ctx, SPX_EINVAL, "server: bad points handle");
     if (pts->cluster_log2)
         return fail(ctx, SPX_EINVAL, "server: a cell-clustered point table has no row order");
+    give_back(ctx); // the server allocates from the device and from a pool of its own
     out.device = ctx->device;
     out.pts = reinterpret_cast<const int2 *>(pts->dev);
     out.n = pts->n;
@@ -1187,7 +1194,7 @@ static spx_status register_disk_index(spx_ctx *ctx, void *mem, size_t total, con
     ix->mem = mem;
     ix->kind = 1;
     double resolved = 0;
-    cudaError_t e = cudaMalloc(&ix->mem2, size_t(2) << (2 * kSumLog2));
+    cudaError_t e = dev_alloc(ctx, &ix->mem2, size_t(2) << (2 * kSumLog2));
     if (e == cudaSuccess)
         e = prepare_disk_words(const_cast<uint32_t *>(cell), g, static_cast<uint16_t *>(ix->mem2), &resolved);
     if (e != cudaSuccess) {
@@ -1303,7 +1310,12 @@ spx_status spx_build_disk_index_device(spx_ctx *ctx, const int32_t *cxy, const i
     const std::vector<int4> disks = disk_array(cxy, r, Q);
     DiskIndexDev d{};
     cudaError_t e = cudaSuccess;
-    const int st = build_disk_index_device(disks.data(), Q, g, d, e);
+    int st = build_disk_index_device(disks.data(), Q, g, d, e);
+    if (st && e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        give_back(ctx);
+        st = build_disk_index_device(disks.data(), Q, g, d, e);
+    }
     if (st == 1)
         return fail(ctx, SPX_EINVAL, "build_disk_index_device: too many disk entries for one index; use a smaller grid");
     if (st != 0)
@@ -1360,6 +1372,7 @@ spx_status spx_build_buffer_index(spx_ctx *ctx, spx_polys polys, const int32_t *
     std::string err;
     if (!build_buffer_edges(pg->xy.data(), pg->off.data(), pg->P, r, g, he, err))
         return fail(ctx, SPX_EINVAL, "build_buffer_index: " + err);
+    give_back(ctx); // the build allocates from the device
     // the polygons' own index answers containment; it becomes part of this one
     spx_index_params prm{};
     prm.fp32_filter = fp32_filter ? 1 : 0;
@@ -1839,6 +1852,10 @@ spx_status spx_join_host(spx_ctx *ctx, const int32_t *xy_host, uint64_t n, spx_i
         // staged when the table, its results and the pairs fit in half the free device memory
         size_t fr = 0, tot = 0;
         cudaMemGetInfo(&fr, &tot);
+        uint64_t kept = 0, used = 0; // what the pool keeps counts as free: dev_alloc gives it back
+        cudaMemPoolGetAttribute(ctx->pool, cudaMemPoolAttrReservedMemCurrent, &kept);
+        cudaMemPoolGetAttribute(ctx->pool, cudaMemPoolAttrUsedMemCurrent, &used);
+        fr += kept - std::min(kept, used);
         const uint64_t staged = n * 8 + n * 4 + cap * 8 + (uint64_t(1) << 26);
         mode = (staged <= fr / 2 || !reach) ? 1 : 2;
     }
