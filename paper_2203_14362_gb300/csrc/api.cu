@@ -1416,6 +1416,10 @@ spx_status spx_build_buffer_index(spx_ctx *ctx, spx_polys polys, const int32_t *
         const int built = build_near_index_device(ix->view, reinterpret_cast<uint32_t *>(p_off),
                                                   reinterpret_cast<uint32_t *>(p_q), reinterpret_cast<int4 *>(p_seg),
                                                   reinterpret_cast<int32_t *>(p_r), g, fx, e);
+        if (built == 3) {
+            drop();
+            return fail(ctx, SPX_EKERNEL, "build_buffer_index: internal error: a list differs from its counted size");
+        }
         if (built == 1) {
             drop();
             // the offsets of a cell's entries have 30 bits; a coarser grid has

@@ -25,6 +25,7 @@
 // results) writes each chunk's pairs in point order.  Small tables take one
 // pass-1 kernel (k_small).  The count aggregate is pass 1 alone, or k_warp.
 // Serving batches (k_multi) and the selection partition (k_part_*) follow.
+#include "cell_filter.h"
 #include "kernels.h"
 #include "spx_internal.h"
 
@@ -449,65 +450,6 @@ __device__ __forceinline__ bool in_disk(const int4 &d, int px, int py)
     const long long dx = (long long)px - d.x, dy = (long long)py - d.y, rr = (long long)d.z * d.z;
     const long long dx2 = dx * dx;
     return dx2 <= rr && dx2 + dy * dy <= rr;
-}
-
-// Is (px, py) within distance r of the closed segment v = (a, b)?  With
-// d = b - a, w = p - a and t = w . d: the distance is |w| when t <= 0, |p - b|
-// when t >= |d|^2, else |d x w| / |d|.  Coordinates lie in [0, 2^30], so every
-// product of two differences is below 2^60 in magnitude (int64 sums stay
-// exact); the last case compares (d x w)^2 with r^2 |d|^2 as 128-bit
-// products.  A zero-length edge takes the first case.
-__device__ __noinline__ bool seg_near_exact(const int4 &v, int px, int py, int64_t r)
-{
-    const int64_t dx = (int64_t)v.z - v.x, dy = (int64_t)v.w - v.y;
-    const int64_t wx = (int64_t)px - v.x, wy = (int64_t)py - v.y, rr = r * r;
-    const int64_t t = wx * dx + wy * dy;
-    if (t <= 0)
-        return wx * wx + wy * wy <= rr;
-    const int64_t dd = dx * dx + dy * dy;
-    if (t >= dd) {
-        const int64_t ux = (int64_t)px - v.z, uy = (int64_t)py - v.w;
-        return ux * ux + uy * uy <= rr;
-    }
-    const int64_t c = dx * wy - dy * wx;
-    const uint64_t ca = (uint64_t)(c < 0 ? -c : c);
-    const uint64_t lh = __umul64hi(ca, ca), ll = ca * ca;
-    const uint64_t rh = __umul64hi((uint64_t)rr, (uint64_t)dd), rl = (uint64_t)rr * (uint64_t)dd;
-    return lh < rh || (lh == rh && ll <= rl);
-}
-
-// The same with an FP32 filter.  Rounding a coordinate difference costs 2^-24
-// relative, so every product of two differences is within 3.01 x 2^-24 of its
-// value and a sum or difference of two within 4.1 x 2^-24 of the sum of their
-// magnitudes; r |d| (one conversion, half of |d|^2's error, two roundings)
-// within 5.2 x 2^-24.  Each comparison trusts FP32 only outside 2^-21 (8 x 2^-24)
-// of the magnitudes involved; the rest (near the radius, or near an end's
-// perpendicular) is decided exactly.
-template <bool FP32>
-__device__ __forceinline__ bool seg_near(const int4 &v, int px, int py, int r)
-{
-    if (FP32) {
-        constexpr float kE = 4.76837158203125e-07f; // 2^-21
-        const float dx = __int2float_rn(v.z - v.x), dy = __int2float_rn(v.w - v.y);
-        const float wx = __int2float_rn(px - v.x), wy = __int2float_rn(py - v.y), rf = __int2float_rn(r);
-        const float t1 = wx * dx, t2 = wy * dy, t = t1 + t2, et = kE * (fabsf(t1) + fabsf(t2));
-        const float dd = dx * dx + dy * dy, rr = rf * rf;
-        float a, b, m; // the point is near iff a <= b; m: the magnitudes compared
-        bool sure = true;
-        if (t < -et) {
-            a = wx * wx + wy * wy, b = rr, m = a + b;
-        } else if (t - dd > et + kE * dd) {
-            const float ux = __int2float_rn(px - v.z), uy = __int2float_rn(py - v.w);
-            a = ux * ux + uy * uy, b = rr, m = a + b;
-        } else {
-            sure = t > et && dd - t > et + kE * dd;
-            const float c1 = dx * wy, c2 = dy * wx;
-            a = fabsf(c1 - c2), b = rf * __fsqrt_rn(dd), m = fabsf(c1) + fabsf(c2) + b;
-        }
-        if (sure && fabsf(a - b) > kE * m)
-            return a < b;
-    }
-    return seg_near_exact(v, px, py, r);
 }
 
 // Does polygon q of its own index hold the in-box point (px, py)?
@@ -3249,9 +3191,7 @@ cudaError_t launch_sum_u64(unsigned long long *dst, const unsigned long long *x,
 //   right  crossed by every ray of a row it straddles, whatever the point's x:
 //          only the parity of such edges per row matters, a step function of y;
 //   near   neither for certain: kept.
-// The ends of the part come from FP32 with 2^-18 of the magnitudes (and 4 units)
-// as margin, 64 times what its few roundings cost; an edge whose own x range is
-// right of the cell needs no arithmetic.  The step function is written as edges
+// (edge_side; in doubt, near.)  The step function is written as edges
 // at x = 2^30, right of every point: one over all rows when it is odd at y0, and
 // one from t up for every y = t where it changes.  A vertex between two right
 // edges changes it twice, so the changes are the few vertices where a chain
@@ -3260,27 +3200,6 @@ constexpr uint32_t kLocalMin = 8;   // shorter lists stay
 constexpr uint32_t kLocalMean = 8;  // mean edges per list from which an index gets local lists
 constexpr int kLocalTurns = 8;      // changes of parity a cell may record; else the list stays
 
-struct LocalCell {
-    int x0, y0, S;
-};
-
-// 0 left or without a row, 1 near, 2 right
-__device__ __forceinline__ int edge_side(const int4 &v, const LocalCell &c)
-{
-    const int ylo = max(c.y0, min(v.y, v.w)), yhi = min(c.y0 + c.S, max(v.y, v.w)) - 1;
-    if (ylo > yhi)
-        return 0; // straddles no integer row of the cell
-    if (min(v.x, v.z) >= c.x0 + c.S)
-        return 2;
-    const float ax = __int2float_rn(v.x - c.x0), dx = __int2float_rn(v.z - v.x);
-    const float slope = dx / __int2float_rn(v.w - v.y);
-    const float xa = ax + slope * __int2float_rn(ylo - v.y), xb = ax + slope * __int2float_rn(yhi - v.y);
-    const float margin = 4.f + 3.814697265625e-06f * (fabsf(ax) + fabsf(dx)); // 2^-18
-    if (fminf(xa, xb) - margin >= __int2float_rn(c.S))
-        return 2;
-    return fmaxf(xa, xb) + margin < 0.f ? 0 : 1;
-}
-
 // The parity of the right edges over the rows of a cell: at y0 (odd), and the y
 // where it changes.  add() is false when there are more changes than fit.
 struct LocalTurns {
@@ -3288,7 +3207,7 @@ struct LocalTurns {
     int nt = 0;
     uint32_t odd = 0;
 
-    __device__ __forceinline__ bool add(const int4 &v, const LocalCell &c)
+    __device__ __forceinline__ bool add(const int4 &v, const CellBox &c)
     {
         odd ^= (v.y > c.y0) != (v.w > c.y0) ? 1u : 0u;
 #pragma unroll
@@ -3385,7 +3304,7 @@ __global__ void __launch_bounds__(256) k_local_size(IndexView ix, const uint4 *e
     for (uint64_t i = (uint64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (uint64_t)gridDim.x * 256) {
         const uint4 it = items[i];
         const uint4 en = ent[it.x];
-        const LocalCell c{int(it.y), int(it.z), 1 << ix.sf};
+        const CellBox c{int(it.y), int(it.z), 1 << ix.sf};
         LocalTurns tn;
         uint32_t near = 0;
         bool fits = true;
@@ -3414,7 +3333,9 @@ __global__ void __launch_bounds__(256) k_local_size(IndexView ix, const uint4 *e
 }
 
 // A lane per long list: writes the changed ones and their records, at places that
-// each warp takes from totals[0..1] (zeroed), in no particular order.
+// each warp takes from totals[0..1] (zeroed), in no particular order.  A list that
+// does not come out as k_local_size counted it stays what it was (never seen: the
+// two kernels decide alike; the bound keeps every write in the list's own place).
 __global__ void __launch_bounds__(256) k_local_write(IndexView ix, uint4 *ent, uint64_t n, const uint4 *items,
                                                      unsigned long long *totals, int4 *loc, uint4 *undo)
 {
@@ -3444,28 +3365,36 @@ __global__ void __launch_bounds__(256) k_local_write(IndexView ix, uint4 *ent, u
         if (!take)
             continue;
         const uint4 en = ent[it.x];
-        const LocalCell c{int(it.y), int(it.z), 1 << ix.sf};
+        const CellBox c{int(it.y), int(it.z), 1 << ix.sf};
         LocalTurns tn;
+        const uint32_t near = it.w & (kLocalMaxList - 1);
         int4 *d = loc + at_loc + odd + nt;
+        uint32_t kept = 0;
+        bool fits = true;
         for (uint32_t k = 0; k < en.z; k += kLocalLoads) { // in the list's order: right ends descending
             int4 v[kLocalLoads];
             load_list(ix, en, k, v);
 #pragma unroll
             for (uint32_t u = 0; u < kLocalLoads; ++u) {
                 const int side = k + u < en.z ? edge_side(v[u], c) : 0;
-                if (side == 1)
-                    *d++ = v[u];
-                else if (side == 2)
-                    tn.add(v[u], c);
+                if (side == 1) {
+                    if (kept < near)
+                        d[kept] = v[u];
+                    ++kept;
+                } else if (side == 2) {
+                    fits = fits && tn.add(v[u], c);
+                }
             }
         }
+        undo[at_ent] = make_uint4(it.x, en.y, en.z, 0u);
+        if (!fits || kept != near || tn.odd != odd || (uint32_t)tn.nt != nt)
+            continue;
         const int far = int(kBox);
         d = loc + at_loc;
         if (odd)
             *d++ = make_int4(far, c.y0, far, c.y0 + c.S);
         for (uint32_t k = 0; k < nt; ++k)
             *d++ = make_int4(far, tn.turn[k], far, c.y0 + c.S);
-        undo[at_ent] = make_uint4(it.x, en.y, en.z, 0u);
         ent[it.x].y = kLocalEdge | (uint32_t)at_loc;
         ent[it.x].z = size;
     }
@@ -4034,27 +3963,11 @@ static cudaError_t launch_buffer_mask(const IndexView &ix, const uint32_t *cell_
 //           FP32 with the coordinate differences' rounding (2^-24 relative, a
 //           few of them) covered by 2^-18 of their sum;
 //   none    neither cross nor edges: no point of the cell meets the polygon.
-struct NearCell {
-    int x0, y0, S;
-};
-
-__device__ __forceinline__ bool edge_reaches(const int4 &v, const NearCell &c, int r)
-{
-    const float dx = __int2float_rn(v.z - v.x), dy = __int2float_rn(v.w - v.y), m = 0.5f * __int2float_rn(c.S - 1);
-    const float wx = __int2float_rn(c.x0 - v.x) + m, wy = __int2float_rn(c.y0 - v.y) + m;
-    const float dd = dx * dx + dy * dy;
-    const float t = dd > 0.f ? fminf(1.f, fmaxf(0.f, (wx * dx + wy * dy) / dd)) : 0.f;
-    const float ex = wx - t * dx, ey = wy - t * dy;
-    const float reach = __int2float_rn(r) + 1.41421366f * m + 2.f;
-    const float slack = 3.814697265625e-06f * (fabsf(wx) + fabsf(wy) + fabsf(dx) + fabsf(dy) + reach); // 2^-18
-    return sqrtf(ex * ex + ey * ey) <= reach + slack;
-}
-
 // Calls add(q, first item, end, flags) for every group of the cell but those
 // that no point meets: flags 0 for whole, else kEntBoundary and kEntCross.
 template <class F>
 __device__ __forceinline__ void near_groups(const IndexView &in, const uint32_t *item_q, const int4 *item_seg,
-                                            const int32_t *rad, uint32_t k, uint32_t kend, const NearCell &c, F add)
+                                            const int32_t *rad, uint32_t k, uint32_t kend, const CellBox &c, F add)
 {
     const int x1 = c.x0 + c.S - 1, y1 = c.y0 + c.S - 1;
     auto group = [&](uint32_t q, bool holds) {
@@ -4101,12 +4014,14 @@ __device__ __forceinline__ void near_groups(const IndexView &in, const uint32_t 
 
 // Coarse level, a thread per cell.  COUNT: the cell's word (kinds kCellSub and
 // kCellCoarseList without their payload), its entries when it is a coarse list,
-// and 1 when it is split.  Else: the payloads and the coarse lists.
+// and 1 when it is split.  Else: the payloads and the coarse lists, each within the
+// place that was counted for it (*wrong counts those that come out otherwise).
 template <bool COUNT>
 __global__ void __launch_bounds__(256) k_near_coarse(IndexView in, const uint32_t *cell_off, const uint32_t *item_q,
                                                      const int4 *item_seg, const int32_t *rad, const uint32_t *mask,
                                                      int g, unsigned long long *n_ent, unsigned long long *n_blk,
-                                                     uint32_t *cell, uint4 *ent)
+                                                     uint32_t *cell, uint4 *ent, uint64_t ent_end,
+                                                     unsigned long long *wrong)
 {
     const uint32_t ncell = 1u << (2 * g);
     const int sh = kBoxLog2 - g;
@@ -4123,14 +4038,14 @@ __global__ void __launch_bounds__(256) k_near_coarse(IndexView in, const uint32_
             cell[c] |= (uint32_t)n_blk[c];
             continue;
         }
-        const NearCell nc{int((c & ((1u << g) - 1)) << sh), int((c >> g) << sh), 1 << sh};
-        const uint64_t off = COUNT ? 0 : n_ent[c];
+        const CellBox nc{int((c & ((1u << g) - 1)) << sh), int((c >> g) << sh), 1 << sh};
+        const uint64_t off = COUNT ? 0 : n_ent[c], room = COUNT ? 0 : (c + 1 < ncell ? n_ent[c + 1] : ent_end) - off;
         uint32_t n = 0, one = 0;
         bool lists = false;
         near_groups(in, item_q, item_seg, rad, cell_off[c], cell_off[c + 1], nc,
                     [&](uint32_t q, uint32_t, uint32_t, uint32_t flags) {
-                        if (!COUNT)
-                            ent[off + n] = make_uint4(q, 0u, 0u, 0u);
+                        if (!COUNT && n < room)
+                            ent[off + n] = make_uint4(q, 0u, 0u, n + 1 == room ? kEntLast : 0u);
                         one = q;
                         lists = lists || flags;
                         ++n;
@@ -4140,7 +4055,8 @@ __global__ void __launch_bounds__(256) k_near_coarse(IndexView in, const uint32_
             n_blk[c] = lists ? 1 : 0;
             cell[c] = lists ? kCellSub << 30 : n > 1 ? kCellCoarseList << 30 : n ? (kCellInsideOne << 30) | one : 0u;
         } else {
-            ent[off + n - 1].w = kEntLast;
+            if (n != room || lists)
+                atomicAdd(wrong, 1ull);
             cell[c] |= uint32_t(off);
         }
     }
@@ -4156,13 +4072,14 @@ __global__ void __launch_bounds__(256) k_near_blocks(uint32_t ncell, const uint3
 }
 
 // Fine level, a thread per fine cell of every block.  COUNT: its word (a list's
-// without its offset), its entries and its edges; else the lists.
+// without its offset), its entries and its edges; else the lists, as above.
 template <bool COUNT>
 __global__ void __launch_bounds__(256) k_near_fine(IndexView in, const uint32_t *cell_off, const uint32_t *item_q,
                                                    const int4 *item_seg, const int32_t *rad, int g, int sb,
                                                    const uint32_t *blk_cell, uint64_t n_fine, unsigned long long *n_ent,
                                                    unsigned long long *n_edge, uint64_t ent0, uint32_t *fine, uint4 *ent,
-                                                   int4 *edge)
+                                                   int4 *edge, uint64_t ent_end, uint64_t edge_end,
+                                                   unsigned long long *wrong)
 {
     const int sh = kBoxLog2 - g, sf = sh - sb;
     const uint32_t fm = (1u << sb) - 1;
@@ -4170,9 +4087,11 @@ __global__ void __launch_bounds__(256) k_near_fine(IndexView in, const uint32_t 
         if (!COUNT && (fine[t] >> 30) != kCellList)
             continue;
         const uint32_t c = blk_cell[t >> (2 * sb)], f = (uint32_t)t & ((1u << (2 * sb)) - 1);
-        const NearCell nc{int(((c & ((1u << g) - 1)) << sh) | ((f & fm) << sf)), int(((c >> g) << sh) | ((f >> sb) << sf)),
+        const CellBox nc{int(((c & ((1u << g) - 1)) << sh) | ((f & fm) << sf)), int(((c >> g) << sh) | ((f >> sb) << sf)),
                           1 << sf};
         const uint64_t off = COUNT ? 0 : ent0 + n_ent[t], eoff = COUNT ? 0 : n_edge[t];
+        const uint64_t room = COUNT ? 0 : (t + 1 < n_fine ? n_ent[t + 1] : ent_end) - n_ent[t];
+        const uint64_t eroom = COUNT ? 0 : (t + 1 < n_fine ? n_edge[t + 1] : edge_end) - eoff;
         uint32_t n = 0, one = 0, ne = 0;
         bool whole = false;
         near_groups(in, item_q, item_seg, rad, cell_off[c], cell_off[c + 1], nc,
@@ -4181,13 +4100,14 @@ __global__ void __launch_bounds__(256) k_near_fine(IndexView in, const uint32_t 
                         for (uint32_t k = k0; k < k1; ++k) {
                             const int4 v = item_seg[k];
                             if (edge_reaches(v, nc, rad[q])) {
-                                if (!COUNT)
+                                if (!COUNT && ne < eroom)
                                     edge[eoff + ne] = v;
                                 ++ne;
                             }
                         }
-                        if (!COUNT)
-                            ent[off + n] = make_uint4(q, uint32_t(eoff + first), ne - first, flags);
+                        if (!COUNT && n < room)
+                            ent[off + n] = make_uint4(q, uint32_t(eoff + first), ne - first,
+                                                      flags | (n + 1 == room ? kEntLast : 0u));
                         one = q;
                         whole = !flags;
                         ++n;
@@ -4198,7 +4118,8 @@ __global__ void __launch_bounds__(256) k_near_fine(IndexView in, const uint32_t 
             n_edge[t] = lst ? ne : 0;
             fine[t] = lst ? kCellList << 30 : n ? (kCellInsideOne << 30) | one : 0u;
         } else {
-            ent[off + n - 1].w |= kEntLast;
+            if (n != room || ne != eroom)
+                atomicAdd(wrong, 1ull);
             fine[t] = (kCellList << 30) | uint32_t(off);
         }
     }
@@ -4256,13 +4177,15 @@ int build_near_index_device(const IndexView &in, const uint32_t *cell_off, const
     auto *mask = reinterpret_cast<uint32_t *>(tmp + 2 * t_cnt + t_part);
     auto *word = reinterpret_cast<uint32_t *>(tmp + 2 * t_cnt + t_part + t_mask);
     auto *blk_cell = reinterpret_cast<uint32_t *>(tmp + 2 * t_cnt + t_part + t_mask + b_cell);
-    // coarse entries, blocks, fine entries, fine edges, resolved summary blocks
+    // coarse entries, blocks, fine entries, fine edges, resolved summary blocks,
+    // lists that the two passes over their cell see differently
     auto *tot = reinterpret_cast<unsigned long long *>(tmp + 2 * t_cnt + t_part + t_mask + 2 * b_cell);
-    unsigned long long h[5] = {};
+    unsigned long long h[6] = {};
     if ((e = cudaMemset(mask, 0, t_mask)) != cudaSuccess || (e = cudaMemset(tot, 0, sizeof(h))) != cudaSuccess ||
         (e = launch_buffer_mask(in, cell_off, mask, g)) != cudaSuccess)
         return done(2);
-    k_near_coarse<true><<<blocks(ncell), 256>>>(in, cell_off, item_q, item_seg, rad, mask, g, n_ent, n_blk, word, nullptr);
+    k_near_coarse<true><<<blocks(ncell), 256>>>(in, cell_off, item_q, item_seg, rad, mask, g, n_ent, n_blk, word, nullptr,
+                                               0, nullptr);
     if ((e = cudaGetLastError()) != cudaSuccess || (e = launch_scan(n_ent, ncell, tot, part, nullptr)) != cudaSuccess ||
         (e = launch_scan(n_blk, ncell, tot + 1, part, nullptr)) != cudaSuccess ||
         (e = cudaMemcpy(h, tot, 16, cudaMemcpyDeviceToHost)) != cudaSuccess)
@@ -4290,7 +4213,7 @@ int build_near_index_device(const IndexView &in, const uint32_t *cell_off, const
         auto *f_word = reinterpret_cast<uint32_t *>(tmp2 + 2 * t_f + t_fp);
         if (NB) {
             k_near_fine<true><<<blocks(nf), 256>>>(in, cell_off, item_q, item_seg, rad, g, sb, blk_cell, nf, f_ent, f_edge, 0,
-                                                   f_word, nullptr, nullptr);
+                                                   f_word, nullptr, nullptr, 0, 0, nullptr);
             if ((e = cudaGetLastError()) != cudaSuccess || (e = launch_scan(f_ent, nf, tot + 2, f_part, nullptr)) != cudaSuccess ||
                 (e = launch_scan(f_edge, nf, tot + 3, f_part, nullptr)) != cudaSuccess ||
                 (e = cudaMemcpy(h, tot, 32, cudaMemcpyDeviceToHost)) != cudaSuccess)
@@ -4329,15 +4252,17 @@ int build_near_index_device(const IndexView &in, const uint32_t *cell_off, const
             (nf && (e = cudaMemcpy(out.fine, f_word, nf * 4, cudaMemcpyDeviceToDevice)) != cudaSuccess))
             return done(2);
         k_near_coarse<false><<<blocks(ncell), 256>>>(in, cell_off, item_q, item_seg, rad, mask, g, n_ent, n_blk, out.cell,
-                                                     out.ent);
+                                                     out.ent, h[0], tot + 5);
         if (NB)
             k_near_fine<false><<<blocks(nf), 256>>>(in, cell_off, item_q, item_seg, rad, g, sb, blk_cell, nf, f_ent, f_edge,
-                                                    h[0], out.fine, out.ent, out.edge);
+                                                    h[0], out.fine, out.ent, out.edge, h[2], h[3], tot + 5);
         k_near_sum<<<((1u << (2 * sg)) + 255) / 256, 256>>>(g, sg, out.cell, out.sum, tot + 4, out.ent + (out.n_ent - 4),
                                                             out.edge + h[3]);
         if ((e = cudaGetLastError()) != cudaSuccess ||
-            (e = cudaMemcpy(h + 4, tot + 4, 8, cudaMemcpyDeviceToHost)) != cudaSuccess)
+            (e = cudaMemcpy(h + 4, tot + 4, 16, cudaMemcpyDeviceToHost)) != cudaSuccess)
             return done(2);
+        if (h[5])
+            return done(3);
         out.sum_resolved = double(h[4]) / double(uint64_t(1) << (2 * sg));
         return done(0);
     }

@@ -172,7 +172,7 @@ cudaError_t build_local_lists(const IndexView &view, uint4 *ent, LocalLists &out
 // device), the radii and the polygons' own index.  out.mem holds cells | fine |
 // entries | edges | summary and belongs to the caller.  Runs on the legacy
 // default stream, synchronises.  Returns 0; 1 when the entries exceed 30-bit
-// offsets; 2 on a CUDA error (in cerr).
+// offsets; 2 on a CUDA error (in cerr); 3 when a list did not come out as counted.
 struct NearIndexDev {
     void *mem;
     size_t bytes;
