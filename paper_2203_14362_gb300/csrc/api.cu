@@ -178,6 +178,12 @@ cudaError_t dev_alloc(spx_ctx *ctx, void **p, size_t bytes)
     return e;
 }
 
+// The end of a call's uploads.  cudaMemcpy from pageable memory may return while
+// its last part is still on the way from the driver's staging buffer, and only the
+// legacy stream waits for that; what comes next runs on the ctx's stream or on a
+// caller's, which do not wait for the legacy stream.
+cudaError_t uploads_done() { return cudaStreamSynchronize(cudaStreamLegacy); }
+
 void free_index_memory(spx_ctx *ctx, IndexObj &ix)
 {
     ix.pooled ? cudaFreeAsync(ix.mem, ctx->stream) : cudaFree(ix.mem);
@@ -556,6 +562,8 @@ spx_status build_index_impl(spx_ctx *ctx, spx_polys polys, const spx_index_param
         e = cudaMemcpy(p_ent, hi.entries.data(), b_ent, cudaMemcpyHostToDevice);
     if (e == cudaSuccess && b_edge)
         e = cudaMemcpy(p_edge, hi.edges.data(), b_edge, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess)
+        e = uploads_done();
     if (e != cudaSuccess) {
         cudaFree(ix->mem);
         return cuda_fail(ctx, e, "build_index upload");
@@ -782,7 +790,9 @@ spx_status spx_load_points(spx_ctx *ctx, const int32_t *xy, uint64_t n, int xy_i
         void *d = nullptr;
         if (dev_alloc(ctx, &d, n ? n * 8 : 16) != cudaSuccess)
             return fail(ctx, SPX_ENOMEM, "load_points: cudaMalloc failed");
-        const cudaError_t e = n ? cudaMemcpy(d, xy, n * 8, cudaMemcpyHostToDevice) : cudaSuccess;
+        cudaError_t e = n ? cudaMemcpy(d, xy, n * 8, cudaMemcpyHostToDevice) : cudaSuccess;
+        if (e == cudaSuccess)
+            e = uploads_done();
         if (e != cudaSuccess) {
             cudaFree(d);
             return cuda_fail(ctx, e, "load_points copy");
