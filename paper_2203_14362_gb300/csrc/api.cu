@@ -3,6 +3,7 @@
 // kernels.  Every step of the join runs in kernels.cu; this file only moves
 // bytes and checks arguments.
 #include "kernels.h"
+#include "optional_buffer.h"
 #include "server_internal.h"
 #include "spx.h"
 #include "spx_internal.h"
@@ -97,6 +98,7 @@ struct spx_ctx {
     char *pinned = nullptr; // kPinnedBytes of host memory: a call's status and total come back here
     void *scratch = nullptr;
     size_t scratch_bytes = 0;
+    OptionalBuffer ids; // distance queries: a point's polygons, 8 B per point, kept by pass 1 for pass 3
     // staging buffers of spx_join_host
     void *st_pts = nullptr, *st_pairs = nullptr, *st_counts = nullptr;
     size_t st_pts_b = 0, st_pairs_b = 0, st_counts_b = 0;
@@ -220,6 +222,26 @@ spx_status ensure(spx_ctx *ctx, void **buf, size_t *have, size_t need, cudaStrea
         return fail(ctx, SPX_ENOMEM, std::string(what) + ": cudaMalloc failed: " + cudaGetErrorString(e));
     *have = sz;
     return SPX_OK;
+}
+
+// The packed ids of a distance query over n points on s, or null where they do not
+// fit (pass 3 then walks those points' lists again).  Not grown under capture.
+uint64_t *packed_ids(spx_ctx *ctx, uint64_t n, cudaStream_t s)
+{
+    const size_t need = n * 8;
+    if (ctx->ids.bytes < need && capturing(s))
+        return nullptr;
+    return static_cast<uint64_t *>(ctx->ids.want(
+        need,
+        [&](void **p, size_t b) {
+            const bool ok = dev_alloc(ctx, p, b) == cudaSuccess;
+            cudaGetLastError();
+            return ok;
+        },
+        [&](void *p) {
+            cudaStreamSynchronize(s);
+            cudaFree(p);
+        }));
 }
 
 // The status of what ran on s (synchronises it): reads the kernel error word,
@@ -362,20 +384,11 @@ spx_status join_common(spx_ctx *ctx, spx_points points, spx_index index, uint32_
     plain = plain && ix->kind == 0; // distance queries have one path
     const bool buffered = ix->kind == 2;
     const size_t need = plain ? plain_scratch_bytes(pts->n) : join_scratch_bytes(pts->n);
-    // buffered polygons overlap: 8 B per point more let pass 1 keep a point's
-    // polygons for pass 3; a call goes without them where the scratch cannot grow
-    const size_t aux_at = (need + 15) & ~size_t(15), with_aux = aux_at + pts->n * 8;
-    bool aux = buffered && ix->nview.P <= kRes16MaxP && (ctx->scratch_bytes >= with_aux || !capturing(s));
-    spx_status st = ensure(ctx, &ctx->scratch, &ctx->scratch_bytes, aux ? with_aux : need, s, "join");
-    if (st == SPX_ENOMEM && aux) {
-        cudaGetLastError();
-        aux = false;
-        st = ensure(ctx, &ctx->scratch, &ctx->scratch_bytes, need, s, "join");
-    }
+    spx_status st = ensure(ctx, &ctx->scratch, &ctx->scratch_bytes, need, s, "join");
     if (st != SPX_OK)
         return st;
     JoinLaunch a = index_launch(ctx, pts, ix);
-    a.aux = aux ? reinterpret_cast<uint64_t *>(static_cast<char *>(ctx->scratch) + aux_at) : nullptr;
+    a.aux = buffered && ix->nview.P <= kRes16MaxP ? packed_ids(ctx, pts->n, s) : nullptr; // buffered polygons overlap
     a.pairs = reinterpret_cast<uint2 *>(pairs_dev);
     a.cap = pairs_dev ? cap : 0;
     a.counts = reinterpret_cast<unsigned long long *>(counts_dev);
@@ -741,6 +754,7 @@ void spx_destroy(spx_ctx *ctx)
     if (ctx->pool)
         cudaMemPoolDestroy(ctx->pool);
     cudaFree(ctx->scratch);
+    cudaFree(ctx->ids.p);
     cudaFree(ctx->st_pts);
     cudaFree(ctx->st_pairs);
     cudaFree(ctx->st_counts);
@@ -1519,21 +1533,16 @@ spx_status spx_select(spx_ctx *ctx, spx_points points, spx_index index, uint32_t
                                          " queries; batched selection takes at most " +
                                          std::to_string(kSelectMaxQueries));
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    // pass 1b keeps the polygons of a point in several for pass 3 in 8 B per point
-    // more; the distance selections go without where the scratch cannot grow
-    const size_t full = select_scratch_bytes(pts->n, PQ, cap, true), least = select_scratch_bytes(pts->n, PQ, cap, false);
-    bool aux = ix->kind == 0 || ctx->scratch_bytes >= full || !capturing(s);
-    spx_status st = ensure(ctx, &ctx->scratch, &ctx->scratch_bytes, aux ? full : least, s, "select");
-    if (st == SPX_ENOMEM && ix->kind) {
-        cudaGetLastError();
-        aux = false;
-        st = ensure(ctx, &ctx->scratch, &ctx->scratch_bytes, least, s, "select");
-    }
+    // pass 1b keeps the polygons of a point in several for pass 3 in 8 B per point:
+    // in the scratch, or, for distance selections, in the packed ids where they fit
+    const bool aux = ix->kind == 0;
+    spx_status st = ensure(ctx, &ctx->scratch, &ctx->scratch_bytes, select_scratch_bytes(pts->n, PQ, cap, aux), s, "select");
     if (st != SPX_OK)
         return st;
-    const JoinLaunch a = index_launch(ctx, pts, ix);
+    JoinLaunch a = index_launch(ctx, pts, ix);
     unsigned long long *offs = reinterpret_cast<unsigned long long *>(offsets_dev);
     if (ix->kind) { // distance selections: not captured
+        a.aux = packed_ids(ctx, pts->n, s);
         const cudaError_t e = launch_select(a, ids_dev, cap, offs, ctx->scratch, s, aux);
         if (e != cudaSuccess)
             return cuda_fail(ctx, e, "select launch");
@@ -2180,6 +2189,7 @@ spx_status spx_free(spx_ctx *ctx, uint64_t handle)
                 ++it;
             }
         free_index_memory(ctx, *ix);
+        ctx->ids.retry();
         PolysObj *pg = lookup(ctx->polys, ix->polys);
         if (pg)
             pg->n_index--;
@@ -2210,6 +2220,7 @@ spx_status spx_free(spx_ctx *ctx, uint64_t handle)
         if (p->owned)
             cudaFree(p->dev);
         cudaFree(p->cell_end);
+        ctx->ids.retry();
         ctx->points.erase(handle);
         return SPX_OK;
     }

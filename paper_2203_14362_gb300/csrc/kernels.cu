@@ -3748,8 +3748,9 @@ cudaError_t launch_select(const JoinLaunch &a, uint32_t *ids, uint64_t cap, unsi
     void *join_scratch = sc;
     sc += (join_scratch_bytes(a.n) + 15) & ~size_t(15);
     // overlapping queries put many points in several polygons: pass 1b packs
-    // their ids so that pass 3 does not walk them again
-    uint64_t *aux = with_aux ? reinterpret_cast<uint64_t *>(sc) : nullptr;
+    // their ids (in the scratch, or where the caller says) so that pass 3 does not
+    // walk them again
+    uint64_t *aux = with_aux ? reinterpret_cast<uint64_t *>(sc) : a.aux;
     sc += with_aux ? a.n * 8 : 0;
     unsigned long long *total = reinterpret_cast<unsigned long long *>(sc);
     sc += 16;
