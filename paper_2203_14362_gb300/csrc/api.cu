@@ -1396,7 +1396,6 @@ spx_status spx_build_buffer_index(spx_ctx *ctx, spx_polys polys, const int32_t *
     std::string err;
     if (!build_buffer_edges(pg->xy.data(), pg->off.data(), pg->P, r, g, he, err))
         return fail(ctx, SPX_EINVAL, "build_buffer_index: " + err);
-    give_back(ctx); // the build allocates from the device
     // the polygons' own index answers containment; it becomes part of this one
     spx_index_params prm{};
     prm.fp32_filter = fp32_filter ? 1 : 0;
@@ -1437,6 +1436,10 @@ spx_status spx_build_buffer_index(spx_ctx *ctx, spx_polys polys, const int32_t *
     if (e == cudaSuccess && P)
         e = cudaMemcpy(p_r, r, size_t(P) * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) {
+        // the build allocates from the device, and without memory it would take
+        // coarser fine cells: what earlier builds, and the local lists of ix, left in
+        // the pool goes back first
+        give_back(ctx);
         const int built = build_near_index_device(ix->view, reinterpret_cast<uint32_t *>(p_off),
                                                   reinterpret_cast<uint32_t *>(p_q), reinterpret_cast<int4 *>(p_seg),
                                                   reinterpret_cast<int32_t *>(p_r), g, fx, e);
