@@ -160,10 +160,11 @@ bool capturing(cudaStream_t s)
     return st != cudaStreamCaptureStatusNone;
 }
 
-// What the ctx's pool keeps goes back to the device.
+// What the ctx's pool keeps goes back to the device.  Waits for the device: scratch
+// of counts is freed on callers' streams, and until then it is not the pool's.
 void give_back(spx_ctx *ctx)
 {
-    cudaStreamSynchronize(ctx->stream);
+    cudaDeviceSynchronize();
     cudaMemPoolTrimTo(ctx->pool, 0);
 }
 
@@ -949,7 +950,12 @@ spx_status spx_build_index_device(spx_ctx *ctx, spx_polys polys, const spx_index
     // temporaries and the index itself from the ctx's pool, in the order of its
     // stream: an index built, used and freed per query reuses its memory (20
     // allocations and frees were half of a query-time build of 1000 cells)
-    const int st = build_grid_index_device(pg->xy.data(), pg->off.data(), pg->P, g, sb, d, why, e, ctx->stream, ctx->pool);
+    int st = build_grid_index_device(pg->xy.data(), pg->off.data(), pg->P, g, sb, d, why, e, ctx->stream, ctx->pool);
+    if (st && e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        give_back(ctx);
+        st = build_grid_index_device(pg->xy.data(), pg->off.data(), pg->P, g, sb, d, why, e, ctx->stream, ctx->pool);
+    }
     cudaDeviceSynchronize(); // as documented
     if (st == 1)
         return fail(ctx, SPX_EINVAL, std::string("build_index_device: ") + why);

@@ -41,3 +41,34 @@ def test_buffered_build_keeps_only_the_index(eng):
     ih = eng.build_buffer_index(gh, np.full(256, 1 << 18, np.int32), grid_log2=9)
     held, own = before - free_bytes(), eng.index_info(ih)["device_bytes"]
     assert held <= own + 64 * MB
+
+
+def test_scratch_freed_on_another_stream(eng):
+    # a count's scratch (32 MB) is still in use on a caller's stream when a table needs
+    # memory that is only there once that scratch goes back
+    n = 1 << 28
+    t = g.quad_tessellation(16, 16, 5, kmin=4, kmax=20)
+    ih = eng.build_index(eng.load_polygons(t.verts, t.ring_off), grid_log2=8)
+    pts = torch.zeros((n, 2), dtype=torch.int32, device="cuda")
+    ph = eng.load_points(pts)
+    counts = torch.zeros(256, dtype=torch.int64, device="cuda")
+    eng.aggregate(ph, ih, counts)
+    want = counts.clone()
+    table = np.zeros((7 * MB, 2), np.int32)  # 56 MB
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        torch.cuda._sleep(1000)
+    hog = torch.empty(free_bytes() - 40 * MB, dtype=torch.uint8, device="cuda")
+    try:
+        with torch.cuda.stream(s):
+            torch.cuda._sleep(1_000_000_000)  # about half a second
+            eng.aggregate(ph, ih, counts, stream=s)
+        few = eng.load_points(table)
+        torch.cuda.synchronize()
+        assert torch.equal(counts, want)
+        eng.aggregate(few, ih, counts)
+        assert counts.sum().item() == (7 * MB if want.sum().item() else 0)
+        assert eng.points_info(few)["n"] == 7 * MB
+    finally:
+        del hog
+        torch.cuda.empty_cache()
