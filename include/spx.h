@@ -157,11 +157,12 @@ spx_status spx_build_index(spx_ctx *ctx, spx_polys polys, const spx_index_params
  * list sorted by right end; per cell: records, fine blocks and entries), and
  * the arrays are byte for byte those of spx_build_index with the same
  * parameters.  Same arguments, results and limits as spx_build_index.
- * Synchronous (the legacy default stream; the device is synchronised).
- * Temporary device memory, and the index's own, come from a pool of the ctx,
- * which keeps up to 4 GiB between calls (given back when another allocation of
- * the ctx fails, and by spx_destroy).  Errors: SPX_EINVAL (bad handle or
- * parameters, an index-format limit exceeded), SPX_ENOMEM, SPX_ECUDA.
+ * Synchronous (a stream of the ctx; the device is synchronised).  Temporary
+ * device memory, and the index's own, come from a pool of the ctx, which keeps up
+ * to 4 GiB between calls (given back when another allocation of the ctx fails,
+ * when a table whose memory the ctx holds is freed, and by spx_destroy).
+ * Errors: SPX_EINVAL (bad handle or parameters, an index-format limit
+ * exceeded), SPX_ENOMEM, SPX_ECUDA.
  */
 spx_status spx_build_index_device(spx_ctx *ctx, spx_polys polys, const spx_index_params *params, spx_index *out);
 

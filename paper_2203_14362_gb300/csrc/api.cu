@@ -2226,8 +2226,10 @@ spx_status spx_free(spx_ctx *ctx, uint64_t handle)
             } else {
                 ++it;
             }
-        if (p->owned)
+        if (p->owned) { // whoever frees a table wants memory for something else
             cudaFree(p->dev);
+            cudaMemPoolTrimTo(ctx->pool, 0);
+        }
         cudaFree(p->cell_end);
         ctx->ids.retry();
         ctx->points.erase(handle);

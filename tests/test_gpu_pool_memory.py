@@ -72,3 +72,16 @@ def test_scratch_freed_on_another_stream(eng):
     finally:
         del hog
         torch.cuda.empty_cache()
+
+
+def test_freed_table_gives_back_the_pool(eng):
+    t = g.quad_tessellation(30, 30, 7, kmin=4, kmax=100)
+    gh = eng.load_polygons(t.verts, t.ring_off)
+    few = np.zeros((1000, 2), np.int32)
+    eng.free(eng.build_index(gh, grid_log2=6, on_device=True))  # kernels loaded
+    eng.free(eng.load_points(few))
+    before = free_bytes()
+    eng.free(eng.build_index(gh, grid_log2=12, on_device=True))
+    assert free_bytes() < before - 256 * MB  # kept for the next build
+    eng.free(eng.load_points(few))
+    assert free_bytes() >= before - 8 * MB
