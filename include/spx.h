@@ -281,7 +281,7 @@ typedef struct {
     int grid_max;           /* largest grid_log2 tried (default 13) */
     int reps;               /* timed launches per candidate, the fastest kept (default 5) */
     int fp32_filter;        /* filter setting of every candidate and of the result: 1 (default) or 0 */
-    uint64_t max_index_bytes; /* skip candidates whose index (local lists aside) would exceed this (default 4 GiB) */
+    uint64_t max_index_bytes; /* skip candidates whose index would exceed this (default 4 GiB) */
     int reserved[4];        /* must be zero */
 } spx_tune_params;
 

@@ -481,7 +481,8 @@ static GridParts device_parts(const GridIndexDev &d)
 }
 
 spx_status register_grid_index(spx_ctx *ctx, spx_polys polys, std::unique_ptr<IndexObj> ix, size_t total, int g, int sb,
-                               int fp32, const GridParts &gp, std::chrono::steady_clock::time_point t0, spx_index *out)
+                               int fp32, const GridParts &gp, std::chrono::steady_clock::time_point t0, spx_index *out,
+                               size_t max_bytes = SIZE_MAX)
 {
     PolysObj *pg = lookup(ctx->polys, polys);
     ix->polys = polys;
@@ -506,7 +507,8 @@ spx_status register_grid_index(spx_ctx *ctx, spx_polys polys, std::unique_ptr<In
     inf.build_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
     inf.sum_resolved = gp.sum_resolved;
     inf.use_sum = ix->view.use_sum;
-    const cudaError_t e = build_local_lists(ix->view, reinterpret_cast<uint4 *>(gp.ent), ix->local, ctx->stream, ctx->pool);
+    const cudaError_t e = build_local_lists(ix->view, reinterpret_cast<uint4 *>(gp.ent), ix->local, max_bytes - total,
+                                            ctx->stream, ctx->pool);
     if (e != cudaSuccess) {
         free_index_memory(ctx, *ix);
         return cuda_fail(ctx, e, "build_index: local edge lists");
@@ -526,7 +528,8 @@ spx_status register_grid_index(spx_ctx *ctx, spx_polys polys, std::unique_ptr<In
 }
 
 // Build the index of polygon set `polys` with the checked parameters prm.  An
-// index of more than max_bytes device bytes is not uploaded: *out is then 0.
+// index of more than max_bytes device bytes is not uploaded: *out is then 0.  (One
+// that only its local lists would take past max_bytes goes without them.)
 spx_status build_index_impl(spx_ctx *ctx, spx_polys polys, const spx_index_params &prm, spx_index *out,
                             size_t max_bytes = SIZE_MAX)
 {
@@ -584,7 +587,7 @@ spx_status build_index_impl(spx_ctx *ctx, spx_polys polys, const spx_index_param
     }
     GridParts gp{p_cell, p_fine, p_ent, p_edge, p_cover, p_sum, hi.cell.size(), hi.fine.size(), hi.entries.size() / 4,
                  hi.edges.size() / 4, hi.n_blocks, hi.n_inside, hi.n_mixed, hi.n_boundary, sum_resolved};
-    return register_grid_index(ctx, polys, std::move(ix), total, g, sb, prm.fp32_filter, gp, t0, out);
+    return register_grid_index(ctx, polys, std::move(ix), total, g, sb, prm.fp32_filter, gp, t0, out, max_bytes);
 }
 
 } // namespace

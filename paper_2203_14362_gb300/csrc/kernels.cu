@@ -3428,7 +3428,8 @@ __global__ void __launch_bounds__(256) k_blk_cell(uint32_t ncell, const uint32_t
             blk_cell[cell[c] & kPayloadMask] = c;
 }
 
-cudaError_t build_local_lists(const IndexView &view, uint4 *ent, LocalLists &out, cudaStream_t s, cudaMemPool_t pool)
+cudaError_t build_local_lists(const IndexView &view, uint4 *ent, LocalLists &out, size_t max_bytes, cudaStream_t s,
+                              cudaMemPool_t pool)
 {
     out = LocalLists{};
     const uint64_t n_blk = view.n_fine >> (2 * view.sb), n_words = n_blk << (2 * view.sb);
@@ -3491,6 +3492,10 @@ cudaError_t build_local_lists(const IndexView &view, uint4 *ent, LocalLists &out
     if (h[0] >= kLocalEdge || !h[1])
         return done(cudaSuccess);
     out.bytes = (h[0] + h[1] + 1) * 16;
+    if (out.bytes > max_bytes) {
+        out = LocalLists{};
+        return done(cudaSuccess);
+    }
     if (cudaMallocFromPoolAsync(&out.mem, out.bytes, pool, s) != cudaSuccess) {
         out = LocalLists{};
         cudaGetLastError();

@@ -156,8 +156,8 @@ struct JoinLaunch {
 // along the cell's rows.  Every point of the cell crosses the new list as often,
 // modulo 2, as the old one.  out.mem (the lists, then a record (entry, y, z, 0)
 // per changed entry) belongs to the caller, who frees it with cudaFreeAsync; null
-// where the lists are short anyway, or there is no memory.  Memory from `pool`, in
-// the order of stream s, which is synchronised.
+// where the lists are short anyway, would take more than max_bytes, or there is no
+// memory.  Memory from `pool`, in the order of stream s, which is synchronised.
 struct LocalLists {
     void *mem;
     size_t bytes;
@@ -165,7 +165,8 @@ struct LocalLists {
     const uint4 *undo;
     uint64_t n_loc, n_undo;
 };
-cudaError_t build_local_lists(const IndexView &view, uint4 *ent, LocalLists &out, cudaStream_t s, cudaMemPool_t pool);
+cudaError_t build_local_lists(const IndexView &view, uint4 *ent, LocalLists &out, size_t max_bytes, cudaStream_t s,
+                              cudaMemPool_t pool);
 
 // The index of buffered polygons (NearView), built on the device from the host's
 // edge grid (cell_off, item_q, item_seg: CSR by cell of a 2^g grid, on the
