@@ -201,9 +201,8 @@ spx_status spx_build_disk_index(spx_ctx *ctx, const int32_t *cxy, const int32_t 
  * "Database Setup and Tuning"; building it on the device keeps that cost small
  * for new query sets): every (cell, disk) pair of each disk's
  * bounding box is classified on the device, bucketed by cell, and the lists
- * laid out in cell order and sorted by disk, so the cell words, entries and
- * cover bitmap are byte for byte those of spx_build_disk_index (see
- * spx_disk_index_arrays).  Same arguments, checks, grid choice and errors;
+ * laid out in cell order and sorted by disk, so the cell words and entries are
+ * byte for byte those of spx_build_disk_index (see spx_disk_index_arrays).  Same arguments, checks, grid choice and errors;
  * the build synchronises the device.  It allocates temporaries of about
  * 20 B per cell of the 4^grid_log2 grid plus 8 B per (cell, disk) record.
  */

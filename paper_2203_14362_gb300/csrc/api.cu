@@ -54,11 +54,10 @@ struct PolysObj {
 
 struct IndexObj {
     uint64_t polys = 0;
-    int kind = 0;        // 0: polygons (view), 1: disks (dview), 2: buffered polygons (view, nview, near)
-    DiskView dview{};
+    int kind = 0;        // 0: polygons (view), 1: disks (nview, near), 2: buffered polygons (view, nview, near)
     IndexView nview{};   // kinds 1 and 2: the grid of the disks or buffered polygons,
     NearView near{};     // and their disks, or radii and containment (view)
-    void *mem2 = nullptr; // buffered polygons: radii
+    void *mem2 = nullptr; // buffered polygons: radii; disks: block summary
     void *mem3 = nullptr; // buffered polygons: their own grid (cells | fine | entries | edges | summary)
     IndexView view{};
     int fp32 = 1;
@@ -1219,17 +1218,19 @@ static std::string check_disks(const int32_t *cxy, const int32_t *r, uint32_t Q)
 
 // Registers a disk index whose arrays are in one device allocation.
 static spx_status register_disk_index(spx_ctx *ctx, void *mem, size_t total, const uint32_t *cell, const uint32_t *ent,
-                                      const int4 *disk, const uint32_t *cover, int g, uint32_t Q, uint64_t n_entries,
-                                      uint64_t n_inside, uint64_t n_boundary,
+                                      const int4 *disk, int g, uint32_t Q, uint64_t n_entries, uint64_t n_inside,
+                                      uint64_t n_boundary,
                                       std::chrono::steady_clock::time_point t0, spx_index *out)
 {
     auto ix = std::make_unique<IndexObj>();
     ix->mem = mem;
     ix->kind = 1;
     double resolved = 0;
-    cudaError_t e = dev_alloc(ctx, &ix->mem2, size_t(2) << (2 * kSumLog2));
+    const size_t b_sum = size_t(2) << (2 * kSumLog2); // and a counter
+    cudaError_t e = dev_alloc(ctx, &ix->mem2, b_sum + 8);
     if (e == cudaSuccess)
-        e = prepare_disk_words(const_cast<uint32_t *>(cell), g, static_cast<uint16_t *>(ix->mem2), &resolved);
+        e = prepare_disk_words(const_cast<uint32_t *>(cell), g, static_cast<uint16_t *>(ix->mem2),
+                               reinterpret_cast<unsigned long long *>(static_cast<char *>(ix->mem2) + b_sum), &resolved);
     if (e != cudaSuccess) {
         free_index_memory(ctx, *ix);
         return e == cudaErrorMemoryAllocation ? fail(ctx, SPX_ENOMEM, "build_disk_index: cudaMalloc failed")
@@ -1237,22 +1238,12 @@ static spx_status register_disk_index(spx_ctx *ctx, void *mem, size_t total, con
     }
     GridParts gp{};
     gp.cell = reinterpret_cast<char *>(const_cast<uint32_t *>(cell));
-    gp.cover = reinterpret_cast<char *>(const_cast<uint32_t *>(cover));
     gp.sum = static_cast<char *>(ix->mem2);
     gp.sum_resolved = resolved;
     ix->nview = grid_view(gp, g, 0, Q);
     ix->nview.err = &ctx->aux->err;
     ix->near.disk = disk;
     ix->near.dent = ent;
-    ix->dview.cell = cell;
-    ix->dview.ent = ent;
-    ix->dview.disk = disk;
-    ix->dview.cover = cover;
-    ix->dview.sc = kBoxLog2 - g;
-    ix->dview.g = g;
-    ix->dview.cg = std::min(g, kCoverLog2);
-    ix->dview.scv = kBoxLog2 - ix->dview.cg;
-    ix->dview.Q = Q;
     spx_index_info &inf = ix->info;
     inf.grid_log2 = g;
     inf.n_polys = Q;
@@ -1260,7 +1251,7 @@ static spx_status register_disk_index(spx_ctx *ctx, void *mem, size_t total, con
     inf.n_entries = n_entries;
     inf.n_inside = n_inside;
     inf.n_boundary = n_boundary;
-    inf.device_bytes = total + (size_t(2) << (2 * kSumLog2));
+    inf.device_bytes = total + b_sum + 8;
     inf.sum_resolved = resolved;
     inf.use_sum = ix->nview.use_sum;
     inf.build_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
@@ -1297,31 +1288,25 @@ spx_status spx_build_disk_index(spx_ctx *ctx, const int32_t *cxy, const int32_t 
     if (!build_disk_index(cxy, r, Q, g, hd, err))
         return fail(ctx, SPX_EINVAL, "build_disk_index: " + err);
     const std::vector<int4> disks = disk_array(cxy, r, Q);
-    const std::vector<uint32_t> cover = cover_bitmap(hd.cell.data(), g);
     auto up = [](size_t v) { return (v + 255) & ~size_t(255); };
-    const size_t b_cell = hd.cell.size() * 4, b_ent = hd.entries.size() * 4, b_disk = disks.size() * sizeof(int4),
-                 b_cover = cover.size() * 4;
-    const size_t total = up(b_cell) + up(b_ent) + up(b_disk) + up(b_cover);
+    const size_t b_cell = hd.cell.size() * 4, b_ent = hd.entries.size() * 4, b_disk = disks.size() * sizeof(int4);
+    const size_t total = up(b_cell) + up(b_ent) + up(b_disk);
     void *mem = nullptr;
     if (dev_alloc(ctx, &mem, total) != cudaSuccess)
         return fail(ctx, SPX_ENOMEM, "build_disk_index: cudaMalloc failed");
-    char *m = static_cast<char *>(mem), *p_ent = m + up(b_cell), *p_disk = p_ent + up(b_ent),
-         *p_cover = p_disk + up(b_disk);
+    char *m = static_cast<char *>(mem), *p_ent = m + up(b_cell), *p_disk = p_ent + up(b_ent);
     cudaError_t e = cudaMemcpy(m, hd.cell.data(), b_cell, cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
         e = cudaMemcpy(p_ent, hd.entries.data(), b_ent, cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
         e = cudaMemcpy(p_disk, disks.data(), b_disk, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess)
-        e = cudaMemcpy(p_cover, cover.data(), b_cover, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         cudaFree(mem);
         return cuda_fail(ctx, e, "build_disk_index upload");
     }
     return register_disk_index(ctx, mem, total, reinterpret_cast<const uint32_t *>(m),
                                reinterpret_cast<const uint32_t *>(p_ent), reinterpret_cast<const int4 *>(p_disk),
-                               reinterpret_cast<const uint32_t *>(p_cover), g, Q, hd.entries.size(), hd.n_inside,
-                               hd.n_boundary, t0, out);
+                               g, Q, hd.entries.size(), hd.n_inside, hd.n_boundary, t0, out);
 }
 
 spx_status spx_build_disk_index_device(spx_ctx *ctx, const int32_t *cxy, const int32_t *r, uint32_t Q, int grid_log2,
@@ -1354,8 +1339,7 @@ spx_status spx_build_disk_index_device(spx_ctx *ctx, const int32_t *cxy, const i
     if (st != 0)
         return e == cudaErrorMemoryAllocation ? fail(ctx, SPX_ENOMEM, "build_disk_index_device: out of device memory")
                                               : cuda_fail(ctx, e, "build_disk_index_device");
-    return register_disk_index(ctx, d.mem, d.bytes, d.cell, d.ent, d.disk, d.cover, g, Q, d.n_ent, d.n_inside,
-                               d.n_boundary, t0, out);
+    return register_disk_index(ctx, d.mem, d.bytes, d.cell, d.ent, d.disk, g, Q, d.n_ent, d.n_inside, d.n_boundary, t0, out);
 }
 
 spx_status spx_disk_index_arrays(spx_ctx *ctx, spx_index index, uint32_t *cell, uint32_t *entries, uint64_t sizes[3])
@@ -1371,12 +1355,12 @@ spx_status spx_disk_index_arrays(spx_ctx *ctx, spx_index index, uint32_t *cell, 
     sizes[1] = ix->info.n_entries;
     sizes[2] = uint64_t(ix->info.grid_log2);
     if (cell)
-        SPX_CUDA(cudaMemcpy(cell, ix->dview.cell, sizes[0] * 4, cudaMemcpyDeviceToHost), "disk_index_arrays copy");
+        SPX_CUDA(cudaMemcpy(cell, ix->nview.cell, sizes[0] * 4, cudaMemcpyDeviceToHost), "disk_index_arrays copy");
     for (uint64_t c = 0; cell && c < sizes[0]; ++c) // as built: prepare_disk_words set the lists' lower kind bit
         if ((cell[c] >> 30) == kCellCoarseList)
             cell[c] ^= 1u << 30;
     if (entries)
-        SPX_CUDA(cudaMemcpy(entries, ix->dview.ent, sizes[1] * 4, cudaMemcpyDeviceToHost), "disk_index_arrays copy");
+        SPX_CUDA(cudaMemcpy(entries, ix->near.dent, sizes[1] * 4, cudaMemcpyDeviceToHost), "disk_index_arrays copy");
     return SPX_OK;
 }
 

@@ -195,10 +195,11 @@ __device__ __forceinline__ int orient_sign(int ax, int ay, int bx, int by, int p
 // Parity of the crossings of the rightward ray from (px, py) with a fine-row
 // edge list sorted by max x descending.  Edges are loaded RW at a time so a
 // list costs one L2 round trip per RW edges.
-template <bool FP32, int RW = 4>
+template <bool FP32>
 __device__ __forceinline__ uint32_t row_parity(const int4 *__restrict__ e, uint32_t n, int px, int py,
                                                uint32_t &tests, uint32_t &esc, uint64_t pol)
 {
+    constexpr int RW = 4;
     uint32_t par = 0;
     for (uint32_t k = 0; k < n; k += RW) {
         int4 v[RW];
@@ -380,7 +381,7 @@ __device__ __forceinline__ void point_emit(const IndexView &ix, int px, int py, 
 // arrays (both end with a sentinel), and selects the results; divergent lanes
 // of a warp would otherwise serialise their memory round trips.  Longer lists
 // finish in a loop.
-template <bool FP32, int RW = 4>
+template <bool FP32>
 __device__ __forceinline__ uint32_t walk_list(const IndexView &ix, uint32_t e0, int px, int py, uint32_t &first,
                                               uint32_t &tests, uint32_t &esc, uint64_t pol)
 {
@@ -411,9 +412,9 @@ __device__ __forceinline__ uint32_t walk_list(const IndexView &ix, uint32_t e0, 
     }
     // lists longer than four edges: the rest, in row order
     if ((en0.w & kEntBoundary) && en0.z > 4 && max(v0[3].x, v0[3].z) > px)
-        p0 ^= row_parity<FP32, RW>(edge_at(ix, en0.y) + 4, en0.z - 4, px, py, tests, esc, pol);
+        p0 ^= row_parity<FP32>(edge_at(ix, en0.y) + 4, en0.z - 4, px, py, tests, esc, pol);
     if (two && (en1.w & kEntBoundary) && en1.z > 4 && max(v1[3].x, v1[3].z) > px)
-        p1 ^= row_parity<FP32, RW>(edge_at(ix, en1.y) + 4, en1.z - 4, px, py, tests, esc, pol);
+        p1 ^= row_parity<FP32>(edge_at(ix, en1.y) + 4, en1.z - 4, px, py, tests, esc, pol);
     const uint32_t in0 = (en0.w & kEntBoundary) ? p0 : 1u;
     const uint32_t in1 = two ? ((en1.w & kEntBoundary) ? p1 : 1u) : 0u;
     uint32_t c = in0 + in1;
@@ -1303,7 +1304,7 @@ __global__ void __launch_bounds__(THREADS, TMA ? 6 : kResolveMinBlocks)
             if (lane == 0 && nx < nchunks && full(nx))
                 bulk_load(s_buf, a.pts + (uint64_t)nx * kWChunk, kWChunk * sizeof(int2), s_bar);
         } else {
-            if (kPrefetchChunks > 0 && lane == 0) {
+            if (!TMA && kPrefetchChunks > 0 && lane == 0) { // (with TMA only a ragged last chunk comes here)
                 // this warp's chunk kPrefetchChunks ahead goes to L2 while this one is resolved
                 const uint64_t nb = base + (uint64_t)kPrefetchChunks * nw * kWChunk;
                 if (nb + kWChunk <= a.n)
@@ -2900,25 +2901,11 @@ __global__ void k_dbuild_sort(uint32_t ncell, const uint32_t *cell_word, uint32_
     }
 }
 
-// Cover bitmap: a bit per block of cells that holds a non-empty cell.
-__global__ void k_dbuild_cover(uint32_t ncell, int g, int cg, const uint32_t *cell_word, uint32_t *cover)
-{
-    for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < ncell; c += gridDim.x * blockDim.x) {
-        if (!cell_word[c])
-            continue;
-        const uint32_t cx = c & ((1u << g) - 1), cy = c >> g;
-        const uint32_t b = ((cy >> (g - cg)) << cg) | (cx >> (g - cg));
-        atomicOr(cover + (b >> 5), 1u << (b & 31));
-    }
-}
-
 int build_disk_index_device(const int4 *disks_host, uint32_t Q, int g, DiskIndexDev &out, cudaError_t &cerr)
 {
     out = DiskIndexDev{};
     cerr = cudaSuccess;
     const uint32_t ncell = 1u << (2 * g);
-    const int cg = g < kCoverLog2 ? g : kCoverLog2;
-    const size_t cover_words = ((size_t(1) << (2 * cg)) / 32) > 0 ? ((size_t(1) << (2 * cg)) / 32) : 1;
     const size_t nd = Q ? Q : 1;
     const uint64_t nparts = scan_partials(ncell > nd ? ncell : nd) + 2;
     // temporaries: disks | per-disk record counts | totals | scan partials |
@@ -2978,9 +2965,9 @@ int build_disk_index_device(const int4 *disks_host, uint32_t Q, int g, DiskIndex
     const uint64_t E = 1 + T;
     if (E > kPayloadMask)
         return done(1, cudaSuccess);
-    // the index's own allocation: cells | entries | disks | cover, as the host path lays it out
-    const size_t b_cell = size_t(ncell) * 4, b_ent = size_t(E) * 4, b_disk = nd * sizeof(int4), b_cover = cover_words * 4;
-    out.bytes = up(b_cell) + up(b_ent) + up(b_disk) + up(b_cover);
+    // the index's own allocation: cells | entries | disks, as the host path lays it out
+    const size_t b_cell = size_t(ncell) * 4, b_ent = size_t(E) * 4, b_disk = nd * sizeof(int4);
+    out.bytes = up(b_cell) + up(b_ent) + up(b_disk);
     if ((e = cudaMalloc(&out.mem, out.bytes)) != cudaSuccess) {
         out.mem = nullptr;
         return done(2, e);
@@ -2989,9 +2976,7 @@ int build_disk_index_device(const int4 *disks_host, uint32_t Q, int g, DiskIndex
     out.cell = reinterpret_cast<uint32_t *>(m);
     out.ent = reinterpret_cast<uint32_t *>(m + up(b_cell));
     out.disk = reinterpret_cast<int4 *>(m + up(b_cell) + up(b_ent));
-    out.cover = reinterpret_cast<uint32_t *>(m + up(b_cell) + up(b_ent) + up(b_disk));
     if ((e = cudaMemset(out.cell, 0, b_cell)) != cudaSuccess || (e = cudaMemset(out.ent, 0, b_ent)) != cudaSuccess ||
-        (e = cudaMemset(out.cover, 0, b_cover)) != cudaSuccess ||
         (e = cudaMemcpy(out.disk, d_disk, b_disk, cudaMemcpyDeviceToDevice)) != cudaSuccess)
         return done(2, e);
     k_dbuild_cells<<<cblocks, 256>>>(ncell, cell_cnt, cell_bnd, words, out.cell, out.ent);
@@ -3003,7 +2988,6 @@ int build_disk_index_device(const int4 *disks_host, uint32_t Q, int g, DiskIndex
                                            out.cell, out.ent);
         k_dbuild_sort<<<cblocks, 256>>>(ncell, out.cell, out.ent);
     }
-    k_dbuild_cover<<<cblocks, 256>>>(ncell, g, cg, out.cell, out.cover);
     if ((e = cudaGetLastError()) != cudaSuccess || (e = cudaDeviceSynchronize()) != cudaSuccess)
         return done(2, e);
     out.n_ent = E;
@@ -3688,8 +3672,8 @@ cudaError_t launch_aggregate(const JoinLaunch &a, void *scratch, cudaStream_t s,
         k_agg_cells<<<grid, 256, 0, s>>>(a.cell_end, a.cluster_log2, a.ix, a.counts, rows, a.stats);
         if ((e = cudaGetLastError()) != cudaSuccess)
             return e;
-        e = a.fp32 ? launch_walk<true, kOutCount, false, true>(a, rows, s)
-                   : launch_walk<false, kOutCount, false, true>(a, rows, s);
+        e = a.fp32 ? launch_walk<true, kOutCount, kPoly, true>(a, rows, s)
+                   : launch_walk<false, kOutCount, kPoly, true>(a, rows, s);
     } else if (a.clustered)
         e = a.fp32 ? launch_warp_kernel<true, true>(a, use_hist, s) : launch_warp_kernel<false, true>(a, use_hist, s);
     else
@@ -4282,22 +4266,19 @@ __global__ void __launch_bounds__(256) k_disk_words(uint32_t ncell, uint32_t *ce
             cell[c] |= kCellCoarseList << 30;
 }
 
-cudaError_t prepare_disk_words(uint32_t *cell, int g, uint16_t *sum, double *sum_resolved)
+cudaError_t prepare_disk_words(uint32_t *cell, int g, uint16_t *sum, unsigned long long *n, double *sum_resolved)
 {
     const uint32_t ncell = 1u << (2 * g);
     const int sg = std::min(g, kSumLog2);
-    unsigned long long *n = nullptr, h = 0;
-    cudaError_t e = cudaMalloc(&n, 8);
-    if (e != cudaSuccess)
-        return e;
-    if ((e = cudaMemset(n, 0, 8)) == cudaSuccess) {
+    unsigned long long h = 0;
+    cudaError_t e = cudaMemset(n, 0, 8);
+    if (e == cudaSuccess) {
         k_disk_words<<<std::min<uint32_t>((ncell + 255) / 256, uint32_t(device_sm_count()) * 32), 256>>>(ncell, cell);
         k_near_sum<<<((1u << (2 * sg)) + 255) / 256, 256>>>(g, sg, cell, sum, n, nullptr, nullptr);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess)
         e = cudaMemcpy(&h, n, 8, cudaMemcpyDeviceToHost);
-    cudaFree(n);
     *sum_resolved = double(h) / double(uint64_t(1) << (2 * sg));
     return e;
 }
