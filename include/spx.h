@@ -124,7 +124,9 @@ spx_status spx_load_polygons(spx_ctx *ctx, const int32_t *xy, const uint64_t *ri
 typedef struct {
     int grid_log2;   /* coarse grid of 2^grid_log2 cells per side, 1..13; 0 = choose automatically
                         (about 80 cells across the median polygon bounding box, clamped to 5..13) */
-    int fp32_filter; /* 1: orientation in FP32 with exact int64 redo inside the error bound; 0: int64 only */
+    int fp32_filter; /* 1: orientation in FP32 with exact int64 redo inside the error bound; 0: int64 only.
+                        (The tests of points.  Which edges a cell lists is decided in FP32 either way, with
+                        a margin that keeps every edge the exact test could need.) */
     int sub_log2;    /* a coarse cell cut by a polygon boundary is split into 2^sub_log2 x 2^sub_log2
                         fine cells, 1..3 (grid_log2 + sub_log2 <= 16); 0 = default (3) */
     int reserved[5]; /* must be zero */
@@ -402,7 +404,9 @@ spx_status spx_join_plain_static(spx_ctx *ctx, spx_points points, spx_index inde
  * Aggregations", the plan for point data): counts_dev[q] (uint64, P entries,
  * device) = number of points inside polygon q.  Large tables take a bit per point
  * of scratch in the stream's order (none shared with other calls; a slower pass
- * without it when there is no memory).
+ * without it when there is no memory).  Captured, the scratch is a pair of
+ * allocation nodes of the graph, which CUDA instantiates once at a time and neither
+ * clones nor nests.
  */
 spx_status spx_aggregate(spx_ctx *ctx, spx_points points, spx_index index, uint64_t *counts_dev, void *stream);
 
@@ -536,12 +540,13 @@ typedef struct {
     uint64_t pairs_emitted;
     uint64_t timed_joins;      /* joins timed since the last reset */
     uint64_t timed_aggregates; /* aggregates timed since the last reset */
-    double ms_resolve;         /* join pass 1 (distance join: all of it; polygon join: 1a, index lookups
-                                  of every point, results and counts of points that need no exact test) */
+    double ms_resolve;         /* join pass 1a, of polygon and disk indexes: index lookups of every point,
+                                  results and counts of points that need no exact test (small tables: 1b
+                                  too) */
     double ms_scan;            /* join pass 2: scan of per-tile pair totals */
     double ms_emit;            /* join pass 3: pairs written in point order */
     double ms_aggregate;       /* count-only aggregate */
-    double ms_walk;            /* polygon join pass 1b: exact tests of the points whose cell lists edges */
+    double ms_walk;            /* join pass 1b: exact tests of the points whose cell lists edges or disks */
     uint64_t points_from_directory; /* of points_scanned, those an aggregate over a clustered table counted
                                        from its cell directory without reading them */
 } spx_stats_t;

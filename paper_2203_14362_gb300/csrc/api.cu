@@ -440,8 +440,6 @@ struct GridParts {
     double sum_resolved;
 };
 
-// Views and info of a polygon index whose allocation ix->mem holds `gp`;
-// takes the index into the ctx and returns its handle.
 // The kernels' view of a polygon index whose arrays are `gp`.
 static IndexView grid_view(const GridParts &gp, int g, int sb, uint32_t P)
 {
@@ -479,6 +477,9 @@ static GridParts device_parts(const GridIndexDev &d)
                      d.n_ent, d.n_edge, d.n_blocks, d.n_inside, d.n_mixed, d.n_boundary, d.sum_resolved};
 }
 
+// Views and info of a polygon index whose allocation ix->mem (total bytes) holds
+// `gp`, and its local lists (max_bytes: what the index may take with them); takes
+// the index into the ctx and returns its handle.
 spx_status register_grid_index(spx_ctx *ctx, spx_polys polys, std::unique_ptr<IndexObj> ix, size_t total, int g, int sb,
                                int fp32, const GridParts &gp, std::chrono::steady_clock::time_point t0, spx_index *out,
                                size_t max_bytes = SIZE_MAX)

@@ -1372,8 +1372,7 @@ __global__ void __launch_bounds__(THREADS, TMA ? 6 : kResolveMinBlocks)
     add_stats(a.stats, n_pts, 0u, 0u, n_pairs);
 }
 
-//
-// Up to kSmallHist polygons are counted in shared memory: where many points lie
+// Pass 1b.  Up to kSmallHist polygons are counted in shared memory: where many points lie
 // in several polygons (overlapping queries) a global atomic per hit on a few
 // hundred counters was what this pass waited for (20M points x 256 buffered
 // queries: 1545 -> 185 us).
@@ -1578,8 +1577,10 @@ cudaError_t launch_walk(const JoinLaunch &a, uint32_t *pend, cudaStream_t s)
 // summary for a few chunks each.  CTA of kThreads, no barrier between its warps
 // but for the counters (a CTA's points counted in shared memory when P is at
 // most kSmallHist).  Whole join with k_wemit16<SELF>, against pass 1a + 1b + scan
-// + pass 3, 2000-cell map: 20k points 18.5 against 28.8 us, 500k 20.6 / 32.8,
-// 1M 32.8 / 39.0, 1.5M 39.0 / 39.1, 2M 53.7 / 43.1; the line is at 1M points.
+// + pass 3, 2000-cell map: 20k points 19.1 against 30.9 us, 500k 21.2 / 32.9, 1M
+// 26.7 / 35.9, 1.5M 39.3 / 41.1, 2M 48.5 / 41.1, 3M 71.0 / 51.5; 256 stars: 1M 24.1 /
+// 32.9, 2M 35.1 / 35.0.  The two cross between 1.5M and 2M points.  The line is
+// below that, at 1M, where an earlier form of this kernel had it.
 constexpr uint32_t kSmallChunks = 4096;
 
 template <bool FP32, int OUT, int KIND>
@@ -1813,7 +1814,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_wemit(const __grid_constant__ J
 constexpr uint32_t kEmitStage = 320; // pairs; a full chunk's lie nine apart per lane of eight (no bank conflict)
 constexpr uint32_t kEmitQueue = kWChunk + 32; // a chunk's rows and a partial round
 constexpr size_t kEmit16Warp = (kEmitStage * 8 + size_t(kEmitQueue) * 12 + kWaveWords * 4 + 15) & ~size_t(15);
-constexpr size_t kEmit16Smem = kWarps * kEmit16Warp; // 53 KB: four CTAs per SM
+constexpr size_t kEmit16Smem = kWarps * kEmit16Warp; // 49 KB: four CTAs per SM
 static_assert(kWItems == 8, "a lane's rows: one 16-byte load of 2-byte results");
 
 template <bool FP32, bool SELF, int KIND>
@@ -2244,6 +2245,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_multi(const __grid_constant__ M
 // room for 207k ids: count + emit 170 -> 11.6 us; 84M ids of 256 queries keep
 // 32768).
 constexpr int kSuperTileMax = 32768, kSuperTileMin = 1024;
+constexpr uint32_t kSuperTiles = 2 * 152;  // two per SM
 constexpr int kSelMaxQ = 1024;            // queries per index (shared-memory counters)
 constexpr int kPartTile = 4096;           // pairs that k_part_emit orders in shared memory at a time
 constexpr int kPartRounds = kPartTile / kThreads; // rounds of 32 pairs per warp and tile
@@ -2252,7 +2254,7 @@ static_assert(kSelMaxQ == 4 * kThreads, "k_part_emit: at most four queries per t
 uint32_t super_tile(uint64_t cap)
 {
     uint32_t t = kSuperTileMax;
-    while (t > kSuperTileMin && (cap + t - 1) / t < 2 * 152)
+    while (t > kSuperTileMin && (cap + t - 1) / t < kSuperTiles)
         t >>= 1;
     return t;
 }
@@ -3181,7 +3183,13 @@ cudaError_t launch_sum_u64(unsigned long long *dst, const unsigned long long *x,
 // edges changes it twice, so the changes are the few vertices where a chain
 // passes from right to near or left.
 constexpr uint32_t kLocalMin = 8;   // shorter lists stay
-constexpr uint32_t kLocalMean = 8;  // mean edges per list from which an index gets local lists
+// Mean edges per list from which an index gets local lists.  50M points x 2000 cells,
+// without and with: at a mean of 4.2 the join takes 307 / 302 us, the build 4.0 / 4.7
+// ms and the index 463 / 519 MB; at 7.7 434 / 387 us, 1.6 / 2.1 ms, 66 / 86 MB; at
+// 11.1 627 / 491 us, 1.2 / 1.8 ms, 36 / 55 MB.  Shorter lists repay the build and the
+// memory only over many joins, so the line lies above the automatic grids' lists of
+// a map of small polygons.
+constexpr uint32_t kLocalMean = 8;
 constexpr int kLocalTurns = 8;      // changes of parity a cell may record; else the list stays
 
 // The parity of the right edges over the rows of a cell: at y0 (odd), and the y
@@ -3449,10 +3457,9 @@ cudaError_t build_local_lists(const IndexView &view, uint4 *ent, LocalLists &out
     k_list_edges<<<blocks(view.n_ent), 256, 0, s>>>(ent, view.n_ent, totals + 2);
     if ((e = cudaGetLastError()) != cudaSuccess || (e = read(5)) != cudaSuccess)
         return done(e);
-    // Lists of four edges (maps of 500 to 5000 cells with about 500 vertices each)
-    // gain nothing: 2000 cells, walk 81 us without, 92 with, and the build costs
-    // 2 ms.  40 (queries of up to 5000 vertices) or 15 (40000 cells of up to 10000):
-    // the walk of 500M points x 256 queries 4.39 -> 2.74 ms.
+    // Maps of 500 to 5000 cells with about 500 vertices each list four edges on
+    // average, queries of up to 5000 vertices 40 and 40000 cells of up to 10000
+    // vertices 15: the walk of 500M points x 256 queries 4.39 -> 2.74 ms.
     if (h[2] < kLocalMean * h[3] || !h[4])
         return done(cudaSuccess);
     if (cudaMallocFromPoolAsync(&tmp2, h[4] * 16, pool, s) != cudaSuccess) {
@@ -3690,10 +3697,10 @@ size_t select_scratch_bytes(uint64_t n, uint32_t P, uint64_t cap, bool aux)
 
 size_t partition_scratch_bytes(uint64_t cap, uint32_t P)
 {
-    // super_tile leaves fewer than 608 tiles, or takes the largest or the
+    // super_tile leaves fewer than 2 kSuperTiles tiles, or takes the largest or the
     // smallest size; this bound, unlike the count itself, grows with cap
     const uint64_t n_super = std::max((cap + kSuperTileMax - 1) / kSuperTileMax,
-                                      std::min<uint64_t>((cap + kSuperTileMin - 1) / kSuperTileMin, 608));
+                                      std::min<uint64_t>((cap + kSuperTileMin - 1) / kSuperTileMin, 2 * kSuperTiles));
     const uint64_t tab = uint64_t(P) * (n_super ? n_super : 1);
     return size_t(tab * 8 + (scan_partials(tab) + 2) * 8 + 64);
 }
