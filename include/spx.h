@@ -203,8 +203,9 @@ spx_status spx_build_disk_index(spx_ctx *ctx, const int32_t *cxy, const int32_t 
  * "Database Setup and Tuning"; building it on the device keeps that cost small
  * for new query sets): every (cell, disk) pair of each disk's
  * bounding box is classified on the device, bucketed by cell, and the lists
- * laid out in cell order and sorted by disk, so the cell words and entries are
- * byte for byte those of spx_build_disk_index (see spx_disk_index_arrays).  Same arguments, checks, grid choice and errors;
+ * laid out in cell order and sorted by disk, so the cell words, entries and
+ * cover bitmap are byte for byte those of spx_build_disk_index (see
+ * spx_disk_index_arrays).  Same arguments, checks, grid choice and errors;
  * the build synchronises the device.  It allocates temporaries of about
  * 20 B per cell of the 4^grid_log2 grid plus 8 B per (cell, disk) record.
  */
@@ -540,9 +541,9 @@ typedef struct {
     uint64_t pairs_emitted;
     uint64_t timed_joins;      /* joins timed since the last reset */
     uint64_t timed_aggregates; /* aggregates timed since the last reset */
-    double ms_resolve;         /* join pass 1a, of polygon and disk indexes: index lookups of every point,
-                                  results and counts of points that need no exact test (small tables: 1b
-                                  too) */
+    double ms_resolve;         /* join pass 1a: index lookups of every point, results and counts of points
+                                  that need no exact test (all of pass 1 where it is one kernel: small
+                                  tables, more than 2048 disks) */
     double ms_scan;            /* join pass 2: scan of per-tile pair totals */
     double ms_emit;            /* join pass 3: pairs written in point order */
     double ms_aggregate;       /* count-only aggregate */

@@ -1219,8 +1219,8 @@ static std::string check_disks(const int32_t *cxy, const int32_t *r, uint32_t Q)
 
 // Registers a disk index whose arrays are in one device allocation.
 static spx_status register_disk_index(spx_ctx *ctx, void *mem, size_t total, const uint32_t *cell, const uint32_t *ent,
-                                      const int4 *disk, int g, uint32_t Q, uint64_t n_entries, uint64_t n_inside,
-                                      uint64_t n_boundary,
+                                      const int4 *disk, const uint32_t *cover, int g, uint32_t Q, uint64_t n_entries,
+                                      uint64_t n_inside, uint64_t n_boundary,
                                       std::chrono::steady_clock::time_point t0, spx_index *out)
 {
     auto ix = std::make_unique<IndexObj>();
@@ -1230,8 +1230,8 @@ static spx_status register_disk_index(spx_ctx *ctx, void *mem, size_t total, con
     const size_t b_sum = size_t(2) << (2 * kSumLog2); // and a counter
     cudaError_t e = dev_alloc(ctx, &ix->mem2, b_sum + 8);
     if (e == cudaSuccess)
-        e = prepare_disk_words(const_cast<uint32_t *>(cell), g, static_cast<uint16_t *>(ix->mem2),
-                               reinterpret_cast<unsigned long long *>(static_cast<char *>(ix->mem2) + b_sum), &resolved);
+        e = disk_summary(cell, g, static_cast<uint16_t *>(ix->mem2),
+                         reinterpret_cast<unsigned long long *>(static_cast<char *>(ix->mem2) + b_sum), &resolved);
     if (e != cudaSuccess) {
         free_index_memory(ctx, *ix);
         return e == cudaErrorMemoryAllocation ? fail(ctx, SPX_ENOMEM, "build_disk_index: cudaMalloc failed")
@@ -1239,6 +1239,7 @@ static spx_status register_disk_index(spx_ctx *ctx, void *mem, size_t total, con
     }
     GridParts gp{};
     gp.cell = reinterpret_cast<char *>(const_cast<uint32_t *>(cell));
+    gp.cover = reinterpret_cast<char *>(const_cast<uint32_t *>(cover));
     gp.sum = static_cast<char *>(ix->mem2);
     gp.sum_resolved = resolved;
     ix->nview = grid_view(gp, g, 0, Q);
@@ -1289,25 +1290,31 @@ spx_status spx_build_disk_index(spx_ctx *ctx, const int32_t *cxy, const int32_t 
     if (!build_disk_index(cxy, r, Q, g, hd, err))
         return fail(ctx, SPX_EINVAL, "build_disk_index: " + err);
     const std::vector<int4> disks = disk_array(cxy, r, Q);
+    const std::vector<uint32_t> cover = cover_bitmap(hd.cell.data(), g);
     auto up = [](size_t v) { return (v + 255) & ~size_t(255); };
-    const size_t b_cell = hd.cell.size() * 4, b_ent = hd.entries.size() * 4, b_disk = disks.size() * sizeof(int4);
-    const size_t total = up(b_cell) + up(b_ent) + up(b_disk);
+    const size_t b_cell = hd.cell.size() * 4, b_ent = hd.entries.size() * 4, b_disk = disks.size() * sizeof(int4),
+                 b_cover = cover.size() * 4;
+    const size_t total = up(b_cell) + up(b_ent) + up(b_disk) + up(b_cover);
     void *mem = nullptr;
     if (dev_alloc(ctx, &mem, total) != cudaSuccess)
         return fail(ctx, SPX_ENOMEM, "build_disk_index: cudaMalloc failed");
-    char *m = static_cast<char *>(mem), *p_ent = m + up(b_cell), *p_disk = p_ent + up(b_ent);
+    char *m = static_cast<char *>(mem), *p_ent = m + up(b_cell), *p_disk = p_ent + up(b_ent),
+         *p_cover = p_disk + up(b_disk);
     cudaError_t e = cudaMemcpy(m, hd.cell.data(), b_cell, cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
         e = cudaMemcpy(p_ent, hd.entries.data(), b_ent, cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
         e = cudaMemcpy(p_disk, disks.data(), b_disk, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess)
+        e = cudaMemcpy(p_cover, cover.data(), b_cover, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         cudaFree(mem);
         return cuda_fail(ctx, e, "build_disk_index upload");
     }
     return register_disk_index(ctx, mem, total, reinterpret_cast<const uint32_t *>(m),
                                reinterpret_cast<const uint32_t *>(p_ent), reinterpret_cast<const int4 *>(p_disk),
-                               g, Q, hd.entries.size(), hd.n_inside, hd.n_boundary, t0, out);
+                               reinterpret_cast<const uint32_t *>(p_cover), g, Q, hd.entries.size(), hd.n_inside,
+                               hd.n_boundary, t0, out);
 }
 
 spx_status spx_build_disk_index_device(spx_ctx *ctx, const int32_t *cxy, const int32_t *r, uint32_t Q, int grid_log2,
@@ -1340,7 +1347,8 @@ spx_status spx_build_disk_index_device(spx_ctx *ctx, const int32_t *cxy, const i
     if (st != 0)
         return e == cudaErrorMemoryAllocation ? fail(ctx, SPX_ENOMEM, "build_disk_index_device: out of device memory")
                                               : cuda_fail(ctx, e, "build_disk_index_device");
-    return register_disk_index(ctx, d.mem, d.bytes, d.cell, d.ent, d.disk, g, Q, d.n_ent, d.n_inside, d.n_boundary, t0, out);
+    return register_disk_index(ctx, d.mem, d.bytes, d.cell, d.ent, d.disk, d.cover, g, Q, d.n_ent, d.n_inside,
+                               d.n_boundary, t0, out);
 }
 
 spx_status spx_disk_index_arrays(spx_ctx *ctx, spx_index index, uint32_t *cell, uint32_t *entries, uint64_t sizes[3])
@@ -1357,9 +1365,6 @@ spx_status spx_disk_index_arrays(spx_ctx *ctx, spx_index index, uint32_t *cell, 
     sizes[2] = uint64_t(ix->info.grid_log2);
     if (cell)
         SPX_CUDA(cudaMemcpy(cell, ix->nview.cell, sizes[0] * 4, cudaMemcpyDeviceToHost), "disk_index_arrays copy");
-    for (uint64_t c = 0; cell && c < sizes[0]; ++c) // as built: prepare_disk_words set the lists' lower kind bit
-        if ((cell[c] >> 30) == kCellCoarseList)
-            cell[c] ^= 1u << 30;
     if (entries)
         SPX_CUDA(cudaMemcpy(entries, ix->near.dent, sizes[1] * 4, cudaMemcpyDeviceToHost), "disk_index_arrays copy");
     return SPX_OK;

@@ -23,7 +23,8 @@
 // (k_walk) walks those lists 32 rows at a time.  A device-wide scan turns the
 // chunks' pair totals into offsets, and pass 3 (k_wemit16; k_wemit for 4-byte
 // results) writes each chunk's pairs in point order.  Small tables take one
-// pass-1 kernel (k_small).  The count aggregate is pass 1 alone, or k_warp.
+// pass-1 kernel (k_small), and so do many disks (k_disk_pass1).  The count aggregate
+// is pass 1 alone, or k_warp.
 // Serving batches (k_multi) and the selection partition (k_part_*) follow.
 #include "cell_filter.h"
 #include "kernels.h"
@@ -78,28 +79,42 @@ __device__ __forceinline__ uint32_t lanemask_lt()
     return m;
 }
 // L2 eviction policies: the index stays resident (evict_last) while the
-// streamed points pass through (evict_first).  Index words are read once per point
-// at random, 32 lines a warp: they take no L1 line (tess. join 100M x 2000 cells
-// 618 -> 604 us, count x 5000 cells 521 -> 487).
+// streamed points pass through (evict_first).
 __device__ __forceinline__ uint64_t policy_evict_last()
 {
     uint64_t p;
     asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
     return p;
 }
+// Pass 1a of polygons reads index words past L1: once per point, at random, 32 lines a
+// warp (100M points x 2000 cells 571 -> 549 us, count x 5000 cells 497 -> 467).
+// Everywhere else they take an L1 line.  Disk lists are read word after word, and
+// where points crowd into few cells their words are in L1: past it, 20M points, 90 %
+// of them in 256 cells of 64 disks, joined in 586 us instead of 257.
+template <bool L1 = true>
 __device__ __forceinline__ uint32_t ld_idx(const uint32_t *p, uint64_t pol)
 {
     uint32_t v;
-    asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.u32 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(pol));
+    if (L1)
+        asm volatile("ld.global.nc.L2::cache_hint.u32 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(pol));
+    else
+        asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.u32 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(pol));
     return v;
 }
 // The same where `on`, else v stays; without a branch.
+template <bool L1>
 __device__ __forceinline__ void ld_idx_if(uint32_t &v, const uint32_t *p, uint64_t pol, bool on)
 {
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\t"
-                 "@p ld.global.nc.L1::no_allocate.L2::cache_hint.u32 %0, [%1], %2;\n\t}"
-                 : "+r"(v)
-                 : "l"(p), "l"(pol), "r"((uint32_t)on));
+    if (L1)
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\t"
+                     "@p ld.global.nc.L2::cache_hint.u32 %0, [%1], %2;\n\t}"
+                     : "+r"(v)
+                     : "l"(p), "l"(pol), "r"((uint32_t)on));
+    else
+        asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\t"
+                     "@p ld.global.nc.L1::no_allocate.L2::cache_hint.u32 %0, [%1], %2;\n\t}"
+                     : "+r"(v)
+                     : "l"(p), "l"(pol), "r"((uint32_t)on));
 }
 __device__ __forceinline__ uint4 ld_idx(const uint4 *p, uint64_t pol)
 {
@@ -258,25 +273,33 @@ __device__ __forceinline__ bool edges_ok(const IndexView &ix, const uint4 &en)
            ((en.y & ix.loc_bit) ? (uint64_t)(en.y & ~kLocalEdge) + en.z <= ix.n_loc : (uint64_t)en.y + en.z < ix.n_edge);
 }
 
+template <bool L1 = true>
 __device__ __forceinline__ uint32_t coarse_word(const IndexView &ix, uint32_t px, uint32_t py, uint64_t pol)
 {
-    return ld_idx(ix.cell + (((py >> ix.sc) << ix.gc) | (px >> ix.sc)), pol);
+    return ld_idx<L1>(ix.cell + (((py >> ix.sc) << ix.gc) | (px >> ix.sc)), pol);
 }
+template <bool L1 = true>
 __device__ __forceinline__ uint32_t fine_word(const IndexView &ix, uint32_t w, uint32_t px, uint32_t py,
                                               uint64_t pol)
 {
     const uint32_t fm = (1u << ix.sb) - 1;
     if (!in_bounds(((uint64_t)(w & kPayloadMask) + 1) << (2 * ix.sb) <= ix.n_fine, ix))
         return 0u;
-    return ld_idx(ix.fine + (((w & kPayloadMask) << (2 * ix.sb)) | (((py >> ix.sf) & fm) << ix.sb) |
+    return ld_idx<L1>(ix.fine + (((w & kPayloadMask) << (2 * ix.sb)) | (((py >> ix.sf) & fm) << ix.sb) |
                              ((px >> ix.sf) & fm)),
                   pol);
 }
-// Resolved word of an in-box point: kind 0 none, 1 one INSIDE polygon, 2 list.
+// What an index's entry lists hold: polygons with crossing edges, buffered
+// polygons with edges that may be near, or disks.
+constexpr int kPoly = 0, kNear = 1, kDisk = 2;
+
+// Resolved word of an in-box point: kind 0 none, 1 one INSIDE polygon, 2 list (a disk
+// index has one level, whose words are that already).
+template <int KIND = kPoly>
 __device__ __forceinline__ uint32_t resolve(const IndexView &ix, uint32_t px, uint32_t py, uint64_t pol)
 {
     const uint32_t w = coarse_word(ix, px, py, pol);
-    return (w >> 30) == kCellSub ? fine_word(ix, w, px, py, pol) : w;
+    return KIND != kDisk && (w >> 30) == kCellSub ? fine_word(ix, w, px, py, pol) : w;
 }
 
 // One edge's contribution to the crossing parity of (px, py).
@@ -438,10 +461,6 @@ __device__ __forceinline__ uint32_t walk_list(const IndexView &ix, uint32_t e0, 
     }
     return c;
 }
-
-// What an index's entry lists hold: polygons with crossing edges, buffered
-// polygons with edges that may be near, or disks.
-constexpr int kPoly = 0, kNear = 1, kDisk = 2;
 
 // A point is within distance r of a centre c iff (px-cx)^2 + (py-cy)^2 <= r^2,
 // exact in int64 (differences < 2^31; r < 2^30; the x term is compared with
@@ -1118,7 +1137,7 @@ __host__ __device__ constexpr size_t resolve_smem_head(int warps, bool sum, int 
 // aggregate, whose pass 1b only counts).
 constexpr int kOut32 = 0, kOut16 = 1, kOutCount = 2;
 
-template <int OUT>
+template <int OUT, bool DISK>
 __global__ void __launch_bounds__(kResolveSumThreads, 1)
     k_resolve_sum(const __grid_constant__ JoinLaunch a, uint32_t *pend, uint32_t nchunks, int use_hist)
 {
@@ -1173,12 +1192,12 @@ __global__ void __launch_bounds__(kResolveSumThreads, 1)
             const bool ok = (px | py) < kBox; // both in [0, 2^30)
             const uint32_t sv = s_sum[(((py >> ix.ssh) << ix.sg) | (px >> ix.ssh)) & smask];
             w[j] = ok && sv != kSumEmpty ? (kCellInsideOne << 30) | sv : 0u;
-            ld_idx_if(w[j], ix.cell + (((py >> ix.sc) << ix.gc) | (px >> ix.sc)), keep, ok && sv == kSumMixed);
+            ld_idx_if<DISK>(w[j], ix.cell + (((py >> ix.sc) << ix.gc) | (px >> ix.sc)), keep, ok && sv == kSumMixed);
         }
 #pragma unroll
         for (int j = 0; j < kWItems; ++j)
-            if ((w[j] >> 30) == kCellSub)
-                w[j] = fine_word(ix, w[j], (uint32_t)p[j].x, (uint32_t)p[j].y, keep);
+            if (!DISK && (w[j] >> 30) == kCellSub) // a disk index has one level
+                w[j] = fine_word<false>(ix, w[j], (uint32_t)p[j].x, (uint32_t)p[j].y, keep);
         uint32_t bl[kWItems];
 #pragma unroll
         for (int j = 0; j < kWItems; ++j)
@@ -1250,7 +1269,7 @@ __global__ void __launch_bounds__(kResolveSumThreads, 1)
 // with plain loads.
 //
 // Without the summary.
-template <int THREADS, bool TMA, int OUT>
+template <int THREADS, bool TMA, int OUT, bool DISK>
 __global__ void __launch_bounds__(THREADS, TMA ? 6 : kResolveMinBlocks)
     k_resolve(const __grid_constant__ JoinLaunch a, uint32_t *pend, uint32_t nchunks, int use_hist)
 {
@@ -1323,12 +1342,12 @@ __global__ void __launch_bounds__(THREADS, TMA ? 6 : kResolveMinBlocks)
             const uint32_t px = ok ? (uint32_t)p[j].x : 0u, py = ok ? (uint32_t)p[j].y : 0u;
             w[j] = 0u;
             if (ok)
-                w[j] = coarse_word(ix, px, py, keep);
+                w[j] = coarse_word<DISK>(ix, px, py, keep);
         }
 #pragma unroll
         for (int j = 0; j < kWItems; ++j)
-            if ((w[j] >> 30) == kCellSub)
-                w[j] = fine_word(ix, w[j], (uint32_t)p[j].x, (uint32_t)p[j].y, keep);
+            if (!DISK && (w[j] >> 30) == kCellSub) // a disk index has one level
+                w[j] = fine_word<false>(ix, w[j], (uint32_t)p[j].x, (uint32_t)p[j].y, keep);
         uint32_t total = 0, mask = 0;
 #pragma unroll
         for (int j = 0; j < kWItems; ++j) {
@@ -1425,7 +1444,7 @@ __global__ void __launch_bounds__(kThreads, KIND == kNear ? 3 : kWalkMinBlocks) 
         uint32_t f = 0, c = 0;
         uint64_t ids = 0; // kOut16 and a.aux: the first polygons, aux_bits each
         walk_list_wave<FP32, KIND>(ix, has, it.z, (int)it.x, (int)it.y, n_tests, n_esc, keep, s_par, [&](uint32_t q) {
-            if (OUT == kOut16 && (c + 1) * a.aux_bits <= 64)
+            if (OUT == kOut16 && a.aux && (c + 1) * a.aux_bits <= 64)
                 ids |= (uint64_t)q << (a.aux_bits * c);
             f = c ? f : q;
             ++c;
@@ -1475,7 +1494,7 @@ __global__ void __launch_bounds__(kThreads, KIND == kNear ? 3 : kWalkMinBlocks) 
         if (OUT != kOut32) {
 #pragma unroll
             for (int u = 0; u < B; ++u)
-                if ((w[u] >> 30) == kCellSub)
+                if (KIND != kDisk && (w[u] >> 30) == kCellSub)
                     w[u] = fine_word(ix, w[u], (uint32_t)p[u].x, (uint32_t)p[u].y, keep);
         }
 #pragma unroll
@@ -1553,6 +1572,20 @@ __global__ void __launch_bounds__(kThreads, KIND == kNear ? 3 : kWalkMinBlocks) 
     add_stats(a.stats, n_pts, n_tests, n_esc, n_pairs);
 }
 
+// Opt a kernel in to the shared memory it needs (once per device).
+template <class K>
+cudaError_t smem_opt_in(K kernel, size_t bytes, bool (&done)[64])
+{
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 64 && done[dev])
+        return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
+    if (e == cudaSuccess && dev < 64)
+        done[dev] = true;
+    return e;
+}
+
 template <bool FP32, int OUT, int KIND, bool ALL = false>
 cudaError_t launch_walk(const JoinLaunch &a, uint32_t *pend, cudaStream_t s)
 {
@@ -1627,7 +1660,7 @@ __global__ void __launch_bounds__(kThreads, KIND == kNear ? 3 : 4) k_small(const
         }
 #pragma unroll
         for (int j = 0; j < kWItems; ++j)
-            if ((w[j] >> 30) == kCellSub)
+            if (KIND != kDisk && (w[j] >> 30) == kCellSub)
                 w[j] = fine_word(ix, w[j], (uint32_t)p[j].x, (uint32_t)p[j].y, keep);
         if (lane < kWItems)
             s_m[lane] = 0u;
@@ -1653,7 +1686,7 @@ __global__ void __launch_bounds__(kThreads, KIND == kNear ? 3 : 4) k_small(const
             uint64_t ids = 0; // kOut16 and a.aux: the first polygons, aux_bits each
             walk_list_wave<FP32, KIND>(ix, has, it.z, (int)it.x, (int)it.y, n_tests, n_esc, keep, s_pa + warp * kWaveWords,
                                  [&](uint32_t q) {
-                                     if (OUT == kOut16 && (c + 1) * a.aux_bits <= 64)
+                                     if (OUT == kOut16 && a.aux && (c + 1) * a.aux_bits <= 64)
                                          ids |= (uint64_t)q << (a.aux_bits * c);
                                      f = c ? f : q;
                                      ++c;
@@ -1685,6 +1718,186 @@ __global__ void __launch_bounds__(kThreads, KIND == kNear ? 3 : 4) k_small(const
                 atomicAdd(a.counts + i, (unsigned long long)s_hist[i]);
     }
     add_stats(a.stats, lane == 0 ? npts : 0u, n_tests, n_esc, total);
+}
+
+// Pass 1 of a disk index in one kernel: counts, and joins of more than kDiskSplit
+// disks.  Disk lists are short and their tests cheap: a lane walks its own list as soon
+// as a round of 32 list points is queued (across chunks), with the point at hand.  A
+// point in a block that no disk reaches leaves by the cover bitmap, in shared memory (8
+// KB where the summary takes 128, so four CTAs per SM keep 32 warps).  Counts in shared
+// memory up to kHistMax disks.
+// Counts, against passes 1a and 1b (which re-read their rows): 20M points x 64 / 1024 /
+// 4096 disks 52 / 71 / 82 us against 56 / 68 / 107, over a clustered table 50 / 59 /
+// 73 against 61 / 96 / 158, 300k x 1024 12.1 against 14.5.  Joins: 100M x 1024 disks
+// 500 us against 433, 20M x 1024 125 against 117; 20M x 4096, which k_walk counts in
+// global memory, 140 against 185, x 20000 159 against 198, and with 90 % of 20M points
+// in 512 of 4096 disks, where counters take millions of hits each, 6.8 ms against 59.6.
+constexpr uint32_t kDiskSplit = kSmallHist;
+constexpr uint32_t kDiskCoverWords = 1u << (2 * kCoverLog2 - 5);
+constexpr int kDiskQueue = kWChunk + 32; // a chunk's points plus a partial round
+constexpr size_t kDiskSmem = size_t(kWarps) * kDiskQueue * sizeof(uint4) + kDiskCoverWords * sizeof(uint32_t);
+
+template <int OUT>
+__global__ void __launch_bounds__(kThreads, 4)
+    k_disk_pass1(const __grid_constant__ JoinLaunch a, uint32_t *pend, uint32_t nchunks, int use_hist)
+{
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint4 *s_q = reinterpret_cast<uint4 *>(s_raw) + warp * kDiskQueue; // (x, y, list, row)
+    uint32_t *s_cov = reinterpret_cast<uint32_t *>(s_raw + size_t(kWarps) * kDiskQueue * sizeof(uint4));
+    uint32_t *s_hist = s_cov + kDiskCoverWords;
+    const IndexView &ix = a.ix;
+    const uint64_t keep = policy_evict_last();
+    const bool hist = use_hist && a.counts;
+    for (uint32_t i = threadIdx.x; i < max(1u, (1u << (2 * ix.cg)) >> 5); i += kThreads)
+        s_cov[i] = __ldg(ix.cover + i);
+    if (hist)
+        for (uint32_t i = threadIdx.x; i < ix.P; i += kThreads)
+            s_hist[i] = 0;
+    __syncthreads();
+    auto count1 = [&](bool has, uint32_t q) { // one disk for every lane with has (converged warp)
+        if (!a.counts)
+            return;
+        if (!hist)
+            global_add_warp(a.counts, has, q);
+        else if (has)
+            atomicAdd(s_hist + q, 1u);
+    };
+    unsigned short *res16 = reinterpret_cast<unsigned short *>(a.res);
+    uint32_t n_tests = 0, n_pts = 0, n_pairs = 0, qn = 0; // qn: queued points, < 32 between chunks
+    auto walk = [&](uint32_t k0, uint32_t m) { // queued points [k0, k0 + m), m <= 32
+        const bool has = (uint32_t)lane < m;
+        const uint4 it = s_q[k0 + (has ? lane : 0)]; // idle lanes repeat lane 0's walk, uncounted
+        const uint32_t *e = a.near.dent + it.z;
+        const uint32_t n = ld_idx(e, keep);
+        uint32_t c = 0, f = 0, tests = 0;
+        uint64_t ids = 0; // kOut16 and a.aux: the first disks, aux_bits each
+        for (uint32_t k = 1; k <= n; ++k) {
+            const uint32_t en = ld_idx(e + k, keep), q = en >> 1;
+            bool in = true;
+            if (en & 1u) {
+                ++tests;
+                in = in_disk(__ldg(a.near.disk + q), (int)it.x, (int)it.y);
+            }
+            if (in) {
+                if (OUT == kOut16 && a.aux && (c + 1) * a.aux_bits <= 64)
+                    ids |= (uint64_t)q << (a.aux_bits * c);
+                if (!c)
+                    f = q; // counted with the warp below
+                else if (has && a.counts)
+                    hist ? (void)atomicAdd(s_hist + q, 1u) : (void)atomicAdd(a.counts + q, 1ull);
+                ++c;
+            }
+        }
+        c = has ? c : 0u;
+        n_tests += has ? tests : 0u;
+        n_pairs += c;
+        __syncwarp();
+        count1(c >= 1, f);
+        if (OUT != kOutCount && has) {
+            const uint32_t row = it.w;
+            if (OUT == kOut16) {
+                __stcg(res16 + row, (unsigned short)(c == 0 ? kRes16None : c == 1 ? f : c));
+                if (c >= 2) { // the row's bit: only this warp writes the words of its chunks
+                    atomicOr(pend + (row >> 5), 1u << (row & 31));
+                    if (a.aux && c * a.aux_bits <= 64)
+                        __stcg(reinterpret_cast<unsigned long long *>(a.aux) + row, (unsigned long long)ids);
+                }
+            } else {
+                __stcg(a.res + row, res_encode(c, f));
+            }
+            if (c)
+                atomicAdd(a.tile_tot + row / kWChunk, (unsigned long long)c);
+        }
+        __syncwarp();
+    };
+    const uint32_t nw = gridDim.x * kWarps;
+    for (uint32_t ch = blockIdx.x * kWarps + warp; ch < nchunks; ch += nw) {
+        const uint64_t base = (uint64_t)ch * kWChunk;
+        const uint32_t npts = (uint32_t)min((uint64_t)kWChunk, a.n - base);
+        n_pts += lane == 0 ? npts : 0u;
+        int2 p[kWItems];
+        uint32_t w[kWItems];
+#pragma unroll
+        for (int j = 0; j < kWItems; ++j) {
+            const uint32_t loc = j * 32 + lane;
+            p[j] = loc < npts ? __ldcs(a.pts + base + loc) : make_int2(-1, -1);
+        }
+        if (OUT == kOut16 && lane < kWItems)
+            __stcg(pend + (uint64_t)ch * kWItems + lane, 0u);
+#pragma unroll
+        for (int j = 0; j < kWItems; ++j) {
+            const uint32_t px = (uint32_t)p[j].x, py = (uint32_t)p[j].y;
+            const uint32_t b = (((py & (kBox - 1)) >> ix.scv) << ix.cg) | ((px & (kBox - 1)) >> ix.scv);
+            const bool ok = (px | py) < kBox && ((s_cov[b >> 5] >> (b & 31)) & 1u);
+            w[j] = ok ? ld_idx(ix.cell + ((((py & (kBox - 1)) >> ix.sc) << ix.gc) | ((px & (kBox - 1)) >> ix.sc)), keep) : 0u;
+        }
+        uint32_t total = 0;
+#pragma unroll
+        for (int j = 0; j < kWItems; ++j) {
+            const uint32_t kind = w[j] >> 30, loc = j * 32 + lane, pay = w[j] & kPayloadMask;
+            const bool one = kind == kCellInsideOne && in_bounds(pay < ix.P, ix), lst = kind >= kCellList;
+            total += one ? 1u : 0u;
+            count1(one, pay);
+            if (OUT != kOutCount && loc < npts && !lst) {
+                if (OUT == kOut16)
+                    __stcg(res16 + base + loc, (unsigned short)(one ? pay : kRes16None));
+                else
+                    __stcg(a.res + base + loc, one ? pay : kResNone);
+            }
+            const uint32_t bl = __ballot_sync(kFull, lst);
+            if (lst)
+                s_q[qn + __popc(bl & lanemask_lt())] =
+                    make_uint4((uint32_t)p[j].x, (uint32_t)p[j].y, pay, (uint32_t)(base + loc));
+            qn += __popc(bl);
+        }
+        n_pairs += total;
+        if (OUT != kOutCount) {
+            total = __reduce_add_sync(kFull, total);
+            if (lane == 0)
+                a.tile_tot[ch] = total; // without its queued points, which add theirs
+        }
+        __syncwarp();
+        if (qn >= 32) {
+            uint32_t k0 = 0;
+            for (; qn - k0 >= 32; k0 += 32)
+                walk(k0, 32);
+            const uint32_t rem = qn - k0; // the partial round (< 32, from k0 >= 32) to the front
+            const uint4 it = (uint32_t)lane < rem ? s_q[k0 + lane] : make_uint4(0u, 0u, 0u, 0u);
+            __syncwarp();
+            if ((uint32_t)lane < rem)
+                s_q[lane] = it;
+            qn = rem;
+            __syncwarp();
+        }
+    }
+    if (qn)
+        walk(0, qn);
+    if (hist) {
+        __syncthreads();
+        for (uint32_t i = threadIdx.x; i < ix.P; i += kThreads)
+            if (s_hist[i])
+                atomicAdd(a.counts + i, (unsigned long long)s_hist[i]);
+    }
+    add_stats(a.stats, n_pts, n_tests, 0u, n_pairs);
+}
+
+template <int OUT>
+cudaError_t launch_disk_pass1(const JoinLaunch &a, uint32_t *pend, cudaStream_t s)
+{
+    static bool done[64] = {};
+    if (a.n >= (1ull << 32))
+        return cudaErrorInvalidValue; // rows are 32-bit
+    const uint64_t nchunks = (a.n + kWChunk - 1) / kWChunk;
+    const int use_hist = a.counts && a.ix.P <= (uint32_t)kHistMax ? 1 : 0;
+    const size_t smem = kDiskSmem + (use_hist ? sizeof(uint32_t) * a.ix.P : 0);
+    auto kern = k_disk_pass1<OUT>;
+    const cudaError_t e = smem_opt_in(kern, kDiskSmem + sizeof(uint32_t) * kHistMax, done);
+    if (e != cudaSuccess)
+        return e;
+    const uint32_t nblk = uint32_t((nchunks + kWarps - 1) / kWarps);
+    kern<<<persistent_grid(kern, kThreads, smem, nblk), kThreads, smem, s>>>(a, pend, uint32_t(nchunks), use_hist);
+    return cudaGetLastError();
 }
 
 // Pass 3 of the join with warp chunks: every warp writes the pairs of its
@@ -1779,7 +1992,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_wemit(const __grid_constant__ J
             unsigned long long o = has ? s_o[k0 + lane] : 0ull;
             const int2 p = has ? a.pts[base + loc] : make_int2(0, 0);
             const uint32_t pid = a.pid0 + (uint32_t)(base + loc);
-            const uint32_t w = has ? resolve(a.ix, (uint32_t)p.x, (uint32_t)p.y, keep) : 0u;
+            const uint32_t w = has ? resolve<KIND>(a.ix, (uint32_t)p.x, (uint32_t)p.y, keep) : 0u;
             uint32_t t = 0, e = 0;
             walk_list_wave<FP32, KIND>(a.ix, (w >> 30) >= kCellList, w & kPayloadMask, p.x, p.y, t, e, keep, s_par,
                                  [&](uint32_t q) {
@@ -1811,10 +2024,15 @@ __global__ void __launch_bounds__(kThreads, 3) k_wemit(const __grid_constant__ J
 // With SELF (small tables, a warp per chunk) chunk_off holds the chunks' totals,
 // not their offsets: every CTA sums the totals before its first chunk itself
 // (at most 8 B x kSmallChunks from L2), which saves the scan's launch.
-constexpr uint32_t kEmitStage = 320; // pairs; a full chunk's lie nine apart per lane of eight (no bank conflict)
+// Pairs of the stage; a full chunk's lie nine apart per lane of eight (no bank
+// conflict).  Disks, whose output is sparse, have a small one.
+template <int KIND>
+constexpr uint32_t kEmitStage = KIND == kDisk ? 96 : 320;
 constexpr uint32_t kEmitQueue = kWChunk + 32; // a chunk's rows and a partial round
-constexpr size_t kEmit16Warp = (kEmitStage * 8 + size_t(kEmitQueue) * 12 + kWaveWords * 4 + 15) & ~size_t(15);
-constexpr size_t kEmit16Smem = kWarps * kEmit16Warp; // 49 KB: four CTAs per SM
+template <int KIND>
+constexpr size_t kEmit16Warp = (kEmitStage<KIND> * 8 + size_t(kEmitQueue) * 12 + kWaveWords * 4 + 15) & ~size_t(15);
+template <int KIND>
+constexpr size_t kEmit16Smem = kWarps * kEmit16Warp<KIND>; // 49 KB (disks 35): four CTAs per SM
 static_assert(kWItems == 8, "a lane's rows: one 16-byte load of 2-byte results");
 
 template <bool FP32, bool SELF, int KIND>
@@ -1825,8 +2043,8 @@ __global__ void __launch_bounds__(kThreads, KIND == kNear ? 3 : 4) k_wemit16(con
     __shared__ unsigned long long s_before[SELF ? kWarps : 1];
     extern __shared__ __align__(16) unsigned char s_raw[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint2 *s_st = reinterpret_cast<uint2 *>(s_raw + warp * kEmit16Warp);
-    unsigned long long *s_o = reinterpret_cast<unsigned long long *>(s_st + kEmitStage); // offset | count << 48
+    uint2 *s_st = reinterpret_cast<uint2 *>(s_raw + warp * kEmit16Warp<KIND>);
+    unsigned long long *s_o = reinterpret_cast<unsigned long long *>(s_st + kEmitStage<KIND>); // offset | count << 48
     uint32_t *s_q = reinterpret_cast<uint32_t *>(s_o + kEmitQueue); // rows of the table
     uint32_t *s_par = s_q + kEmitQueue;
     const uint64_t keep = policy_evict_last();
@@ -1887,7 +2105,7 @@ __global__ void __launch_bounds__(kThreads, KIND == kNear ? 3 : 4) k_wemit16(con
         const bool walk = has && !packed; // the whole warp walks these points' lists together
         if (__any_sync(kFull, walk)) {
             const int2 p = walk ? a.pts[row] : make_int2(0, 0);
-            const uint32_t w = walk ? resolve(a.ix, (uint32_t)p.x, (uint32_t)p.y, keep) : 0u;
+            const uint32_t w = walk ? resolve<KIND>(a.ix, (uint32_t)p.x, (uint32_t)p.y, keep) : 0u;
             uint32_t t = 0, e = 0;
             walk_list_wave<FP32, KIND>(a.ix, (w >> 30) >= kCellList, w & kPayloadMask, p.x, p.y, t, e, keep, s_par,
                                        [&](uint32_t q) {
@@ -1925,7 +2143,7 @@ __global__ void __launch_bounds__(kThreads, KIND == kNear ? 3 : 4) k_wemit16(con
                 if ((m >> k) & 1u) // the count of a row in several polygons (never 0xffff: P is below it)
                     mine += r(k) - 1u;
         }
-        if (!any_m && __all_sync(kFull, mine == 8)) { // every row in one polygon
+        if (kEmitStage<KIND> >= 9 * 32 && !any_m && __all_sync(kFull, mine == 8)) { // every row in one polygon
             uint2 *d = s_st + 9 * lane;
 #pragma unroll
             for (int k = 0; k < 8; ++k)
@@ -1957,7 +2175,7 @@ __global__ void __launch_bounds__(kThreads, KIND == kNear ? 3 : 4) k_wemit16(con
         if (tot == 0)
             continue;
         uint32_t at = inc - mine;
-        const bool staged = tot <= kEmitStage;
+        const bool staged = tot <= kEmitStage<KIND>;
         if (!any_m && staged) {
 #pragma unroll
             for (int k = 0; k < 8; ++k)
@@ -2457,20 +2675,6 @@ __global__ void __launch_bounds__(kPlainThreads) k_plain_write(JoinLaunch a, con
     }
 }
 
-// Opt a kernel in to the shared memory it needs (once per device).
-template <class K>
-cudaError_t smem_opt_in(K kernel, size_t bytes, bool (&done)[64])
-{
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 64 && done[dev])
-        return cudaSuccess;
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
-    if (e == cudaSuccess && dev < 64)
-        done[dev] = true;
-    return e;
-}
-
 template <bool FP32, bool CLUSTERED>
 cudaError_t launch_warp_kernel(const JoinLaunch &a, int use_hist, cudaStream_t s)
 {
@@ -2635,11 +2839,11 @@ cudaError_t launch_pass1_as(const JoinLaunch &a, uint32_t *pend, cudaStream_t s,
     if (a.ix.use_sum) {
         // beside the summary, shared memory holds one chunk buffer per warp
         // at most, too shallow to hide a bulk copy: L2 prefetches instead
-        e = launch(k_resolve_sum<OUT>, kResolveSumThreads,
+        e = launch(k_resolve_sum<OUT, KIND == kDisk>, kResolveSumThreads,
                    resolve_smem_head(WS, true, a.ix.sg, false), resolve_smem_head(WS, true, kSumLog2, false), done_r[2]);
     } else {
         const size_t head = kTmaPoints ? resolve_smem_head(kWarps, false, 0, true) : 0;
-        e = launch(k_resolve<kThreads, kTmaPoints, OUT>, kThreads, head, head, done_r[3]);
+        e = launch(k_resolve<kThreads, kTmaPoints, OUT, KIND == kDisk>, kThreads, head, head, done_r[3]);
     }
     if (e != cudaSuccess) // pass 1b must not run on what an earlier call left in the scratch
         return e;
@@ -2663,12 +2867,23 @@ cudaError_t with_switches(const JoinLaunch &a, F f)
 
 cudaError_t launch_pass1(const JoinLaunch &a, uint32_t *pend, cudaStream_t s, cudaEvent_t mid, bool count_only)
 {
-    return with_switches(a, [&](auto fp32, auto kind) {
+    return with_switches(a, [&](auto fp32, auto kind) -> cudaError_t {
         constexpr bool F = decltype(fp32)::value;
         constexpr int N = decltype(kind)::value;
-        return count_only ? launch_pass1_as<F, kOutCount, N>(a, pend, s, mid)
-               : a.narrow ? launch_pass1_as<F, kOut16, N>(a, pend, s, mid)
-                          : launch_pass1_as<F, kOut32, N>(a, pend, s, mid);
+        if constexpr (N == kDisk) {
+            if (!count_only && a.ix.P <= kDiskSplit)
+                return launch_pass1_as<F, kOut16, N>(a, pend, s, mid);
+            const cudaError_t e = count_only ? launch_disk_pass1<kOutCount>(a, nullptr, s)
+                                  : a.narrow ? launch_disk_pass1<kOut16>(a, pend, s)
+                                             : launch_disk_pass1<kOut32>(a, pend, s);
+            if (mid)
+                cudaEventRecord(mid, s);
+            return e;
+        } else {
+            return count_only ? launch_pass1_as<F, kOutCount, N>(a, pend, s, mid)
+                   : a.narrow ? launch_pass1_as<F, kOut16, N>(a, pend, s, mid)
+                              : launch_pass1_as<F, kOut32, N>(a, pend, s, mid);
+        }
     });
 }
 
@@ -2903,11 +3118,25 @@ __global__ void k_dbuild_sort(uint32_t ncell, const uint32_t *cell_word, uint32_
     }
 }
 
+// Cover bitmap: a bit per block of cells that holds a non-empty cell.
+__global__ void k_dbuild_cover(uint32_t ncell, int g, int cg, const uint32_t *cell_word, uint32_t *cover)
+{
+    for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < ncell; c += gridDim.x * blockDim.x) {
+        if (!cell_word[c])
+            continue;
+        const uint32_t cx = c & ((1u << g) - 1), cy = c >> g;
+        const uint32_t b = ((cy >> (g - cg)) << cg) | (cx >> (g - cg));
+        atomicOr(cover + (b >> 5), 1u << (b & 31));
+    }
+}
+
 int build_disk_index_device(const int4 *disks_host, uint32_t Q, int g, DiskIndexDev &out, cudaError_t &cerr)
 {
     out = DiskIndexDev{};
     cerr = cudaSuccess;
     const uint32_t ncell = 1u << (2 * g);
+    const int cg = g < kCoverLog2 ? g : kCoverLog2;
+    const size_t cover_words = ((size_t(1) << (2 * cg)) / 32) > 0 ? ((size_t(1) << (2 * cg)) / 32) : 1;
     const size_t nd = Q ? Q : 1;
     const uint64_t nparts = scan_partials(ncell > nd ? ncell : nd) + 2;
     // temporaries: disks | per-disk record counts | totals | scan partials |
@@ -2967,9 +3196,9 @@ int build_disk_index_device(const int4 *disks_host, uint32_t Q, int g, DiskIndex
     const uint64_t E = 1 + T;
     if (E > kPayloadMask)
         return done(1, cudaSuccess);
-    // the index's own allocation: cells | entries | disks, as the host path lays it out
-    const size_t b_cell = size_t(ncell) * 4, b_ent = size_t(E) * 4, b_disk = nd * sizeof(int4);
-    out.bytes = up(b_cell) + up(b_ent) + up(b_disk);
+    // the index's own allocation: cells | entries | disks | cover, as the host path lays it out
+    const size_t b_cell = size_t(ncell) * 4, b_ent = size_t(E) * 4, b_disk = nd * sizeof(int4), b_cover = cover_words * 4;
+    out.bytes = up(b_cell) + up(b_ent) + up(b_disk) + up(b_cover);
     if ((e = cudaMalloc(&out.mem, out.bytes)) != cudaSuccess) {
         out.mem = nullptr;
         return done(2, e);
@@ -2978,7 +3207,9 @@ int build_disk_index_device(const int4 *disks_host, uint32_t Q, int g, DiskIndex
     out.cell = reinterpret_cast<uint32_t *>(m);
     out.ent = reinterpret_cast<uint32_t *>(m + up(b_cell));
     out.disk = reinterpret_cast<int4 *>(m + up(b_cell) + up(b_ent));
+    out.cover = reinterpret_cast<uint32_t *>(m + up(b_cell) + up(b_ent) + up(b_disk));
     if ((e = cudaMemset(out.cell, 0, b_cell)) != cudaSuccess || (e = cudaMemset(out.ent, 0, b_ent)) != cudaSuccess ||
+        (e = cudaMemset(out.cover, 0, b_cover)) != cudaSuccess ||
         (e = cudaMemcpy(out.disk, d_disk, b_disk, cudaMemcpyDeviceToDevice)) != cudaSuccess)
         return done(2, e);
     k_dbuild_cells<<<cblocks, 256>>>(ncell, cell_cnt, cell_bnd, words, out.cell, out.ent);
@@ -2990,6 +3221,7 @@ int build_disk_index_device(const int4 *disks_host, uint32_t Q, int g, DiskIndex
                                            out.cell, out.ent);
         k_dbuild_sort<<<cblocks, 256>>>(ncell, out.cell, out.ent);
     }
+    k_dbuild_cover<<<cblocks, 256>>>(ncell, g, cg, out.cell, out.cover);
     if ((e = cudaGetLastError()) != cudaSuccess || (e = cudaDeviceSynchronize()) != cudaSuccess)
         return done(2, e);
     out.n_ent = E;
@@ -3123,12 +3355,12 @@ cudaError_t launch_join_emit(const JoinLaunch &a, cudaStream_t s, const uint32_t
         constexpr int N = decltype(kind)::value;
         auto kn = k_wemit16<F, false, N>;
         auto kw = k_wemit<F, N>;
-        const cudaError_t e = a.narrow ? smem_opt_in(kn, kEmit16Smem, done[F + 2 * N])
+        const cudaError_t e = a.narrow ? smem_opt_in(kn, kEmit16Smem<N>, done[F + 2 * N])
                                        : smem_opt_in(kw, kEmitSmem, done[6 + F + 2 * N]);
         if (e != cudaSuccess)
             return e;
         if (a.narrow)
-            kn<<<persistent_grid(kn, kThreads, kEmit16Smem, nblk), kThreads, kEmit16Smem, s>>>(a, a.tile_tot, nchunks, pend);
+            kn<<<persistent_grid(kn, kThreads, kEmit16Smem<N>, nblk), kThreads, kEmit16Smem<N>, s>>>(a, a.tile_tot, nchunks, pend);
         else
             kw<<<persistent_grid(kw, kThreads, kEmitSmem, nblk), kThreads, kEmitSmem, s>>>(a, a.tile_tot, nchunks);
         return cudaGetLastError();
@@ -3145,15 +3377,20 @@ static cudaError_t launch_small(const JoinLaunch &a, uint32_t *pend, cudaStream_
     const uint32_t nchunks = uint32_t((a.n + kWChunk - 1) / kWChunk), nblk = (nchunks + kWarps - 1) / kWarps;
     if (ev)
         cudaEventRecord(ev[0], s);
-    k_small<FP32, kOut16, KIND><<<nblk, kThreads, 0, s>>>(a, pend, nchunks, a.ix.P <= kSmallHist ? 1 : 0);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = cudaSuccess;
+    if (KIND == kDisk && a.ix.P > kDiskSplit) {
+        e = launch_disk_pass1<kOut16>(a, pend, s);
+    } else {
+        k_small<FP32, kOut16, KIND><<<nblk, kThreads, 0, s>>>(a, pend, nchunks, a.ix.P <= kSmallHist ? 1 : 0);
+        e = cudaGetLastError();
+    }
     if (e == cudaSuccess)
-        e = smem_opt_in(k_wemit16<FP32, true, KIND>, kEmit16Smem, done);
+        e = smem_opt_in(k_wemit16<FP32, true, KIND>, kEmit16Smem<KIND>, done);
     if (e != cudaSuccess)
         return e;
     for (int k = 1; ev && k < 4; ++k)
         cudaEventRecord(ev[k], s);
-    k_wemit16<FP32, true, KIND><<<nblk, kThreads, kEmit16Smem, s>>>(a, a.tile_tot, nchunks, pend);
+    k_wemit16<FP32, true, KIND><<<nblk, kThreads, kEmit16Smem<KIND>, s>>>(a, a.tile_tot, nchunks, pend);
     return cudaGetLastError();
 }
 
@@ -3606,7 +3843,7 @@ cudaError_t launch_join(const JoinLaunch &a, void *scratch, cudaStream_t s, cuda
 
 bool use_directory(const JoinLaunch &a)
 {
-    return a.clustered && a.cell_end && a.cluster_log2 >= a.ix.gc && a.cluster_log2 <= 13;
+    return a.clustered && a.cell_end && a.cluster_log2 >= a.ix.gc && a.cluster_log2 <= 13 && !a.near.any();
 }
 
 // A table in row order is counted by the join's pass 1 with nothing kept but the
@@ -3620,7 +3857,7 @@ bool use_directory(const JoinLaunch &a)
 constexpr uint64_t kSplitCountMin = uint64_t(1) << 21;
 bool use_split_count(const JoinLaunch &a)
 {
-    return a.n > kSplitCountMin && (a.near.any() || (!a.clustered && a.ix.use_sum));
+    return a.n > kSplitCountMin && !a.near.disk && (a.near.rad || (!a.clustered && a.ix.use_sum));
 }
 
 static size_t split_count_bytes(uint64_t n)
@@ -3630,9 +3867,9 @@ static size_t split_count_bytes(uint64_t n)
 
 size_t aggregate_scratch_bytes(const JoinLaunch &a)
 {
-    return use_directory(a) && !a.near.any() ? size_t((a.n + kWChunk - 1) / kWChunk) * kWItems * 4
-           : !a.clustered || a.near.any() ? split_count_bytes(a.n)
-                                           : 0;
+    return use_directory(a)                 ? size_t((a.n + kWChunk - 1) / kWChunk) * kWItems * 4
+           : !a.clustered || a.near.rad ? split_count_bytes(a.n)
+                                        : 0;
 }
 
 cudaError_t launch_aggregate(const JoinLaunch &a, void *scratch, cudaStream_t s, cudaEvent_t *ev)
@@ -3653,6 +3890,8 @@ cudaError_t launch_aggregate(const JoinLaunch &a, void *scratch, cudaStream_t s,
             cudaEventRecord(ev[1], s);
         return e;
     }
+    if (a.near.disk)
+        return launch_pass1(a, nullptr, s, nullptr, true);
     if (a.near.any()) { // few points, or no scratch to have: one launch that keeps nothing
         const uint64_t nchunks = (a.n + kWChunk - 1) / kWChunk;
         if (a.n >= (1ull << 32))
@@ -3660,7 +3899,7 @@ cudaError_t launch_aggregate(const JoinLaunch &a, void *scratch, cudaStream_t s,
         const unsigned nblk = unsigned((nchunks + kWarps - 1) / kWarps);
         const int hist = a.ix.P <= kSmallHist ? 1 : 0;
         return with_switches(a, [&](auto fp32, auto kind) {
-            if constexpr (decltype(kind)::value != kPoly)
+            if constexpr (decltype(kind)::value == kNear)
                 k_small<decltype(fp32)::value, kOutCount, decltype(kind)::value>
                     <<<nblk, kThreads, 0, s>>>(a, nullptr, uint32_t(nchunks), hist);
             return cudaGetLastError();
@@ -4265,22 +4504,12 @@ int build_near_index_device(const IndexView &in, const uint32_t *cell_off, const
     }
 }
 
-// A disk index's lists hang from its coarse words directly: kind kCellCoarseList.
-__global__ void __launch_bounds__(256) k_disk_words(uint32_t ncell, uint32_t *cell)
+cudaError_t disk_summary(const uint32_t *cell, int g, uint16_t *sum, unsigned long long *n, double *sum_resolved)
 {
-    for (uint32_t c = blockIdx.x * 256 + threadIdx.x; c < ncell; c += gridDim.x * 256)
-        if ((cell[c] >> 30) == kCellList)
-            cell[c] |= kCellCoarseList << 30;
-}
-
-cudaError_t prepare_disk_words(uint32_t *cell, int g, uint16_t *sum, unsigned long long *n, double *sum_resolved)
-{
-    const uint32_t ncell = 1u << (2 * g);
     const int sg = std::min(g, kSumLog2);
     unsigned long long h = 0;
     cudaError_t e = cudaMemset(n, 0, 8);
     if (e == cudaSuccess) {
-        k_disk_words<<<std::min<uint32_t>((ncell + 255) / 256, uint32_t(device_sm_count()) * 32), 256>>>(ncell, cell);
         k_near_sum<<<((1u << (2 * sg)) + 255) / 256, 256>>>(g, sg, cell, sum, n, nullptr, nullptr);
         e = cudaGetLastError();
     }

@@ -50,9 +50,8 @@ constexpr uint32_t kLocalEdge = 0x80000000u;
 // cell (kEntBoundary), not a crossing list.  kEntCross: the polygon's boundary
 // may also cross the cell, so that a point far from those edges still asks the
 // polygons' own index `in`.
-// A disk index is one too: its words are those of build_disk_index with
-// kCellCoarseList for lists, whose offsets point into dent (n, then n words disk <<
-// 1 | boundary); disks as (cx, cy, r, 0).
+// A disk index is one too, of one level: the words of build_disk_index, whose lists
+// are in dent (n, then n words disk << 1 | boundary); disks as (cx, cy, r, 0).
 struct NearView {
     const int32_t *rad; // P radii, each in [0, 2^30); null: not a buffered index
     IndexView in;
@@ -70,26 +69,25 @@ constexpr uint32_t kSumEmpty = 0xfffeu;
 
 // Device build of the disk index of Q disks (host array of (cx, cy, r, 0),
 // already checked) on a 2^g grid: the same cell words and entries as the host
-// build (build_disk_index), in one new device allocation laid out as the host path
-// lays it out (cells | entries | disks, each part 256-byte aligned); the caller owns
-// out.mem.  Runs on the
+// build (build_disk_index) and the same cover bitmap, in one new device
+// allocation laid out as the host path lays it out (cells | entries | disks |
+// cover, each part 256-byte aligned); the caller owns out.mem.  Runs on the
 // legacy default stream and synchronises the device.  Returns 0, 1 when the
 // entries would not fit 30-bit offsets (use a coarser grid), or 2 on a CUDA
 // error (in cerr).
 struct DiskIndexDev {
     void *mem;
     size_t bytes;
-    uint32_t *cell, *ent;
+    uint32_t *cell, *ent, *cover;
     int4 *disk;
     uint64_t n_ent, n_inside, n_boundary;
 };
 int build_disk_index_device(const int4 *disks_host, uint32_t Q, int g, DiskIndexDev &out, cudaError_t &cerr);
 
-// Turns the lists of a disk index's words (2^g grid, in place) into
-// kCellCoarseList, and writes their block summary (4^min(g, kSumLog2) words) and
+// The block summary of a disk index's words (2^g grid; 4^min(g, kSumLog2) words) and
 // the fraction of it that is not mixed (counted in *n).  Legacy default stream,
 // synchronises.
-cudaError_t prepare_disk_words(uint32_t *cell, int g, uint16_t *sum, unsigned long long *n, double *sum_resolved);
+cudaError_t disk_summary(const uint32_t *cell, int g, uint16_t *sum, unsigned long long *n, double *sum_resolved);
 
 // Device status word bits (ORed into the ctx's persistent error word).
 constexpr unsigned kErrTimeout = 1u;   // a bounded wait (for a bulk copy) gave up
