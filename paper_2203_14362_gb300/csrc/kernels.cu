@@ -1407,7 +1407,7 @@ constexpr uint32_t kSmallHist = 2048;
 // of a mixed coarse cell: rows that its fine cell resolves are counted here.
 template <bool FP32, int OUT, int KIND, bool ALL>
 __global__ void __launch_bounds__(kThreads, KIND == kNear ? 3 : kWalkMinBlocks) k_walk(const __grid_constant__ JoinLaunch a, uint32_t *pend,
-                                                                   uint32_t nwords)
+                                                                   uint32_t nwords, int gl)
 {
     static_assert(!ALL || OUT == kOutCount, "ALL keeps nothing per row");
     __shared__ uint32_t s_qa[kWarps * kWalkQueue];
@@ -1518,16 +1518,19 @@ __global__ void __launch_bounds__(kThreads, KIND == kNear ? 3 : kWalkMinBlocks) 
         while (ln >= 32)
             walk(32);
     };
-    // this warp's words: every nw-th group of 32, so that a run of marked rows (a
-    // clustered table) is shared out; a lane per word, BW groups loaded ahead
+    // this warp's words: every nw-th group of 2^gl (at most 32), so that a run of marked
+    // rows (a clustered table) is shared out; a lane per word, BW groups loaded ahead
     constexpr int BW = 4;
     const uint64_t nw = (uint64_t)gridDim.x * kWarps, g0 = (uint64_t)blockIdx.x * kWarps + warp;
-    auto load = [&](uint64_t g) { return g * 32 + lane < nwords ? __ldcs(pend + g * 32 + lane) : 0u; };
+    auto load = [&](uint64_t g) {
+        const uint64_t i = (g << gl) + lane;
+        return lane < 1 << gl && i < nwords ? __ldcs(pend + i) : 0u;
+    };
     uint32_t nxt[BW];
 #pragma unroll
     for (int k = 0; k < BW; ++k)
         nxt[k] = load(g0 + k * nw);
-    for (uint64_t g = g0; g * 32 < nwords; g += BW * nw) {
+    for (uint64_t g = g0; (g << gl) < nwords; g += BW * nw) {
         uint32_t cur[BW];
 #pragma unroll
         for (int k = 0; k < BW; ++k) {
@@ -1536,13 +1539,30 @@ __global__ void __launch_bounds__(kThreads, KIND == kNear ? 3 : kWalkMinBlocks) 
         }
 #pragma unroll 1
         for (int k = 0; k < BW; ++k) { // not unrolled: one copy of the walk
-            const uint64_t wi = (g + k * nw) * 32 + lane;
+            const uint64_t wi = ((g + k * nw) << gl) + lane;
             uint32_t m = cur[0];
 #pragma unroll
             for (int t = 0; t + 1 < BW; ++t)
                 cur[t] = cur[t + 1];
-            if (ALL)
+            if (ALL) {
+                // marked rows come in runs: a lane per row of a word, so that a round's
+                // points, cells and lists are mostly the same (a row of each lane's word at
+                // a time: 500M points x 40000 cells 1389 us, now 1219)
                 n_pts += __popc(m);
+                for (uint32_t todo = __ballot_sync(kFull, m != 0); todo; todo &= todo - 1) {
+                    const int src = __ffs(todo) - 1;
+                    const uint32_t word = __shfl_sync(kFull, m, src);
+                    const uint32_t row = (uint32_t)((wi - lane + src) * 32) + lane;
+                    if ((word >> lane) & 1u) {
+                        s_q[qn + __popc(word & lanemask_lt())] = row;
+                        prefetch_l2(a.pts + row);
+                    }
+                    qn += __popc(word);
+                    if (qn >= 32 * B)
+                        take(32 * B);
+                }
+                continue;
+            }
             while (__any_sync(kFull, m != 0)) {
                 const bool has = m != 0;
                 const uint32_t b = (uint32_t)__ffs(m) - 1u;
@@ -1589,6 +1609,14 @@ cudaError_t smem_opt_in(K kernel, size_t bytes, bool (&done)[64])
 template <bool FP32, int OUT, int KIND, bool ALL = false>
 cudaError_t launch_walk(const JoinLaunch &a, uint32_t *pend, cudaStream_t s)
 {
+    // Groups of fewer words where the marked rows lie close together: a warp goes through
+    // its own one round after the other.  Over a clustered table (ALL) they come in runs,
+    // and a warp per 1024 rows left most warps without any: 32 groups a warp where the
+    // table has the words (300k points x 120 overlapping queries 310 -> 105 us, 20M
+    // 1437 -> 463; 20M x 300 cells 114 -> 114; 500M x 40000 cells takes whole groups).
+    // With wide results, one (300k points x 70000 buffered squares 88 -> 62 us, 1.5M 170 ->
+    // 146).  Rows of narrow results are spread thin, and a smaller group would only
+    // leave rounds part empty (1.5M x 300 cells 35 -> 37).
     // a warp per group of 32 words, shared out by stride over what the chip holds
     // at once (1M points: 61 warps of 512 words took 20.3 us, 977 of 32 take 7.5;
     // 100M x 2000 cells: 1.8 waves 87 us, one 74), or over up to six times as many
@@ -1596,10 +1624,14 @@ cudaError_t launch_walk(const JoinLaunch &a, uint32_t *pend, cudaStream_t s)
     // queries: one wave 3.15 ms, six 2.95)
     const uint64_t nwords = (a.n + kWChunk - 1) / kWChunk * kWItems;
     auto kern = k_walk<FP32, OUT, KIND, ALL>;
-    const uint32_t nblk = uint32_t((nwords + 32 * kWarps - 1) / (32 * kWarps));
-    const uint32_t wave = (uint32_t)persistent_grid(kern, kThreads, 0, nblk);
+    const uint32_t wave = (uint32_t)persistent_grid(kern, kThreads, 0, UINT32_MAX);
+    int gl = 5;
+    if (ALL || OUT == kOut32)
+        while (gl && (nwords >> gl) < (uint64_t)wave * kWarps * (ALL ? 32 : 1))
+            --gl;
+    const uint32_t nblk = uint32_t((nwords + (kWarps << gl) - 1) / (kWarps << gl));
     const uint32_t waves = std::min(std::max(nblk / (wave * kWalkGroups), 1u), 6u);
-    kern<<<std::min(nblk, wave * waves), kThreads, 0, s>>>(a, pend, uint32_t(nwords));
+    kern<<<std::min(nblk, wave * waves), kThreads, 0, s>>>(a, pend, uint32_t(nwords), gl);
     return cudaGetLastError();
 }
 
