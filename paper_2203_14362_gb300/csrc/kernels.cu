@@ -86,11 +86,12 @@ __device__ __forceinline__ uint64_t policy_evict_last()
     asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
     return p;
 }
-// Pass 1a of polygons reads index words past L1: once per point, at random, 32 lines a
-// warp (100M points x 2000 cells 571 -> 549 us, count x 5000 cells 497 -> 467).
-// Everywhere else they take an L1 line.  Disk lists are read word after word, and
-// where points crowd into few cells their words are in L1: past it, 20M points, 90 %
-// of them in 256 cells of 64 disks, joined in 586 us instead of 257.
+// The join's passes read the index words of polygons past L1: once per point, at
+// random, 32 lines a warp (100M points x 2000 cells 571 -> 549 us, count x 5000 cells
+// 497 -> 467, 20M x 1024 queries 703 -> 673).  The others take an L1 line: disk lists
+// are read word after word, rows of a clustered table share words, and where points
+// crowd into few cells their words are in L1 (past it, 20M points, 90 % of them in 256
+// cells of 64 disks, joined in 586 us instead of 257).
 template <bool L1 = true>
 __device__ __forceinline__ uint32_t ld_idx(const uint32_t *p, uint64_t pol)
 {
@@ -295,11 +296,11 @@ constexpr int kPoly = 0, kNear = 1, kDisk = 2;
 
 // Resolved word of an in-box point: kind 0 none, 1 one INSIDE polygon, 2 list (a disk
 // index has one level, whose words are that already).
-template <int KIND = kPoly>
+template <int KIND = kPoly, bool L1 = true>
 __device__ __forceinline__ uint32_t resolve(const IndexView &ix, uint32_t px, uint32_t py, uint64_t pol)
 {
-    const uint32_t w = coarse_word(ix, px, py, pol);
-    return KIND != kDisk && (w >> 30) == kCellSub ? fine_word(ix, w, px, py, pol) : w;
+    const uint32_t w = coarse_word<L1>(ix, px, py, pol);
+    return KIND != kDisk && (w >> 30) == kCellSub ? fine_word<L1>(ix, w, px, py, pol) : w;
 }
 
 // One edge's contribution to the crossing parity of (px, py).
@@ -1407,9 +1408,11 @@ constexpr uint32_t kSmallHist = 2048;
 // of a mixed coarse cell: rows that its fine cell resolves are counted here.
 template <bool FP32, int OUT, int KIND, bool ALL>
 __global__ void __launch_bounds__(kThreads, KIND == kNear ? 3 : kWalkMinBlocks) k_walk(const __grid_constant__ JoinLaunch a, uint32_t *pend,
-                                                                   uint32_t nwords, int gl)
+                                                                   uint32_t nwords, int group_log2)
 {
     static_assert(!ALL || OUT == kOutCount, "ALL keeps nothing per row");
+    constexpr bool L1 = ALL || KIND == kDisk; // index words
+    const int gl = ALL || OUT == kOut32 ? group_log2 : 5; // see launch_walk
     __shared__ uint32_t s_qa[kWarps * kWalkQueue];
     __shared__ uint4 s_la[kWarps * kWalkQueue];
     __shared__ uint32_t s_pa[kWarps * kWaveWords];
@@ -1490,12 +1493,12 @@ __global__ void __launch_bounds__(kThreads, KIND == kNear ? 3 : kWalkMinBlocks) 
 #pragma unroll
         for (int u = 0; u < B; ++u)
             w[u] = OUT == kOut32 ? (kCellList << 30) | __ldcg(a.res + row[u])
-                                 : coarse_word(ix, (uint32_t)p[u].x, (uint32_t)p[u].y, keep);
+                                 : coarse_word<L1>(ix, (uint32_t)p[u].x, (uint32_t)p[u].y, keep);
         if (OUT != kOut32) {
 #pragma unroll
             for (int u = 0; u < B; ++u)
                 if (KIND != kDisk && (w[u] >> 30) == kCellSub)
-                    w[u] = fine_word(ix, w[u], (uint32_t)p[u].x, (uint32_t)p[u].y, keep);
+                    w[u] = fine_word<L1>(ix, w[u], (uint32_t)p[u].x, (uint32_t)p[u].y, keep);
         }
 #pragma unroll
         for (int u = 0; u < B; ++u) {
@@ -1688,12 +1691,12 @@ __global__ void __launch_bounds__(kThreads, KIND == kNear ? 3 : 4) k_small(const
         for (int j = 0; j < kWItems; ++j) {
             w[j] = 0u;
             if ((uint32_t)(p[j].x | p[j].y) < kBox)
-                w[j] = coarse_word(ix, (uint32_t)p[j].x, (uint32_t)p[j].y, keep);
+                w[j] = coarse_word<KIND == kDisk>(ix, (uint32_t)p[j].x, (uint32_t)p[j].y, keep);
         }
 #pragma unroll
         for (int j = 0; j < kWItems; ++j)
             if (KIND != kDisk && (w[j] >> 30) == kCellSub)
-                w[j] = fine_word(ix, w[j], (uint32_t)p[j].x, (uint32_t)p[j].y, keep);
+                w[j] = fine_word<false>(ix, w[j], (uint32_t)p[j].x, (uint32_t)p[j].y, keep);
         if (lane < kWItems)
             s_m[lane] = 0u;
         uint32_t qn = 0;
@@ -2024,7 +2027,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_wemit(const __grid_constant__ J
             unsigned long long o = has ? s_o[k0 + lane] : 0ull;
             const int2 p = has ? a.pts[base + loc] : make_int2(0, 0);
             const uint32_t pid = a.pid0 + (uint32_t)(base + loc);
-            const uint32_t w = has ? resolve<KIND>(a.ix, (uint32_t)p.x, (uint32_t)p.y, keep) : 0u;
+            const uint32_t w = has ? resolve<KIND, KIND == kDisk>(a.ix, (uint32_t)p.x, (uint32_t)p.y, keep) : 0u;
             uint32_t t = 0, e = 0;
             walk_list_wave<FP32, KIND>(a.ix, (w >> 30) >= kCellList, w & kPayloadMask, p.x, p.y, t, e, keep, s_par,
                                  [&](uint32_t q) {
@@ -2137,7 +2140,7 @@ __global__ void __launch_bounds__(kThreads, KIND == kNear ? 3 : 4) k_wemit16(con
         const bool walk = has && !packed; // the whole warp walks these points' lists together
         if (__any_sync(kFull, walk)) {
             const int2 p = walk ? a.pts[row] : make_int2(0, 0);
-            const uint32_t w = walk ? resolve<KIND>(a.ix, (uint32_t)p.x, (uint32_t)p.y, keep) : 0u;
+            const uint32_t w = walk ? resolve<KIND, KIND == kDisk>(a.ix, (uint32_t)p.x, (uint32_t)p.y, keep) : 0u;
             uint32_t t = 0, e = 0;
             walk_list_wave<FP32, KIND>(a.ix, (w >> 30) >= kCellList, w & kPayloadMask, p.x, p.y, t, e, keep, s_par,
                                        [&](uint32_t q) {
