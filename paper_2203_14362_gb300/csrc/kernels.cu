@@ -1755,18 +1755,18 @@ __global__ void __launch_bounds__(kThreads, KIND == kNear ? 3 : 4) k_small(const
     add_stats(a.stats, lane == 0 ? npts : 0u, n_tests, n_esc, total);
 }
 
-// Pass 1 of a disk index in one kernel: counts, and joins of more than kDiskSplit
-// disks.  Disk lists are short and their tests cheap: a lane walks its own list as soon
-// as a round of 32 list points is queued (across chunks), with the point at hand.  A
-// point in a block that no disk reaches leaves by the cover bitmap, in shared memory (8
-// KB where the summary takes 128, so four CTAs per SM keep 32 warps).  Counts in shared
-// memory up to kHistMax disks.
-// Counts, against passes 1a and 1b (which re-read their rows): 20M points x 64 / 1024 /
-// 4096 disks 52 / 71 / 82 us against 56 / 68 / 107, over a clustered table 50 / 59 /
-// 73 against 61 / 96 / 158, 300k x 1024 12.1 against 14.5.  Joins: 100M x 1024 disks
-// 500 us against 433, 20M x 1024 125 against 117; 20M x 4096, which k_walk counts in
-// global memory, 140 against 185, x 20000 159 against 198, and with 90 % of 20M points
-// in 512 of 4096 disks, where counters take millions of hits each, 6.8 ms against 59.6.
+// Pass 1 of a disk index in one kernel: joins of more than kDiskSplit disks, and the
+// counts but those of large tables in row order (use_split_count).  Disk lists are short
+// and their tests cheap: a lane walks its own list as soon as a round of 32 list points
+// is queued (across chunks), with the point at hand.  A point in a block that no disk
+// reaches leaves by the cover bitmap, in shared memory (8 KB where the summary takes 128,
+// so four CTAs per SM keep 32 warps).  Counts in shared memory up to kHistMax disks.
+// Against passes 1a and 1b, which re-read their rows: counts over a clustered table, 20M
+// points x 64 / 1024 / 4096 disks 50 / 59 / 73 us against 61 / 96 / 158, of 300k x 1024
+// 12.1 against 14.5.  Joins: 100M x 1024 disks 500 us against 433, 20M x 1024 125 against
+// 117; 20M x 4096, which k_walk counts in global memory, 140 against 185, x 20000 159
+// against 198, and with 90 % of 20M points in 512 of 4096 disks, where counters take
+// millions of hits each, 6.8 ms against 59.6.
 constexpr uint32_t kDiskSplit = kSmallHist;
 constexpr uint32_t kDiskCoverWords = 1u << (2 * kCoverLog2 - 5);
 constexpr int kDiskQueue = kWChunk + 32; // a chunk's points plus a partial round
@@ -2906,8 +2906,9 @@ cudaError_t launch_pass1(const JoinLaunch &a, uint32_t *pend, cudaStream_t s, cu
         constexpr bool F = decltype(fp32)::value;
         constexpr int N = decltype(kind)::value;
         if constexpr (N == kDisk) {
-            if (!count_only && a.ix.P <= kDiskSplit)
-                return launch_pass1_as<F, kOut16, N>(a, pend, s, mid);
+            if (pend && a.ix.P <= kDiskSplit)
+                return count_only ? launch_pass1_as<F, kOutCount, N>(a, pend, s, mid)
+                                  : launch_pass1_as<F, kOut16, N>(a, pend, s, mid);
             const cudaError_t e = count_only ? launch_disk_pass1<kOutCount>(a, nullptr, s)
                                   : a.narrow ? launch_disk_pass1<kOut16>(a, pend, s)
                                              : launch_disk_pass1<kOut32>(a, pend, s);
@@ -3890,9 +3891,15 @@ bool use_directory(const JoinLaunch &a)
 // 50.9 / 38.1).  Only with the summary: without it (a 40000-cell map, counts in
 // global memory) the one pass is as fast (2021 / 2068 us).
 constexpr uint64_t kSplitCountMin = uint64_t(1) << 21;
+// A disk index's one pass (k_disk_pass1) holds out longer: 2.5M points x 64 / 1024 disks
+// 14.5 / 19.6 us in one, 21.1 / 26.1 in two, 6M 23.0 / 33.2 and 25.8 / 31.4, 20M 54 / 77
+// and 46 / 61, 100M 231 / 333 and 155 / 234.
+constexpr uint64_t kDiskSplitCountMin = uint64_t(1) << 23;
 bool use_split_count(const JoinLaunch &a)
 {
-    return a.n > kSplitCountMin && !a.near.disk && (a.near.rad || (!a.clustered && a.ix.use_sum));
+    if (a.near.disk)
+        return a.n > kDiskSplitCountMin && !a.clustered && a.ix.use_sum && a.ix.P <= kDiskSplit;
+    return a.n > kSplitCountMin && (a.near.rad || (!a.clustered && a.ix.use_sum));
 }
 
 static size_t split_count_bytes(uint64_t n)

@@ -2,7 +2,7 @@
 2049 disks (two kernels or one for joins), 11776 and 11777 (counters in shared or in
 global memory), a table within and above the small-join limit, points crowded into
 many disks, outputs above and below the emit pass's stage, the smallest grids (whose
-cover bitmap is less than a word).  Whole numbers: equal to the oracle's."""
+cover bitmap is less than a word), counts on both sides of 2^23 points.  Whole numbers: equal to the oracle's."""
 import numpy as np
 import pytest
 
@@ -64,5 +64,23 @@ def test_disk_lines(q, n, gl):
             assert eng.select(ph, ih, ids, offs) == want.shape[0]
             order = np.argsort(want[:, 1], kind="stable")
             assert np.array_equal(ids.cpu().numpy().view(np.uint32), want[order, 0])
+    finally:
+        eng.close()
+
+
+@pytest.mark.parametrize("n", [1 << 23, (1 << 23) + 1])
+def test_disk_count_lines(n):  # one pass, or the join's two
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    c, r, pts = case(60, n)
+    want = oracle.disk_join(pts, c, r)[1]
+    eng = spx.Engine(0)
+    try:
+        dpts = torch.from_numpy(pts).cuda()
+        ph = eng.load_points(dpts)
+        ih = eng.build_disk_index(c, r)
+        counts = torch.full((60,), 7, dtype=torch.int64, device="cuda")
+        eng.aggregate(ph, ih, counts)
+        assert np.array_equal(counts.cpu().numpy().view(np.uint64), want)
     finally:
         eng.close()
