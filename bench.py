@@ -45,7 +45,7 @@ RESOLVE_TRAFFIC_BYTES_PER_POINT = {(12, 3): {"k_resolve_sum": (268.1e6 + 29.26e6
                                              "k_wemit16": (43.18e6 + 100.5e6) / 20e6}}
 # The same for the distance join's pass 1a, from one capture of a 20M-point run
 # of the 1024-disk workload at its default grid (g = 12).
-DISK_RESOLVE_TRAFFIC_BYTES_PER_POINT = (164.3e6 + 6.44e6) / 20e6
+DISK_RESOLVE_TRAFFIC_BYTES_PER_POINT = 170.3e6 / 20e6
 SERVE_SEED = 0x2203143620 + 4  # request indexes of the serving measurement
 
 
